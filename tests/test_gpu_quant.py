@@ -89,3 +89,32 @@ def test_quantize_is_stream_ordered(cuda_device):
         img = emb.quantize(emb.EMB_Q8_0, Wd, stream=s)
     s.synchronize()
     assert np.array_equal(img.cpu().numpy(), oracle.quantize(emb.EMB_Q8_0, W))
+
+
+@pytest.mark.parametrize("fmt", [emb.EMB_Q8_0, emb.EMB_Q4_0, emb.EMB_Q6_0])
+@pytest.mark.parametrize("N,K", [(1, 1024), (1, 1056), (31, 32), (257, 32), (37, 8160), (6, 11008)])
+def test_pack_near_ties_and_padding(cuda_device, fmt, N, K):
+    """Weights on the halves between two codes and one fp32 step beside them, in blocks whose
+    scale is and is not a power of two (the quotients there are where a reciprocal and a division
+    can differ), zero blocks and equal extremes of both signs among them, packed into a buffer
+    that held other bytes: the packing warps' partial last runs and every padding byte."""
+    rng = np.random.default_rng(N + K + fmt)
+    top = {emb.EMB_Q8_0: 127, emb.EMB_Q4_0: 8, emb.EMB_Q6_0: 32}[fmt]
+    nb = N * (K // 32)
+    d = np.where(rng.random((nb, 1)) < 0.3, 0.0078125, rng.uniform(1e-3, 1.0, (nb, 1))).astype(np.float16)
+    d = d.astype(np.float32)
+    w = (d * (rng.integers(-top, top, (nb, 32)) + np.float32(0.5)).astype(np.float32)).astype(np.float32)
+    step = rng.integers(-1, 2, (nb, 32))
+    w = np.where(step < 0, np.nextafter(w, np.float32(-9)), np.where(step > 0, np.nextafter(w, np.float32(9)), w))
+    at = rng.integers(0, 32, nb)
+    w[np.arange(nb), at] = (d[:, 0] * top) * np.where(rng.random(nb) < 0.5, -1, 1)
+    both = rng.random(nb) < 0.3
+    w[both, (at[both] + rng.integers(1, 32, both.sum())) % 32] = -w[both, at[both]]
+    w[rng.random(nb) < 0.05] = 0.0
+    W = np.ascontiguousarray(w.reshape(N, K), dtype=np.float32)
+    out = torch.full((emb.emb_qweight_bytes(fmt, N, K),), 0xA5, dtype=torch.uint8, device="cuda")
+    pack = {emb.EMB_Q8_0: emb.emb_quantize_q8_0, emb.EMB_Q4_0: emb.emb_quantize_q4_0,
+            emb.EMB_Q6_0: emb.emb_quantize_q6_0}[fmt]
+    pack(torch.from_numpy(W).cuda(), N, K, out)
+    diff = np.nonzero(out.cpu().numpy() != oracle.quantize(fmt, W))[0]
+    assert diff.size == 0, f"{diff.size} bytes differ, first at {diff[:8]}"
