@@ -35,8 +35,10 @@ __host__ __device__ inline Layout layout_of(int fmt, int64_t N, int64_t K) {
 
 // ------------------------------------------------------------------ epilogues
 // Activations of the gated epilogues, in fp32 with the CUDA math library.
+// 0.5 (1 + tanh(u)) = 1 / (1 + exp(-2u)): one exponential and one division, no cancellation
+// for negative u.
 __device__ __forceinline__ float act_gelu_tanh(float g) {
-    return 0.5f * g * (1.0f + tanhf(0.7978845608028654f * (g + 0.044715f * g * g * g)));
+    return g / (1.0f + expf(-1.5957691216057308f * (g + 0.044715f * g * g * g)));
 }
 __device__ __forceinline__ float act_silu(float g) { return g / (1.0f + expf(-g)); }
 

@@ -619,31 +619,30 @@ __global__ void __launch_bounds__(kThreads, 1) gemm_tc_kernel(const __grid_const
                     }
                     if (splits == 1) {
                         if (epi >= EMB_EPI_GEGLU) {
-                            // gate row n (even lane) and up row n + 1 (the next lane): rows past N
-                            // hold zeros (their weights were read as zeros), so every lane shuffles
+                            // gate rows sit in even lanes, their up rows in the next lane: of tokens e
+                            // and e + 1 the even lane takes the first and the odd lane the second, each
+                            // getting the other half of its pair by one exchange, so that every lane
+                            // evaluates an activation. Rows past N hold zeros (their weights were read
+                            // as zeros), so every lane shuffles.
+                            const int odd = lane & 1;
 #pragma unroll
-                            for (int e = 0; e < 16; ++e) {
-                                const float up = __shfl_down_sync(0xffffffffu, __uint_as_float(v[e]), 1);
-                                const int m = mt + c0 + e;
-                                if ((lane & 1) == 0 && n < N && m < M)
-                                    epi_store_gated(epi, Y, m, n, N, __uint_as_float(v[e]), up);
+                            for (int e = 0; e < 16; e += 2) {
+                                const float a = __uint_as_float(v[e]), b = __uint_as_float(v[e + 1]);
+                                const float r = __shfl_xor_sync(0xffffffffu, odd ? a : b, 1);
+                                const int m = mt + c0 + e + odd;
+                                if (n < N && m < M)
+                                    epi_store_gated(epi, Y, m, n - odd, N, odd ? r : a, odd ? b : r);
                             }
                         } else if (epi == EMB_EPI_ADD && n < N) {
-                            // reads four at a time ahead of their stores: a read after a store to
-                            // the same buffer would otherwise wait for that store
-                            float* y = reinterpret_cast<float*>(Y);
+                            // every read ahead of the stores: a read after a store to the same buffer
+                            // would otherwise wait for that store
+                            float* y = reinterpret_cast<float*>(Y) + int64_t(mt + c0) * N + n;
+                            float old[16];
 #pragma unroll
-                            for (int e0 = 0; e0 < 16; e0 += 4) {
-                                float old[4];
+                            for (int e = 0; e < 16; ++e) old[e] = (mt + c0 + e < M) ? y[int64_t(e) * N] : 0.0f;
 #pragma unroll
-                                for (int e = 0; e < 4; ++e)
-                                    old[e] = (mt + c0 + e0 + e < M) ? y[int64_t(mt + c0 + e0 + e) * N + n] : 0.0f;
-#pragma unroll
-                                for (int e = 0; e < 4; ++e)
-                                    if (mt + c0 + e0 + e < M)
-                                        y[int64_t(mt + c0 + e0 + e) * N + n] =
-                                            __fadd_rn(old[e], __uint_as_float(v[e0 + e]));
-                            }
+                            for (int e = 0; e < 16; ++e)
+                                if (mt + c0 + e < M) y[int64_t(e) * N] = __fadd_rn(old[e], __uint_as_float(v[e]));
                         } else if (n < N) {
 #pragma unroll
                             for (int e = 0; e < 16; ++e) {
