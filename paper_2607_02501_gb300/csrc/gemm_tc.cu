@@ -9,21 +9,27 @@
 // accumulator D[n][m] sits in TMEM lanes = n. The epilogue reads TMEM lane n (one
 // thread per output feature) and writes Y[m][n] with 128-byte coalesced stores.
 //
-// TMEM (512 columns, one CTA per SM): columns 0..255 the accumulator, 256..511 the ring
-// of bf16 A tiles (32 columns = 64 k per tile, two values per column, row n in lane n).
-// Keeping A out of shared memory leaves shared-memory bandwidth to the X tiles (written
-// by TMA, read by the MMA), which bound this kernel (measured on GB300: 100 -> 70 KB of
-// shared-memory traffic per 64-k step; M = 816 prefill 683 -> 736 TFLOP/s).
+// TMEM (512 columns, one CTA per SM): the accumulators of the CTA's one or two token tiles
+// (T columns each, rounded up to 32), then a ring of up to eight bf16 A tiles (32 columns =
+// 64 k per tile, two values per column, row n in lane n). Keeping A out of shared memory leaves
+// its bandwidth to the X tiles (written by TMA, read by the MMA at 64 bytes per cycle).
 //
-// Roles (352 threads):
-//   warp 0 lane 0 : TMA producer. Raw stages (256 codes of 128 rows + their 8 scales)
-//                   are fetched before griddepcontrol.wait (weights never depend on
-//                   the previous launch); X tiles (64 k x T tokens) after it.
-//   warp 1        : TMEM allocation; lane 0 issues the MMAs (4 x K=16 per 64-k stage).
-//                   It never waits on an mbarrier while MMAs are in flight: warp 10
-//                   waits for each stage and releases it through a named barrier.
+// Roles (320 threads):
+//   warp 0        : TMA producer. Raw stages (256 codes of 128 rows + their 8 scales) are
+//                   fetched before griddepcontrol.wait (weights never depend on the previous
+//                   launch); X tiles (64 k x T tokens) after it.
+//   warp 1        : TMEM allocation; waits for each step's X and A tile and issues its MMAs
+//                   (4 x K=16 per 64-k step and token tile).
 //   warps 2..9    : dequantisation (two threads per weight row, tcgen05.st into the
 //                   warp's lane quarter), then the epilogue.
+// Both issuing warps run converged on warp-uniform operands and elect one lane per instruction
+// (ptx::elect_one says why: behind `lane == 0` an MMA took 100 to 200 cycles to issue, more than
+// its tensor time; with a separate waiter warp in front of it Gemma-2B gate/up at M = 816 took
+// 123 us, now 104). What bounds a 64-k step now (T = 208, cycles): the loads of X and codes into
+// the SM 613 (58 bytes per cycle with all SMs loading), the dequantising warps' chain of barrier,
+// arithmetic and TMEM store ~600, the tensor pipe 416. Sixteen dequantising warps, a separate
+// group of epilogue warps, or a third raw stage (one X stage fewer) are all slower: gate/up
+// 115, 113 and 121 us against 109 then.
 // Grid: x = token tile (fastest: CTAs sharing a weight tile run together), y = weight-row
 // tile, z = K split. With z > 1 the splits of one output tile form a thread-block cluster
 // and are summed in a fixed order through distributed shared memory (deterministic).
@@ -52,14 +58,13 @@ constexpr int kKR = 256;                   // k per raw stage
 constexpr int kStepsPerRaw = kKR / kKC;    // 4
 constexpr int kRawStages = 2;
 constexpr int kDeqWarps = 8;               // dequantisation (then epilogue) warps
-constexpr int kWaitWarp = 2 + kDeqWarps;   // waits on the MMA warp's behalf (see the kernel)
-constexpr int kThreads = 32 * (kWaitWarp + 1);
-constexpr int kAccCols = 256;              // TMEM columns [0, 256): one token tile's accumulator (T <= 256)
+constexpr int kThreads = 32 * (2 + kDeqWarps);
 constexpr int kACols = kKC / 2;            // TMEM columns of one bf16 A tile (two values per column)
 constexpr uint32_t kTmemCols = 512;        // accumulator + A stages
 constexpr int kPlane = kBN * 128;          // 16 KB: 128 rows x 128 bytes of codes
 constexpr int kScaleTile = kBN * 16;       // 2 KB: 128 rows x 8 fp16 scales
-constexpr int kMaxStages = 8;              // A/X ring depth, at most
+constexpr int kMaxStages = 8;              // X ring depth, at most
+constexpr int kMaxAStages = 8;             // A ring depth, at most
 
 struct GemmParams {
     CUtensorMap x_map;                     // X [M][K] bf16, box {64, T}, 128B swizzle
@@ -76,9 +81,8 @@ struct GemmParams {
     int32_t P;                             // token tiles per CTA (1, or 2 sharing each A tile)
     int32_t splits;                        // K splits (cluster size along z)
     int32_t epi;                           // emb_epilogue
-    int32_t stages;                        // A/X ring depth
-    int32_t a_gap0;                        // P = 2: TMEM column of the first A stage after tile 0's
-    int32_t a_per_gap;                     //   accumulator, and A stages per gap (see pick_stages_pair)
+    int32_t stages;                        // X ring depth
+    int32_t a_stages;                      // A ring depth (TMEM)
     uint32_t tmem_cols;
     int32_t persist;                       // 1: CTAs loop over items (no K split)
     int32_t n_tt, n_items;                 // persistent: token tiles per weight tile, items
@@ -102,11 +106,6 @@ struct RawTraits {
 
 __device__ __forceinline__ uint4 lds128(const uint8_t* p) {
     return *reinterpret_cast<const uint4*>(p);
-}
-
-// bar.sync on a named barrier with `count` threads (whole warps).
-__device__ __forceinline__ void named_sync(int id, int count) {
-    asm volatile("bar.sync %0, %1;" ::"r"(id), "r"(count) : "memory");
 }
 
 __device__ __forceinline__ uint32_t pack_bf16(float a, float b) {
@@ -149,13 +148,10 @@ __device__ __forceinline__ void make_chunk(uint32_t u0, uint32_t u1, float d, fl
     }
 }
 
-// TMEM column of A stage s: after the accumulator (P = 1), or in the slots after each of
-// the two accumulators at columns 0 and 256 (P = 2).
-template <int P, bool SPLIT>
-__device__ __forceinline__ uint32_t a_stage_col(int s, int gap0, int per_gap) {
-    if constexpr (P == 1) return uint32_t(kAccCols + s * (SPLIT ? 2 : 1) * kACols);
-    return uint32_t(s < per_gap ? gap0 + s * kACols : kAccCols + gap0 + (s - per_gap) * kACols);
-}
+// TMEM columns: the accumulators of the CTA's P token tiles, each rounded up to 32 columns,
+// then the ring of A tiles (hi and lo tile of a step side by side for the split operand).
+__host__ __device__ constexpr int acc_cols(int T) { return (T + 31) & ~31; }
+__host__ __device__ constexpr int a_stage_cols(bool split) { return (split ? 2 : 1) * kACols; }
 
 template <int FMT, bool SPLIT, int P, bool SK>
 __global__ void __launch_bounds__(kThreads, 1) gemm_tc_kernel(const __grid_constant__ GemmParams p) {
@@ -165,7 +161,8 @@ __global__ void __launch_bounds__(kThreads, 1) gemm_tc_kernel(const __grid_const
     extern __shared__ uint8_t smem_dyn[];
     uint8_t* base = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_dyn) + 1023) &
                                                ~uintptr_t(1023));
-    const int S = p.stages, T = p.T;
+    const int S = p.stages, SA = p.a_stages, T = p.T;
+    const int a_col0 = P * acc_cols(T);  // TMEM column of the A ring
     uint8_t* x_ring = base;                                     // S x P x T x 128 B
     uint8_t* r_ring = x_ring + S * P * T * 128;                 // 2 x RT::bytes
     uint8_t* s_ring = r_ring + kRawStages * RT::bytes;          // 2 x 2 KB
@@ -174,22 +171,22 @@ __global__ void __launch_bounds__(kThreads, 1) gemm_tc_kernel(const __grid_const
     uint64_t* raw_full = bars;
     uint64_t* raw_empty = bars + kRawStages;
     uint64_t* x_full = bars + 2 * kRawStages;
-    uint64_t* a_full = x_full + S;
-    uint64_t* ax_empty = a_full + S;
-    uint64_t* acc_full = ax_empty + S;
+    uint64_t* x_empty = x_full + S;
+    uint64_t* a_full = x_empty + S;
+    uint64_t* a_empty = a_full + SA;
+    uint64_t* acc_full = a_empty + SA;
     uint64_t* acc_empty = acc_full + 1;  // the epilogue warps have read the accumulator
     uint64_t* sk_full = acc_empty + 1;   // stream-K head: a chunk of a tail is in the X ring
     uint64_t* sk_free = sk_full + 1;     // stream-K head: every epilogue warp has added it
     uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(sk_free + 1);
     volatile int* abort_flag = reinterpret_cast<volatile int*>(tmem_slot + 1);
-    volatile int* mma_stop = abort_flag + 1;  // set by the waiter warp when a wait gave up
-    int* sk_cnt = const_cast<int*>(mma_stop) + 1;  // stream-K: epilogue warps done with the tail
+    int* sk_cnt = const_cast<int*>(abort_flag) + 1;  // stream-K: epilogue warps done with the tail
     int* sk_seen = sk_cnt + 1;                     // stream-K: epilogue warps done with the head
     // split-K partial tile [T][128] fp32 (token-major): reuses the X ring once every MMA
     // has completed
     float* part = reinterpret_cast<float*>(x_ring);
 
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int warp = ptx::warp_uniform(int(threadIdx.x >> 5)), lane = threadIdx.x & 31;
     const int M = p.M, K = p.K;
     const int splits = gridDim.z, split = blockIdx.z;
     const int nr_all = (K + kKR - 1) / kKR, nk_all = (K + kKC - 1) / kKC;
@@ -273,15 +270,17 @@ __global__ void __launch_bounds__(kThreads, 1) gemm_tc_kernel(const __grid_const
         }
         for (int i = 0; i < S; ++i) {
             ptx::mbar_init(&x_full[i], 1);
+            ptx::mbar_init(&x_empty[i], 1);
+        }
+        for (int i = 0; i < SA; ++i) {
             ptx::mbar_init(&a_full[i], kDeqWarps);
-            ptx::mbar_init(&ax_empty[i], 1);
+            ptx::mbar_init(&a_empty[i], 1);
         }
         ptx::mbar_init(acc_full, 1);
         ptx::mbar_init(acc_empty, kDeqWarps);
         ptx::mbar_init(sk_full, 1);
         ptx::mbar_init(sk_free, kDeqWarps);
         *abort_flag = 0;
-        *mma_stop = 0;
         *sk_cnt = 0;
         *sk_seen = 0;
         ptx::fence_mbar_init();
@@ -300,26 +299,29 @@ __global__ void __launch_bounds__(kThreads, 1) gemm_tc_kernel(const __grid_const
     ptx::tc_fence_before();
     __syncthreads();
     ptx::tc_fence_after();
-    const uint32_t tmem = *tmem_slot;
+    const uint32_t tmem = ptx::warp_uniform(*tmem_slot);
     ptx::griddep_launch_dependents();
     int items_done = 0;  // this CTA's items started by its role (phase of acc_full / acc_empty)
 
     if (warp == 0) {
-        if (lane == 0) {
-            // ---------------------------------------------------------------- producer
-            const uint64_t pol_w = ptx::policy_evict_first();
-            const uint64_t pol_x = ptx::policy_evict_last();
-            int raw_issued = 0, x_issued = 0;  // over all items of the CTA
-            bool stop = false, waited = false;
-            int rbase = 0, xbase = 0;  // raw stages and steps of the earlier segments
-            for (int j = 0; j < n_seg && !stop; ++j, ++items_done) {
-                const Seg sg = seg_at(j);
-                const Item I = item_at(sg.it);
-                const int nr = sg.r1 - sg.r0, nk = seg_nk(sg), ks0 = sg.r0 * kStepsPerRaw;
-                auto issue_raw = [&](int r) {  // raw stage r of this segment (global rbase + r)
-                    const int rg_all = rbase + r;
-                    const int slot = rg_all % kRawStages;
-                    const int rg = sg.r0 + r;  // raw stage index within the whole row
+        // -------------------------------------------------------------------- producer
+        // the whole warp runs the loop; one elected lane issues the copies (see ptx::elect_one)
+        const unsigned full = 0xffffffffu;
+        const uint64_t pol_w = ptx::policy_evict_first();
+        const uint64_t pol_x = ptx::policy_evict_last();
+        int raw_issued = 0, x_issued = 0;  // over all items of the CTA
+        bool stop = false, waited = false;
+        int rbase = 0;         // raw stages of the earlier segments
+        int s = 0;             // X stage, and how often the ring has gone round
+        uint32_t xround = 0;
+        for (int j = 0; j < n_seg && !stop; ++j, ++items_done) {
+            const Seg sg = seg_at(j);
+            const Item I = item_at(sg.it);
+            const int nr = sg.r1 - sg.r0, nk = seg_nk(sg), ks0 = sg.r0 * kStepsPerRaw;
+            auto issue_raw = [&](int r) {  // raw stage r of this segment (global rbase + r)
+                const int slot = (rbase + r) % kRawStages;
+                const int rg = sg.r0 + r;  // raw stage index within the whole row
+                if (ptx::elect_one()) {
                     ptx::mbar_arrive_expect_tx(&raw_full[slot], RT::bytes + RT::hbytes + kScaleTile);
 #pragma unroll
                     for (int pl = 0; pl < RT::planes; ++pl)
@@ -330,136 +332,117 @@ __global__ void __launch_bounds__(kThreads, 1) gemm_tc_kernel(const __grid_const
                                          rg * 64, I.n0, pol_w);
                     ptx::tma_load_2d(s_ring + slot * kScaleTile, &p.scales_map[I.g], &raw_full[slot],
                                      rg * (kKR / kQBlock), I.n0, pol_w);
-                };
-                if (!waited) {
-                    // the first raw stages before griddepcontrol.wait: weights never depend on
-                    // the previous launch; X may be written by it, so only its rows' way towards
-                    // L2 starts now (a hint: the TMA loads after the wait read the written values)
-                    for (; raw_issued < nr && raw_issued < kRawStages; ++raw_issued) issue_raw(raw_issued);
-                    const int x_rows = min(M - I.m0, P * T);
-                    if (x_rows > 0 && I.n0 == 0 && I.g == 0 && sg.r0 == 0)  // one CTA per token tile
-                        ptx::prefetch_l2(reinterpret_cast<const uint8_t*>(p.X) + int64_t(I.m0) * K * 2,
-                                         uint32_t(min(int64_t(x_rows) * K * 2, int64_t(1) << 20)));
-                    ptx::griddep_wait();
-                    waited = true;
                 }
-                for (int i = 0; i < nk; ++i) {
-                    if (i % kStepsPerRaw == 0) {
-                        const int rg_all = rbase + i / kStepsPerRaw;
-                        if (rg_all >= raw_issued) {
-                            if (rg_all >= kRawStages &&
-                                !ptx::mbar_wait(&raw_empty[rg_all % kRawStages], ((rg_all / kRawStages) - 1) & 1,
-                                                abort_flag, p.status, kWaitLimitNs)) {
-                                stop = true;
-                                break;
-                            }
-                            issue_raw(i / kStepsPerRaw);
-                            ++raw_issued;
+                __syncwarp();
+            };
+            if (!waited) {
+                // the first raw stages before griddepcontrol.wait: weights never depend on
+                // the previous launch; X may be written by it, so only its rows' way towards
+                // L2 starts now (a hint: the TMA loads after the wait read the written values)
+                for (; raw_issued < nr && raw_issued < kRawStages; ++raw_issued) issue_raw(raw_issued);
+                const int x_rows = min(M - I.m0, P * T);
+                if (lane == 0 && x_rows > 0 && I.n0 == 0 && I.g == 0 && sg.r0 == 0)  // one CTA per token tile
+                    ptx::prefetch_l2(reinterpret_cast<const uint8_t*>(p.X) + int64_t(I.m0) * K * 2,
+                                     uint32_t(min(int64_t(x_rows) * K * 2, int64_t(1) << 20)));
+                ptx::griddep_wait();
+                waited = true;
+            }
+            for (int i = 0; i < nk; ++i) {
+                if (i % kStepsPerRaw == 0) {
+                    const int rg_all = rbase + i / kStepsPerRaw;
+                    if (rg_all >= raw_issued) {
+                        if (rg_all >= kRawStages &&
+                            !__all_sync(full, ptx::mbar_wait(&raw_empty[rg_all % kRawStages], ((rg_all / kRawStages) - 1) & 1,
+                                                             abort_flag, p.status, kWaitLimitNs))) {
+                            stop = true;
+                            break;
                         }
+                        issue_raw(i / kStepsPerRaw);
+                        ++raw_issued;
                     }
-                    const int xs = xbase + i;
-                    const int s = xs % S;
-                    if (xs >= S && !ptx::mbar_wait(&ax_empty[s], ((xs / S) - 1) & 1, abort_flag, p.status,
-                                                   kWaitLimitNs)) {
-                        stop = true;
-                        break;
-                    }
+                }
+                if (xround > 0 && !__all_sync(full, ptx::mbar_wait(&x_empty[s], (xround - 1) & 1, abort_flag, p.status,
+                                                                   kWaitLimitNs))) {
+                    stop = true;
+                    break;
+                }
+                if (ptx::elect_one()) {
                     ptx::mbar_arrive_expect_tx(&x_full[s], uint32_t(P * T) * 128u);
 #pragma unroll
                     for (int q = 0; q < P; ++q)  // a tile past M reads zeros (its outputs are not stored)
                         ptx::tma_load_2d(x_ring + (s * P + q) * T * 128, &p.x_map, &x_full[s],
                                          (ks0 + i) * kKC, I.m0 + q * T, pol_x);
-                    ++x_issued;
                 }
-                rbase += nr;
-                xbase += nk;
+                __syncwarp();
+                ++x_issued;
+                if (++s == S) {
+                    s = 0;
+                    ++xround;
+                }
             }
-            // every issued copy must land before this CTA's shared memory can be released
-            for (int r = raw_issued - 1; r >= 0 && r >= raw_issued - kRawStages; --r)
-                ptx::mbar_wait(&raw_full[r % kRawStages], (r / kRawStages) & 1, nullptr, p.status,
-                               kWaitLimitNs);
-            for (int i = x_issued - 1; i >= 0 && i >= x_issued - S; --i)
-                ptx::mbar_wait(&x_full[i % S], (i / S) & 1, nullptr, p.status, kWaitLimitNs);
+            rbase += nr;
         }
+        // every issued copy must land before this CTA's shared memory can be released
+        for (int r = raw_issued - 1; r >= 0 && r >= raw_issued - kRawStages; --r)
+            ptx::mbar_wait(&raw_full[r % kRawStages], (r / kRawStages) & 1, nullptr, p.status,
+                           kWaitLimitNs);
+        for (int i = x_issued - 1; i >= 0 && i >= x_issued - S; --i)
+            ptx::mbar_wait(&x_full[i % S], (i / S) & 1, nullptr, p.status, kWaitLimitNs);
     } else if (warp == 1) {
         // ---------------------------------------------------------------- MMA issuer
-        // Step i is released by the waiter warp through named barrier 1; this warp itself
-        // runs no mbarrier wait while MMAs are in flight (see kWaitWarp below).
+        // the whole warp waits for step i's X tile and A tile (and, at an item's first step, for
+        // the previous item's epilogue to have read the accumulator); one elected lane issues
+        const unsigned full = 0xffffffffu;
         const uint32_t idesc = ptx::idesc_bf16_f32(kBN, T);
         const uint32_t x0 = ptx::smem_u32(x_ring);
         bool stop = false;
         int commits = 0;  // accumulator commits (one per finished segment)
-        int xbase = 0;
+        int s = 0, a = 0;  // X and A ring stages of the step and their phases
+        uint32_t ph = 0, pha = 0;
         for (int j = 0; j < n_seg && !stop; ++j, ++items_done) {
             const int nk = seg_nk(seg_at(j));
             for (int i = 0; i < nk; ++i) {
-                named_sync(1, 64);
-                if (*mma_stop) {
+                bool ok = true;
+                if (i == 0 && items_done > 0)
+                    ok = ptx::mbar_wait(acc_empty, (items_done - 1) & 1, abort_flag, p.status, kWaitLimitNs);
+                ok = ok && ptx::mbar_wait(&x_full[s], ph, abort_flag, p.status, kWaitLimitNs) &&
+                     ptx::mbar_wait(&a_full[a], pha, abort_flag, p.status, kWaitLimitNs);
+                if (!__all_sync(full, ok)) {
                     stop = true;
                     break;
                 }
-                if (lane == 0) {
-                    const int s = (xbase + i) % S;
-                    ptx::tc_fence_after();
-                    const uint32_t a_tm = tmem + a_stage_col<P, SPLIT>(s, p.a_gap0, p.a_per_gap);
+                ptx::tc_fence_after();
+                const uint32_t a_tm = tmem + uint32_t(a_col0 + a * a_stage_cols(SPLIT));
 #pragma unroll
-                    for (int q = 0; q < P; ++q) {
-                        // token tile q: its own X tile and accumulator, the same A tile
-                        const uint32_t x_addr = x0 + (s * P + q) * T * 128;
-                        const uint32_t d_tm = tmem + uint32_t(q * kAccCols);
+                for (int q = 0; q < P; ++q) {
+                    // token tile q: its own X tile and accumulator, the same A tile
+                    const uint64_t bdesc = ptx::smem_desc_sw128(x0 + (s * P + q) * T * 128);
+                    const uint32_t d_tm = tmem + uint32_t(q * acc_cols(T));
 #pragma unroll
-                        for (int k = 0; k < kKC / 16; ++k) {
-                            const uint64_t bdesc = ptx::smem_desc_sw128(x_addr + 32 * k);
-                            ptx::mma_bf16_ta(d_tm, a_tm + 8 * k, bdesc, idesc, (i | k) != 0);
-                            if constexpr (SPLIT) ptx::mma_bf16_ta(d_tm, a_tm + kACols + 8 * k, bdesc, idesc, 1u);
-                        }
+                    for (int k = 0; k < kKC / 16; ++k) {  // 32 bytes along K: two 16-byte units
+                        ptx::mma_bf16_ta(d_tm, a_tm + 8 * k, bdesc + 2 * k, idesc, (i | k) != 0);
+                        if constexpr (SPLIT) ptx::mma_bf16_ta(d_tm, a_tm + kACols + 8 * k, bdesc + 2 * k, idesc, 1u);
                     }
-                    ptx::mma_commit(&ax_empty[s]);
                 }
-                __syncwarp();
+                ptx::mma_commit(&a_empty[a]);
+                ptx::mma_commit(&x_empty[s]);
+                if (++s == S) {
+                    s = 0;
+                    ph ^= 1u;
+                }
+                if (++a == SA) {
+                    a = 0;
+                    pha ^= 1u;
+                }
             }
             // the item's accumulator is complete once every MMA issued so far has finished
-            if (stop) break;
-            if (lane == 0) ptx::mma_commit(acc_full);
+            // (after a wait gave up: the MMAs issued so far, so that they finish before TMEM is freed)
+            ptx::mma_commit(acc_full);
             ++commits;
-            xbase += nk;
-            __syncwarp();
         }
-        if (lane == 0 && commits > 0)  // the last item's MMAs finish before TMEM is freed
+        if (commits > 0)  // the last item's MMAs finish before TMEM is freed
             ptx::mbar_wait(acc_full, (commits - 1) & 1, nullptr, p.status, kWaitLimitNs);
-    } else if (warp == kWaitWarp) {
-        // ---------------------------------------------------------------- waiter
-        // An mbarrier wait executed by the warp that issues tcgen05 MMAs is ordered behind
-        // that warp's in-flight MMAs, which drains the tensor pipe at every step (measured
-        // on GB300: 104 -> 330+ cycles per 128x208x16 MMA). This warp waits for step i's
-        // X tile and A tile (and, at an item's first step, for the previous item's epilogue
-        // to have read the accumulator) and then releases the MMA warp through named barrier 1.
-        bool stop = false;
-        int xbase = 0;
-        for (int j = 0; j < n_seg && !stop; ++j, ++items_done) {
-            const int nk = seg_nk(seg_at(j));
-            for (int i = 0; i < nk; ++i) {
-                const int xs = xbase + i;
-                const int s = xs % S;
-                const uint32_t ph = (xs / S) & 1;
-                if (lane == 0) {
-                    bool ok = true;
-                    if (i == 0 && items_done > 0)
-                        ok = ptx::mbar_wait(acc_empty, (items_done - 1) & 1, abort_flag, p.status, kWaitLimitNs);
-                    ok = ok && ptx::mbar_wait(&x_full[s], ph, abort_flag, p.status, kWaitLimitNs) &&
-                         ptx::mbar_wait(&a_full[s], ph, abort_flag, p.status, kWaitLimitNs);
-                    if (!ok) *mma_stop = 1;
-                }
-                __syncwarp();
-                named_sync(1, 64);
-                if (*mma_stop) {
-                    stop = true;
-                    break;
-                }
-            }
-            xbase += nk;
-        }
-    } else if (warp < 2 + kDeqWarps) {
+    } else {
         // ---------------------------------------------------------------- dequant
         // two threads per weight row: thread (row t, half h) produces 32 of the 64 bf16 of
         // each 64-k step (32-block 2j+h of step j) and stores them into its TMEM lane t,
@@ -507,8 +490,8 @@ __global__ void __launch_bounds__(kThreads, 1) gemm_tc_kernel(const __grid_const
                     const int i = r * kStepsPerRaw + j;
                     if (i >= nk) break;
                     const int xs = xbase + i;
-                    const int s = xs % S;
-                    const uint32_t a_dst = a_lane + a_stage_col<P, SPLIT>(s, p.a_gap0, p.a_per_gap);
+                    const int s = xs % SA;
+                    const uint32_t a_dst = a_lane + uint32_t(a_col0 + s * a_stage_cols(SPLIT));
                     const int sx = t & 7;  // raw codes: 16-byte chunk c of row t lives at c ^ (t & 7)
                     uint32_t va[16], vl[16];  // this thread's 16 columns of the hi (and lo) tile
                     if constexpr (FMT == EMB_Q8_0) {
@@ -566,8 +549,8 @@ __global__ void __launch_bounds__(kThreads, 1) gemm_tc_kernel(const __grid_const
                         }
                     }
                     signal_pending();
-                    if (xs >= S) {
-                        ok = __all_sync(full, ptx::mbar_wait(&ax_empty[s], ((xs / S) - 1) & 1, abort_flag,
+                    if (xs >= SA) {
+                        ok = __all_sync(full, ptx::mbar_wait(&a_empty[s], ((xs / SA) - 1) & 1, abort_flag,
                                                              p.status, kWaitLimitNs));
                         if (!ok) break;
                         ptx::tc_fence_after();  // the MMAs that read this A stage have completed
@@ -593,17 +576,15 @@ __global__ void __launch_bounds__(kThreads, 1) gemm_tc_kernel(const __grid_const
             const bool sk_head = streamk && sg.r0 == 0 && sg.r1 < nr_all;
             if (ok) {
                 ptx::tc_fence_after();
-                // warps 2..9: TMEM lane quarter = warp % 4; the two warps of a quarter split the
-                // columns of one token tile, or (P = 2) take one token tile each
-                const int quarter = warp & 3, half = (warp - 2) >> 2;
-                const int csplit = ((T >> 1) + 15) & ~15;
-                const int tt = (P == 2) ? half : 0;  // token tile read by this warp
-                const int cbeg = (P == 2 || !half) ? 0 : csplit;
-                const int cend = (P == 2 || half) ? T : min(csplit, T);
+                // TMEM lane quarter = warp % 4; the warps of a quarter take the 16-column groups of
+                // the item's P * T token columns in turn
+                const int quarter = warp & 3, slot = (warp - 2) >> 2;
+                constexpr int kStride = 16 * (kDeqWarps / 4);
                 const int row = quarter * 32 + lane;
-                const uint32_t taddr = tmem + (uint32_t(quarter * 32) << 16) + uint32_t(tt * kAccCols);
+                const uint32_t tlane = tmem + (uint32_t(quarter * 32) << 16);
+                auto tcol = [&](int c) { return uint32_t(P == 2 && c >= T ? c - T + acc_cols(T) : c); };
                 const int n = I.n0 + row, N = I.N;
-                const int mt = I.m0 + tt * T;  // first token of that tile
+                const int mt = I.m0;  // token of column 0
                 void* Y = p.Y[I.g];
                 const int epi = p.epi;
                 // Emit 16 accumulator columns c0 .. c0+15 of this warp's rows, plus (stream-K
@@ -615,7 +596,7 @@ __global__ void __launch_bounds__(kThreads, 1) gemm_tc_kernel(const __grid_const
 #pragma unroll
                         for (int e = 0; e < 16; ++e)
                             v[e] = __float_as_uint(__fadd_rn(
-                                __uint_as_float(v[e]), ptx::ld_shared_f32(staged + uint32_t(((tt * T + c0 + e) * kBN + row) * 4))));
+                                __uint_as_float(v[e]), ptx::ld_shared_f32(staged + uint32_t(((c0 + e) * kBN + row) * 4))));
                     }
                     if (splits == 1) {
                         if (epi >= EMB_EPI_GEGLU) {
@@ -690,17 +671,16 @@ __global__ void __launch_bounds__(kThreads, 1) gemm_tc_kernel(const __grid_const
                                 add_staged = true;  // the store pass adds it
                                 break;
                             }
-                            for (int c0 = cbeg; c0 < cend; c0 += 16) {
-                                const int sc = tt * T + c0;  // slot column (chunks are whole 16-column groups)
-                                if (sc < k0 || sc >= k1) continue;
+                            for (int c0 = 16 * slot; c0 < P * T; c0 += kStride) {
+                                if (c0 < k0 || c0 >= k1) continue;  // chunks are whole 16-column groups
                                 uint32_t v[16];
-                                ptx::tmem_ld_16(taddr + uint32_t(c0), v);
+                                ptx::tmem_ld_16(tlane + tcol(c0), v);
                                 ptx::tmem_ld_wait();
 #pragma unroll
                                 for (int e = 0; e < 16; ++e)
                                     v[e] = __float_as_uint(__fadd_rn(
-                                        __uint_as_float(v[e]), ptx::ld_shared_f32(staged + uint32_t(((sc - k0 + e) * kBN + row) * 4))));
-                                ptx::tmem_st_16(taddr + uint32_t(c0), v);
+                                        __uint_as_float(v[e]), ptx::ld_shared_f32(staged + uint32_t(((c0 - k0 + e) * kBN + row) * 4))));
+                                ptx::tmem_st_16(tlane + tcol(c0), v);
                             }
                             ptx::tmem_st_wait();
                             __syncwarp();
@@ -709,12 +689,12 @@ __global__ void __launch_bounds__(kThreads, 1) gemm_tc_kernel(const __grid_const
                     }
                 }
                 if (sk_tail) {
-                    float* slot = p.ws_part + int64_t(blockIdx.x) * p.slot_floats;
-                    for (int c0 = cbeg; c0 < cend; c0 += 16) {
+                    float* part_out = p.ws_part + int64_t(blockIdx.x) * p.slot_floats;
+                    for (int c0 = 16 * slot; c0 < P * T; c0 += kStride) {
                         uint32_t v[16];
-                        ptx::tmem_ld_16(taddr + uint32_t(c0), v);
+                        ptx::tmem_ld_16(tlane + tcol(c0), v);
                         ptx::tmem_ld_wait();
-                        float* dst = slot + int64_t(tt * T + c0) * kBN + row;  // a warp writes 32 consecutive rows
+                        float* dst = part_out + int64_t(c0) * kBN + row;  // a warp writes 32 consecutive rows
 #pragma unroll
                         for (int e = 0; e < 16; ++e) __stcg(dst + e * kBN, __uint_as_float(v[e]));
                     }
@@ -728,9 +708,9 @@ __global__ void __launch_bounds__(kThreads, 1) gemm_tc_kernel(const __grid_const
                 } else if (ok) {
                     // one TMEM load per wait (two per wait measured slower on GB300: the kernel's
                     // register count rose by 16 and the main loop lost 10-17 %)
-                    for (int c0 = cbeg; c0 < cend; c0 += 16) {
+                    for (int c0 = 16 * slot; c0 < P * T; c0 += kStride) {
                         uint32_t v[16];
-                        ptx::tmem_ld_16(taddr + uint32_t(c0), v);
+                        ptx::tmem_ld_16(tlane + tcol(c0), v);
                         ptx::tmem_ld_wait();
                         emit(v, c0);
                     }
@@ -761,7 +741,7 @@ __global__ void __launch_bounds__(kThreads, 1) gemm_tc_kernel(const __grid_const
         // [s*128/splits, (s+1)*128/splits) over the cluster in a fixed order through
         // distributed shared memory and stores them (deterministic, no global scratch)
         ptx::cluster_sync();
-        if (threadIdx.x >= 64 && !*abort_flag) {
+        if (warp >= 2 && !*abort_flag) {
             // one thread = 4 consecutive rows of one token: 16-byte remote loads and
             // 16-byte coalesced stores to Y[m][n..n+3]
             const int rows = kBN / splits, r0 = split * rows, q4 = rows / 4;
@@ -850,29 +830,31 @@ template <int FMT, bool SPLIT>
 int smem_bytes(int T, int S, int P) {
     const int need = 1024 + S * P * T * 128 +
                      kRawStages * (RawTraits<FMT>::bytes + RawTraits<FMT>::hbytes + kScaleTile) +
-                     (2 * kRawStages + 3 * S + 4) * 8 + 32;
+                     (2 * kRawStages + 2 * S + 2 * kMaxAStages + 4) * 8 + 32;
     return need > kOneCtaPerSm ? need : kOneCtaPerSm;
 }
 
-// Ring depth: as many X stages as shared memory holds, at most as many A stages as fit
-// in TMEM beside the accumulator (8 single tiles or 4 hi/lo pairs).
+// X ring depth: as many stages as shared memory holds, at most kMaxStages.
 template <int FMT, bool SPLIT>
 int pick_stages(int T) {
-    int S = (int(kTmemCols) - kAccCols) / ((SPLIT ? 2 : 1) * kACols);
+    int S = kMaxStages;
     while (S > 2 && smem_bytes<FMT, SPLIT>(T, S, 1) > kSmemLimit) --S;
     return S;
 }
 
-// Two token tiles per CTA (P = 2): the accumulators sit at TMEM columns 0 and 256 and the
-// A stages in the 32-column slots after each (so T <= 224). Returns the ring depth that
-// fits TMEM and shared memory (0 if fewer than two) and fills the stages' columns.
+// A ring depth: the tiles that fit TMEM beside the accumulators, at most kMaxAStages.
+int a_stages_of(bool split, int T, int P) {
+    return std::min(kMaxAStages, (int(kTmemCols) - P * acc_cols(T)) / a_stage_cols(split));
+}
+
+// X ring depth with two token tiles per CTA (P = 2), each at most 224 tokens; 0 if fewer than
+// two stages fit shared memory or two A tiles TMEM.
 template <int FMT>
-int pick_stages_pair(int T, int& gap0, int& per_gap) {
-    gap0 = int(roundup(T, 32));
-    per_gap = (kAccCols - gap0) / kACols;
-    int S = std::min(2 * per_gap, kMaxStages);
+int pick_stages_pair(int T) {
+    if (a_stages_of(false, T, 2) < 2) return 0;
+    int S = kMaxStages;
     while (S > 2 && smem_bytes<FMT, false>(T, S, 2) > kSmemLimit) --S;
-    if (S < 2 || smem_bytes<FMT, false>(T, S, 2) > kSmemLimit) return 0;
+    if (smem_bytes<FMT, false>(T, S, 2) > kSmemLimit) return 0;
     return S;
 }
 
@@ -965,7 +947,7 @@ namespace {
 struct GemmPlan {
     int T = 0, S = 0, P = 1, splits = 1;
     int grid_x = 0, grid_y = 0, persist = 0, streamk = 0;
-    int a_gap0 = 0, a_per_gap = 0, n_tt = 0, n_items = 0;
+    int n_tt = 0, n_items = 0;
     size_t ws_bytes = 0;  // stream-K workspace: flags, then grid_x partial-tile slots
 };
 
@@ -974,6 +956,14 @@ struct GemmPlan {
 constexpr int kSkFlagBytes = 4096;  // room for 1024 CTAs
 size_t sk_slot_bytes(int P, int T) { return size_t(roundup(int64_t(P) * T * kBN * 4, 256)); }
 size_t sk_ws_bytes(int G, int P, int T) { return kSkFlagBytes + size_t(G) * sk_slot_bytes(P, T); }
+
+// Cycle model of the plans (GB300, fitted to both formats' measured launches). A 64-k step of a
+// CTA with P token tiles of T takes the largest of: the dequantisation warps' chain per A tile,
+// ~620; moving its X tiles and raw codes into the SM, (128 P T + 8.7 K) bytes at the ~58 bytes
+// per cycle an SM gets with all of them loading; the MMAs (2 per token of the CTA, always less
+// than the loads). An item adds its drain, epilogue and restart.
+double step_cycles(int P, int T) { return std::max(620.0, 2.22 * P * T + 150.0); }
+double item_cycles(int P, int T) { return 6300.0 + 22.6 * P * T; }
 
 // The launch shape of one group. With streamk_ok the plan may take the stream-K schedule,
 // which needs plan.ws_bytes of zero-filled workspace.
@@ -991,17 +981,16 @@ GemmPlan plan_gemm(const GroupRef& g, bool streamk_ok) {
     int splits = pick_splits(int64_t(t_tiles) * tiles, T, g.K, S, split);
     // Prefill shapes whose weight tiles x token tiles leave SMs idle (narrow layers: the
     // vision tower's 1152-wide ones give 9-36 weight tiles) may take more, smaller token
-    // tiles: per the cycle model below (per 64-k step the larger of the dequantisation,
-    // ~1050 cycles, and the MMA work, ~5.2 cycles per token; ~3900 per CTA; times the
-    // waves), up to three more tiles when that is at least 3 % faster. ViT M = 768: four
-    // tiles of 192 instead of three of 256 (qkv 81 -> 108 CTAs, fc1 108 -> 144).
+    // tiles: up to three more when the cycle model says at least 3 % faster. ViT M = 768: fc1
+    // takes four tiles of 192 instead of three of 256 (108 -> 144 CTAs), q/k/v five of 160
+    // (81 -> 135).
     if (!split && g.M >= 256) {
         const int sms = sm_count();
         if (sms > 0) {
             const double nk = double((g.K + kKC - 1) / kKC);
             auto cost = [&](int64_t tt, int Tc, int sp) {
                 return double((tt * tiles * sp + sms - 1) / sms) *
-                       (std::ceil(nk / sp) * std::max(1050.0, 5.2 * Tc) + 3900.0);
+                       (std::ceil(nk / sp) * step_cycles(1, Tc) + item_cycles(1, Tc));
             };
             double best = cost(t_tiles, T, splits);
             const int64_t t0 = t_tiles;
@@ -1024,36 +1013,30 @@ GemmPlan plan_gemm(const GroupRef& g, bool streamk_ok) {
         }
     }
     int P = 1, grid_x = int(t_tiles);
-    // Two token tiles per CTA halve the dequantisation per token (each A tile feeds the MMAs
-    // of both). Time model in cycles, fitted to GB300 measurements of both formats: per
-    // 64-k step the larger of the dequantisation (~1050) and the MMA work (~5.2 per token
-    // of the CTA), plus ~3900 of pipeline fill and drain per CTA, times the waves of CTAs
-    // over the SMs. Pairs win where one tile per CTA is dequantisation-bound (T <= ~200)
-    // and the pairs do not add a wave: Llama-7B qkv at M = 280, 455 -> 678 TFLOP/s; gate/up
-    // 547 -> 610. At M = 816 (T = 208) one tile per CTA is already MMA-bound and pairs lose
-    // (847 -> 772); narrow layers keep one tile per CTA and split K instead.
+    // Two token tiles per CTA halve the dequantisation and the code loads per token (each A tile
+    // feeds the MMAs of both), for half as many CTAs: taken where the cycle model gains 5 %.
+    // Llama-7B q/k/v at M = 280 (one wave of 96 CTAs instead of two of 192), Gemma-2B gate/up at
+    // M = 816 (four rounds of two tiles instead of seven of one: 111 -> 104 us); narrow layers
+    // keep one tile per CTA and split K instead.
     if (!split && t_tiles >= 2) {
         const int64_t t2 = 2 * ((g.M + 447) / 448);  // even count of tiles of at most 224
         const int T2 = int(roundup((g.M + t2 - 1) / t2, 16));
-        int gap0 = 0, per_gap = 0;
-        const int S2 = (g.fmt == EMB_Q8_0)   ? pick_stages_pair<EMB_Q8_0>(T2, gap0, per_gap)
-                       : (g.fmt == EMB_Q4_0) ? pick_stages_pair<EMB_Q4_0>(T2, gap0, per_gap)
-                                             : pick_stages_pair<EMB_Q6_0>(T2, gap0, per_gap);
+        const int S2 = (g.fmt == EMB_Q8_0)   ? pick_stages_pair<EMB_Q8_0>(T2)
+                       : (g.fmt == EMB_Q4_0) ? pick_stages_pair<EMB_Q4_0>(T2)
+                                             : pick_stages_pair<EMB_Q6_0>(T2);
         const int sms = sm_count();
         if (S2 >= 2 && T2 <= 224 && sms > 0) {
             const double nk = double((g.K + kKC - 1) / kKC);
             auto waves = [&](int64_t ctas) { return double((ctas + sms - 1) / sms); };
             const double c1 = waves(int64_t(t_tiles) * tiles * splits) *
-                              (std::ceil(nk / splits) * std::max(1050.0, 5.2 * T) + 3900.0);
-            const double c2 = waves(int64_t(t2 / 2) * tiles) * (nk * std::max(1050.0, 5.2 * 2 * T2) + 3900.0);
+                              (std::ceil(nk / splits) * step_cycles(1, T) + item_cycles(1, T));
+            const double c2 = waves(int64_t(t2 / 2) * tiles) * (nk * step_cycles(2, T2) + item_cycles(2, T2));
             if (c2 < 0.95 * c1) {
                 P = 2;
                 T = T2;
                 S = S2;
                 splits = 1;
                 grid_x = int(t2 / 2);
-                pl.a_gap0 = gap0;
-                pl.a_per_gap = per_gap;
             }
         }
     }
@@ -1064,7 +1047,7 @@ GemmPlan plan_gemm(const GroupRef& g, bool streamk_ok) {
     {
         const int sms = sm_count();
         const int64_t items = int64_t(grid_x) * tiles;
-        if (P == 1 && splits == 1 && sms > 0 && items > sms && items < (int64_t(1) << 30)) {
+        if (splits == 1 && sms > 0 && items > sms && items < (int64_t(1) << 30)) {
             persist = 1;
             pl.n_tt = grid_x;
             pl.n_items = int32_t(items);
@@ -1081,26 +1064,25 @@ GemmPlan plan_gemm(const GroupRef& g, bool streamk_ok) {
     pl.persist = persist;
     // Stream-K: when the waves of whole items leave SMs idle (a last wave that is mostly
     // empty), cut the raw stages of all items into one equal range per SM. Both plans are
-    // costed with per 64-k step max(900, 4.1 per token of the CTA) cycles (measured on
-    // GB300: 922 at one tile of 208, 1170 at two of 144) plus ~3900 of fill per CTA (and
-    // ~5000 for a K split's cluster exchange); stream-K adds ~17000 for writing, publishing,
-    // staging and adding a partial tile and ~3300 for every further tail a head adds
-    // (per-CTA %globaltimer stamps: 147 KB written in ~3 us, staged and added in ~1.7 us, a
-    // slower store pass after it). So it is taken only where it is clearly faster (10 %):
-    // Llama-7B gate/up at M = 280, 172 tiles on 152 SMs, 84 -> 61 us; the q/k/v, o and down
-    // projections, whose tiles fill more of the SMs, gain nothing or lose.
+    // costed with the cycle model (and ~5000 for a K split's cluster exchange); stream-K adds, per
+    // token of the CTA, 59 cycles for writing, publishing, staging and adding a partial tile and
+    // 11.5 for every further tail a head adds (per-CTA %globaltimer stamps at 288 tokens: 147 KB
+    // written in ~3 us, staged and added in ~1.7 us, a slower store pass after it). It is taken
+    // where that gains 8 %. Measured with and without it, us per launch: Llama-7B gate/up at
+    // M = 280 49.8 / 63.8; 24000 x 4096 at M = 130 44.2 / 61.0; 5000 x 5056 at M = 300 30.0 / 35.2;
+    // not taken: Llama-7B o 22.9 / 20.2, Gemma-2B gate/up at M = 816 (every CTA ends several
+    // items) 108 / 104, ViT q/k/v 19.6 / 11.1.
     const int sms = sm_count();
     if (streamk_ok && !split && g.M >= 128 && sms > 0) {
         const int64_t nr_all = (g.K + kKR - 1) / kKR;
         const double nk = double((g.K + kKC - 1) / kKC);
-        auto step = [](int Pc, int Tc) { return std::max(900.0, 4.1 * Pc * Tc); };
         double cur;
         if (pl.persist)
-            cur = double((int64_t(pl.n_items) + sms - 1) / sms) * nk * step(P, T) + 3900.0;
+            cur = double((int64_t(pl.n_items) + sms - 1) / sms) * (nk * step_cycles(P, T) + item_cycles(P, T));
         else
             cur = double((int64_t(grid_x) * grid_y * splits + sms - 1) / sms) *
-                  (std::ceil(nk / splits) * step(P, T) + 3900.0 + (splits > 1 ? 5000.0 : 0.0));
-        struct Cand { int P, T, S, gap0, per_gap; int64_t n_tt; };
+                  (std::ceil(nk / splits) * step_cycles(P, T) + item_cycles(P, T) + (splits > 1 ? 5000.0 : 0.0));
+        struct Cand { int P, T, S; int64_t n_tt; };
         Cand cands[2];
         int nc = 0;
         {
@@ -1109,16 +1091,15 @@ GemmPlan plan_gemm(const GroupRef& g, bool streamk_ok) {
             const int S1 = g.fmt == EMB_Q8_0   ? pick_stages<EMB_Q8_0, false>(T1)
                            : g.fmt == EMB_Q4_0 ? pick_stages<EMB_Q4_0, false>(T1)
                                                : pick_stages<EMB_Q6_0, false>(T1);
-            cands[nc++] = Cand{1, T1, S1, 0, 0, tt1};
+            cands[nc++] = Cand{1, T1, S1, tt1};
             const int64_t t2 = 2 * ((g.M + 447) / 448);
             const int T2 = int(roundup((g.M + t2 - 1) / t2, 16));
-            int gap0 = 0, per_gap = 0;
-            const int S2 = g.fmt == EMB_Q8_0   ? pick_stages_pair<EMB_Q8_0>(T2, gap0, per_gap)
-                           : g.fmt == EMB_Q4_0 ? pick_stages_pair<EMB_Q4_0>(T2, gap0, per_gap)
-                                               : pick_stages_pair<EMB_Q6_0>(T2, gap0, per_gap);
-            if (S2 >= 2 && T2 <= 224) cands[nc++] = Cand{2, T2, S2, gap0, per_gap, t2 / 2};
+            const int S2 = g.fmt == EMB_Q8_0   ? pick_stages_pair<EMB_Q8_0>(T2)
+                           : g.fmt == EMB_Q4_0 ? pick_stages_pair<EMB_Q4_0>(T2)
+                                               : pick_stages_pair<EMB_Q6_0>(T2);
+            if (S2 >= 2 && T2 <= 224) cands[nc++] = Cand{2, T2, S2, t2 / 2};
         }
-        double best = cur / 1.1;
+        double best = cur / 1.08;
         for (int c = 0; c < nc; ++c) {
             const Cand& cd = cands[c];
             const int64_t items = cd.n_tt * tiles;
@@ -1128,15 +1109,14 @@ GemmPlan plan_gemm(const GroupRef& g, bool streamk_ok) {
             // a head adds the tails of the CTAs whose ranges start inside its item
             const int64_t per = std::max<int64_t>(1, U / G);
             const double tails = double(std::max<int64_t>(1, (nr_all + per - 1) / per));
-            const double t = double((U + G - 1) / G) * kStepsPerRaw * step(cd.P, cd.T) + 3900.0 + 17000.0 +
-                             3300.0 * (tails - 1.0);
+            const double ends = std::max(1.0, double(per) / double(nr_all));  // items a CTA ends
+            const double t = double((U + G - 1) / G) * kStepsPerRaw * step_cycles(cd.P, cd.T) +
+                             ends * item_cycles(cd.P, cd.T) + cd.P * cd.T * (59.0 + 11.5 * (tails - 1.0));
             if (t < best) {
                 best = t;
                 pl.T = cd.T;
                 pl.S = cd.S;
                 pl.P = cd.P;
-                pl.a_gap0 = cd.gap0;
-                pl.a_per_gap = cd.per_gap;
                 pl.splits = 1;
                 pl.persist = 1;
                 pl.streamk = 1;
@@ -1160,8 +1140,6 @@ cudaError_t launch_plan(const GroupRef& g, const GemmPlan& pl, bool pdl, int* st
     p.streamk = pl.streamk;
     p.n_tt = pl.n_tt;
     p.n_items = pl.n_items;
-    p.a_gap0 = pl.a_gap0;
-    p.a_per_gap = pl.a_per_gap;
     if (pl.streamk) {
         p.slot_floats = int32_t(sk_slot_bytes(P, T) / 4);
         p.ws_flag = static_cast<uint32_t*>(g.ws);
@@ -1202,6 +1180,7 @@ cudaError_t launch_plan(const GroupRef& g, const GemmPlan& pl, bool pdl, int* st
     p.T = T;
     p.P = P;
     p.stages = S;
+    p.a_stages = a_stages_of(split, T, P);
     p.splits = splits;
     p.epi = g.epi;
     p.tmem_cols = kTmemCols;

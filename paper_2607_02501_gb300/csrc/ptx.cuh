@@ -52,6 +52,19 @@ __device__ __forceinline__ bool mbar_try_wait(uint64_t* bar, uint32_t parity) {
     return ok != 0;
 }
 
+// Whether the phase with the given parity has completed; never suspends the thread.
+__device__ __forceinline__ bool mbar_test_wait(uint64_t* bar, uint32_t parity) {
+    uint32_t ok;
+    asm volatile(
+        "{\n\t.reg .pred p;\n\t"
+        "mbarrier.test_wait.parity.shared::cta.b64 p, [%1], %2;\n\t"
+        "selp.u32 %0, 1, 0, p;\n\t}"
+        : "=r"(ok)
+        : "r"(smem_u32(bar)), "r"(parity)
+        : "memory");
+    return ok != 0;
+}
+
 // Wait until the phase with the given parity has completed. Gives up after limit_ns,
 // or as soon as *abort is set by another thread of the CTA; returns false then.
 // On its own expiry it records kStatusTimeout and sets *abort for the other roles.
@@ -237,34 +250,48 @@ __device__ __forceinline__ void tc_fence_after() {
     asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
 }
 
-// D[tmem] (+)= A[smem desc] x B[smem desc]^T, bf16 inputs, fp32 accumulation.
-__device__ __forceinline__ void mma_bf16(uint32_t d_tmem, uint64_t a_desc, uint64_t b_desc,
-                                         uint32_t idesc, uint32_t accumulate) {
+// One thread of the (converged) warp, the same one every time. Tensor-core and TMA issue is
+// written as `if (elect_one())` in warp-uniform code on warp-uniform operands: the compiler then
+// keeps the operands in uniform registers, and a 128 x 64 x 16 MMA issues every 32 cycles, its
+// tensor time. Behind `if (lane == 0)`, or with operands it cannot prove uniform, every MMA cost
+// 100 to 200 cycles to issue whatever its size (measured on GB300, 4 MMAs per step: N = 64
+// 417-810 cycles per step against 129, N = 208 417-815 against 416).
+__device__ __forceinline__ bool elect_one() {
+    uint32_t p;
     asm volatile(
-        "{\n\t.reg .pred p;\n\t"
-        "setp.ne.b32 p, %4, 0;\n\t"
-        "tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n\t}" ::"r"(d_tmem),
-        "l"(a_desc), "l"(b_desc), "r"(idesc), "r"(accumulate)
-        : "memory");
+        "{\n\t.reg .pred q;\n\t"
+        "elect.sync _|q, 0xffffffff;\n\t"
+        "selp.u32 %0, 1, 0, q;\n\t}"
+        : "=r"(p));
+    return p != 0;
+}
+// A value that every lane of the warp holds alike, in a form the compiler knows to be uniform.
+template <typename T>
+__device__ __forceinline__ T warp_uniform(T v) {
+    return __shfl_sync(0xffffffffu, v, 0);
 }
 
 // D[tmem] (+)= A[tmem] x B[smem desc]^T: A (M = 128 rows) sits in TMEM, row i in lane i,
-// K along the columns, two bf16 per 32-bit column.
+// K along the columns, two bf16 per 32-bit column; issued by one elected thread of the warp
+// (call it converged, operands warp-uniform).
 __device__ __forceinline__ void mma_bf16_ta(uint32_t d_tmem, uint32_t a_tmem, uint64_t b_desc,
                                             uint32_t idesc, uint32_t accumulate) {
     asm volatile(
-        "{\n\t.reg .pred p;\n\t"
+        "{\n\t.reg .pred p, q;\n\t"
+        "elect.sync _|q, 0xffffffff;\n\t"
         "setp.ne.b32 p, %4, 0;\n\t"
-        "tcgen05.mma.cta_group::1.kind::f16 [%0], [%1], %2, %3, p;\n\t}" ::"r"(d_tmem),
+        "@q tcgen05.mma.cta_group::1.kind::f16 [%0], [%1], %2, %3, p;\n\t}" ::"r"(d_tmem),
         "r"(a_tmem), "l"(b_desc), "r"(idesc), "r"(accumulate)
         : "memory");
 }
 
-// Arrive (once) on the mbarrier when every tcgen05 operation issued so far by this
-// thread has completed.
+// Arrive (once) on the mbarrier when every tcgen05 operation issued so far by the elected
+// thread has completed (call it converged).
 __device__ __forceinline__ void mma_commit(uint64_t* bar) {
     asm volatile(
-        "tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(
+        "{\n\t.reg .pred q;\n\t"
+        "elect.sync _|q, 0xffffffff;\n\t"
+        "@q tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];\n\t}" ::"r"(
             smem_u32(bar))
         : "memory");
 }

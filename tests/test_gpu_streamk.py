@@ -145,3 +145,23 @@ def test_workspace_errors(cuda_device):
     with pytest.raises(emb.EmbError) as e:
         emb.emb_qlayer_seq(layers, M, ws[16:], n)
     assert e.value.status == emb.EMB_EALIGN
+
+
+@pytest.mark.parametrize("fmt,M,N,K", [(Q4, 280, 20600, 2048), (Q6, 300, 20100, 2112), (Q8, 250, 11500, 8160)])
+def test_streamk_parity_where_the_cycle_model_takes_it(cuda_device, fmt, M, N, K):
+    """Shapes whose whole tiles need a nearly empty second round (two token tiles per CTA, 161
+    and 158 tiles; one token tile, 90 tiles of a long row whose heads add two tails), ragged in
+    every dimension: stream-K is taken, within the bound of the plain schedule's operands, twice
+    alike, and the workspace comes back zero."""
+    W, Xb, img, X = _setup(fmt, M, N, K, 5 + N + K)
+    Y = torch.full((M, N), float("nan"), device="cuda")
+    n = emb.emb_qlayer_seq_workspace([(fmt, img, N, K, X, Y)], M)
+    assert n > 4096
+    ws = torch.zeros(n, dtype=torch.uint8, device="cuda")
+    _run(fmt, img, X, Y, M, N, K, ws)
+    Y2 = torch.full_like(Y, float("nan"))
+    _run(fmt, img, X, Y2, M, N, K, ws)
+    assert torch.equal(Y, Y2) and int(ws[:4096].count_nonzero()) == 0
+    rows = np.r_[0:N:97, N - 1]
+    Yref, B = oracle.qmatmul(fmt, oracle.quantize(fmt, W[rows]), Xb, len(rows), K)
+    check_close(Y.cpu().numpy()[:, rows], Yref, B, f"stream-K fmt={fmt} M={M} N={N} K={K}")
