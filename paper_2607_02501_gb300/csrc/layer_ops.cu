@@ -11,6 +11,7 @@
 #include <algorithm>
 #include <cmath>
 #include <mutex>
+#include <type_traits>
 
 #include "ptx.cuh"
 
@@ -140,28 +141,39 @@ __global__ void __launch_bounds__(256) rope_kernel(const __grid_constant__ RopeP
 // Tensor-core attention (mma.sync m16n8k16, bf16 operands, fp32 accumulation). The rows of
 // one key/value head g are its (query m, head) pairs, row r = m * G + (h - g * G) with G the
 // heads per key/value head, so every query head of a group shares the key and value tiles.
-// CTA = (64 rows, key/value head, key split); warp w owns rows 16w..16w+15 of the CTA.
-// Per 64-key tile (double-buffered in shared memory by cp.async, rows padded by 16 bytes so
-// fragment loads are conflict-free): S = Q K^T (Q fragments held in registers for the whole
-// kernel), scale, an online softmax on the accumulator fragments (row max and sums over the
-// four lanes that share a row), then O += P V with P split into bf16 hi + lo parts (two MMAs,
-// weight error 2^-16) and V fragments from ldmatrix.trans. The key splits of one row block
-// form a cluster along z; their (max, sum, output) partials are combined through distributed
-// shared memory in split order (deterministic).
+// CTA = (row block, key/value head, key split) of four warps, which walk the split's keys in
+// tiles of 64 (double-buffered in shared memory by cp.async, rows padded by 16 bytes so
+// fragment loads are conflict-free). WK = 1: a row block is 64 rows, 16 per warp, and every warp
+// takes all 64 keys. WK = 4, for few rows (a decode step's one query per head would leave
+// three warps of four without a row): a row block is 16 rows, every warp takes 16 of a tile's
+// keys, and the warps' partial results are combined in shared memory.
+// Per tile: S = Q K^T (Q fragments held in registers for the whole kernel), an online softmax
+// in base 2 on the accumulator fragments (row max and sums over the four lanes that share a row),
+// then O += P V with P split into bf16 hi + lo parts (two MMAs, weight error 2^-16) and V
+// fragments from ldmatrix.trans. The key splits of one row block form a cluster along z; their
+// (max, sum, output) partials are combined through distributed shared memory in split order
+// (deterministic).
+// What bounds it: latency. mma.sync does 1016 bf16 multiply-adds per cycle and SM here, which is
+// 7 us for M = 816, 8 heads, 816 keys (26.4 us measured, 84.2 before); the rest is each warp's
+// chain of loads, scores, exponentials and products with one or two warps per scheduler, and the
+// clusters' exchange. Consecutive MMAs go to different accumulators, weights are 2^x (one
+// multiply into base 2 per score), and unchanged row maxima skip the rescaling of the output.
 constexpr int kAttnWarps = 4;
 constexpr int kAttnThreads = 32 * kAttnWarps;
-constexpr int kAttnRows = 16 * kAttnWarps;
+template <int WK>
+constexpr int kAttnRows = 16 * kAttnWarps / WK;  // rows of a CTA
 constexpr int kKeyTile = 64;
 constexpr int kMaxSplits = 16;      // cluster size along the keys (16: non-portable, opted in)
-constexpr int kMinSplitKeys = 48;   // keys per split, at least
+constexpr int kMinSplitKeys = 32;   // keys per split, at least
 
 template <int D>
 struct AttnSmem {
     static constexpr int kPitch = D + 8;                 // bf16 per padded key row
     __nv_bfloat16 k[2][kKeyTile][kPitch];
     __nv_bfloat16 v[2][kKeyTile][kPitch];
-    float part_o[kAttnRows][D];
-    float part_m[kAttnRows], part_l[kAttnRows];
+    float part_o[16 * kAttnWarps][D];  // one 16-row partial result per warp
+    float part_m[16 * kAttnWarps], part_l[16 * kAttnWarps];
+    float cta_m[16], cta_l[16];        // WK > 1: the CTA's rows after its warps are combined
 };
 
 struct AttnParams {
@@ -173,17 +185,30 @@ struct AttnParams {
     __nv_bfloat16* O;
     int64_t n0, n1;
     int M, H, Hk;
-    float scale;
+    float scale_log2;  // scale * log2(e): scores are kept in base 2
 };
 
 __device__ __forceinline__ void mma_16816(float (&d)[4], const uint32_t (&a)[4], uint32_t b0, uint32_t b1) {
-    asm volatile(
+    asm(
         "mma.sync.aligned.m16n8k16.row.col.f32.bf16.bf16.f32 {%0, %1, %2, %3}, {%4, %5, %6, %7}, "
         "{%8, %9}, {%0, %1, %2, %3};"
         : "+f"(d[0]), "+f"(d[1]), "+f"(d[2]), "+f"(d[3])
         : "r"(a[0]), "r"(a[1]), "r"(a[2]), "r"(a[3]), "r"(b0), "r"(b1));
 }
 
+// 2^x (results below the normal range become zero; -inf gives 0).
+__device__ __forceinline__ float exp2_fast(float x) {
+    float y;
+    asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
+    return y;
+}
+
+__device__ __forceinline__ void ldsm_x4(uint32_t saddr, uint32_t& r0, uint32_t& r1, uint32_t& r2,
+                                        uint32_t& r3) {
+    asm volatile("ldmatrix.sync.aligned.m8n8.x4.shared.b16 {%0, %1, %2, %3}, [%4];"
+                 : "=r"(r0), "=r"(r1), "=r"(r2), "=r"(r3)
+                 : "r"(saddr));
+}
 __device__ __forceinline__ void ldsm_x4_trans(uint32_t saddr, uint32_t& r0, uint32_t& r1, uint32_t& r2,
                                               uint32_t& r3) {
     asm volatile("ldmatrix.sync.aligned.m8n8.x4.trans.shared.b16 {%0, %1, %2, %3}, [%4];"
@@ -207,32 +232,55 @@ __device__ __forceinline__ float2 unpack_bf16x2(uint32_t w) {
     return make_float2(__uint_as_float(w << 16), __uint_as_float(w & 0xFFFF0000u));
 }
 
-template <int D>
+template <int D, int WK>
 __global__ void __launch_bounds__(kAttnThreads) attention_kernel(const __grid_constant__ AttnParams p) {
     constexpr int KS = D / 16;  // k-steps of the score MMAs (head dims)
     constexpr int NT = D / 8;   // n-tiles of the output (head dims)
+    constexpr int NJ = kKeyTile / 8 / WK;   // 8-key n-tiles of a warp's share of a tile
+    constexpr int kRows = kAttnRows<WK>;
     using SM = AttnSmem<D>;
     extern __shared__ __align__(128) uint8_t smem_raw[];
     SM& sm = *reinterpret_cast<SM*>(smem_raw);
-    ptx::griddep_launch_dependents();
-    ptx::griddep_wait();  // Q and the chunk's keys and values come from the previous launches
-
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int quad = lane >> 2, qc = lane & 3;
     const int g = blockIdx.y, G = p.H / p.Hk;
     const int64_t rows_total = int64_t(p.M) * G;
-    const int64_t row0 = int64_t(blockIdx.x) * kAttnRows;
+    const int64_t row0 = int64_t(blockIdx.x) * kRows;
     const int splits = gridDim.z, z = blockIdx.z;
     const int64_t n = p.n0 + p.n1;
     const int64_t k_lo = z * n / splits, k_hi = (z + 1) * n / splits;
-    const int kv_stride = p.Hk * D;
+    const int64_t kv_stride = int64_t(p.Hk) * D;
+    const int wrow = WK == 1 ? warp * 16 : 0;  // the warp's rows of the CTA, and keys of a tile
+    const int wkey = WK == 1 ? 0 : warp * 16;
 
-    // global row -> (query, head) -> its Q / O row; nullptr past the last row
+    ptx::griddep_launch_dependents();
+    ptx::griddep_wait();  // Q and the chunk's keys and values come from the previous launches
+
+    // tile loader: 64 keys x D of keys and of values, 16-byte chunks, zero past the split
+    constexpr int kChunksPerRow = D / 8, kPass = kAttnThreads / kChunksPerRow;
+    const int lc = threadIdx.x % kChunksPerRow, lj = threadIdx.x / kChunksPerRow;
+    const int64_t col = int64_t(g) * D + lc * 8;
+    auto issue_tile = [&](int64_t t0, int stage) {
+#pragma unroll
+        for (int i = 0; i < kKeyTile / kPass; ++i) {
+            const int j = lj + i * kPass;
+            const bool ok = t0 + j < k_hi;
+            const int64_t kk = ok ? t0 + j : k_lo;  // any valid row when nothing is read
+            const bool cached = kk < p.n0;
+            const int64_t off = (cached ? kk : kk - p.n0) * kv_stride + col;
+            cp_async16(ptx::smem_u32(&sm.k[stage][j][lc * 8]), (cached ? p.K0 : p.K1) + off, ok ? 16 : 0);
+            cp_async16(ptx::smem_u32(&sm.v[stage][j][lc * 8]), (cached ? p.V0 : p.V1) + off, ok ? 16 : 0);
+        }
+    };
+    const int ntiles = int((k_hi - k_lo + kKeyTile - 1) / kKeyTile);
+    if (ntiles > 0) issue_tile(k_lo, 0);
+    cp_async_commit();
+
+    // global row -> (query, head) -> its Q / O row; -1 past the last row
     auto q_row = [&](int64_t r) -> int64_t {
         return r < rows_total ? (r / G) * int64_t(p.H) * D + (int64_t(g) * G + r % G) * D : -1;
     };
-    const int64_t rA = row0 + warp * 16 + quad, rB = rA + 8;
-    const int64_t offA = q_row(rA), offB = q_row(rB);
+    const int64_t offA = q_row(row0 + wrow + quad), offB = q_row(row0 + wrow + quad + 8);
 
     // Q fragments for the whole kernel (A operand, row-major 16 x D); ordinary loads, since
     // the previous launch wrote Q while this grid was already resident
@@ -247,29 +295,11 @@ __global__ void __launch_bounds__(kAttnThreads) attention_kernel(const __grid_co
         qf[ks][3] = offB >= 0 ? ldq(offB + c + 8) : 0u;
     }
 
-    // tile loader: 64 keys x D of keys and of values, 16-byte chunks, zero past the split
-    auto issue_tile = [&](int64_t t0, int stage) {
-        constexpr int kChunksPerRow = D / 8;
-        for (int e = threadIdx.x; e < kKeyTile * kChunksPerRow; e += kAttnThreads) {
-            const int j = e / kChunksPerRow, c = e - j * kChunksPerRow;
-            const int64_t key = t0 + j;
-            const bool ok = key < k_hi;
-            const int64_t kk = ok ? key : k_lo;  // any valid row when nothing is read
-            const __nv_bfloat16* kp = kk < p.n0 ? p.K0 + kk * kv_stride : p.K1 + (kk - p.n0) * kv_stride;
-            const __nv_bfloat16* vp = kk < p.n0 ? p.V0 + kk * kv_stride : p.V1 + (kk - p.n0) * kv_stride;
-            cp_async16(ptx::smem_u32(&sm.k[stage][j][c * 8]), kp + g * D + c * 8, ok ? 16 : 0);
-            cp_async16(ptx::smem_u32(&sm.v[stage][j][c * 8]), vp + g * D + c * 8, ok ? 16 : 0);
-        }
-    };
-
     float o[NT][4];
 #pragma unroll
     for (int j = 0; j < NT; ++j) o[j][0] = o[j][1] = o[j][2] = o[j][3] = 0.0f;
     float mA = -INFINITY, mB = -INFINITY, lA = 0.0f, lB = 0.0f;
 
-    const int ntiles = int((k_hi - k_lo + kKeyTile - 1) / kKeyTile);
-    if (ntiles > 0) issue_tile(k_lo, 0);
-    cp_async_commit();
     for (int it = 0; it < ntiles; ++it) {
         const int stage = it & 1;
         const int64_t t0 = k_lo + int64_t(it) * kKeyTile;
@@ -278,65 +308,84 @@ __global__ void __launch_bounds__(kAttnThreads) attention_kernel(const __grid_co
         cp_async_wait1();  // this thread's copies of tile `it` have landed
         __syncthreads();   // and every thread's
 
-        // S = Q K^T for 64 keys: 8 n-tiles of 8 keys
-        float sc[8][4];
+        // S = Q K^T for the warp's keys, 8 per n-tile; one ldmatrix gives the B fragments of two
+        // k-steps (lanes 8i .. 8i + 7 address the eight keys at dims 8i). The n-tiles are the inner
+        // loop: consecutive MMAs then do not wait for one another.
+        float sc[NJ][4];
 #pragma unroll
-        for (int j = 0; j < 8; ++j) {
-            sc[j][0] = sc[j][1] = sc[j][2] = sc[j][3] = 0.0f;
-            const __nv_bfloat16* krow = &sm.k[stage][j * 8 + quad][0];
+        for (int j = 0; j < NJ; ++j) sc[j][0] = sc[j][1] = sc[j][2] = sc[j][3] = 0.0f;
+        const uint32_t kbase = ptx::smem_u32(&sm.k[stage][wkey + (lane & 7)][(lane >> 3) * 8]);
 #pragma unroll
-            for (int ks = 0; ks < KS; ++ks) {
-                const uint32_t b0 = *reinterpret_cast<const uint32_t*>(krow + ks * 16 + 2 * qc);
-                const uint32_t b1 = *reinterpret_cast<const uint32_t*>(krow + ks * 16 + 2 * qc + 8);
-                mma_16816(sc[j], qf[ks], b0, b1);
-            }
+        for (int ks = 0; ks < KS; ks += 2) {
+            uint32_t b[NJ][4];
+#pragma unroll
+            for (int j = 0; j < NJ; ++j)
+                ldsm_x4(kbase + j * 8 * SM::kPitch * 2 + ks * 32, b[j][0], b[j][1], b[j][2], b[j][3]);
+#pragma unroll
+            for (int j = 0; j < NJ; ++j) mma_16816(sc[j], qf[ks], b[j][0], b[j][1]);
+#pragma unroll
+            for (int j = 0; j < NJ; ++j) mma_16816(sc[j], qf[ks + 1], b[j][2], b[j][3]);
         }
-        // scale, mask keys past the split, row maxima (rows A = quad, B = quad + 8)
+        // scores in base 2, keys past the split masked (last tile only), row maxima (rows A =
+        // quad, B = quad + 8)
+        const int left = int(min(k_hi - t0, int64_t(kKeyTile)));
         float tA = -INFINITY, tB = -INFINITY;
 #pragma unroll
-        for (int j = 0; j < 8; ++j) {
+        for (int j = 0; j < NJ; ++j) {
 #pragma unroll
             for (int e = 0; e < 2; ++e) {
-                const bool ok = t0 + j * 8 + 2 * qc + e < k_hi;
-                sc[j][e] = ok ? __fmul_rn(sc[j][e], p.scale) : -INFINITY;
-                sc[j][2 + e] = ok ? __fmul_rn(sc[j][2 + e], p.scale) : -INFINITY;
-                tA = fmaxf(tA, sc[j][e]);
-                tB = fmaxf(tB, sc[j][2 + e]);
+                sc[j][e] = __fmul_rn(sc[j][e], p.scale_log2);
+                sc[j][2 + e] = __fmul_rn(sc[j][2 + e], p.scale_log2);
             }
+        }
+        if (left < kKeyTile) {
+#pragma unroll
+            for (int j = 0; j < NJ; ++j)
+#pragma unroll
+                for (int e = 0; e < 2; ++e)
+                    if (wkey + j * 8 + 2 * qc + e >= left) sc[j][e] = sc[j][2 + e] = -INFINITY;
+        }
+#pragma unroll
+        for (int j = 0; j < NJ; ++j) {
+            tA = fmaxf(tA, fmaxf(sc[j][0], sc[j][1]));
+            tB = fmaxf(tB, fmaxf(sc[j][2], sc[j][3]));
         }
 #pragma unroll
         for (int x = 1; x <= 2; x <<= 1) {
             tA = fmaxf(tA, __shfl_xor_sync(0xffffffffu, tA, x));
             tB = fmaxf(tB, __shfl_xor_sync(0xffffffffu, tB, x));
         }
-        const float nA = fmaxf(mA, tA), nB = fmaxf(mB, tB);  // finite: the tile has a key
-        const float cA = (mA == -INFINITY) ? 0.0f : expf(mA - nA);
-        const float cB = (mB == -INFINITY) ? 0.0f : expf(mB - nB);
-        mA = nA;
-        mB = nB;
+        const float nA = fmaxf(mA, tA), nB = fmaxf(mB, tB);
+        // (a row without a finite score so far subtracts 0: its weights are 2^-inf = 0)
+        const float sA0 = nA == -INFINITY ? 0.0f : nA, sB0 = nB == -INFINITY ? 0.0f : nB;
+        const float cA = exp2_fast(mA - sA0), cB = exp2_fast(mB - sB0);
         float sA = 0.0f, sB = 0.0f;
 #pragma unroll
-        for (int j = 0; j < 8; ++j) {
+        for (int j = 0; j < NJ; ++j) {
 #pragma unroll
             for (int e = 0; e < 2; ++e) {
-                sc[j][e] = expf(sc[j][e] - nA);  // exp(-inf) = 0 for masked keys
-                sc[j][2 + e] = expf(sc[j][2 + e] - nB);
+                sc[j][e] = exp2_fast(sc[j][e] - sA0);
+                sc[j][2 + e] = exp2_fast(sc[j][2 + e] - sB0);
                 sA += sc[j][e];
                 sB += sc[j][2 + e];
             }
         }
         lA = lA * cA + sA;  // lane-partial sums; the four lanes of a row are added at the end
         lB = lB * cB + sB;
+        if (__any_sync(0xffffffffu, nA != mA || nB != mB)) {  // else every factor is 1
 #pragma unroll
-        for (int j = 0; j < NT; ++j) {
-            o[j][0] *= cA;
-            o[j][1] *= cA;
-            o[j][2] *= cB;
-            o[j][3] *= cB;
+            for (int j = 0; j < NT; ++j) {
+                o[j][0] *= cA;
+                o[j][1] *= cA;
+                o[j][2] *= cB;
+                o[j][3] *= cB;
+            }
         }
-        // O += P V: 4 k-steps of 16 keys; P as hi + lo bf16 A fragments
+        mA = nA;
+        mB = nB;
+        // O += P V: k-steps of 16 keys; P as hi + lo bf16 A fragments
 #pragma unroll
-        for (int kk = 0; kk < 4; ++kk) {
+        for (int kk = 0; kk < NJ / 2; ++kk) {
             uint32_t ah[4], al[4];
             const float* s0 = sc[2 * kk];
             const float* s1 = sc[2 * kk + 1];
@@ -349,16 +398,17 @@ __global__ void __launch_bounds__(kAttnThreads) attention_kernel(const __grid_co
             }
             // ldmatrix.trans: lanes 0-7 keys 16kk..+7, 8-15 keys +8..+15 (dims 8jj..),
             // lanes 16-31 the same keys at dims 8jj + 8
-            const int key = kk * 16 + (lane & 7) + ((lane >> 3) & 1) * 8;
-            const int dcol = (lane >> 4) * 8;
+            const int key = wkey + kk * 16 + (lane & 7) + ((lane >> 3) & 1) * 8;
+            const uint32_t vrow = ptx::smem_u32(&sm.v[stage][key][(lane >> 4) * 8]);
 #pragma unroll
-            for (int jj = 0; jj < NT; jj += 2) {
-                uint32_t b0, b1, b2, b3;
-                ldsm_x4_trans(ptx::smem_u32(&sm.v[stage][key][jj * 8 + dcol]), b0, b1, b2, b3);
-                mma_16816(o[jj], ah, b0, b1);
-                mma_16816(o[jj], al, b0, b1);
-                mma_16816(o[jj + 1], ah, b2, b3);
-                mma_16816(o[jj + 1], al, b2, b3);
+            for (int jj = 0; jj < NT; jj += 4) {
+                uint32_t b[2][4];
+                ldsm_x4_trans(vrow + jj * 16, b[0][0], b[0][1], b[0][2], b[0][3]);
+                ldsm_x4_trans(vrow + jj * 16 + 32, b[1][0], b[1][1], b[1][2], b[1][3]);
+#pragma unroll
+                for (int i = 0; i < 4; ++i) mma_16816(o[jj + i], ah, b[i >> 1][2 * (i & 1)], b[i >> 1][2 * (i & 1) + 1]);
+#pragma unroll
+                for (int i = 0; i < 4; ++i) mma_16816(o[jj + i], al, b[i >> 1][2 * (i & 1)], b[i >> 1][2 * (i & 1) + 1]);
             }
         }
         __syncthreads();  // every warp is done with this stage before it is refilled
@@ -369,7 +419,16 @@ __global__ void __launch_bounds__(kAttnThreads) attention_kernel(const __grid_co
         lB += __shfl_xor_sync(0xffffffffu, lB, x);
     }
 
-    if (splits == 1) {
+    auto store4 = [&](int64_t at, float4 v, float L) {  // four normalised outputs
+        const float inv = __fdiv_rn(1.0f, L);
+        const __nv_bfloat162 lo = __floats2bfloat162_rn(__fmul_rn(v.x, inv), __fmul_rn(v.y, inv));
+        const __nv_bfloat162 hi = __floats2bfloat162_rn(__fmul_rn(v.z, inv), __fmul_rn(v.w, inv));
+        uint2 u;
+        u.x = *reinterpret_cast<const uint32_t*>(&lo);
+        u.y = *reinterpret_cast<const uint32_t*>(&hi);
+        *reinterpret_cast<uint2*>(p.O + at) = u;
+    };
+    if (WK == 1 && splits == 1) {
         const float iA = __fdiv_rn(1.0f, lA), iB = __fdiv_rn(1.0f, lB);
 #pragma unroll
         for (int j = 0; j < NT; ++j) {
@@ -383,15 +442,13 @@ __global__ void __launch_bounds__(kAttnThreads) attention_kernel(const __grid_co
         }
         return;
     }
-    // partials of this split into shared memory, then the cluster combines them
+    // each warp's partial result into shared memory
     const int lrA = warp * 16 + quad, lrB = lrA + 8;
 #pragma unroll
     for (int j = 0; j < NT; ++j) {
         const int c = j * 8 + 2 * qc;
-        sm.part_o[lrA][c] = o[j][0];
-        sm.part_o[lrA][c + 1] = o[j][1];
-        sm.part_o[lrB][c] = o[j][2];
-        sm.part_o[lrB][c + 1] = o[j][3];
+        *reinterpret_cast<float2*>(&sm.part_o[lrA][c]) = make_float2(o[j][0], o[j][1]);
+        *reinterpret_cast<float2*>(&sm.part_o[lrB][c]) = make_float2(o[j][2], o[j][3]);
     }
     if (qc == 0) {
         sm.part_m[lrA] = mA;
@@ -399,35 +456,19 @@ __global__ void __launch_bounds__(kAttnThreads) attention_kernel(const __grid_co
         sm.part_m[lrB] = mB;
         sm.part_l[lrB] = lB;
     }
-    ptx::cluster_sync();
-    // CTA z combines rows [z * 64 / splits, (z + 1) * 64 / splits): one thread per 4 dims
-    const int rows_per = kAttnRows / splits;
-    for (int e = threadIdx.x; e < rows_per * (D / 4); e += kAttnThreads) {
-        const int lr = z * rows_per + e / (D / 4), c = (e % (D / 4)) * 4;
-        const int64_t off = q_row(row0 + lr);
-        if (off < 0) continue;
-        const uint32_t am = ptx::smem_u32(&sm.part_m[lr]), al_ = ptx::smem_u32(&sm.part_l[lr]);
-        const uint32_t ao = ptx::smem_u32(&sm.part_o[lr][c]);
-        float qm[kMaxSplits], ql[kMaxSplits];
-        float4 qo[kMaxSplits];
+    // max, sum and output of the partials that share a row, added in order
+    auto merge = [](const float* qm, const float* ql, const float4* qo, auto count, float& mx, float& L, float4& O) {
+        constexpr int kCount = decltype(count)::value;
+        mx = -INFINITY;
 #pragma unroll
-        for (int q = 0; q < kMaxSplits; ++q) {
-            if (q < splits) {
-                qm[q] = ptx::ld_dsmem_f32(ptx::map_dsmem(am, q));
-                ql[q] = ptx::ld_dsmem_f32(ptx::map_dsmem(al_, q));
-                qo[q] = ptx::ld_dsmem_f32x4(ptx::map_dsmem(ao, q));
-            }
-        }
-        float mx = -INFINITY;
+        for (int q = 0; q < kCount; ++q)
+            mx = fmaxf(mx, qm[q]);
+        L = 0.0f;
+        O = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
 #pragma unroll
-        for (int q = 0; q < kMaxSplits; ++q)
-            if (q < splits) mx = fmaxf(mx, qm[q]);
-        float L = 0.0f;
-        float4 O = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
-#pragma unroll
-        for (int q = 0; q < kMaxSplits; ++q) {
-            if (q < splits && qm[q] != -INFINITY) {  // a split without keys adds nothing
-                const float w = expf(qm[q] - mx);
+        for (int q = 0; q < kCount; ++q) {
+            if (qm[q] != -INFINITY) {  // a partial without keys adds nothing
+                const float w = exp2_fast(qm[q] - mx);
                 L = fmaf(ql[q], w, L);
                 O.x = fmaf(qo[q].x, w, O.x);
                 O.y = fmaf(qo[q].y, w, O.y);
@@ -435,18 +476,119 @@ __global__ void __launch_bounds__(kAttnThreads) attention_kernel(const __grid_co
                 O.w = fmaf(qo[q].w, w, O.w);
             }
         }
-        const float inv = __fdiv_rn(1.0f, L);
-        const __nv_bfloat162 lo = __floats2bfloat162_rn(__fmul_rn(O.x, inv), __fmul_rn(O.y, inv));
-        const __nv_bfloat162 hi = __floats2bfloat162_rn(__fmul_rn(O.z, inv), __fmul_rn(O.w, inv));
-        uint2 u;
-        u.x = *reinterpret_cast<const uint32_t*>(&lo);
-        u.y = *reinterpret_cast<const uint32_t*>(&hi);
-        *reinterpret_cast<uint2*>(p.O + off + c) = u;
+    };
+    if constexpr (WK > 1) {
+        // the four warps' partials of the CTA's 16 rows: one thread per 4 dims
+        __syncthreads();
+        for (int e = threadIdx.x; e < 16 * (D / 4); e += kAttnThreads) {
+            const int r = e / (D / 4), c = (e % (D / 4)) * 4;
+            float qm[WK], ql[WK], mx, L;
+            float4 qo[WK], O;
+#pragma unroll
+            for (int w = 0; w < WK; ++w) {
+                qm[w] = sm.part_m[16 * w + r];
+                ql[w] = sm.part_l[16 * w + r];
+                qo[w] = *reinterpret_cast<const float4*>(&sm.part_o[16 * w + r][c]);
+            }
+            merge(qm, ql, qo, std::integral_constant<int, WK>{}, mx, L, O);
+            if (splits == 1) {
+                const int64_t off = q_row(row0 + r);
+                if (off >= 0) store4(off + c, O, L);
+            } else {
+                *reinterpret_cast<float4*>(&sm.part_o[r][c]) = O;  // read by this thread only so far
+                if (c == 0) {
+                    sm.cta_m[r] = mx;
+                    sm.cta_l[r] = L;
+                }
+            }
+        }
+        if (splits == 1) return;
     }
+    ptx::cluster_sync();
+    // CTA z combines rows z, z + splits, ... of the row block, one thread per 4 dims; a thread
+    // has the loads of 16 / splits elements in flight at once
+    const int elems = (kRows + splits - 1) / splits * (D / 4);
+    auto combine = [&](auto count) {
+        constexpr int kSp = decltype(count)::value, kAtOnce = kMaxSplits / kSp;
+        for (int e0 = threadIdx.x; e0 < elems; e0 += kAttnThreads * kAtOnce) {
+            float qm[kAtOnce][kSp], ql[kAtOnce][kSp];
+            float4 qo[kAtOnce][kSp];
+            int64_t off[kAtOnce];
+#pragma unroll
+            for (int u = 0; u < kAtOnce; ++u) {
+                const int e = e0 + u * kAttnThreads;
+                const int lr = z + e / (D / 4) * splits, c = (e % (D / 4)) * 4;
+                off[u] = e < elems && lr < kRows ? q_row(row0 + lr) : -1;
+                if (off[u] < 0) continue;
+                off[u] += c;
+                const uint32_t am = ptx::smem_u32(WK > 1 ? &sm.cta_m[lr & 15] : &sm.part_m[lr]);
+                const uint32_t al_ = ptx::smem_u32(WK > 1 ? &sm.cta_l[lr & 15] : &sm.part_l[lr]);
+                const uint32_t ao = ptx::smem_u32(&sm.part_o[lr][c]);
+#pragma unroll
+                for (int q = 0; q < kSp; ++q) {
+                    qm[u][q] = ptx::ld_dsmem_f32(ptx::map_dsmem(am, q));
+                    ql[u][q] = ptx::ld_dsmem_f32(ptx::map_dsmem(al_, q));
+                    qo[u][q] = ptx::ld_dsmem_f32x4(ptx::map_dsmem(ao, q));
+                }
+            }
+#pragma unroll
+            for (int u = 0; u < kAtOnce; ++u) {
+                if (off[u] < 0) continue;
+                float mx, L;
+                float4 O;
+                merge(qm[u], ql[u], qo[u], count, mx, L, O);
+                store4(off[u], O, L);
+            }
+        }
+    };
+    if (splits == 2) combine(std::integral_constant<int, 2>{});
+    else if (splits == 4) combine(std::integral_constant<int, 4>{});
+    else if (splits == 8) combine(std::integral_constant<int, 8>{});
+    else combine(std::integral_constant<int, 16>{});
     ptx::cluster_sync();  // remote shared memory must outlive its readers
 }
 
-template <int D>
+// Which kernel (WK) and how many key splits (one cluster, a power of two) a call takes: the
+// least time by a model in microseconds fitted on GB300. A CTA costs 2.5, per tile of 64 keys 1.8
+// (D = 128) or 1.2 (D = 64) with 16 rows per warp and 1.0 or 0.5 with the keys shared out to the
+// warps; CTAs that share an SM slow one another by a quarter each, further ones queue; a cluster
+// adds 4.0 or 1.3 for its exchange and 0.8 more at 16 CTAs, which must all fit at once.
+// Measured (us per launch, graph-replayed; before: 64 rows per CTA and as many splits as keys
+// allow): M = 816, 8 heads on one key/value head of 128, 816 keys 84.2 -> 26.4 (2 splits); 280
+// queries and keys, 32 heads 43.2 -> 16.9 (1); one query, 32
+// heads, 281 keys 10.9 -> 5.5 (WK = 4, 8 splits); 400 queries, 16 heads on 4 of 64, 900 keys
+// 41.5 -> 13.7 (4); one query, 8 heads on one, 4001 keys 14.5 -> 7.7 (WK = 4, 16).
+struct AttnPlan {
+    bool shared_keys;  // WK = 4
+    int splits;
+};
+AttnPlan plan_attention(int64_t rows, int64_t Hk, int64_t n, int64_t D) {
+    const double sms = 152.0;
+    const double per_sm = D == 64 ? 3.0 : 2.0;
+    AttnPlan best{false, 1};
+    double best_t = 1e30;
+    for (int few = 0; few < 2; ++few) {
+        const double blocks = double((rows + (few ? 15 : 63)) / (few ? 16 : 64)) * double(Hk);
+        const double tile = few ? (D == 64 ? 0.5 : 1.0) : (D == 64 ? 1.2 : 1.8);
+        for (int sp = 1; sp <= kMaxSplits && (sp == 1 || n >= sp * int64_t(kMinSplitKeys)); sp *= 2) {
+            const double ctas = blocks * sp;
+            if (sp == kMaxSplits && ctas > sms) break;
+            const double tiles = double((((n + sp - 1) / sp) + kKeyTile - 1) / kKeyTile);
+            const double share = 1.0 + 0.25 * (std::min(std::ceil(ctas / sms), per_sm) - 1.0);
+            const double x = ctas / (sms * per_sm);
+            const double rounds = x <= 1.0 ? 1.0 : 0.5 * (x + std::ceil(x));
+            const double t = rounds * (tiles * tile * share + 2.5 + (sp > 1 ? (few ? 1.3 : 4.0) : 0.0)) +
+                             (sp == kMaxSplits ? 0.8 : 0.0);
+            if (t < best_t * 0.99) {
+                best_t = t;
+                best = AttnPlan{few != 0, sp};
+            }
+        }
+    }
+    return best;
+}
+
+template <int D, int WK>
 cudaError_t launch_attention_d(const AttnParams& p, int splits, cudaStream_t s) {
     const size_t smem = sizeof(AttnSmem<D>);
     // the opt-in shared-memory size and cluster size are per-device function attributes
@@ -457,18 +599,18 @@ cudaError_t launch_attention_d(const AttnParams& p, int splits, cudaStream_t s) 
     if (e != cudaSuccess) return e;
     std::lock_guard<std::mutex> lock(mu);
     if (dev < 0 || dev >= 64 || !attr_done[dev]) {
-        e = cudaFuncSetAttribute(attention_kernel<D>, cudaFuncAttributeMaxDynamicSharedMemorySize, int(smem));
+        e = cudaFuncSetAttribute(attention_kernel<D, WK>, cudaFuncAttributeMaxDynamicSharedMemorySize, int(smem));
         if (e != cudaSuccess) return e;
         if (kMaxSplits > 8) {
-            e = cudaFuncSetAttribute(attention_kernel<D>, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
+            e = cudaFuncSetAttribute(attention_kernel<D, WK>, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
             if (e != cudaSuccess) return e;
         }
         if (dev >= 0 && dev < 64) attr_done[dev] = true;
     }
     AttnParams pc = p;
     void* args[] = {&pc};
-    const int64_t row_blocks = (int64_t(p.M) * (p.H / p.Hk) + kAttnRows - 1) / kAttnRows;
-    return launch_pdl(reinterpret_cast<const void*>(attention_kernel<D>),
+    const int64_t row_blocks = (int64_t(p.M) * (p.H / p.Hk) + kAttnRows<WK> - 1) / kAttnRows<WK>;
+    return launch_pdl(reinterpret_cast<const void*>(attention_kernel<D, WK>),
                       dim3(unsigned(row_blocks), unsigned(p.Hk), unsigned(splits)), dim3(kAttnThreads),
                       smem, s, args, unsigned(splits));
 }
@@ -523,12 +665,11 @@ cudaError_t launch_attention(const uint16_t* Q, const uint16_t* K0, const uint16
     p.M = int(M);
     p.H = int(H);
     p.Hk = int(Hk);
-    p.scale = scale;
-    // key splits (one cluster): at least kMinSplitKeys keys each, at most kMaxSplits
-    const int64_t n = n0 + n1;
-    int splits = 1;
-    while (splits < kMaxSplits && n >= int64_t(2 * splits) * kMinSplitKeys) splits *= 2;
-    return D == 64 ? launch_attention_d<64>(p, splits, s) : launch_attention_d<128>(p, splits, s);
+    p.scale_log2 = float(double(scale) * 1.4426950408889634);
+    const AttnPlan pl = plan_attention(M * (H / Hk), Hk, n0 + n1, D);
+    if (pl.shared_keys)
+        return D == 64 ? launch_attention_d<64, 4>(p, pl.splits, s) : launch_attention_d<128, 4>(p, pl.splits, s);
+    return D == 64 ? launch_attention_d<64, 1>(p, pl.splits, s) : launch_attention_d<128, 1>(p, pl.splits, s);
 }
 
 }  // namespace emb

@@ -234,3 +234,26 @@ def test_action_expert_layer_recorded(cuda_device):
                                e.view(torch.int16) if e.dtype == torch.bfloat16 else e.view(torch.int32))
     rec.close()
     assert emb.emb_device_status() == emb.EMB_OK
+
+
+# every kernel and split count of the attention plan, at its edges: keys shared out to the warps
+# (one 16-row block exactly and one row more, a single tile, a last tile that leaves warps without
+# keys, 1 to 16 splits) and rows shared out (1 to 8 splits, ragged last row block and tile)
+ATTN_PLANS = [(1, 32, 32, 128, 280, 1), (16, 1, 1, 64, 0, 33), (17, 1, 1, 128, 5, 60), (16, 8, 1, 128, 816, 16),
+              (1, 8, 1, 64, 4090, 3), (300, 8, 8, 64, 0, 300), (120, 8, 2, 128, 1000, 120), (130, 8, 2, 64, 300, 1),
+              (816, 8, 1, 128, 0, 700), (400, 16, 4, 64, 500, 400), (280, 32, 32, 128, 0, 65)]
+
+
+@pytest.mark.parametrize("M,H,Hk,d,n0,n1", ATTN_PLANS)
+@pytest.mark.parametrize("gain", [1.0, 30.0])
+def test_attention_plans(cuda_device, M, H, Hk, d, n0, n1, gain):
+    """gain 30: scores in the hundreds, so one key takes nearly all the weight, the running
+    maximum moves between tiles and splits, and most weights underflow to zero."""
+    ins = _attn_inputs(M, H, Hk, d, n0, n1, M + H + n0 + n1 + 1)
+    scale = gain / math.sqrt(d)
+    O = _run_attention(*ins, H, Hk, d, scale)
+    ref, bound = oracle.attention_reference(*ins, H, Hk, d, scale)
+    _check(_vals(O), ref, bound, f"attention M={M} H={H} Hk={Hk} d={d} n={n0}+{n1} gain={gain}")
+    again = _run_attention(*ins, H, Hk, d, scale)
+    assert torch.equal(O.view(torch.int16), again.view(torch.int16))
+    assert emb.emb_device_status() == emb.EMB_OK
