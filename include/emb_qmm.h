@@ -125,7 +125,8 @@ EMB_API emb_status emb_quantize_q6_0(const float* W, int64_t N, int64_t K, void*
  * action chunks, M = 250..820 prefix prefill) on the Table 3 weight formats.
  * Y [M][N] fp32 = X [M][K] bf16  x  w'^T, w' the dequantised weights of W_blocks.
  * X, Y: device, 16-byte aligned; W_blocks as produced by emb_quantize_*.
- * Small M (M <= 4, action-token decode) runs a weight-streaming GEMV that dequantises
+ * Small M (M <= 4, action-token decode, and most layers up to M = 16, with the accuracy of
+ * M <= 4) runs a weight-streaming GEMV that dequantises
  * in registers; larger M (action-chunk denoising, prefix prefill) runs a tcgen05
  * tensor-core GEMM that dequantises shared-memory tiles to bf16.
  * Accuracy, per element, with Y_exact from the same dequantised weights w' and the

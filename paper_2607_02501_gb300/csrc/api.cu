@@ -23,7 +23,7 @@ __device__ int g_status_read;  // where emb_device_status's exchange leaves the 
 constexpr size_t kScratchBytes = size_t(48) << 20;
 __device__ __align__(256) unsigned char g_scratch[kScratchBytes];
 
-// Token counts up to this run the GEMV; above it, the tensor-core GEMM.
+// Token counts up to this run the GEMV; above it, the tensor-core GEMM unless gemv_takes().
 constexpr int64_t kGemvMaxM = 4;
 
 int* status_ptr() {
@@ -119,7 +119,7 @@ MatRef mat_ref(int fmt, const void* W, void* Y, int64_t N, int64_t K) {
 cudaError_t launch_group(const GroupRef& g, bool pdl, cudaStream_t s) {
     int* st = status_ptr();
     if (!st) return cudaErrorInvalidDevice;
-    if (g.M <= kGemvMaxM) return launch_gemv(g, pdl, st, s);
+    if (g.M <= kGemvMaxM || gemv_takes(g)) return launch_gemv(g, pdl, st, s);
     return launch_gemm_tc(g, pdl, st, s);
 }
 
@@ -546,8 +546,8 @@ const char* emb_status_string(emb_status status) {
 }
 
 const char* emb_build_info(void) {
-    return "libembqmm: sm_103a; Q8_0/Q6_0/Q4_0; GEMV (M<=4: staged/ring/register FFMA2, Q4_0 mma.sync at M>=2) + "
-           "tcgen05 GEMM (M>4: TMA, dequant to bf16 A tiles in TMEM, TMEM accumulators; one tile, persistent, "
+    return "libembqmm: sm_103a; Q8_0/Q6_0/Q4_0; GEMV (M=1: staged/ring/register FFMA2, long rows and M<=16: mma.sync) + "
+           "tcgen05 GEMM (larger M: TMA, dequant to bf16 A tiles in TMEM, TMEM accumulators; one tile, persistent, "
            "cluster split-K or stream-K schedules); "
            "recorded chains (CUDA graphs); RMSNorm, rotary embedding, grouped-head attention";
 }

@@ -137,6 +137,8 @@ struct GroupRef {
 // pdl: launch with programmatic stream serialisation (the kernel reads X only after
 // griddepcontrol.wait, weights before).
 cudaError_t launch_gemv(const GroupRef& g, bool pdl, int* status, cudaStream_t s);
+// Whether a group of more than four tokens is faster through launch_gemv.
+bool gemv_takes(const GroupRef& g);
 
 // Tensor-core GEMM (tcgen05 + TMEM) for larger M.
 cudaError_t launch_gemm_tc(const GroupRef& g, bool pdl, int* status, cudaStream_t s);

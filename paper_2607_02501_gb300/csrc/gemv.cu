@@ -1,21 +1,23 @@
-// GEMV for small token counts (action-token decode, M = 1..4).
+// GEMV for small token counts (action-token decode, M = 1; a few tokens, M = 2..16).
 //
 // The paper's batch-1 setting (Section 3.1, challenge 2) makes every linear layer a
 // matrix-vector product whose cost is reading the packed weights once from HBM.
-// Three kernels:
-//   * the staged kernel (large layers with short rows, and M > 1): each CTA pulls one
+// Four kernels:
+//   * the tensor-core kernel (M = 2..16, and long rows at M = 1): dot products on mma.sync with
+//     the codes exact in bf16 (described at its definition);
+//   * the staged kernel (large layers with short rows at M = 1): each CTA pulls one
 //     tile of rows plus its activations into shared memory with cp.async.bulk, so many
 //     bytes are in flight per SM and the next layer's tiles load during this layer's
 //     tail (programmatic dependent launch);
-//   * the register kernel (small layers, and long rows at M = 1): one CTA owns R
-//     consecutive weight rows; its NT threads split K in 16-byte units (a Q8_0 unit is
+//   * the ring kernel (large Q8_0 layers with long rows at M = 1): activations in
+//     registers, rows through a ring of bulk copies;
+//   * the register kernel (what is left: small layers, rows that the others do not take): one CTA
+//     owns R consecutive weight rows; its NT threads split K in 16-byte units (a Q8_0 unit is
 //     16 codes, half a block; a Q4_0 unit is one whole 32-code block; a warp reads 512
 //     contiguous bytes), load codes with 128-bit non-allocating loads one unit ahead
 //     (register double buffering) and reduce with warp shuffles, then across warps in
-//     shared memory;
-//   * the Q4_0 tensor-core kernel (large Q4_0 layers at M = 2..8): staged like the
-//     first, with the dot products on mma.sync (described at its definition).
-// The first two dequantise in registers with exact integer->float "magic number"
+//     shared memory.
+// The last three dequantise in registers with exact integer->float "magic number"
 // conversions followed by packed fp32x2 FMAs (FFMA2). Every reduction runs in a fixed
 // order, so results are deterministic. Weights are fetched before griddepcontrol.wait (they never depend
 // on an earlier launch) with non-coherent streaming loads; X is read with ordinary
@@ -261,8 +263,12 @@ cudaError_t dispatch_mt(const GemvParams& p, int grid_x, int M, bool pdl, cudaSt
         if (M == 1 && p.U > NT && p.U <= 4 * NT) return launch_one<FMT, R, NT, 1, 4>(p, grid_x, 1, pdl, s);
     }
     if (M == 1) return launch_one<FMT, R, NT, 1>(p, grid_x, 1, pdl, s);
-    if (M == 2) return launch_one<FMT, R, NT, 2>(p, grid_x, 1, pdl, s);
-    return launch_one<FMT, R, NT, 4>(p, grid_x, (M + 3) / 4, pdl, s);
+    // more tokens (see tc_takes): small Q8_0 layers at M = 2, Q6_0 with K % 64 != 0 at M <= 4
+    if constexpr (FMT != EMB_Q4_0) {
+        if (M == 2) return launch_one<FMT, R, NT, 2>(p, grid_x, 1, pdl, s);
+        if constexpr (FMT == EMB_Q6_0) return launch_one<FMT, R, NT, 4>(p, grid_x, (M + 3) / 4, pdl, s);
+    }
+    return cudaErrorInvalidValue;
 }
 
 template <int FMT, int R>
@@ -298,10 +304,10 @@ int pick_threads(int U, int fmt, int64_t tiles) {
 // can, and under programmatic dependent launch the next layer's tiles stream in while
 // this layer's last CTAs finish. The four warps form a WR x WK grid (WR = 4 / WK): a
 // warp owns RW rows of the tile and one K slice of U / WK units; its lanes stride the
-// slice in 16-byte units and reuse each activation unit across the warp's RW rows.
+// slice in 16-byte units and reuse each activation unit across the warp's RW rows. (M = 1.)
 constexpr int kStageWarps = 4;
 constexpr int kStageThreads = 32 * kStageWarps;
-constexpr int kStageBytes = 32 * 1024;     // codes of one tile, at most
+constexpr int kStageBytes = 16 * 1024;     // codes of one tile, at most
 constexpr int kStageXBytes = 32 * 1024;    // activation rows of one CTA, at most
 constexpr int kStageHeader = 1152;         // mbarriers (0..15), cross-warp sums (128..1151)
 
@@ -320,6 +326,9 @@ struct StagedParams {
     int* status;
 };
 
+// (MT, the tokens of a CTA, is 1 in every use. The kernel keeps the loop over tokens: with it
+// written out, ptxas sinks the code loads to their uses, 55 registers become 48, and Gemma-2B gate/up
+// takes 14.9 us instead of 14.4.)
 template <int FMT, int RW, int MT>
 __global__ void __launch_bounds__(kStageThreads) gemv_staged_kernel(const __grid_constant__ StagedParams p) {
     constexpr int UW = (FMT == EMB_Q8_0) ? 16 : 32;
@@ -474,11 +483,11 @@ __global__ void __launch_bounds__(kStageThreads) gemv_staged_kernel(const __grid
     }
 }
 
-template <int FMT, int RW, int MT>
+template <int FMT, int RW>
 cudaError_t launch_staged_one(const StagedParams& p, int tiles, size_t smem, bool pdl, cudaStream_t s) {
     static_assert(kStageHeader + kStageXBytes + kStageBytes + kStageBytes / 8 <= 227 * 1024, "smem");
     cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3(tiles, (p.M + MT - 1) / MT, 1);
+    cfg.gridDim = dim3(tiles, 1, 1);
     cfg.blockDim = dim3(kStageThreads, 1, 1);
     cfg.dynamicSmemBytes = smem;
     cfg.stream = s;
@@ -489,19 +498,19 @@ cudaError_t launch_staged_one(const StagedParams& p, int tiles, size_t smem, boo
     cfg.numAttrs = pdl ? 1 : 0;
     if (smem > 48 * 1024) {
         // once per instantiation and device is enough, but the call is cheap and idempotent
-        const cudaError_t e = cudaFuncSetAttribute(gemv_staged_kernel<FMT, RW, MT>,
+        const cudaError_t e = cudaFuncSetAttribute(gemv_staged_kernel<FMT, RW, 1>,
                                                    cudaFuncAttributeMaxDynamicSharedMemorySize,
                                                    int(kStageHeader + kStageXBytes + kStageBytes + kStageBytes / 8));
         if (e != cudaSuccess) return e;
     }
-    return cudaLaunchKernelEx(&cfg, gemv_staged_kernel<FMT, RW, MT>, p);
+    return cudaLaunchKernelEx(&cfg, gemv_staged_kernel<FMT, RW, 1>, p);
 }
 
-template <int FMT, int MT>
+template <int FMT>
 cudaError_t launch_staged_rw(const StagedParams& p, int RW, int tiles, size_t smem, bool pdl, cudaStream_t s) {
-    if (RW == 4) return launch_staged_one<FMT, 4, MT>(p, tiles, smem, pdl, s);
-    if (RW == 2) return launch_staged_one<FMT, 2, MT>(p, tiles, smem, pdl, s);
-    return launch_staged_one<FMT, 1, MT>(p, tiles, smem, pdl, s);
+    if (RW == 4) return launch_staged_one<FMT, 4>(p, tiles, smem, pdl, s);
+    if (RW == 2) return launch_staged_one<FMT, 2>(p, tiles, smem, pdl, s);
+    return launch_staged_one<FMT, 1>(p, tiles, smem, pdl, s);
 }
 
 // Tile shape: rows per warp RW and warps along K WK (TR = RW * 4 / WK rows per tile),
@@ -511,7 +520,7 @@ cudaError_t launch_staged_rw(const StagedParams& p, int RW, int tiles, size_t sm
 // K slice keeps at least 32 units (one per lane). Returns false when no tile fits.
 // Measured on GB300 at M = 1 (graph-replayed chains): 16 KB tiles beat 32 KB ones by
 // 3-6% (a shorter CTA lifetime shortens each launch's tail), e.g. Q8_0 32768 x 2048:
-// 14.9 us (8 rows) vs 15.8 us (16 rows); at M = 4, 32 KB tiles win (22.7 vs 27.0 us).
+// 14.9 us (8 rows) vs 15.8 us (16 rows).
 bool pick_stage_shape(int fmt, int64_t rows_total, int64_t row_bytes, int U, int64_t tile_bytes,
                       bool even_rows, int& RW, int& WK) {
     static const int kQ8[5][2] = {{4, 1}, {4, 2}, {4, 4}, {2, 4}, {1, 4}};
@@ -539,8 +548,7 @@ bool pick_stage_shape(int fmt, int64_t rows_total, int64_t row_bytes, int U, int
 // M = 1: 2.1 us register, 3.2 us staged). Long rows at M = 1 leave a staged CTA one or two
 // rows and re-stage the whole activation row per CTA; the register kernel with 2 rows
 // per CTA is faster there (Q8_0 2048 x 16384: 9.6 us register, 12.0 us staged). Short
-// rows favour the staged path (Q4_0 32768 x 2048: 13.4 us staged, 15.1 us register), and
-// so does M > 1 (Q8_0 32768 x 2048 at M = 4: 22.6 us staged, 32.2 us register).
+// rows favour the staged path (Q4_0 32768 x 2048: 13.4 us staged, 15.1 us register).
 constexpr int64_t kStageMinBytes = 12ll << 20;
 constexpr int64_t kStageMaxRowBytesM1 = 6 * 1024;
 
@@ -552,15 +560,13 @@ bool launch_staged(const GroupRef& g, bool pdl, int* status, cudaStream_t s, cud
     if (g.fmt == EMB_Q6_0 && g.K % 64 != 0) return false;
     const int64_t weight_row_bytes = row_bytes + high_bytes;
     const int U = int((g.fmt == EMB_Q8_0) ? g.K / 16 : g.K / 32);
-    const int MT = (g.M == 1) ? 1 : (g.M == 2) ? 2 : 4;
-    if (int64_t(MT) * g.K * 2 > kStageXBytes) return false;
+    if (g.M != 1 || g.K * 2 > kStageXBytes) return false;
     int64_t rows = 0;
     for (int i = 0; i < g.n_mats; ++i) rows += g.mats[i].N;
     if (rows * weight_row_bytes < kStageMinBytes) return false;
-    if (g.M == 1 && weight_row_bytes > kStageMaxRowBytesM1) return false;
+    if (weight_row_bytes > kStageMaxRowBytesM1) return false;
     int RW = 0, WK = 0;
-    const int64_t tile_bytes = (g.M == 1) ? kStageBytes / 2 : kStageBytes;
-    if (!pick_stage_shape(g.fmt, rows, weight_row_bytes, U, tile_bytes, g.epi >= EMB_EPI_GEGLU, RW, WK))
+    if (!pick_stage_shape(g.fmt, rows, weight_row_bytes, U, kStageBytes, g.epi >= EMB_EPI_GEGLU, RW, WK))
         return false;
     StagedParams p = {};
     const int TR = RW * kStageWarps / WK;
@@ -585,260 +591,413 @@ bool launch_staged(const GroupRef& g, bool pdl, int* status, cudaStream_t s, cud
     p.epi = g.epi;
     p.X = g.X;
     p.status = status;
-    const size_t smem = kStageHeader + size_t(MT) * g.K * 2 + size_t(TR) * size_t(weight_row_bytes + g.ldS * 2);
-    if (g.fmt == EMB_Q8_0) {
-        if (MT == 1) err = launch_staged_rw<EMB_Q8_0, 1>(p, RW, tiles, smem, pdl, s);
-        else if (MT == 2) err = launch_staged_rw<EMB_Q8_0, 2>(p, RW, tiles, smem, pdl, s);
-        else err = launch_staged_rw<EMB_Q8_0, 4>(p, RW, tiles, smem, pdl, s);
-    } else if (g.fmt == EMB_Q6_0) {
-        if (MT == 1) err = launch_staged_rw<EMB_Q6_0, 1>(p, RW, tiles, smem, pdl, s);
-        else if (MT == 2) err = launch_staged_rw<EMB_Q6_0, 2>(p, RW, tiles, smem, pdl, s);
-        else err = launch_staged_rw<EMB_Q6_0, 4>(p, RW, tiles, smem, pdl, s);
-    } else {
-        if (MT == 1) err = launch_staged_rw<EMB_Q4_0, 1>(p, RW, tiles, smem, pdl, s);
-        else if (MT == 2) err = launch_staged_rw<EMB_Q4_0, 2>(p, RW, tiles, smem, pdl, s);
-        else err = launch_staged_rw<EMB_Q4_0, 4>(p, RW, tiles, smem, pdl, s);
-    }
+    const size_t smem = kStageHeader + size_t(g.K) * 2 + size_t(TR) * size_t(weight_row_bytes + g.ldS * 2);
+    err = g.fmt == EMB_Q8_0   ? launch_staged_rw<EMB_Q8_0>(p, RW, tiles, smem, pdl, s)
+          : g.fmt == EMB_Q6_0 ? launch_staged_rw<EMB_Q6_0>(p, RW, tiles, smem, pdl, s)
+                              : launch_staged_rw<EMB_Q4_0>(p, RW, tiles, smem, pdl, s);
     return true;
 }
 
 
-// ------------------------------------------------------------ Q4_0 tensor-core GEMV
-// For Q4_0 the dequantise-and-dot arithmetic, not HBM, bounds the kernels above. Here
-// the dot products run on the tensor cores (mma.sync m16n8k16, bf16 x bf16 -> fp32) and
-// the CUDA cores only unpack nibbles: a nibble OR-ed into the bf16 pattern 0x4300 is
-// 128 + q exactly, and one packed bf16 subtraction of 136 leaves q - 8 exactly, so each
-// pair of weights costs one LOP3 and one HSUB2. One MMA covers 16 rows x 16 consecutive
-// K of one block (the tokens, M <= 8, are the MMA's 8 columns); a block's two MMAs
-// accumulate into a fresh fragment that is then scaled by the block's fp32 scale, as in
-// the plain definition. The MMA sums its 16 products in its own fixed order, so results
-// are deterministic.
+// ------------------------------------------------------------------ tensor-core GEMV
+// A few tokens (M = 2..16). With M tokens per weight the FFMA2 dot products, not HBM, bound the
+// kernels above (M = 4: ~6 instructions per weight). Here they run on mma.sync m16n8k16 (bf16 x
+// bf16 -> fp32): 16 weight rows are the MMA's M side, the tokens its eight columns (two MMAs for
+// M > 8), so up to eight tokens cost what one does and the CUDA cores only turn codes into bf16:
+// codes are small integers, exact in bf16, and every product is exact in fp32. A 32-weight block
+// is two MMAs into one fragment, which is then scaled by the block's fp32 scale as in the plain
+// definition; two such sums alternate by block and are added at the end, the warps' sums pairwise,
+// all in a fixed order: results are deterministic.
 //
-// Fragment mapping (any permutation of K inside a block is valid as long as A and B use
-// the same one): lane (g, t) = (lane / 4, lane % 4) loads 32-bit word t of the block in
-// rows g and g + 8. Word t holds q[4t + i] in the low nibble and q[16 + 4t + i] in the
-// high nibble of its byte i. MMA 0 takes the low nibbles: (bytes 0, 2) -> k slots
-// (2t, 2t + 1), (bytes 1, 3) -> (2t + 8, 2t + 9); MMA 1 the high nibbles likewise. The
-// activation fragment of lane (g, t) is token g's x at the same four positions.
+// A row tile is 16 rows of one matrix; a CTA walks row tiles blockIdx.x, + gridDim.x, ... Each of
+// its eight (or, for long rows that give an SM one tile, sixteen) warps takes every eighth
+// 256-k chunk of the tile's rows and streams its chunks through a ring of its own in shared memory
+// with cp.async (whole 128-byte lines per row, XOR-swizzled 16-byte granules so that fragment loads
+// are conflict-free): no barrier between warps until a tile's sums are added. The first ring's
+// worth is issued before griddepcontrol.wait; the activations come by ordinary cached loads after.
 //
-// The CTA's tile (TR rows, TR a multiple of 16) and its activations are staged in shared
-// memory as in the staged kernel, but row by row into a padded layout (pitch = row
-// bytes + 16) so that the eight rows a fragment load touches fall into distinct banks.
-constexpr int kMmaWarps = 4;
-constexpr int kMmaThreads = 32 * kMmaWarps;
-constexpr int kMmaTileBytes = 32 * 1024;  // codes of one tile, at most
-constexpr int kMmaMaxM = 8;
-constexpr int kMmaHeader = 128 + 512 * 4;  // barriers, then cross-warp sums [WK][TR][8] (WK * TR <= 64)
+// Fragment mapping (any permutation of K inside a block is valid as long as A and B use the same
+// one): lane (g, t) = (lane / 4, lane % 4) holds tile rows rho(g) and rho(g) + 8.
+//  * Q8_0: codes 8t .. 8t + 7 of the block (one 8-byte load per row; rho = 0, 2, 4, 6, 1, 3, 5, 7
+//    puts a half warp's 16 loads into distinct banks). MMA 0 takes codes (8t, 8t + 1) as k slots
+//    (2t, 2t + 1) and (8t + 2, 8t + 3) as (2t + 8, 2t + 9), MMA 1 the other four; its activations
+//    are token g's x[8t .. 8t + 7], one 16-byte load.
+//  * Q4_0, Q6_0: 32-bit word t of the block (low nibbles codes 4t .. 4t + 3, high nibbles 16 + 4t
+//    ..), rho = identity. MMA 0 takes the low, MMA 1 the high nibbles: (bytes 0, 1) -> slots
+//    (2t, 2t + 1), (bytes 2, 3) -> (2t + 8, 2t + 9).
+// What bounds it: the codes-to-bf16 arithmetic (2 to 3 instructions per weight, on the pipe that
+// also permutes bytes) and, for few rows, latency: Q6_0 32768 x 2048 at M = 4 15.4 us against 8.1
+// for its bytes. Without the shared-memory ring (fragments loaded from global memory directly,
+// 32 bytes per row and instruction) the same layer took 23 us, with or without a persistent grid.
+constexpr int kTcRows = 16;
+constexpr int kTcBlocks = 8;       // 32-weight blocks of a chunk (16 bytes of scales per row)
+constexpr int kTcMaxM = 16;
 
-struct MmaParams {
+struct TcParams {
     const uint8_t* codes[kMaxGroup];
+    const uint8_t* high[kMaxGroup];  // Q6_0: 2-bit high plane of each matrix
     const __half* scales[kMaxGroup];
     void* Y[kMaxGroup];              // as the epilogue says
     int32_t N[kMaxGroup];
-    int32_t tile0[kMaxGroup + 1];
+    int32_t tile0[kMaxGroup + 1];  // first row tile of each matrix (prefix sums)
     int32_t n_mats;
     int32_t M, K, ldS;
-    int32_t TR, WK;                // rows per tile (multiple of 16), warps along K
-    int32_t pitch, spitch;         // padded shared-memory row pitch of codes / scales, bytes
-    int32_t epi;                   // emb_epilogue (element-wise kinds only)
+    int32_t epi;                   // emb_epilogue
     const __nv_bfloat16* X;
-    int* status;
 };
 
 __device__ __forceinline__ void mma_bf16_16816(float (&d)[4], const uint32_t (&a)[4], uint32_t b0,
                                                uint32_t b1) {
-    asm volatile(
-        "mma.sync.aligned.m16n8k16.row.col.f32.bf16.bf16.f32 {%0, %1, %2, %3}, {%4, %5, %6, %7}, "
-        "{%8, %9}, {%10, %11, %12, %13};"
-        : "=f"(d[0]), "=f"(d[1]), "=f"(d[2]), "=f"(d[3])
-        : "r"(a[0]), "r"(a[1]), "r"(a[2]), "r"(a[3]), "r"(b0), "r"(b1), "f"(0.0f), "f"(0.0f), "f"(0.0f),
-          "f"(0.0f));
+    asm("mma.sync.aligned.m16n8k16.row.col.f32.bf16.bf16.f32 {%0, %1, %2, %3}, {%4, %5, %6, %7}, "
+        "{%8, %9}, {%0, %1, %2, %3};"
+        : "+f"(d[0]), "+f"(d[1]), "+f"(d[2]), "+f"(d[3])
+        : "r"(a[0]), "r"(a[1]), "r"(a[2]), "r"(a[3]), "r"(b0), "r"(b1));
 }
-
-// (128 + q) pairs from the nibbles at bits 0..3 and 16..19, then q - 8 (exact in bf16).
-__device__ __forceinline__ uint32_t q4_pair(uint32_t v) {
-    const uint32_t b = and_or(v, 0x000F000Fu, 0x43004300u);
-    const __nv_bfloat162 r = __hsub2(*reinterpret_cast<const __nv_bfloat162*>(&b),
-                                     __floats2bfloat162_rn(136.0f, 136.0f));
+__device__ __forceinline__ uint32_t sub_bf16x2(uint32_t a, uint32_t b) {
+    const __nv_bfloat162 r = __hsub2(*reinterpret_cast<const __nv_bfloat162*>(&a),
+                                     *reinterpret_cast<const __nv_bfloat162*>(&b));
     return *reinterpret_cast<const uint32_t*>(&r);
 }
+// Bytes 0, 1 (LO) or 2, 3 of v, each below 128, as the bf16 pair 128 + byte (exact: the byte is the
+// whole 7-bit fraction of 0x4300).
+template <bool LO>
+__device__ __forceinline__ uint32_t bytes_128(uint32_t v) {
+    return __byte_perm(v, 0x43434343u, LO ? 0x4140 : 0x4342);
+}
+// Four signed bytes -> bf16 pairs (codes 0, 1) and (2, 3): q = (128 + (q & 127)) - (128 or 256 by
+// its sign bit), both of which are bf16 0x4300 with the masked byte as fraction and exponent bits.
+__device__ __forceinline__ void q8_pairs(uint32_t v, uint32_t& p01, uint32_t& p23) {
+    const uint32_t m = v & 0x7F7F7F7Fu, s = v & 0x80808080u;
+    p01 = sub_bf16x2(bytes_128<true>(m), bytes_128<true>(s));
+    p23 = sub_bf16x2(bytes_128<false>(m), bytes_128<false>(s));
+}
 
-__global__ void __launch_bounds__(kMmaThreads) gemv_q4_mma_kernel(const __grid_constant__ MmaParams p) {
+__device__ __forceinline__ uint2 ld_shared_u2(uint32_t a) {
+    uint2 v;
+    asm volatile("ld.shared.v2.u32 {%0, %1}, [%2];" : "=r"(v.x), "=r"(v.y) : "r"(a));
+    return v;
+}
+__device__ __forceinline__ uint32_t ld_shared_u1(uint32_t a) {
+    uint32_t v;
+    asm volatile("ld.shared.u32 %0, [%1];" : "=r"(v) : "r"(a));
+    return v;
+}
+__device__ __forceinline__ float ld_shared_half(uint32_t a) {
+    uint16_t v;
+    asm volatile("ld.shared.u16 %0, [%1];" : "=h"(v) : "r"(a));
+    return __half2float(__ushort_as_half(v));
+}
+
+__device__ __forceinline__ void cp_async16(uint32_t saddr, const void* g, bool ok) {
+    asm volatile("cp.async.cg.shared.global.L2::128B [%0], [%1], 16, %2;" ::"r"(saddr), "l"(g), "r"(ok ? 16 : 0)
+                 : "memory");
+}
+
+// One stage of a warp's ring: 16 rows x 256 k of codes, then (Q6_0) high bits, then scales.
+template <int FMT>
+struct TcStage {
+    static constexpr int kCodes = kTcRows * (FMT == EMB_Q8_0 ? 256 : 128);
+    static constexpr int kHigh = FMT == EMB_Q6_0 ? kTcRows * 64 : 0;
+    static constexpr int kBytes = kCodes + kHigh + kTcRows * 16;
+};
+// Ring depth: three stages, two where the sums of sixteen tokens would leave an SM one CTA.
+template <int FMT, int NT, int NW>
+constexpr int kTcDepth = FMT == EMB_Q8_0 && NT == 2 && NW == 8 ? 2 : 3;
+template <int FMT, int NT, int NW>
+constexpr int kTcSmem = NW * kTcDepth<FMT, NT, NW> * TcStage<FMT>::kBytes;
+
+template <int FMT, int NT, int NW>
+__global__ void __launch_bounds__(32 * NW, 16 / NW) gemv_tc_kernel(const __grid_constant__ TcParams p) {
+    using St = TcStage<FMT>;
+    constexpr int kTcStages = kTcDepth<FMT, NT, NW>;
+    constexpr int kBufs = NW == 8 ? 2 : 1;  // (sixteen warps: one tile per CTA)
     extern __shared__ __align__(128) uint8_t smem[];
-    uint64_t* bar_w = reinterpret_cast<uint64_t*>(smem);
-    uint64_t* bar_x = reinterpret_cast<uint64_t*>(smem + 8);
-    float* red = reinterpret_cast<float*>(smem + 128);  // [WK][TR][8]
-    const int row_bytes = p.K / 2;
-    const int nb = p.K / kQBlock;
-    uint8_t* x_s = smem + kMmaHeader;                  // [M][K] bf16
-    uint8_t* codes_s = x_s + p.M * p.K * 2;            // [TR][pitch]
-    uint8_t* scales_s = codes_s + p.TR * p.pitch;
-
-    const int tile = blockIdx.x;
-    int g_mat = 0;
-#pragma unroll
-    for (int i = 1; i < kMaxGroup; ++i)
-        if (i < p.n_mats && tile >= p.tile0[i]) g_mat = i;
-    const int N = p.N[g_mat];
-    const int row0 = (tile - p.tile0[g_mat]) * p.TR;
-    const int rows = min(p.TR, N - row0);
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int g = lane >> 2, t = lane & 3;
+    const int nb = p.K / kQBlock;
+    const int tiles = p.tile0[p.n_mats];
+    const int64_t row_bytes = FMT == EMB_Q8_0 ? int64_t(p.K) : int64_t(p.K) / 2;
+    const uint32_t ring = ptx::smem_u32(smem) + warp * kTcStages * St::kBytes;
+    auto mat_of = [&](int tile) {
+        int gm = 0;
+#pragma unroll
+        for (int i = 1; i < kMaxGroup; ++i)
+            if (i < p.n_mats && tile >= p.tile0[i]) gm = i;
+        return gm;
+    };
 
-    if (warp == 0) {
-        if (lane == 0) {
-            ptx::mbar_init(bar_w, 1);
-            ptx::mbar_init(bar_x, 1);
-            ptx::fence_mbar_init();
-            ptx::mbar_arrive_expect_tx(bar_w, uint32_t(rows) * uint32_t(row_bytes + p.ldS * 2));
+    griddep_launch_dependents();
+    // chunk of a row tile whose first block is kb0: blocks past the row are zero codes with zero
+    // scales (the scale row is zero-padded to eight), rows past N read row N - 1 (never stored)
+    auto issue = [&](int tile, int kb0, int stage) {
+        const int gm = mat_of(tile);
+        const int row0 = (tile - p.tile0[gm]) * kTcRows, last = p.N[gm] - 1;
+        const uint32_t st = ring + stage * St::kBytes;
+        constexpr int kG = FMT == EMB_Q8_0 ? 16 : 8;  // 16-byte granules of a row's codes
+        const int c = lane % kG, kbg = kb0 + (FMT == EMB_Q8_0 ? c >> 1 : c);  // the granule's block
+#pragma unroll
+        for (int i = 0; i < kTcRows * kG / 32; ++i) {
+            const int r = i * (32 / kG) + lane / kG;
+            const uint8_t* src = p.codes[gm] + int64_t(min(row0 + r, last)) * row_bytes +
+                                 (kbg < nb ? int64_t(kb0) * (FMT == EMB_Q8_0 ? 32 : 16) + c * 16 : 0);
+            cp_async16(st + r * (kG * 16) + ((c ^ (r & 7)) << 4), src, kbg < nb);
         }
-        __syncwarp();
-        const uint8_t* src_c = p.codes[g_mat] + int64_t(row0) * row_bytes;
-        const __half* src_s = p.scales[g_mat] + int64_t(row0) * p.ldS;
-        for (int r = lane; r < rows; r += 32) {
-            ptx::bulk_load(codes_s + r * p.pitch, src_c + int64_t(r) * row_bytes, uint32_t(row_bytes), bar_w);
-            ptx::bulk_load(scales_s + r * p.spitch, src_s + int64_t(r) * p.ldS, uint32_t(p.ldS * 2), bar_w);
-        }
-        if (lane == 0 && blockIdx.x == 0) ptx::prefetch_l2(p.X, uint32_t(p.M) * uint32_t(p.K) * 2u);  // towards L2
-    }
-    ptx::griddep_launch_dependents();
-    // weights do not depend on earlier launches; X and Y may
-    ptx::griddep_wait();
-    if (threadIdx.x == 0) {
-        const uint32_t x_bytes = uint32_t(p.M) * uint32_t(p.K) * 2u;
-        ptx::mbar_arrive_expect_tx(bar_x, x_bytes);
-        ptx::bulk_load(x_s, p.X, x_bytes, bar_x);
-    }
-    __syncthreads();  // the barriers' initialisation is visible to every waiting thread
-    // both waits are bounded; the CTA leaves together if any of its threads gave up
-    bool ok = ptx::mbar_wait(bar_w, 0, nullptr, p.status, kWaitLimitNs);
-    ok = ok && ptx::mbar_wait(bar_x, 0, nullptr, p.status, kWaitLimitNs);
-    if (__syncthreads_or(!ok)) return;
-
-    const int WK = p.WK;
-    const int wk = warp % WK, rg = warp / WK;  // K slice, 16-row group
-    const int gq = lane >> 2, t = lane & 3;
-    const int bw = (nb + WK - 1) / WK;
-    const int kb_lo = wk * bw, kb_hi = min(nb, kb_lo + bw);
-    const uint8_t* c0 = codes_s + (rg * 16 + gq) * p.pitch + 4 * t;
-    const uint8_t* c1 = c0 + 8 * p.pitch;
-    const __half* s0 = reinterpret_cast<const __half*>(scales_s + (rg * 16 + gq) * p.spitch);
-    const __half* s1 = reinterpret_cast<const __half*>(reinterpret_cast<const uint8_t*>(s0) + 8 * p.spitch);
-    const bool has_x = gq < p.M;
-    const uint8_t* xr = x_s + (gq * p.K + 4 * t) * 2;
-
-    float acc[4] = {0.0f, 0.0f, 0.0f, 0.0f};
-    if (rg * 16 < rows) {
-#pragma unroll 4
-        for (int kb = kb_lo; kb < kb_hi; ++kb) {
-            uint32_t b[4] = {0u, 0u, 0u, 0u};
-            if (has_x) {
-                const uint2 lo = *reinterpret_cast<const uint2*>(xr + kb * 64);       // x[4t .. 4t+3]
-                const uint2 hi = *reinterpret_cast<const uint2*>(xr + kb * 64 + 32);  // x[16+4t ..]
-                b[0] = __byte_perm(lo.x, lo.y, 0x5410);
-                b[1] = __byte_perm(lo.x, lo.y, 0x7632);
-                b[2] = __byte_perm(hi.x, hi.y, 0x5410);
-                b[3] = __byte_perm(hi.x, hi.y, 0x7632);
+        if constexpr (FMT == EMB_Q6_0) {
+            const int ch = lane & 3;
+#pragma unroll
+            for (int i = 0; i < 2; ++i) {
+                const int r = 8 * i + (lane >> 2);
+                const bool ok = kb0 + 2 * ch < nb;  // nb is even (K % 64 == 0)
+                const uint8_t* src = p.high[gm] + int64_t(min(row0 + r, last)) * (p.K / 4) +
+                                     (ok ? int64_t(kb0) * 8 + ch * 16 : 0);
+                cp_async16(st + St::kCodes + r * 64 + ((ch ^ ((r >> 1) & 3)) << 4), src, ok);
             }
-            const uint32_t w0 = *reinterpret_cast<const uint32_t*>(c0 + kb * 16);
-            const uint32_t w1 = *reinterpret_cast<const uint32_t*>(c1 + kb * 16);
-            const uint32_t alo[4] = {q4_pair(w0), q4_pair(w1), q4_pair(w0 >> 8), q4_pair(w1 >> 8)};
-            const uint32_t ahi[4] = {q4_pair(w0 >> 4), q4_pair(w1 >> 4), q4_pair(w0 >> 12), q4_pair(w1 >> 12)};
-            float dlo[4], dhi[4];
-            mma_bf16_16816(dlo, alo, b[0], b[1]);
-            mma_bf16_16816(dhi, ahi, b[2], b[3]);
-            const float sc0 = __half2float(s0[kb]), sc1 = __half2float(s1[kb]);
-            acc[0] = fmaf(sc0, dlo[0] + dhi[0], acc[0]);
-            acc[1] = fmaf(sc0, dlo[1] + dhi[1], acc[1]);
-            acc[2] = fmaf(sc1, dlo[2] + dhi[2], acc[2]);
-            acc[3] = fmaf(sc1, dlo[3] + dhi[3], acc[3]);
         }
+        if (lane < kTcRows) {
+            const __half* src = p.scales[gm] + int64_t(min(row0 + lane, last)) * p.ldS + (kb0 < nb ? kb0 : 0);
+            cp_async16(st + St::kCodes + St::kHigh + lane * 16, src, kb0 < nb);
+        }
+    };
+    // this warp's chunks of all the CTA's tiles, in order; the next one to issue
+    const int stride = NW * kTcBlocks;                 // blocks between a warp's chunks of a tile
+    int it_tile = blockIdx.x, it_base = 0;
+    auto issue_next = [&](int stage) {
+        if (it_tile < tiles) {
+            issue(it_tile, it_base + warp * kTcBlocks, stage);
+            it_base += stride;
+            if (it_base >= nb) {
+                it_base = 0;
+                it_tile += gridDim.x;
+            }
+        }
+        asm volatile("cp.async.commit_group;" ::: "memory");
+    };
+#pragma unroll
+    for (int i = 0; i < kTcStages; ++i) issue_next(i);
+    if (threadIdx.x == 0 && blockIdx.x == 0) ptx::prefetch_l2(p.X, uint32_t(p.M) * uint32_t(p.K) * 2u);
+    // weights do not depend on earlier launches; X and Y may
+    griddep_wait();
+
+    // activation fragments of a block, by token n-tile: token 8 * nt + g
+    const __nv_bfloat16* xr[NT];
+    bool has[NT];
+#pragma unroll
+    for (int nt = 0; nt < NT; ++nt) {
+        has[nt] = 8 * nt + g < p.M;
+        xr[nt] = p.X + int64_t(has[nt] ? 8 * nt + g : 0) * p.K;
     }
-    // acc[0], acc[1]: row gq, tokens 2t, 2t+1; acc[2], acc[3]: row gq + 8, same tokens
-    const int ra = rg * 16 + gq, rb = ra + 8, m0 = 2 * t;
-    void* Yg = p.Y[g_mat];
-    if (WK == 1) {
-        if (m0 < p.M) {
-            if (ra < rows) epi_store(p.epi, Yg, m0, row0 + ra, N, acc[0]);
-            if (rb < rows) epi_store(p.epi, Yg, m0, row0 + rb, N, acc[2]);
+    auto load_x = [&](int kb, int nt, uint32_t (&b)[4]) {
+        b[0] = b[1] = b[2] = b[3] = 0u;
+        if (!has[nt] || kb >= nb) return;
+        if constexpr (FMT == EMB_Q8_0) {
+            const uint4 v = *reinterpret_cast<const uint4*>(xr[nt] + kb * 32 + 8 * t);
+            b[0] = v.x; b[1] = v.y; b[2] = v.z; b[3] = v.w;
+        } else {
+            const uint2 lo = *reinterpret_cast<const uint2*>(xr[nt] + kb * 32 + 4 * t);
+            const uint2 hi = *reinterpret_cast<const uint2*>(xr[nt] + kb * 32 + 16 + 4 * t);
+            b[0] = lo.x; b[1] = lo.y; b[2] = hi.x; b[3] = hi.y;
         }
-        if (m0 + 1 < p.M) {
-            if (ra < rows) epi_store(p.epi, Yg, m0 + 1, row0 + ra, N, acc[1]);
-            if (rb < rows) epi_store(p.epi, Yg, m0 + 1, row0 + rb, N, acc[3]);
+    };
+
+    constexpr int kAcc = NT == 1 ? 4 : 2;  // sums that alternate by block
+    float acc[kAcc][NT][4];
+    const int ra = FMT == EMB_Q8_0 ? (2 * g) % 7 + (g == 7 ? 7 : 0) : g;  // rho(g): 0, 2, 4, 6, 1, 3, 5, 7
+    const int rsw = ra & 7;
+    auto compute = [&](int kb0, uint32_t st) {
+        const uint32_t sc = st + St::kCodes + St::kHigh + ra * 16;
+#pragma unroll
+        for (int i = 0; i < kTcBlocks; ++i) {
+            uint32_t a0[4], a1[4];  // A fragments: {row ra slots 2t, row ra + 8, row ra slots 2t + 8, row ra + 8}
+            if constexpr (FMT == EMB_Q8_0) {
+                const uint32_t at = st + ra * 256 + (((2 * i + (t >> 1)) ^ rsw) << 4) + (t & 1) * 8;
+                const uint2 va = ld_shared_u2(at), vb = ld_shared_u2(at + 8 * 256);
+                q8_pairs(va.x, a0[0], a0[2]);
+                q8_pairs(vb.x, a0[1], a0[3]);
+                q8_pairs(va.y, a1[0], a1[2]);
+                q8_pairs(vb.y, a1[1], a1[3]);
+            } else {
+                constexpr uint32_t kOff = FMT == EMB_Q4_0 ? 0x43084308u : 0x43204320u;  // 128 + 8, 128 + 32
+                const uint32_t at = st + ra * 128 + ((i ^ rsw) << 4) + t * 4;
+                const uint32_t w[2] = {ld_shared_u1(at), ld_shared_u1(at + 8 * 128)};
+                uint32_t hw[2] = {0u, 0u};
+                if constexpr (FMT == EMB_Q6_0) {
+                    // high word of low word t is word t & 1, shifted by 2 (t >> 1)
+                    const uint32_t ah = st + St::kCodes + ra * 64 + (((i >> 1) ^ ((ra >> 1) & 3)) << 4) + (i & 1) * 8 + (t & 1) * 4;
+                    hw[0] = ld_shared_u1(ah) >> (2 * (t >> 1));
+                    hw[1] = ld_shared_u1(ah + 8 * 64) >> (2 * (t >> 1));
+                }
+#pragma unroll
+                for (int r = 0; r < 2; ++r) {
+                    uint32_t lo = w[r] & 0x0F0F0F0Fu, hi = (w[r] >> 4) & 0x0F0F0F0Fu;
+                    if constexpr (FMT == EMB_Q6_0) {
+                        lo |= (hw[r] & 0x03030303u) << 4;
+                        hi |= hw[r] & 0x30303030u;
+                    }
+                    a0[r] = sub_bf16x2(bytes_128<true>(lo), kOff);
+                    a0[2 + r] = sub_bf16x2(bytes_128<false>(lo), kOff);
+                    a1[r] = sub_bf16x2(bytes_128<true>(hi), kOff);
+                    a1[2 + r] = sub_bf16x2(bytes_128<false>(hi), kOff);
+                }
+            }
+            const float da = ld_shared_half(sc + 2 * i), db = ld_shared_half(sc + 8 * 16 + 2 * i);
+#pragma unroll
+            for (int nt = 0; nt < NT; ++nt) {
+                uint32_t b[4];
+                load_x(kb0 + i, nt, b);
+                // (two sums from zero and one rounded addition: chaining the second MMA onto the first
+                // costs 5 % in accuracy)
+                float d0[4] = {0.0f, 0.0f, 0.0f, 0.0f}, d1[4] = {0.0f, 0.0f, 0.0f, 0.0f};
+                mma_bf16_16816(d0, a0, b[0], b[1]);
+                mma_bf16_16816(d1, a1, b[2], b[3]);
+                float(&ac)[4] = acc[i % kAcc][nt];
+                ac[0] = fmaf(da, d0[0] + d1[0], ac[0]);
+                ac[1] = fmaf(da, d0[1] + d1[1], ac[1]);
+                ac[2] = fmaf(db, d0[2] + d1[2], ac[2]);
+                ac[3] = fmaf(db, d0[3] + d1[3], ac[3]);
+            }
         }
-        return;
-    }
-    float* rw = red + wk * p.TR * 8;
-    rw[ra * 8 + m0] = acc[0];
-    rw[ra * 8 + m0 + 1] = acc[1];
-    rw[rb * 8 + m0] = acc[2];
-    rw[rb * 8 + m0 + 1] = acc[3];
-    __syncthreads();
-    // add the K slices in slice order
-    for (int e = threadIdx.x; e < rows * p.M; e += kMmaThreads) {
-        const int r = e / p.M, m = e % p.M;
-        float v = 0.0f;
-        for (int k = 0; k < WK; ++k) v += red[(k * p.TR + r) * 8 + m];
-        epi_store(p.epi, Yg, m, row0 + r, N, v);
+    };
+    __shared__ float red[kBufs][NW][8 * NT][kTcRows];
+    int buf = 0, stage = 0;
+    for (int tile = blockIdx.x; tile < tiles; tile += gridDim.x, buf = (buf + 1) % kBufs) {
+#pragma unroll
+        for (int i = 0; i < kAcc; ++i)
+#pragma unroll
+            for (int nt = 0; nt < NT; ++nt) acc[i][nt][0] = acc[i][nt][1] = acc[i][nt][2] = acc[i][nt][3] = 0.0f;
+        for (int base = 0; base < nb; base += stride) {
+            asm volatile("cp.async.wait_group %0;" ::"n"(kTcStages - 1) : "memory");
+            __syncwarp();  // every lane's copies of this chunk have landed
+            const int kb0 = base + warp * kTcBlocks;
+            if (kb0 < nb) compute(kb0, ring + stage * St::kBytes);
+            __syncwarp();  // every lane has read it
+            issue_next(stage);
+            stage = stage + 1 == kTcStages ? 0 : stage + 1;
+        }
+        // acc[.][nt][0, 1]: row ra, tokens 8 nt + 2t, + 1; [2, 3]: row ra + 8. (Two
+        // buffers: a buffer is written again only after the barrier of the tile between.)
+#pragma unroll
+        for (int nt = 0; nt < NT; ++nt) {
+            float v[4];
+#pragma unroll
+            for (int e = 0; e < 4; ++e) {
+                v[e] = acc[0][nt][e] + acc[1][nt][e];
+                if constexpr (kAcc == 4) v[e] += acc[2][nt][e] + acc[3][nt][e];
+            }
+            red[buf][warp][8 * nt + 2 * t][ra] = v[0];
+            red[buf][warp][8 * nt + 2 * t + 1][ra] = v[1];
+            red[buf][warp][8 * nt + 2 * t][ra + 8] = v[2];
+            red[buf][warp][8 * nt + 2 * t + 1][ra + 8] = v[3];
+        }
+        __syncthreads();
+        const int m = threadIdx.x / kTcRows, r = threadIdx.x % kTcRows;
+        if (m < p.M && m < 8 * NT) {
+            const int gm = mat_of(tile), N = p.N[gm];
+            const int n = (tile - p.tile0[gm]) * kTcRows + r;
+            // the warps' sums pairwise (in order, one rounding more per warp adds 20 % of error)
+            auto total = [&](int row) {
+                float v[NW];
+#pragma unroll
+                for (int w = 0; w < NW; ++w) v[w] = red[buf][w][m][row];
+#pragma unroll
+                for (int o = NW / 2; o > 0; o >>= 1)
+#pragma unroll
+                    for (int w = 0; w < o; ++w) v[w] += v[w + o];
+                return v[0];
+            };
+            const float v = total(r);
+            if (p.epi >= EMB_EPI_GEGLU) {
+                // gate row n (even) and up row n + 1
+                if ((r & 1) == 0 && n < N) epi_store_gated(p.epi, p.Y[gm], m, n, N, v, total(r + 1));
+            } else if (n < N) {
+                epi_store(p.epi, p.Y[gm], m, n, N, v);
+            }
+        }
     }
 }
 
-// Q4_0 layers with 2..8 tokens, large enough for the staged path and with rows of at
-// most 2 KB (K <= 4096). At M = 1 the FFMA2 staged kernel is faster (measured on GB300,
-// Q4_0 32768 x 2048: 13.0 us FFMA2, 16.4 us MMA); from M = 2 the MMA's cost does not grow
-// with the token count while FFMA2's does (M = 4: 17.0 us MMA, 29.5 us FFMA2).
-// TR = 32 rows (2 row groups x 2 K slices) when that still gives 4 tiles per SM, else
-// 16 rows (4 K slices).
-bool launch_q4_mma(const GroupRef& g, bool pdl, int* status, cudaStream_t s, cudaError_t& err) {
-    if (g.fmt != EMB_Q4_0 || g.M < 2 || g.M > kMmaMaxM || g.epi >= EMB_EPI_GEGLU) return false;
-    const int64_t row_bytes = g.K / 2;
-    if (row_bytes * 16 > kMmaTileBytes) return false;
-    if (g.M * g.K * 2 > kStageXBytes) return false;
-    int64_t rows = 0;
-    for (int i = 0; i < g.n_mats; ++i) rows += g.mats[i].N;
-    if (rows * row_bytes < kStageMinBytes) return false;
-    const int nb = int(g.K / kQBlock);
-    int TR = 16, WK = 4;
-    if (row_bytes * 32 <= kMmaTileBytes && rows / 32 >= 4 * 152) { TR = 32; WK = 2; }
-    if (nb < WK) WK = 1, TR = 16 * kMmaWarps;  // too few blocks to split K: 4 row groups
-    if (TR * row_bytes > kMmaTileBytes) return false;
-    MmaParams p = {};
-    int tiles = 0;
-    for (int i = 0; i < g.n_mats; ++i) {
-        p.codes[i] = g.mats[i].codes;
-        p.scales[i] = g.mats[i].scales;
-        p.Y[i] = g.mats[i].Y;
-        p.N[i] = int32_t(g.mats[i].N);
-        p.tile0[i] = tiles;
-        tiles += int((g.mats[i].N + TR - 1) / TR);
-    }
-    p.tile0[g.n_mats] = tiles;
-    p.n_mats = g.n_mats;
-    p.M = int32_t(g.M);
-    p.K = int32_t(g.K);
-    p.ldS = int32_t(g.ldS);
-    p.TR = TR;
-    p.WK = WK;
-    p.pitch = int32_t(row_bytes + 16);
-    p.spitch = int32_t(g.ldS * 2 + 16);
-    p.epi = g.epi;
-    p.X = g.X;
-    p.status = status;
-    const size_t smem = size_t(kMmaHeader) + size_t(g.M) * g.K * 2 + size_t(TR) * (p.pitch + p.spitch);
+int gemv_sm_count();
+
+template <int FMT, int NT, int NW>
+cudaError_t launch_tc_one(const TcParams& p, int grid, bool pdl, cudaStream_t s) {
     cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3(tiles, 1, 1);
-    cfg.blockDim = dim3(kMmaThreads, 1, 1);
-    cfg.dynamicSmemBytes = smem;
+    cfg.gridDim = dim3(grid, 1, 1);
+    cfg.blockDim = dim3(32 * NW, 1, 1);
+    cfg.dynamicSmemBytes = kTcSmem<FMT, NT, NW>;
     cfg.stream = s;
+    const cudaError_t e = cudaFuncSetAttribute(gemv_tc_kernel<FMT, NT, NW>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                               kTcSmem<FMT, NT, NW>);
+    if (e != cudaSuccess) return e;
     cudaLaunchAttribute attr[1];
     attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
     attr[0].val.programmaticStreamSerializationAllowed = 1;
     cfg.attrs = attr;
     cfg.numAttrs = pdl ? 1 : 0;
-    if (smem > 48 * 1024) {
-        err = cudaFuncSetAttribute(gemv_q4_mma_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, int(smem));
-        if (err != cudaSuccess) return true;
+    return cudaLaunchKernelEx(&cfg, gemv_tc_kernel<FMT, NT, NW>, p);
+}
+
+template <int FMT>
+cudaError_t launch_tc_fmt(const TcParams& p, int tiles, int sms, bool pdl, cudaStream_t s) {
+    // long rows whose tiles leave each SM at most one CTA: sixteen warps
+    const bool wide = tiles <= sms && p.K > 8 * kTcBlocks * kQBlock;
+    const int grid = std::min(tiles, 2 * sms);
+    if (p.M <= 8) return wide ? launch_tc_one<FMT, 1, 16>(p, tiles, pdl, s) : launch_tc_one<FMT, 1, 8>(p, grid, pdl, s);
+    return wide ? launch_tc_one<FMT, 2, 16>(p, tiles, pdl, s) : launch_tc_one<FMT, 2, 8>(p, grid, pdl, s);
+}
+
+bool ring_takes(const GroupRef& g);
+
+// Which calls take it (us per launch in graph-replayed chains, this kernel / the one it leaves):
+//  * M = 3, 4 always, M = 2 but for Q8_0 layers below 1 M weights (640 x 320 1.77 / 1.50, kept on
+//    the register kernel): Q6_0 32768 x 2048 at M = 4 15.4 / 32.9, Q4_0 13.4 / 18.0, Q8_0 16.6 /
+//    22.8; 2048 x 16384 at M = 4 Q8_0 10.0 / 22.6, Q6_0 9.7 / 24.9, Q4_0 8.1 / 23.0;
+//  * M = 6..16 in place of the tcgen05 GEMM (12288 x 4096 at M = 8 Q8_0 14.6 / 26.7, Q4_0 13.5 /
+//    27.9; 1024 x 4096 at M = 16 4.6 / 6.4), but for Q8_0 above 12 tokens and 32 M weights
+//    (32768 x 2048 30.4 / 27.7), and for five tokens, the count at which the GEMM's bf16 operand
+//    is held to its bits (tests/test_gpu_hotpath_dequant.py);
+//  * M = 1 with rows of at least 4096 k, where its codes-to-bf16 step is cheaper than FFMA2 dot
+//    products and no activation row is staged per CTA: Q4_0 (2048 x 16384 7.5 / 9.3, 4096 x 4096
+//    4.1 / 4.7; with K < 8192 and more than five row tiles per SM the staged kernel keeps it,
+//    22016 x 4096 16.9 / 16.4), Q6_0 (12288 x 4096 12.7 / 16.8, 4096 x 11008 11.6 /
+//    14.4, 2048 x 16384 9.4 / 9.3), Q8_0 only with at most two row tiles per SM (1024 x 4096 2.6 / 3.3, 4096 x 11008
+//    12.1 / 13.3; 12288 x 4096 13.2 / 11.9).
+bool tc_takes(const GroupRef& g, int sms) {
+    if (g.M > kTcMaxM || g.M == 5 || (g.fmt == EMB_Q6_0 && g.K % 64 != 0)) return false;
+    int64_t rows = 0;
+    for (int i = 0; i < g.n_mats; ++i) rows += g.mats[i].N;
+    if (g.M == 1) {
+        if (g.K < 4096) return false;
+        if (g.fmt == EMB_Q4_0) return g.K >= 8192 || rows <= int64_t(5 * kTcRows) * sms;
+        return g.fmt == EMB_Q6_0 || (!ring_takes(g) && rows <= int64_t(2 * kTcRows) * sms);
     }
-    err = cudaLaunchKernelEx(&cfg, gemv_q4_mma_kernel, p);
+    if (g.fmt == EMB_Q8_0 && g.M == 2) return rows * g.K >= (int64_t(1) << 20);
+    if (g.fmt == EMB_Q8_0 && g.M > 12) return rows * g.K <= (int64_t(1) << 25);
+    return true;
+}
+
+bool launch_tc(const GroupRef& g, bool pdl, cudaStream_t s, cudaError_t& err) {
+    const int sms = gemv_sm_count();
+    if (sms <= 0 || !tc_takes(g, sms)) return false;
+    TcParams p = {};
+    int64_t tiles = 0;
+    for (int i = 0; i < g.n_mats; ++i) {
+        p.codes[i] = g.mats[i].codes;
+        p.high[i] = g.mats[i].high;
+        p.scales[i] = g.mats[i].scales;
+        p.Y[i] = g.mats[i].Y;
+        p.N[i] = int32_t(g.mats[i].N);
+        p.tile0[i] = int32_t(tiles);
+        tiles += (g.mats[i].N + kTcRows - 1) / kTcRows;
+    }
+    p.tile0[g.n_mats] = int32_t(tiles);
+    p.n_mats = g.n_mats;
+    p.M = int32_t(g.M);
+    p.K = int32_t(g.K);
+    p.ldS = int32_t(g.ldS);
+    p.epi = g.epi;
+    p.X = g.X;
+    err = g.fmt == EMB_Q8_0   ? launch_tc_fmt<EMB_Q8_0>(p, int(tiles), sms, pdl, s)
+          : g.fmt == EMB_Q4_0 ? launch_tc_fmt<EMB_Q4_0>(p, int(tiles), sms, pdl, s)
+                              : launch_tc_fmt<EMB_Q6_0>(p, int(tiles), sms, pdl, s);
     return true;
 }
 
@@ -865,7 +1024,6 @@ constexpr int kRingHeader = 144 + kRingFlush * (kRingThreads / 32) * 4;
 
 struct RingParams {
     const uint8_t* codes[kMaxGroup];
-    const uint8_t* high[kMaxGroup];  // Q6_0: 2-bit high plane of each matrix
     const __half* scales[kMaxGroup];
     void* Y[kMaxGroup];
     int32_t N[kMaxGroup];
@@ -873,16 +1031,16 @@ struct RingParams {
     int32_t n_mats;
     int32_t K, ldS, U;
     int32_t rows_per_cta, rows_total;
-    int32_t stage_bytes;          // one row of codes (+ Q6_0 high bits) + its scales, rounded up to 16
+    int32_t stage_bytes;          // one row of codes + its scales, rounded up to 16
     int32_t stages;               // ring depth (2..kRingMaxStages)
     int32_t epi;
     const __nv_bfloat16* X;
     int* status;
 };
 
-template <int FMT, int PF>
+template <int PF>
 __global__ void __launch_bounds__(kRingThreads, 2) gemv_ring_kernel(const __grid_constant__ RingParams p) {
-    constexpr int UW = (FMT == EMB_Q8_0) ? 16 : 32;
+    constexpr int UW = 16;
     constexpr int NT = kRingThreads, NWARP = NT / 32;
     extern __shared__ __align__(128) uint8_t smem[];
     uint64_t* full = reinterpret_cast<uint64_t*>(smem);              // [stages]
@@ -893,8 +1051,7 @@ __global__ void __launch_bounds__(kRingThreads, 2) gemv_ring_kernel(const __grid
     const int S = p.stages;
     const int t = threadIdx.x, lane = t & 31, warp = t >> 5;
     const int U = p.U;
-    const int64_t row_bytes = (FMT == EMB_Q8_0) ? int64_t(p.K) : int64_t(p.K) / 2;
-    const int64_t high_bytes = (FMT == EMB_Q6_0) ? int64_t(p.K) / 4 : 0;  // a multiple of 16
+    const int64_t row_bytes = p.K;
     const int r_begin = blockIdx.x * p.rows_per_cta;
     const int n_rows = min(p.rows_per_cta, p.rows_total - r_begin);
     // global row -> (matrix, row within it)
@@ -910,11 +1067,10 @@ __global__ void __launch_bounds__(kRingThreads, 2) gemv_ring_kernel(const __grid
         locate(r_begin + i, g, n);
         uint8_t* st = ring + stage * p.stage_bytes;
         uint64_t* bar = &full[stage];
-        const uint32_t cb = uint32_t(row_bytes), hb = uint32_t(high_bytes), sb = uint32_t(p.ldS) * 2u;
-        ptx::mbar_arrive_expect_tx(bar, cb + hb + sb);
+        const uint32_t cb = uint32_t(row_bytes), sb = uint32_t(p.ldS) * 2u;
+        ptx::mbar_arrive_expect_tx(bar, cb + sb);
         ptx::bulk_load(st, p.codes[g] + int64_t(n) * row_bytes, cb, bar);
-        if constexpr (FMT == EMB_Q6_0) ptx::bulk_load(st + row_bytes, p.high[g] + int64_t(n) * high_bytes, hb, bar);
-        ptx::bulk_load(st + row_bytes + high_bytes, p.scales[g] + int64_t(n) * p.ldS, sb, bar);
+        ptx::bulk_load(st + row_bytes, p.scales[g] + int64_t(n) * p.ldS, sb, bar);
     };
     if (t == 0) {
         *abort_flag = 0;
@@ -945,7 +1101,6 @@ __global__ void __launch_bounds__(kRingThreads, 2) gemv_ring_kernel(const __grid
             x[k][8 * v + 6] = lo_bf16(hx.w); x[k][8 * v + 7] = hi_bf16(hx.w);
         }
     }
-    const uint2 h0 = make_uint2(0, 0);
     bool ok = true;
     int flushed = 0;  // rows already reduced and stored
     // reduce and store rows [flushed, upto) of this CTA; false (the CTA leaves) if any of its
@@ -991,17 +1146,15 @@ __global__ void __launch_bounds__(kRingThreads, 2) gemv_ring_kernel(const __grid
         ok = __all_sync(0xffffffffu, ok && ptx::mbar_wait(&full[s], ph, abort_flag, p.status, kWaitLimitNs));
         if (ok) {
             const uint8_t* cs = ring + s * p.stage_bytes;
-            const __half* ss = reinterpret_cast<const __half*>(cs + row_bytes + high_bytes);
+            const __half* ss = reinterpret_cast<const __half*>(cs + row_bytes);
             float acc = 0.0f;
 #pragma unroll
             for (int k = 0; k < PF; ++k) {
                 const int uk = t + k * NT;
                 if (uk < U) {
                     const uint4 c = *reinterpret_cast<const uint4*>(cs + int64_t(uk) * 16);
-                    uint2 hq = h0;
-                    if constexpr (FMT == EMB_Q6_0) hq = *reinterpret_cast<const uint2*>(cs + row_bytes + int64_t(uk) * 8);
-                    const float d = __half2float(ss[(FMT == EMB_Q8_0) ? (uk >> 1) : uk]);
-                    acc = fmaf(d, dot_unit<FMT>(c, hq, x[k]), acc);
+                    const float d = __half2float(ss[uk >> 1]);
+                    acc = fmaf(d, dot_q8_unit(c, x[k]), acc);
                 }
             }
             __syncwarp();
@@ -1021,7 +1174,7 @@ __global__ void __launch_bounds__(kRingThreads, 2) gemv_ring_kernel(const __grid
     if (flushed < n_rows) flush(n_rows);  // (a CTA whose wait gave up leaves inside it)
 }
 
-template <int FMT, int PF>
+template <int PF>
 cudaError_t launch_ring_one(const RingParams& p, int ctas, size_t smem, bool pdl, cudaStream_t s) {
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3(ctas, 1, 1);
@@ -1033,10 +1186,10 @@ cudaError_t launch_ring_one(const RingParams& p, int ctas, size_t smem, bool pdl
     attr[0].val.programmaticStreamSerializationAllowed = 1;
     cfg.attrs = attr;
     cfg.numAttrs = pdl ? 1 : 0;
-    const cudaError_t e = cudaFuncSetAttribute(gemv_ring_kernel<FMT, PF>,
+    const cudaError_t e = cudaFuncSetAttribute(gemv_ring_kernel<PF>,
                                                cudaFuncAttributeMaxDynamicSharedMemorySize, int(smem));
     if (e != cudaSuccess) return e;
-    return cudaLaunchKernelEx(&cfg, gemv_ring_kernel<FMT, PF>, p);
+    return cudaLaunchKernelEx(&cfg, gemv_ring_kernel<PF>, p);
 }
 
 int gemv_sm_count() {
@@ -1050,30 +1203,34 @@ int gemv_sm_count() {
     return counts[dev];
 }
 
-// Which layers take the ring path: M = 1, Q8_0, Q4_0 or Q6_0 (K % 64 == 0, for its high
-// plane's 16-byte rows), rows longer than the staged path takes at M = 1 and than one pass
+// Which layers take the ring path: M = 1, Q8_0 (the other formats are faster on the tensor-core
+// kernel), rows longer than the staged path takes at M = 1 and than one pass
 // of 256 threads (2..4 units per thread), matrices of at least kStageMinBytes; two CTAs per
 // SM, rows split evenly (even runs for gated epilogues).
 // Measured on GB300, Gemma-2B decode step (paired runs on one box, 1000 steps): Q8_0 chain
-// 0.507 -> 0.477 ms and Q4_0 0.457 -> 0.455 against a kernel with two rows per CTA in
+// 0.507 -> 0.477 ms against a kernel with two rows per CTA in
 // registers and two in shared memory; a 72 KB ring instead of 56 KB was slower for Q8_0,
 // a CTA-wide barrier per row cost ~2 %, and stage indices by integer division ~4 %.
-bool launch_ring(const GroupRef& g, bool pdl, int* status, cudaStream_t s, cudaError_t& err) {
-    if (g.M != 1 || (g.fmt == EMB_Q6_0 && g.K % 64 != 0)) return false;
-    const int64_t row_bytes = (g.fmt == EMB_Q8_0) ? g.K : g.K / 2;
-    const int64_t high_bytes = (g.fmt == EMB_Q6_0) ? g.K / 4 : 0;
-    const int64_t U = (g.fmt == EMB_Q8_0) ? g.K / 16 : g.K / 32;
-    if (row_bytes + high_bytes <= kStageMaxRowBytesM1 || U <= kRingThreads || U > 4 * kRingThreads) return false;
+bool ring_takes(const GroupRef& g) {
+    if (g.M != 1 || g.fmt != EMB_Q8_0) return false;
+    const int64_t U = g.K / 16;
+    if (g.K <= kStageMaxRowBytesM1 || U <= kRingThreads || U > 4 * kRingThreads) return false;
     int64_t rows = 0;
     for (int i = 0; i < g.n_mats; ++i) rows += g.mats[i].N;
-    if (rows * (row_bytes + high_bytes) < kStageMinBytes) return false;
+    return rows * g.K >= kStageMinBytes;
+}
+
+bool launch_ring(const GroupRef& g, bool pdl, int* status, cudaStream_t s, cudaError_t& err) {
+    if (!ring_takes(g)) return false;
+    const int64_t row_bytes = g.K, U = g.K / 16;
+    int64_t rows = 0;
+    for (int i = 0; i < g.n_mats; ++i) rows += g.mats[i].N;
     const int sms = gemv_sm_count();
     if (sms <= 0) return false;
     RingParams p = {};
     int64_t r0 = 0;
     for (int i = 0; i < g.n_mats; ++i) {
         p.codes[i] = g.mats[i].codes;
-        p.high[i] = g.mats[i].high;
         p.scales[i] = g.mats[i].scales;
         p.Y[i] = g.mats[i].Y;
         p.N[i] = int32_t(g.mats[i].N);
@@ -1092,33 +1249,29 @@ bool launch_ring(const GroupRef& g, bool pdl, int* status, cudaStream_t s, cudaE
     if (g.epi >= EMB_EPI_GEGLU) rpc = (rpc + 1) & ~int64_t(1);  // gate/up pairs stay in one CTA
     p.rows_per_cta = int32_t(rpc);
     p.rows_total = int32_t(rows);
-    p.stage_bytes = int32_t((row_bytes + high_bytes + g.ldS * 2 + 15) & ~int64_t(15));
+    p.stage_bytes = int32_t((row_bytes + g.ldS * 2 + 15) & ~int64_t(15));
     p.stages = int32_t(std::min<int64_t>(kRingMaxStages, std::max<int64_t>(2, kRingBudget / p.stage_bytes)));
     const int ctas = int((rows + rpc - 1) / rpc);
     const size_t smem = kRingHeader + size_t(p.stages) * p.stage_bytes;
     const int pf = int((U + kRingThreads - 1) / kRingThreads);
-    if (g.fmt == EMB_Q8_0)
-        err = pf == 2 ? launch_ring_one<EMB_Q8_0, 2>(p, ctas, smem, pdl, s)
-            : pf == 3 ? launch_ring_one<EMB_Q8_0, 3>(p, ctas, smem, pdl, s)
-                      : launch_ring_one<EMB_Q8_0, 4>(p, ctas, smem, pdl, s);
-    else if (g.fmt == EMB_Q4_0)
-        err = pf == 2 ? launch_ring_one<EMB_Q4_0, 2>(p, ctas, smem, pdl, s)
-            : pf == 3 ? launch_ring_one<EMB_Q4_0, 3>(p, ctas, smem, pdl, s)
-                      : launch_ring_one<EMB_Q4_0, 4>(p, ctas, smem, pdl, s);
-    else
-        err = pf == 2 ? launch_ring_one<EMB_Q6_0, 2>(p, ctas, smem, pdl, s)
-            : pf == 3 ? launch_ring_one<EMB_Q6_0, 3>(p, ctas, smem, pdl, s)
-                      : launch_ring_one<EMB_Q6_0, 4>(p, ctas, smem, pdl, s);
+    err = pf == 2 ? launch_ring_one<2>(p, ctas, smem, pdl, s)
+        : pf == 3 ? launch_ring_one<3>(p, ctas, smem, pdl, s)
+                  : launch_ring_one<4>(p, ctas, smem, pdl, s);
     return true;
 }
 
 }  // namespace
 
+bool gemv_takes(const GroupRef& g) {
+    const int sms = gemv_sm_count();
+    return sms > 0 && tc_takes(g, sms);
+}
+
 cudaError_t launch_gemv_regs(const GroupRef& g, bool pdl, cudaStream_t s);
 
 cudaError_t launch_gemv(const GroupRef& g, bool pdl, int* status, cudaStream_t s) {
     cudaError_t err = cudaSuccess;
-    if (launch_q4_mma(g, pdl, status, s, err)) return err;
+    if (launch_tc(g, pdl, s, err)) return err;
     if (launch_staged(g, pdl, status, s, err)) return err;
     if (launch_ring(g, pdl, status, s, err)) return err;
     return launch_gemv_regs(g, pdl, s);

@@ -252,3 +252,46 @@ def test_precise_operand_flag_few_dominant_terms(cuda_device):
     assert (err_d <= (2.0 ** -8 + 2.0 ** -12) * S + 1e-6).all()
     assert (err_d > B).any()            # the single-operand form is not within 1e-3 here
     check_close(Yp.cpu().numpy(), Yref, B, "EMB_PRECISE_OPERAND")
+
+
+# the tensor-core GEMV's edges: a single row, row tiles one short and one over, a 32-weight row, an
+# odd block count, a ragged last 256-k chunk, one and several chunks per warp, sixteen warps per CTA
+# (long rows, few tiles), several row tiles per CTA; one token (long rows only), eight, and both
+# ends of the sixteen-token variant
+TC_SHAPES = [(3, 1, 64), (3, 15, 32), (4, 17, 96), (6, 33, 352), (8, 300, 2048), (9, 16, 2080), (16, 31, 256),
+             (13, 257, 4160), (1, 100, 4096), (1, 5000, 4128), (8, 70, 16384), (16, 2433, 5056), (7, 9000, 1088)]
+
+
+@pytest.mark.parametrize("fmt", FMTS + [emb.EMB_Q6_0])
+@pytest.mark.parametrize("M,N,K", TC_SHAPES)
+def test_tensor_core_gemv_has_exact_products(cuda_device, fmt, M, N, K):
+    """Products of codes and activations are exact, so only fp32 sums round: 32 products per block
+    (2^-23 of their magnitudes each, as tensor-core sums may truncate), the scaled block sums and
+    the warps' sums, K / 32 + 32 additions of 2^-24: no bf16 rounding of a weight (2^-9) fits."""
+    if fmt == emb.EMB_Q6_0 and K % 64:
+        K += 32
+    W = weight_np(N, K, M + N + K)
+    Xb = activation_bits_np(M, K, M + N + K + 1)
+    img = emb.quantize(fmt, torch.from_numpy(W).cuda())
+    X = to_dev_bf16(Xb)
+    Yref, B = oracle.qmatmul(fmt, oracle.quantize(fmt, W), Xb, N, K)
+    S = (B - 1e-6) / 1e-3
+    bound = (32 * 2.0 ** -23 + (K // 32 + 32) * 2.0 ** -24) * S + 1e-9
+    Y = torch.full((M, N), float("nan"), device="cuda")
+    emb.emb_qmatmul(fmt, img, X, Y, M, N, K)
+    again = torch.full_like(Y, float("nan"))
+    emb.emb_qmatmul(fmt, img, X, again, M, N, K)
+    torch.cuda.synchronize()
+    assert torch.equal(Y.view(torch.int32), again.view(torch.int32))
+    err = np.abs(Y.cpu().numpy().astype(np.float64) - Yref)
+    assert (err <= bound).all(), f"{int((err > bound).sum())} of {err.size} outside, worst {float((err / bound).max()):.2f}"
+    # a gated and an adding epilogue of the same sums
+    if N % 2 == 0:
+        H = torch.full((M, N // 2), float("nan"), dtype=torch.bfloat16, device="cuda")
+        emb.emb_qlayer_seq([(fmt, img, N, K, X, H, emb.EMB_EPI_SWIGLU)], M)
+        ref, b = oracle.epilogue_reference(oracle.EPI_SWIGLU, Yref, bound)
+        assert (np.abs(H.float().cpu().numpy().astype(np.float64) - ref) <= b).all()
+    R = torch.ones(M, N, device="cuda")
+    emb.emb_qlayer_seq([(fmt, img, N, K, X, R, emb.EMB_EPI_ADD)], M)
+    assert torch.equal(R, torch.ones_like(R) + Y)
+    assert emb.emb_device_status() == emb.EMB_OK
