@@ -257,3 +257,18 @@ def test_attention_plans(cuda_device, M, H, Hk, d, n0, n1, gain):
     again = _run_attention(*ins, H, Hk, d, scale)
     assert torch.equal(O.view(torch.int16), again.view(torch.int16))
     assert emb.emb_device_status() == emb.EMB_OK
+
+
+# the pairs per thread follow from head_dim (half divisible by 8, 4, 2, 1) and from the size
+@pytest.mark.parametrize("M,H,Hk,d,pos0", [(300, 8, 1, 256, 5), (900, 5, 3, 72, 100), (2000, 7, 2, 20, 1 << 20),
+                                           (3000, 3, 1, 6, 7), (1, 2, 1, 16, 0), (40, 4, 4, 512, 16000000)])
+def test_rope_access_widths(cuda_device, M, H, Hk, d, pos0):
+    rng = np.random.default_rng(M + H + d)
+    qb = oracle.bf16_round(rng.standard_normal((M, H * d)))
+    kb = oracle.bf16_round(rng.standard_normal((M, Hk * d)))
+    q, k = _bf16_dev(qb), _bf16_dev(kb)
+    emb.emb_rope_qk(q, H, k, Hk, d, pos0, 10000.0)
+    torch.cuda.synchronize()
+    for t, xb, heads in ((q, qb, H), (k, kb, Hk)):
+        ref, bound = oracle.rope_reference(xb, heads, d, pos0, 10000.0)
+        _check(_vals(t), ref, bound, f"rope d={d} heads={heads}")
