@@ -134,8 +134,8 @@ struct GroupRef {
 };
 
 // Weight-streaming GEMV for small M (register dequant, shuffle reductions).
-// pdl: launch with programmatic stream serialisation (the kernel reads X only after
-// griddepcontrol.wait, weights before).
+// pdl: the kernel reads weights before griddepcontrol.wait (X only after it); otherwise it waits
+// before it reads anything. Both are launched with programmatic stream serialisation.
 cudaError_t launch_gemv(const GroupRef& g, bool pdl, int* status, cudaStream_t s);
 // Whether a group of more than four tokens is faster through launch_gemv.
 bool gemv_takes(const GroupRef& g);

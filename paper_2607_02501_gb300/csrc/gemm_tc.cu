@@ -87,6 +87,7 @@ struct GemmParams {
     int32_t persist;                       // 1: CTAs loop over items (no K split)
     int32_t n_tt, n_items;                 // persistent: token tiles per weight tile, items
     int32_t streamk;                       // 1: the items' raw stages split evenly over the CTAs
+    int32_t wait_first;                    // 1: nothing is read before griddepcontrol.wait
     int32_t slot_floats;                   // stream-K: floats of one partial tile (P * T * 128)
     float* ws_part;                        // stream-K: one partial-tile slot per CTA
     uint32_t* ws_flag;                     // stream-K: one ready flag per CTA (zero between launches)
@@ -339,6 +340,7 @@ __global__ void __launch_bounds__(kThreads, 1) gemm_tc_kernel(const __grid_const
                 // the first raw stages before griddepcontrol.wait: weights never depend on
                 // the previous launch; X may be written by it, so only its rows' way towards
                 // L2 starts now (a hint: the TMA loads after the wait read the written values)
+                if (p.wait_first) ptx::griddep_wait();  // (the previous launch may have written the weights)
                 for (; raw_issued < nr && raw_issued < kRawStages; ++raw_issued) issue_raw(raw_issued);
                 const int x_rows = min(M - I.m0, P * T);
                 if (lane == 0 && x_rows > 0 && I.n0 == 0 && I.g == 0 && sg.r0 == 0)  // one CTA per token tile
@@ -859,7 +861,7 @@ int pick_stages_pair(int T) {
 }
 
 template <int FMT, bool SPLIT, int P, bool SK = false>
-cudaError_t launch_kernel(const GemmParams& p, int grid_x, int grid_y, bool pdl, cudaStream_t s) {
+cudaError_t launch_kernel(const GemmParams& p, int grid_x, int grid_y, cudaStream_t s) {
     // grid: x = token tile (fastest, so the CTAs sharing a weight tile run together and
     // read it from L2 after the first), y = weight-row tile, z = K split (one cluster)
     const int bytes = smem_bytes<FMT, SPLIT>(p.T, p.stages, p.P);
@@ -884,12 +886,9 @@ cudaError_t launch_kernel(const GemmParams& p, int grid_x, int grid_y, bool pdl,
     cfg.dynamicSmemBytes = size_t(bytes);
     cfg.stream = s;
     cudaLaunchAttribute attr[2];
-    int na = 0;
-    if (pdl) {
-        attr[na].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-        attr[na].val.programmaticStreamSerializationAllowed = 1;
-        ++na;
-    }
+    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[0].val.programmaticStreamSerializationAllowed = 1;
+    int na = 1;
     if (p.splits > 1) {
         attr[na].id = cudaLaunchAttributeClusterDimension;
         attr[na].val.clusterDim.x = 1;
@@ -1185,27 +1184,28 @@ cudaError_t launch_plan(const GroupRef& g, const GemmPlan& pl, bool pdl, int* st
     p.epi = g.epi;
     p.tmem_cols = kTmemCols;
     p.status = status;
+    p.wait_first = pdl ? 0 : 1;
     if (pl.streamk) {
         if (g.fmt == EMB_Q8_0)
-            return P == 2 ? launch_kernel<EMB_Q8_0, false, 2, true>(p, grid_x, grid_y, pdl, s)
-                          : launch_kernel<EMB_Q8_0, false, 1, true>(p, grid_x, grid_y, pdl, s);
+            return P == 2 ? launch_kernel<EMB_Q8_0, false, 2, true>(p, grid_x, grid_y, s)
+                          : launch_kernel<EMB_Q8_0, false, 1, true>(p, grid_x, grid_y, s);
         if (g.fmt == EMB_Q4_0)
-            return P == 2 ? launch_kernel<EMB_Q4_0, false, 2, true>(p, grid_x, grid_y, pdl, s)
-                          : launch_kernel<EMB_Q4_0, false, 1, true>(p, grid_x, grid_y, pdl, s);
-        return P == 2 ? launch_kernel<EMB_Q6_0, false, 2, true>(p, grid_x, grid_y, pdl, s)
-                      : launch_kernel<EMB_Q6_0, false, 1, true>(p, grid_x, grid_y, pdl, s);
+            return P == 2 ? launch_kernel<EMB_Q4_0, false, 2, true>(p, grid_x, grid_y, s)
+                          : launch_kernel<EMB_Q4_0, false, 1, true>(p, grid_x, grid_y, s);
+        return P == 2 ? launch_kernel<EMB_Q6_0, false, 2, true>(p, grid_x, grid_y, s)
+                      : launch_kernel<EMB_Q6_0, false, 1, true>(p, grid_x, grid_y, s);
     }
     if (g.fmt == EMB_Q8_0)
-        return split    ? launch_kernel<EMB_Q8_0, true, 1>(p, grid_x, grid_y, pdl, s)
-               : P == 2 ? launch_kernel<EMB_Q8_0, false, 2>(p, grid_x, grid_y, pdl, s)
-                        : launch_kernel<EMB_Q8_0, false, 1>(p, grid_x, grid_y, pdl, s);
+        return split    ? launch_kernel<EMB_Q8_0, true, 1>(p, grid_x, grid_y, s)
+               : P == 2 ? launch_kernel<EMB_Q8_0, false, 2>(p, grid_x, grid_y, s)
+                        : launch_kernel<EMB_Q8_0, false, 1>(p, grid_x, grid_y, s);
     if (g.fmt == EMB_Q4_0)
-        return split    ? launch_kernel<EMB_Q4_0, true, 1>(p, grid_x, grid_y, pdl, s)
-               : P == 2 ? launch_kernel<EMB_Q4_0, false, 2>(p, grid_x, grid_y, pdl, s)
-                        : launch_kernel<EMB_Q4_0, false, 1>(p, grid_x, grid_y, pdl, s);
-    return split    ? launch_kernel<EMB_Q6_0, true, 1>(p, grid_x, grid_y, pdl, s)
-           : P == 2 ? launch_kernel<EMB_Q6_0, false, 2>(p, grid_x, grid_y, pdl, s)
-                    : launch_kernel<EMB_Q6_0, false, 1>(p, grid_x, grid_y, pdl, s);
+        return split    ? launch_kernel<EMB_Q4_0, true, 1>(p, grid_x, grid_y, s)
+               : P == 2 ? launch_kernel<EMB_Q4_0, false, 2>(p, grid_x, grid_y, s)
+                        : launch_kernel<EMB_Q4_0, false, 1>(p, grid_x, grid_y, s);
+    return split    ? launch_kernel<EMB_Q6_0, true, 1>(p, grid_x, grid_y, s)
+           : P == 2 ? launch_kernel<EMB_Q6_0, false, 2>(p, grid_x, grid_y, s)
+                    : launch_kernel<EMB_Q6_0, false, 1>(p, grid_x, grid_y, s);
 }
 
 }  // namespace

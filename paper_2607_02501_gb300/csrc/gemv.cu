@@ -50,6 +50,7 @@ struct GemvParams {
     int32_t n_mats;
     int32_t M, K, ldS, U;          // U = 16-byte code units per row
     int32_t epi;                   // emb_epilogue (gated: R even, gate/up row pairs)
+    int32_t wait_first;            // 1: nothing is read before griddepcontrol.wait
     const __nv_bfloat16* X;
 };
 
@@ -105,6 +106,7 @@ __global__ void __launch_bounds__(NT) gemv_kernel(const __grid_constant__ GemvPa
     const int U = p.U;
 
     griddep_launch_dependents();
+    if (p.wait_first) griddep_wait();  // (the previous launch may have written the weights)
     // the activation rows towards L2 while the previous launch finishes (measured on GB300:
     // cold, they arrive ~2 us after the dependency wait, behind the weight stream); one CTA
     // per row block asks, since every CTA reads the same rows
@@ -238,7 +240,7 @@ __global__ void __launch_bounds__(NT) gemv_kernel(const __grid_constant__ GemvPa
 }
 
 template <int FMT, int R, int NT, int MT, int PF = 1>
-cudaError_t launch_one(const GemvParams& p, int grid_x, int grid_y, bool pdl, cudaStream_t s) {
+cudaError_t launch_one(const GemvParams& p, int grid_x, int grid_y, cudaStream_t s) {
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3(grid_x, grid_y, 1);
     cfg.blockDim = dim3(NT, 1, 1);
@@ -248,35 +250,35 @@ cudaError_t launch_one(const GemvParams& p, int grid_x, int grid_y, bool pdl, cu
     attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
     attr[0].val.programmaticStreamSerializationAllowed = 1;
     cfg.attrs = attr;
-    cfg.numAttrs = pdl ? 1 : 0;
+    cfg.numAttrs = 1;
     return cudaLaunchKernelEx(&cfg, gemv_kernel<FMT, R, NT, MT, PF>, p);
 }
 
 template <int FMT, int R, int NT>
-cudaError_t dispatch_mt(const GemvParams& p, int grid_x, int M, bool pdl, cudaStream_t s) {
+cudaError_t dispatch_mt(const GemvParams& p, int grid_x, int M, cudaStream_t s) {
     // Q8_0 rows longer than one pass of the CTA's threads (at most four) are loaded whole
     // before the wait (measured on GB300 on the Gemma-2B decode chain at M = 1, whose down
     // projection 2048 x 16384 took this path before the ring kernel: Q8_0 3899 -> 3987
     // GB/s). Not for Q4_0: its variant needs ~100 registers, halves the resident CTAs and
     // lost (2265 -> 2068).
     if constexpr (FMT == EMB_Q8_0 && R <= 2) {
-        if (M == 1 && p.U > NT && p.U <= 4 * NT) return launch_one<FMT, R, NT, 1, 4>(p, grid_x, 1, pdl, s);
+        if (M == 1 && p.U > NT && p.U <= 4 * NT) return launch_one<FMT, R, NT, 1, 4>(p, grid_x, 1, s);
     }
-    if (M == 1) return launch_one<FMT, R, NT, 1>(p, grid_x, 1, pdl, s);
+    if (M == 1) return launch_one<FMT, R, NT, 1>(p, grid_x, 1, s);
     // more tokens (see tc_takes): small Q8_0 layers at M = 2, Q6_0 with K % 64 != 0 at M <= 4
     if constexpr (FMT != EMB_Q4_0) {
-        if (M == 2) return launch_one<FMT, R, NT, 2>(p, grid_x, 1, pdl, s);
-        if constexpr (FMT == EMB_Q6_0) return launch_one<FMT, R, NT, 4>(p, grid_x, (M + 3) / 4, pdl, s);
+        if (M == 2) return launch_one<FMT, R, NT, 2>(p, grid_x, 1, s);
+        if constexpr (FMT == EMB_Q6_0) return launch_one<FMT, R, NT, 4>(p, grid_x, (M + 3) / 4, s);
     }
     return cudaErrorInvalidValue;
 }
 
 template <int FMT, int R>
-cudaError_t dispatch_nt(const GemvParams& p, int grid_x, int M, int NT, bool pdl, cudaStream_t s) {
-    if (NT == 256) return dispatch_mt<FMT, R, 256>(p, grid_x, M, pdl, s);
-    if (NT == 128) return dispatch_mt<FMT, R, 128>(p, grid_x, M, pdl, s);
-    if (NT == 64) return dispatch_mt<FMT, R, 64>(p, grid_x, M, pdl, s);
-    return dispatch_mt<FMT, R, 32>(p, grid_x, M, pdl, s);
+cudaError_t dispatch_nt(const GemvParams& p, int grid_x, int M, int NT, cudaStream_t s) {
+    if (NT == 256) return dispatch_mt<FMT, R, 256>(p, grid_x, M, s);
+    if (NT == 128) return dispatch_mt<FMT, R, 128>(p, grid_x, M, s);
+    if (NT == 64) return dispatch_mt<FMT, R, 64>(p, grid_x, M, s);
+    return dispatch_mt<FMT, R, 32>(p, grid_x, M, s);
 }
 
 // Threads per CTA (they split K): about 8 (Q8_0) or 4 (Q4_0) 16-byte units per thread
@@ -322,6 +324,7 @@ struct StagedParams {
     int32_t M, K, ldS, U;
     int32_t TR, WK;                // rows per tile, warps along K
     int32_t epi;                   // emb_epilogue (gated: RW and TR even)
+    int32_t wait_first;            // 1: nothing is read before griddepcontrol.wait
     const __nv_bfloat16* X;
     int* status;
 };
@@ -362,6 +365,7 @@ __global__ void __launch_bounds__(kStageThreads) gemv_staged_kernel(const __grid
         ptx::mbar_init(bar_w, 1);
         ptx::mbar_init(bar_x, 1);
         ptx::fence_mbar_init();
+        if (p.wait_first) ptx::griddep_wait();  // (the previous launch may have written the weights)
         ptx::mbar_arrive_expect_tx(bar_w, codes_bytes + hi_bytes + scales_bytes);
         ptx::bulk_load(codes_s, p.codes[g] + int64_t(row0) * row_bytes, codes_bytes, bar_w);
         if constexpr (FMT == EMB_Q6_0)
@@ -484,7 +488,7 @@ __global__ void __launch_bounds__(kStageThreads) gemv_staged_kernel(const __grid
 }
 
 template <int FMT, int RW>
-cudaError_t launch_staged_one(const StagedParams& p, int tiles, size_t smem, bool pdl, cudaStream_t s) {
+cudaError_t launch_staged_one(const StagedParams& p, int tiles, size_t smem, cudaStream_t s) {
     static_assert(kStageHeader + kStageXBytes + kStageBytes + kStageBytes / 8 <= 227 * 1024, "smem");
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3(tiles, 1, 1);
@@ -495,7 +499,7 @@ cudaError_t launch_staged_one(const StagedParams& p, int tiles, size_t smem, boo
     attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
     attr[0].val.programmaticStreamSerializationAllowed = 1;
     cfg.attrs = attr;
-    cfg.numAttrs = pdl ? 1 : 0;
+    cfg.numAttrs = 1;
     if (smem > 48 * 1024) {
         // once per instantiation and device is enough, but the call is cheap and idempotent
         const cudaError_t e = cudaFuncSetAttribute(gemv_staged_kernel<FMT, RW, 1>,
@@ -507,10 +511,10 @@ cudaError_t launch_staged_one(const StagedParams& p, int tiles, size_t smem, boo
 }
 
 template <int FMT>
-cudaError_t launch_staged_rw(const StagedParams& p, int RW, int tiles, size_t smem, bool pdl, cudaStream_t s) {
-    if (RW == 4) return launch_staged_one<FMT, 4>(p, tiles, smem, pdl, s);
-    if (RW == 2) return launch_staged_one<FMT, 2>(p, tiles, smem, pdl, s);
-    return launch_staged_one<FMT, 1>(p, tiles, smem, pdl, s);
+cudaError_t launch_staged_rw(const StagedParams& p, int RW, int tiles, size_t smem, cudaStream_t s) {
+    if (RW == 4) return launch_staged_one<FMT, 4>(p, tiles, smem, s);
+    if (RW == 2) return launch_staged_one<FMT, 2>(p, tiles, smem, s);
+    return launch_staged_one<FMT, 1>(p, tiles, smem, s);
 }
 
 // Tile shape: rows per warp RW and warps along K WK (TR = RW * 4 / WK rows per tile),
@@ -590,11 +594,12 @@ bool launch_staged(const GroupRef& g, bool pdl, int* status, cudaStream_t s, cud
     p.WK = WK;
     p.epi = g.epi;
     p.X = g.X;
+    p.wait_first = pdl ? 0 : 1;
     p.status = status;
     const size_t smem = kStageHeader + size_t(g.K) * 2 + size_t(TR) * size_t(weight_row_bytes + g.ldS * 2);
-    err = g.fmt == EMB_Q8_0   ? launch_staged_rw<EMB_Q8_0>(p, RW, tiles, smem, pdl, s)
-          : g.fmt == EMB_Q6_0 ? launch_staged_rw<EMB_Q6_0>(p, RW, tiles, smem, pdl, s)
-                              : launch_staged_rw<EMB_Q4_0>(p, RW, tiles, smem, pdl, s);
+    err = g.fmt == EMB_Q8_0   ? launch_staged_rw<EMB_Q8_0>(p, RW, tiles, smem, s)
+          : g.fmt == EMB_Q6_0 ? launch_staged_rw<EMB_Q6_0>(p, RW, tiles, smem, s)
+                              : launch_staged_rw<EMB_Q4_0>(p, RW, tiles, smem, s);
     return true;
 }
 
@@ -643,6 +648,7 @@ struct TcParams {
     int32_t n_mats;
     int32_t M, K, ldS;
     int32_t epi;                   // emb_epilogue
+    int32_t wait_first;            // 1: nothing is read before griddepcontrol.wait
     const __nv_bfloat16* X;
 };
 
@@ -772,6 +778,7 @@ __global__ void __launch_bounds__(32 * NW, 16 / NW) gemv_tc_kernel(const __grid_
         }
         asm volatile("cp.async.commit_group;" ::: "memory");
     };
+    if (p.wait_first) griddep_wait();  // (the previous launch may have written the weights)
 #pragma unroll
     for (int i = 0; i < kTcStages; ++i) issue_next(i);
     if (threadIdx.x == 0 && blockIdx.x == 0) ptx::prefetch_l2(p.X, uint32_t(p.M) * uint32_t(p.K) * 2u);
@@ -918,7 +925,7 @@ __global__ void __launch_bounds__(32 * NW, 16 / NW) gemv_tc_kernel(const __grid_
 int gemv_sm_count();
 
 template <int FMT, int NT, int NW>
-cudaError_t launch_tc_one(const TcParams& p, int grid, bool pdl, cudaStream_t s) {
+cudaError_t launch_tc_one(const TcParams& p, int grid, cudaStream_t s) {
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3(grid, 1, 1);
     cfg.blockDim = dim3(32 * NW, 1, 1);
@@ -931,17 +938,17 @@ cudaError_t launch_tc_one(const TcParams& p, int grid, bool pdl, cudaStream_t s)
     attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
     attr[0].val.programmaticStreamSerializationAllowed = 1;
     cfg.attrs = attr;
-    cfg.numAttrs = pdl ? 1 : 0;
+    cfg.numAttrs = 1;
     return cudaLaunchKernelEx(&cfg, gemv_tc_kernel<FMT, NT, NW>, p);
 }
 
 template <int FMT>
-cudaError_t launch_tc_fmt(const TcParams& p, int tiles, int sms, bool pdl, cudaStream_t s) {
+cudaError_t launch_tc_fmt(const TcParams& p, int tiles, int sms, cudaStream_t s) {
     // long rows whose tiles leave each SM at most one CTA: sixteen warps
     const bool wide = tiles <= sms && p.K > 8 * kTcBlocks * kQBlock;
     const int grid = std::min(tiles, 2 * sms);
-    if (p.M <= 8) return wide ? launch_tc_one<FMT, 1, 16>(p, tiles, pdl, s) : launch_tc_one<FMT, 1, 8>(p, grid, pdl, s);
-    return wide ? launch_tc_one<FMT, 2, 16>(p, tiles, pdl, s) : launch_tc_one<FMT, 2, 8>(p, grid, pdl, s);
+    if (p.M <= 8) return wide ? launch_tc_one<FMT, 1, 16>(p, tiles, s) : launch_tc_one<FMT, 1, 8>(p, grid, s);
+    return wide ? launch_tc_one<FMT, 2, 16>(p, tiles, s) : launch_tc_one<FMT, 2, 8>(p, grid, s);
 }
 
 bool ring_takes(const GroupRef& g);
@@ -995,9 +1002,10 @@ bool launch_tc(const GroupRef& g, bool pdl, cudaStream_t s, cudaError_t& err) {
     p.ldS = int32_t(g.ldS);
     p.epi = g.epi;
     p.X = g.X;
-    err = g.fmt == EMB_Q8_0   ? launch_tc_fmt<EMB_Q8_0>(p, int(tiles), sms, pdl, s)
-          : g.fmt == EMB_Q4_0 ? launch_tc_fmt<EMB_Q4_0>(p, int(tiles), sms, pdl, s)
-                              : launch_tc_fmt<EMB_Q6_0>(p, int(tiles), sms, pdl, s);
+    p.wait_first = pdl ? 0 : 1;
+    err = g.fmt == EMB_Q8_0   ? launch_tc_fmt<EMB_Q8_0>(p, int(tiles), sms, s)
+          : g.fmt == EMB_Q4_0 ? launch_tc_fmt<EMB_Q4_0>(p, int(tiles), sms, s)
+                              : launch_tc_fmt<EMB_Q6_0>(p, int(tiles), sms, s);
     return true;
 }
 
@@ -1034,6 +1042,7 @@ struct RingParams {
     int32_t stage_bytes;          // one row of codes + its scales, rounded up to 16
     int32_t stages;               // ring depth (2..kRingMaxStages)
     int32_t epi;
+    int32_t wait_first;            // 1: nothing is read before griddepcontrol.wait
     const __nv_bfloat16* X;
     int* status;
 };
@@ -1079,6 +1088,7 @@ __global__ void __launch_bounds__(kRingThreads, 2) gemv_ring_kernel(const __grid
             ptx::mbar_init(&empty[i], NWARP);
         }
         ptx::fence_mbar_init();
+        if (p.wait_first) ptx::griddep_wait();  // (the previous launch may have written the weights)
         for (int i = 0; i < S && i < n_rows; ++i) issue(i, i);
         // the activation row towards L2 while the previous launch finishes (one CTA asks)
         if (blockIdx.x == 0) ptx::prefetch_l2(p.X, uint32_t(p.K) * 2u);
@@ -1175,7 +1185,7 @@ __global__ void __launch_bounds__(kRingThreads, 2) gemv_ring_kernel(const __grid
 }
 
 template <int PF>
-cudaError_t launch_ring_one(const RingParams& p, int ctas, size_t smem, bool pdl, cudaStream_t s) {
+cudaError_t launch_ring_one(const RingParams& p, int ctas, size_t smem, cudaStream_t s) {
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3(ctas, 1, 1);
     cfg.blockDim = dim3(kRingThreads, 1, 1);
@@ -1185,7 +1195,7 @@ cudaError_t launch_ring_one(const RingParams& p, int ctas, size_t smem, bool pdl
     attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
     attr[0].val.programmaticStreamSerializationAllowed = 1;
     cfg.attrs = attr;
-    cfg.numAttrs = pdl ? 1 : 0;
+    cfg.numAttrs = 1;
     const cudaError_t e = cudaFuncSetAttribute(gemv_ring_kernel<PF>,
                                                cudaFuncAttributeMaxDynamicSharedMemorySize, int(smem));
     if (e != cudaSuccess) return e;
@@ -1244,6 +1254,7 @@ bool launch_ring(const GroupRef& g, bool pdl, int* status, cudaStream_t s, cudaE
     p.U = int32_t(U);
     p.epi = g.epi;
     p.X = g.X;
+    p.wait_first = pdl ? 0 : 1;
     p.status = status;
     int64_t rpc = (rows + 2 * sms - 1) / (2 * sms);
     if (g.epi >= EMB_EPI_GEGLU) rpc = (rpc + 1) & ~int64_t(1);  // gate/up pairs stay in one CTA
@@ -1254,9 +1265,9 @@ bool launch_ring(const GroupRef& g, bool pdl, int* status, cudaStream_t s, cudaE
     const int ctas = int((rows + rpc - 1) / rpc);
     const size_t smem = kRingHeader + size_t(p.stages) * p.stage_bytes;
     const int pf = int((U + kRingThreads - 1) / kRingThreads);
-    err = pf == 2 ? launch_ring_one<2>(p, ctas, smem, pdl, s)
-        : pf == 3 ? launch_ring_one<3>(p, ctas, smem, pdl, s)
-                  : launch_ring_one<4>(p, ctas, smem, pdl, s);
+    err = pf == 2 ? launch_ring_one<2>(p, ctas, smem, s)
+        : pf == 3 ? launch_ring_one<3>(p, ctas, smem, s)
+                  : launch_ring_one<4>(p, ctas, smem, s);
     return true;
 }
 
@@ -1306,19 +1317,20 @@ cudaError_t launch_gemv_regs(const GroupRef& g, bool pdl, cudaStream_t s) {
     p.U = U;
     p.epi = g.epi;
     p.X = g.X;
+    p.wait_first = pdl ? 0 : 1;
     const int NT = pick_threads(U, g.fmt, tiles);
     const int M = int(g.M);
     if (g.fmt == EMB_Q8_0)
-        return R == 4 ? dispatch_nt<EMB_Q8_0, 4>(p, tiles, M, NT, pdl, s)
-             : R == 2 ? dispatch_nt<EMB_Q8_0, 2>(p, tiles, M, NT, pdl, s)
-                      : dispatch_nt<EMB_Q8_0, 1>(p, tiles, M, NT, pdl, s);
+        return R == 4 ? dispatch_nt<EMB_Q8_0, 4>(p, tiles, M, NT, s)
+             : R == 2 ? dispatch_nt<EMB_Q8_0, 2>(p, tiles, M, NT, s)
+                      : dispatch_nt<EMB_Q8_0, 1>(p, tiles, M, NT, s);
     if (g.fmt == EMB_Q4_0)
-        return R == 4 ? dispatch_nt<EMB_Q4_0, 4>(p, tiles, M, NT, pdl, s)
-             : R == 2 ? dispatch_nt<EMB_Q4_0, 2>(p, tiles, M, NT, pdl, s)
-                      : dispatch_nt<EMB_Q4_0, 1>(p, tiles, M, NT, pdl, s);
-    return R == 4 ? dispatch_nt<EMB_Q6_0, 4>(p, tiles, M, NT, pdl, s)
-         : R == 2 ? dispatch_nt<EMB_Q6_0, 2>(p, tiles, M, NT, pdl, s)
-                  : dispatch_nt<EMB_Q6_0, 1>(p, tiles, M, NT, pdl, s);
+        return R == 4 ? dispatch_nt<EMB_Q4_0, 4>(p, tiles, M, NT, s)
+             : R == 2 ? dispatch_nt<EMB_Q4_0, 2>(p, tiles, M, NT, s)
+                      : dispatch_nt<EMB_Q4_0, 1>(p, tiles, M, NT, s);
+    return R == 4 ? dispatch_nt<EMB_Q6_0, 4>(p, tiles, M, NT, s)
+         : R == 2 ? dispatch_nt<EMB_Q6_0, 2>(p, tiles, M, NT, s)
+                  : dispatch_nt<EMB_Q6_0, 1>(p, tiles, M, NT, s);
 }
 
 }  // namespace emb
