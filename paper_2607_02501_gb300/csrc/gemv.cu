@@ -25,6 +25,7 @@
 // just written X, and after griddepcontrol.wait its writes are visible to ordinary loads.
 // Up to kMaxGroup matrices that read the same X (q/k/v or gate/up) share one launch.
 #include <algorithm>
+#include <atomic>
 #include <mutex>
 
 #include "dequant_dot.cuh"
@@ -39,6 +40,20 @@ using dq::dot_q6_unit;
 using dq::dot_q8_unit;
 using dq::hi_bf16;
 using dq::lo_bf16;
+
+// cudaFuncSetAttribute(MaxDynamicSharedMemorySize) once per kernel and device (the call is
+// idempotent, and threads may race to make it).
+template <typename K>
+cudaError_t allow_smem(K* kernel, int bytes, std::atomic<uint64_t>& done) {
+    int dev = 0;
+    cudaError_t e = cudaGetDevice(&dev);
+    if (e != cudaSuccess) return e;
+    const uint64_t bit = dev >= 0 && dev < 64 ? uint64_t(1) << dev : 0;
+    if (bit && (done.load(std::memory_order_relaxed) & bit)) return cudaSuccess;
+    e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
+    if (e == cudaSuccess) done.fetch_or(bit, std::memory_order_relaxed);
+    return e;
+}
 
 struct GemvParams {
     const uint8_t* codes[kMaxGroup];
@@ -501,10 +516,9 @@ cudaError_t launch_staged_one(const StagedParams& p, int tiles, size_t smem, cud
     cfg.attrs = attr;
     cfg.numAttrs = 1;
     if (smem > 48 * 1024) {
-        // once per instantiation and device is enough, but the call is cheap and idempotent
-        const cudaError_t e = cudaFuncSetAttribute(gemv_staged_kernel<FMT, RW, 1>,
-                                                   cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                                   int(kStageHeader + kStageXBytes + kStageBytes + kStageBytes / 8));
+        static std::atomic<uint64_t> done{0};
+        const cudaError_t e = allow_smem(gemv_staged_kernel<FMT, RW, 1>,
+                                         int(kStageHeader + kStageXBytes + kStageBytes + kStageBytes / 8), done);
         if (e != cudaSuccess) return e;
     }
     return cudaLaunchKernelEx(&cfg, gemv_staged_kernel<FMT, RW, 1>, p);
@@ -931,8 +945,8 @@ cudaError_t launch_tc_one(const TcParams& p, int grid, cudaStream_t s) {
     cfg.blockDim = dim3(32 * NW, 1, 1);
     cfg.dynamicSmemBytes = kTcSmem<FMT, NT, NW>;
     cfg.stream = s;
-    const cudaError_t e = cudaFuncSetAttribute(gemv_tc_kernel<FMT, NT, NW>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                               kTcSmem<FMT, NT, NW>);
+    static std::atomic<uint64_t> done{0};
+    const cudaError_t e = allow_smem(gemv_tc_kernel<FMT, NT, NW>, kTcSmem<FMT, NT, NW>, done);
     if (e != cudaSuccess) return e;
     cudaLaunchAttribute attr[1];
     attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
@@ -1196,8 +1210,9 @@ cudaError_t launch_ring_one(const RingParams& p, int ctas, size_t smem, cudaStre
     attr[0].val.programmaticStreamSerializationAllowed = 1;
     cfg.attrs = attr;
     cfg.numAttrs = 1;
-    const cudaError_t e = cudaFuncSetAttribute(gemv_ring_kernel<PF>,
-                                               cudaFuncAttributeMaxDynamicSharedMemorySize, int(smem));
+    // (two stages of the longest row, 16 KB of codes, fit the budget too)
+    static std::atomic<uint64_t> done{0};
+    const cudaError_t e = allow_smem(gemv_ring_kernel<PF>, kRingHeader + kRingBudget, done);
     if (e != cudaSuccess) return e;
     return cudaLaunchKernelEx(&cfg, gemv_ring_kernel<PF>, p);
 }
