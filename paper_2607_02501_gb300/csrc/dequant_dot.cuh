@@ -1,5 +1,6 @@
 // Exact in-register dequantisation and dot products of one 16-byte unit of packed codes
-// with fp32 activations, used by the GEMV kernels (gemv.cu). Each code becomes an exact fp32 value through a "magic number"
+// with fp32 activations, used by the GEMV kernels (gemv.cu), and exact weights for the bf16 operands of
+// the tensor-core kernels (gemm_tc.cu, gemv.cu). Each code becomes an exact fp32 value through a "magic number"
 // (the code placed in the mantissa of a float with a fixed exponent, the offset subtracted
 // exactly); products and their sums are fp32 FMAs on packed pairs (FFMA2) in a fixed order.
 #pragma once
@@ -20,6 +21,26 @@ __device__ __forceinline__ uint32_t and_or(uint32_t a, uint32_t mask, uint32_t b
 }
 // Nibble field of v selected by mask, as the binary32 2^23 + field (exact).
 __device__ __forceinline__ float magic(uint32_t v, uint32_t mask) { return __uint_as_float(and_or(v, mask, 0x4B000000u)); }
+
+__device__ __forceinline__ uint32_t pack_bf16(float a, float b) {
+    __nv_bfloat162 h = __floats2bfloat162_rn(a, b);
+    return *reinterpret_cast<uint32_t*>(&h);
+}
+
+// Four 8-bit values b_i (the bytes of u) -> w'_i = d*(b_i - bias) exactly, as two fp32 pairs.
+// __byte_perm(u, 0x47000000, 0x7504 | i<<4) is the binary32 with exponent 15 whose
+// fraction holds b_i at bits 8..15, i.e. 2^15 + b_i; one FMA with (d, -bias*d) gives
+// d*(b_i - bias) exactly (the product has at most 19 significant bits; bias*d at most 24).
+__device__ __forceinline__ void bytes_to_w(uint32_t u, float d, float nbd, float2& w01,
+                                           float2& w23) {
+    const float2 dd = make_float2(d, d), oo = make_float2(nbd, nbd);
+    w01 = __ffma2_rn(make_float2(__uint_as_float(__byte_perm(u, 0x47000000u, 0x7504u)),
+                                 __uint_as_float(__byte_perm(u, 0x47000000u, 0x7514u))),
+                     dd, oo);
+    w23 = __ffma2_rn(make_float2(__uint_as_float(__byte_perm(u, 0x47000000u, 0x7524u)),
+                                 __uint_as_float(__byte_perm(u, 0x47000000u, 0x7534u))),
+                     dd, oo);
+}
 
 // 16 Q8_0 codes (one unit) times 16 fp32 activations -> fp32 partial sum.
 // __byte_perm(v ^ 0x80808080, 0x4B000000, 0x7540 + i) is the binary32 2^23 + (q_i + 128)

@@ -47,6 +47,7 @@
 #include <cstring>
 #include <mutex>
 
+#include "dequant_dot.cuh"
 #include "ptx.cuh"
 
 namespace emb {
@@ -109,25 +110,8 @@ __device__ __forceinline__ uint4 lds128(const uint8_t* p) {
     return *reinterpret_cast<const uint4*>(p);
 }
 
-__device__ __forceinline__ uint32_t pack_bf16(float a, float b) {
-    __nv_bfloat162 h = __floats2bfloat162_rn(a, b);
-    return *reinterpret_cast<uint32_t*>(&h);
-}
-
-// Four 8-bit values b_i (the bytes of u) -> w'_i = d*(b_i - bias) exactly, as two fp32 pairs.
-// __byte_perm(u, 0x47000000, 0x7504 | i<<4) is the binary32 with exponent 15 whose
-// fraction holds b_i at bits 8..15, i.e. 2^15 + b_i; one FMA with (d, -bias*d) gives
-// d*(b_i - bias) exactly (the product has at most 19 significant bits; bias*d at most 24).
-__device__ __forceinline__ void bytes_to_w(uint32_t u, float d, float nbd, float2& w01,
-                                           float2& w23) {
-    const float2 dd = make_float2(d, d), oo = make_float2(nbd, nbd);
-    w01 = __ffma2_rn(make_float2(__uint_as_float(__byte_perm(u, 0x47000000u, 0x7504u)),
-                                 __uint_as_float(__byte_perm(u, 0x47000000u, 0x7514u))),
-                     dd, oo);
-    w23 = __ffma2_rn(make_float2(__uint_as_float(__byte_perm(u, 0x47000000u, 0x7524u)),
-                                 __uint_as_float(__byte_perm(u, 0x47000000u, 0x7534u))),
-                     dd, oo);
-}
+using dq::bytes_to_w;
+using dq::pack_bf16;
 
 // 8 consecutive w' (two input words) -> one 16-byte chunk of bf16 (hi), and for the split
 // variant the residual chunk lo = bf16(w' - hi).

@@ -1,8 +1,10 @@
-// GEMV for small token counts (action-token decode, M = 1; a few tokens, M = 2..16).
+// GEMV for small token counts (action-token decode, M = 1; a few tokens, M = 2..16), and the
+// tensor-core kernel for an action chunk (M = 17..64).
 //
 // The paper's batch-1 setting (Section 3.1, challenge 2) makes every linear layer a
 // matrix-vector product whose cost is reading the packed weights once from HBM.
-// Four kernels:
+// Five kernels:
+//   * the chunk kernel (M = 17..64, K >= 1024; described at its definition);
 //   * the tensor-core kernel (M = 2..16, and long rows at M = 1): dot products on mma.sync with
 //     the codes exact in bf16 (described at its definition);
 //   * the staged kernel (large layers with short rows at M = 1): each CTA pulls one
@@ -636,14 +638,12 @@ bool launch_staged(const GroupRef& g, bool pdl, int* status, cudaStream_t s, cud
 // worth is issued before griddepcontrol.wait; the activations come by ordinary cached loads after.
 //
 // Fragment mapping (any permutation of K inside a block is valid as long as A and B use the same
-// one): lane (g, t) = (lane / 4, lane % 4) holds tile rows rho(g) and rho(g) + 8.
-//  * Q8_0: codes 8t .. 8t + 7 of the block (one 8-byte load per row; rho = 0, 2, 4, 6, 1, 3, 5, 7
-//    puts a half warp's 16 loads into distinct banks). MMA 0 takes codes (8t, 8t + 1) as k slots
-//    (2t, 2t + 1) and (8t + 2, 8t + 3) as (2t + 8, 2t + 9), MMA 1 the other four; its activations
-//    are token g's x[8t .. 8t + 7], one 16-byte load.
-//  * Q4_0, Q6_0: 32-bit word t of the block (low nibbles codes 4t .. 4t + 3, high nibbles 16 + 4t
-//    ..), rho = identity. MMA 0 takes the low, MMA 1 the high nibbles: (bytes 0, 1) -> slots
-//    (2t, 2t + 1), (bytes 2, 3) -> (2t + 8, 2t + 9).
+// one): lane (g, t) = (lane / 4, lane % 4) holds tile rows rho(g) and rho(g) + 8
+// (rho is the identity but for Q8_0, where 0, 2, 4, 6, 1, 3, 5, 7 puts a half warp's loads into
+// distinct banks) and of each block the codes 8t .. 8t + 7: 8 bytes of Q8_0, or one nibble of each byte
+// of words 2(t & 1) and 2(t & 1) + 1. MMA 0 takes codes (8t, 8t + 1) as k slots (2t, 2t + 1) and
+// (8t + 2, 8t + 3) as (2t + 8, 2t + 9), MMA 1 the other four; the activations are token g's
+// x[8t .. 8t + 7], one 16-byte load.
 // What bounds it: the codes-to-bf16 arithmetic (2 to 3 instructions per weight, on the pipe that
 // also permutes bytes) and, for few rows, latency: Q6_0 32768 x 2048 at M = 4 15.4 us against 8.1
 // for its bytes. Without the shared-memory ring (fragments loaded from global memory directly,
@@ -697,11 +697,6 @@ __device__ __forceinline__ uint2 ld_shared_u2(uint32_t a) {
     asm volatile("ld.shared.v2.u32 {%0, %1}, [%2];" : "=r"(v.x), "=r"(v.y) : "r"(a));
     return v;
 }
-__device__ __forceinline__ uint32_t ld_shared_u1(uint32_t a) {
-    uint32_t v;
-    asm volatile("ld.shared.u32 %0, [%1];" : "=r"(v) : "r"(a));
-    return v;
-}
 __device__ __forceinline__ float ld_shared_half(uint32_t a) {
     uint16_t v;
     asm volatile("ld.shared.u16 %0, [%1];" : "=h"(v) : "r"(a));
@@ -720,6 +715,79 @@ struct TcStage {
     static constexpr int kHigh = FMT == EMB_Q6_0 ? kTcRows * 64 : 0;
     static constexpr int kBytes = kCodes + kHigh + kTcRows * 16;
 };
+// Matrix of a row tile.
+__device__ __forceinline__ int tc_mat_of(const TcParams& p, int tile) {
+    int gm = 0;
+#pragma unroll
+    for (int i = 1; i < kMaxGroup; ++i)
+        if (i < p.n_mats && tile >= p.tile0[i]) gm = i;
+    return gm;
+}
+
+// Issue the copies of one chunk (256 k from block kb0) of a row tile into a stage: blocks past the
+// row are zero codes with zero scales (the scale row is zero-padded to eight), rows past N read row
+// N - 1 (never stored).
+template <int FMT>
+__device__ __forceinline__ void tc_issue(const TcParams& p, int tile, int kb0, uint32_t st, int lane) {
+    using St = TcStage<FMT>;
+    const int nb = p.K / kQBlock;
+    const int64_t row_bytes = FMT == EMB_Q8_0 ? int64_t(p.K) : int64_t(p.K) / 2;
+    const int gm = tc_mat_of(p, tile);
+    const int row0 = (tile - p.tile0[gm]) * kTcRows, last = p.N[gm] - 1;
+    constexpr int kG = FMT == EMB_Q8_0 ? 16 : 8;  // 16-byte granules of a row's codes
+    const int c = lane % kG, kbg = kb0 + (FMT == EMB_Q8_0 ? c >> 1 : c);  // the granule's block
+#pragma unroll
+    for (int i = 0; i < kTcRows * kG / 32; ++i) {
+        const int r = i * (32 / kG) + lane / kG;
+        const uint8_t* src = p.codes[gm] + int64_t(min(row0 + r, last)) * row_bytes +
+                             (kbg < nb ? int64_t(kb0) * (FMT == EMB_Q8_0 ? 32 : 16) + c * 16 : 0);
+        cp_async16(st + r * (kG * 16) + ((c ^ (r & 7)) << 4), src, kbg < nb);
+    }
+    if constexpr (FMT == EMB_Q6_0) {
+        const int ch = lane & 3;
+#pragma unroll
+        for (int i = 0; i < 2; ++i) {
+            const int r = 8 * i + (lane >> 2);
+            const bool ok = kb0 + 2 * ch < nb;  // nb is even (K % 64 == 0)
+            const uint8_t* src =
+                p.high[gm] + int64_t(min(row0 + r, last)) * (p.K / 4) + (ok ? int64_t(kb0) * 8 + ch * 16 : 0);
+            cp_async16(st + St::kCodes + r * 64 + ((ch ^ ((r >> 1) & 3)) << 4), src, ok);
+        }
+    }
+    if (lane < kTcRows) {
+        const __half* src = p.scales[gm] + int64_t(min(row0 + lane, last)) * p.ldS + (kb0 < nb ? kb0 : 0);
+        cp_async16(st + St::kCodes + St::kHigh + lane * 16, src, kb0 < nb);
+    }
+}
+
+// The tile row whose fragment lane (g, t) holds as MMA row g (+ 8 for MMA row g + 8).
+template <int FMT>
+__device__ __forceinline__ int tc_row(int g) {
+    return FMT == EMB_Q8_0 ? (2 * g) % 7 + (g == 7 ? 7 : 0) : g;  // rho(g): 0, 2, 4, 6, 1, 3, 5, 7
+}
+// Codes 8t .. 8t + 7 of block i of a stage's row, one per byte (Q8_0 signed, else unsigned).
+template <int FMT>
+__device__ __forceinline__ uint2 tc_codes(uint32_t st, int row, int i, int t) {
+    if constexpr (FMT == EMB_Q8_0) {
+        return ld_shared_u2(st + row * 256 + (((2 * i + (t >> 1)) ^ (row & 7)) << 4) + (t & 1) * 8);
+    } else {
+        // words 2(t & 1), 2(t & 1) + 1 of the block, low nibbles for t < 2, high ones for t >= 2
+        const uint32_t m = 0x0F0F0F0Fu;
+        uint2 w = ld_shared_u2(st + row * 128 + ((i ^ (row & 7)) << 4) + (t & 1) * 8);
+        w.x = (w.x >> (4 * (t >> 1))) & m;
+        w.y = (w.y >> (4 * (t >> 1))) & m;
+        if constexpr (FMT == EMB_Q6_0) {
+            // the high bits of word j are in high word j & 1, shifted by 2 (j >> 1), by 4 more for
+            // the high nibbles' codes
+            const uint2 h = ld_shared_u2(st + TcStage<FMT>::kCodes + row * 64 + (((i >> 1) ^ ((row >> 1) & 3)) << 4) + (i & 1) * 8);
+            const int sh = 2 * (t & 1) + 4 * (t >> 1);
+            w.x |= ((h.x >> sh) & 0x03030303u) << 4;
+            w.y |= ((h.y >> sh) & 0x03030303u) << 4;
+        }
+        return w;
+    }
+}
+
 // Ring depth: three stages, two where the sums of sixteen tokens would leave an SM one CTA.
 template <int FMT, int NT, int NW>
 constexpr int kTcDepth = FMT == EMB_Q8_0 && NT == 2 && NW == 8 ? 2 : 3;
@@ -736,54 +804,14 @@ __global__ void __launch_bounds__(32 * NW, 16 / NW) gemv_tc_kernel(const __grid_
     const int g = lane >> 2, t = lane & 3;
     const int nb = p.K / kQBlock;
     const int tiles = p.tile0[p.n_mats];
-    const int64_t row_bytes = FMT == EMB_Q8_0 ? int64_t(p.K) : int64_t(p.K) / 2;
     const uint32_t ring = ptx::smem_u32(smem) + warp * kTcStages * St::kBytes;
-    auto mat_of = [&](int tile) {
-        int gm = 0;
-#pragma unroll
-        for (int i = 1; i < kMaxGroup; ++i)
-            if (i < p.n_mats && tile >= p.tile0[i]) gm = i;
-        return gm;
-    };
-
     griddep_launch_dependents();
-    // chunk of a row tile whose first block is kb0: blocks past the row are zero codes with zero
-    // scales (the scale row is zero-padded to eight), rows past N read row N - 1 (never stored)
-    auto issue = [&](int tile, int kb0, int stage) {
-        const int gm = mat_of(tile);
-        const int row0 = (tile - p.tile0[gm]) * kTcRows, last = p.N[gm] - 1;
-        const uint32_t st = ring + stage * St::kBytes;
-        constexpr int kG = FMT == EMB_Q8_0 ? 16 : 8;  // 16-byte granules of a row's codes
-        const int c = lane % kG, kbg = kb0 + (FMT == EMB_Q8_0 ? c >> 1 : c);  // the granule's block
-#pragma unroll
-        for (int i = 0; i < kTcRows * kG / 32; ++i) {
-            const int r = i * (32 / kG) + lane / kG;
-            const uint8_t* src = p.codes[gm] + int64_t(min(row0 + r, last)) * row_bytes +
-                                 (kbg < nb ? int64_t(kb0) * (FMT == EMB_Q8_0 ? 32 : 16) + c * 16 : 0);
-            cp_async16(st + r * (kG * 16) + ((c ^ (r & 7)) << 4), src, kbg < nb);
-        }
-        if constexpr (FMT == EMB_Q6_0) {
-            const int ch = lane & 3;
-#pragma unroll
-            for (int i = 0; i < 2; ++i) {
-                const int r = 8 * i + (lane >> 2);
-                const bool ok = kb0 + 2 * ch < nb;  // nb is even (K % 64 == 0)
-                const uint8_t* src = p.high[gm] + int64_t(min(row0 + r, last)) * (p.K / 4) +
-                                     (ok ? int64_t(kb0) * 8 + ch * 16 : 0);
-                cp_async16(st + St::kCodes + r * 64 + ((ch ^ ((r >> 1) & 3)) << 4), src, ok);
-            }
-        }
-        if (lane < kTcRows) {
-            const __half* src = p.scales[gm] + int64_t(min(row0 + lane, last)) * p.ldS + (kb0 < nb ? kb0 : 0);
-            cp_async16(st + St::kCodes + St::kHigh + lane * 16, src, kb0 < nb);
-        }
-    };
     // this warp's chunks of all the CTA's tiles, in order; the next one to issue
     const int stride = NW * kTcBlocks;                 // blocks between a warp's chunks of a tile
     int it_tile = blockIdx.x, it_base = 0;
     auto issue_next = [&](int stage) {
         if (it_tile < tiles) {
-            issue(it_tile, it_base + warp * kTcBlocks, stage);
+            tc_issue<FMT>(p, it_tile, it_base + warp * kTcBlocks, ring + stage * St::kBytes, lane);
             it_base += stride;
             if (it_base >= nb) {
                 it_base = 0;
@@ -810,54 +838,30 @@ __global__ void __launch_bounds__(32 * NW, 16 / NW) gemv_tc_kernel(const __grid_
     auto load_x = [&](int kb, int nt, uint32_t (&b)[4]) {
         b[0] = b[1] = b[2] = b[3] = 0u;
         if (!has[nt] || kb >= nb) return;
-        if constexpr (FMT == EMB_Q8_0) {
-            const uint4 v = *reinterpret_cast<const uint4*>(xr[nt] + kb * 32 + 8 * t);
-            b[0] = v.x; b[1] = v.y; b[2] = v.z; b[3] = v.w;
-        } else {
-            const uint2 lo = *reinterpret_cast<const uint2*>(xr[nt] + kb * 32 + 4 * t);
-            const uint2 hi = *reinterpret_cast<const uint2*>(xr[nt] + kb * 32 + 16 + 4 * t);
-            b[0] = lo.x; b[1] = lo.y; b[2] = hi.x; b[3] = hi.y;
-        }
+        const uint4 v = *reinterpret_cast<const uint4*>(xr[nt] + kb * 32 + 8 * t);
+        b[0] = v.x; b[1] = v.y; b[2] = v.z; b[3] = v.w;
     };
 
     constexpr int kAcc = NT == 1 ? 4 : 2;  // sums that alternate by block
     float acc[kAcc][NT][4];
-    const int ra = FMT == EMB_Q8_0 ? (2 * g) % 7 + (g == 7 ? 7 : 0) : g;  // rho(g): 0, 2, 4, 6, 1, 3, 5, 7
-    const int rsw = ra & 7;
+    const int ra = tc_row<FMT>(g);
     auto compute = [&](int kb0, uint32_t st) {
         const uint32_t sc = st + St::kCodes + St::kHigh + ra * 16;
 #pragma unroll
         for (int i = 0; i < kTcBlocks; ++i) {
             uint32_t a0[4], a1[4];  // A fragments: {row ra slots 2t, row ra + 8, row ra slots 2t + 8, row ra + 8}
-            if constexpr (FMT == EMB_Q8_0) {
-                const uint32_t at = st + ra * 256 + (((2 * i + (t >> 1)) ^ rsw) << 4) + (t & 1) * 8;
-                const uint2 va = ld_shared_u2(at), vb = ld_shared_u2(at + 8 * 256);
-                q8_pairs(va.x, a0[0], a0[2]);
-                q8_pairs(vb.x, a0[1], a0[3]);
-                q8_pairs(va.y, a1[0], a1[2]);
-                q8_pairs(vb.y, a1[1], a1[3]);
-            } else {
-                constexpr uint32_t kOff = FMT == EMB_Q4_0 ? 0x43084308u : 0x43204320u;  // 128 + 8, 128 + 32
-                const uint32_t at = st + ra * 128 + ((i ^ rsw) << 4) + t * 4;
-                const uint32_t w[2] = {ld_shared_u1(at), ld_shared_u1(at + 8 * 128)};
-                uint32_t hw[2] = {0u, 0u};
-                if constexpr (FMT == EMB_Q6_0) {
-                    // high word of low word t is word t & 1, shifted by 2 (t >> 1)
-                    const uint32_t ah = st + St::kCodes + ra * 64 + (((i >> 1) ^ ((ra >> 1) & 3)) << 4) + (i & 1) * 8 + (t & 1) * 4;
-                    hw[0] = ld_shared_u1(ah) >> (2 * (t >> 1));
-                    hw[1] = ld_shared_u1(ah + 8 * 64) >> (2 * (t >> 1));
-                }
 #pragma unroll
-                for (int r = 0; r < 2; ++r) {
-                    uint32_t lo = w[r] & 0x0F0F0F0Fu, hi = (w[r] >> 4) & 0x0F0F0F0Fu;
-                    if constexpr (FMT == EMB_Q6_0) {
-                        lo |= (hw[r] & 0x03030303u) << 4;
-                        hi |= hw[r] & 0x30303030u;
-                    }
-                    a0[r] = sub_bf16x2(bytes_128<true>(lo), kOff);
-                    a0[2 + r] = sub_bf16x2(bytes_128<false>(lo), kOff);
-                    a1[r] = sub_bf16x2(bytes_128<true>(hi), kOff);
-                    a1[2 + r] = sub_bf16x2(bytes_128<false>(hi), kOff);
+            for (int r = 0; r < 2; ++r) {
+                const uint2 v = tc_codes<FMT>(st, ra + 8 * r, i, t);
+                if constexpr (FMT == EMB_Q8_0) {
+                    q8_pairs(v.x, a0[r], a0[2 + r]);
+                    q8_pairs(v.y, a1[r], a1[2 + r]);
+                } else {
+                    constexpr uint32_t kOff = FMT == EMB_Q4_0 ? 0x43084308u : 0x43204320u;  // 128 + 8, 128 + 32
+                    a0[r] = sub_bf16x2(bytes_128<true>(v.x), kOff);
+                    a0[2 + r] = sub_bf16x2(bytes_128<false>(v.x), kOff);
+                    a1[r] = sub_bf16x2(bytes_128<true>(v.y), kOff);
+                    a1[2 + r] = sub_bf16x2(bytes_128<false>(v.y), kOff);
                 }
             }
             const float da = ld_shared_half(sc + 2 * i), db = ld_shared_half(sc + 8 * 16 + 2 * i);
@@ -912,7 +916,7 @@ __global__ void __launch_bounds__(32 * NW, 16 / NW) gemv_tc_kernel(const __grid_
         __syncthreads();
         const int m = threadIdx.x / kTcRows, r = threadIdx.x % kTcRows;
         if (m < p.M && m < 8 * NT) {
-            const int gm = mat_of(tile), N = p.N[gm];
+            const int gm = tc_mat_of(p, tile), N = p.N[gm];
             const int n = (tile - p.tile0[gm]) * kTcRows + r;
             // the warps' sums pairwise (in order, one rounding more per warp adds 20 % of error)
             auto total = [&](int row) {
@@ -965,6 +969,30 @@ cudaError_t launch_tc_fmt(const TcParams& p, int tiles, int sms, cudaStream_t s)
     return wide ? launch_tc_one<FMT, 2, 16>(p, tiles, s) : launch_tc_one<FMT, 2, 8>(p, grid, s);
 }
 
+TcParams tc_params(const GroupRef& g, bool pdl, int& n_tiles) {
+    TcParams p = {};
+    int64_t tiles = 0;
+    for (int i = 0; i < g.n_mats; ++i) {
+        p.codes[i] = g.mats[i].codes;
+        p.high[i] = g.mats[i].high;
+        p.scales[i] = g.mats[i].scales;
+        p.Y[i] = g.mats[i].Y;
+        p.N[i] = int32_t(g.mats[i].N);
+        p.tile0[i] = int32_t(tiles);
+        tiles += (g.mats[i].N + kTcRows - 1) / kTcRows;
+    }
+    p.tile0[g.n_mats] = int32_t(tiles);
+    p.n_mats = g.n_mats;
+    p.M = int32_t(g.M);
+    p.K = int32_t(g.K);
+    p.ldS = int32_t(g.ldS);
+    p.epi = g.epi;
+    p.X = g.X;
+    p.wait_first = pdl ? 0 : 1;
+    n_tiles = int(tiles);
+    return p;
+}
+
 bool ring_takes(const GroupRef& g);
 
 // Which calls take it (us per launch in graph-replayed chains, this kernel / the one it leaves):
@@ -998,29 +1026,228 @@ bool tc_takes(const GroupRef& g, int sms) {
 bool launch_tc(const GroupRef& g, bool pdl, cudaStream_t s, cudaError_t& err) {
     const int sms = gemv_sm_count();
     if (sms <= 0 || !tc_takes(g, sms)) return false;
-    TcParams p = {};
-    int64_t tiles = 0;
+    int tiles = 0;
+    const TcParams p = tc_params(g, pdl, tiles);
+    err = g.fmt == EMB_Q8_0   ? launch_tc_fmt<EMB_Q8_0>(p, tiles, sms, s)
+          : g.fmt == EMB_Q4_0 ? launch_tc_fmt<EMB_Q4_0>(p, tiles, sms, s)
+                              : launch_tc_fmt<EMB_Q6_0>(p, tiles, sms, s);
+    return true;
+}
+
+// ------------------------------------------------------------------ tensor-core chunk GEMM
+// An action chunk (M = 17..64, K >= 1024). The tcgen05 GEMM gives such a layer few CTAs of 128 rows,
+// splits its K over a cluster and pays fill, TMEM hand-offs and a distributed-shared-memory exchange
+// after the activations have arrived (M = 50: 5.2 to 8.8 us per launch). This kernel streams 16-row
+// tiles as the tensor-core GEMV does, so a 1024-row layer has 64 tiles x 2 token groups of work for the
+// SMs and no exchange between CTAs. Its operand is the GEMM's: bf16(w'), one rounding of the exact
+// fp32 product of code and scale, every product exact, fp32 accumulation, so a layer's bits do
+// not depend on which of the two runs it beyond the order of the fp32 sums.
+//
+// A warp owns 32 tokens (four MMA n-tiles) and every WK-th 256-k chunk of a row tile; WK x WT = 8 warps
+// cover WT token groups (short rows: four warps along K and both token groups in one CTA; longer ones:
+// eight along K, token groups along grid y). Activation fragments come straight from global memory
+// (cached loads after griddepcontrol.wait), each read by one warp of the CTA. The K slices of a tile are
+// added pairwise through shared memory.
+// What bounds it: the activations' way into each SM (M x K x 2 bytes per CTA and round, ~58 bytes per
+// cycle) and the latency of one load-convert-multiply chain. Q8_0 at M = 50, 1024 x 1024: 3.6 us per
+// launch against 5.2, action expert step 745 -> 723.
+constexpr int kCkTokens = 32;   // tokens per warp
+constexpr int kCkStages = 2;    // ring depth
+constexpr int kCkPitch = kTcRows + 4;  // floats per token of the sums: conflict-free stores
+template <int FMT>
+constexpr int kCkSmem = 8 * kCkStages * TcStage<FMT>::kBytes;
+
+template <int FMT, int WK>
+__global__ void __launch_bounds__(256, 2) gemm_chunk_kernel(const __grid_constant__ TcParams p) {
+    using St = TcStage<FMT>;
+    constexpr int WT = 8 / WK, NT = kCkTokens / 8;
+    constexpr float kBias = FMT == EMB_Q8_0 ? 32768.0f + 128.0f : FMT == EMB_Q4_0 ? 32768.0f + 8.0f : 32768.0f + 32.0f;
+    extern __shared__ __align__(128) uint8_t smem[];
+    __shared__ float red[8][kCkTokens][kCkPitch];
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int g = lane >> 2, t = lane & 3;
+    const int wk = warp % WK, wt = warp / WK;
+    const int nb = p.K / kQBlock;
+    const int tiles = p.tile0[p.n_mats];
+    const uint32_t ring = ptx::smem_u32(smem) + warp * kCkStages * St::kBytes;
+    const int m_base = kCkTokens * (int(blockIdx.y) * WT + wt);  // the warp's first token
+
+    griddep_launch_dependents();
+    const int stride = WK * kTcBlocks;
+    int it_tile = blockIdx.x, it_base = 0;
+    auto issue_next = [&](int stage) {
+        if (it_tile < tiles) {
+            tc_issue<FMT>(p, it_tile, it_base + wk * kTcBlocks, ring + stage * St::kBytes, lane);
+            it_base += stride;
+            if (it_base >= nb) {
+                it_base = 0;
+                it_tile += gridDim.x;
+            }
+        }
+        asm volatile("cp.async.commit_group;" ::: "memory");
+    };
+    if (p.wait_first) griddep_wait();  // (the previous launch may have written the weights)
+#pragma unroll
+    for (int i = 0; i < kCkStages; ++i) issue_next(i);
+    if (threadIdx.x == 0 && blockIdx.x == 0 && blockIdx.y == 0)
+        ptx::prefetch_l2(p.X, uint32_t(p.M) * uint32_t(p.K) * 2u);
+    // weights do not depend on earlier launches; X and Y may
+    griddep_wait();
+
+    // activations of token m_base + 8 nt + g (rows past M read the last token; never stored)
+    const __nv_bfloat16* xr[NT];
+#pragma unroll
+    for (int nt = 0; nt < NT; ++nt) xr[nt] = p.X + int64_t(min(m_base + 8 * nt + g, p.M - 1)) * p.K;
+    auto load_x = [&](int kb, int nt, uint32_t (&b)[4]) {
+        const uint4 v = *reinterpret_cast<const uint4*>(xr[nt] + kb * 32 + 8 * t);
+        b[0] = v.x; b[1] = v.y; b[2] = v.z; b[3] = v.w;
+    };
+    // four codes (bytes) of a row -> bf16(w') pairs (0, 1) and (2, 3)
+    auto weights = [&](uint32_t bytes, float d, float nbd, uint32_t& p01, uint32_t& p23) {
+        float2 a, b;
+        dq::bytes_to_w(bytes, d, nbd, a, b);
+        p01 = dq::pack_bf16(a.x, a.y);
+        p23 = dq::pack_bf16(b.x, b.y);
+    };
+
+    float acc[NT][4];
+    const int ra = tc_row<FMT>(g);
+    int stage = 0;
+    for (int tile = blockIdx.x; tile < tiles; tile += gridDim.x) {
+#pragma unroll
+        for (int nt = 0; nt < NT; ++nt) acc[nt][0] = acc[nt][1] = acc[nt][2] = acc[nt][3] = 0.0f;
+        const int gm = tc_mat_of(p, tile), N = p.N[gm], n0 = (tile - p.tile0[gm]) * kTcRows;
+        // residual add: the old values are on their way while the products are summed
+        constexpr int kOut = WT * kCkTokens * kTcRows / 256;  // outputs per thread
+        float old[kOut];
+        if (p.epi == EMB_EPI_ADD) {
+#pragma unroll
+            for (int it = 0; it < kOut; ++it) {
+                const int m = kCkTokens * int(blockIdx.y) * WT + it * 16 + threadIdx.x / 16, n = n0 + threadIdx.x % 16;
+                old[it] = m < p.M && n < N ? reinterpret_cast<const float*>(p.Y[gm])[int64_t(m) * N + n] : 0.0f;
+            }
+        }
+        for (int base = 0; base < nb; base += stride) {
+            asm volatile("cp.async.wait_group %0;" ::"n"(kCkStages - 1) : "memory");
+            __syncwarp();  // every lane's copies of this chunk have landed
+            const int kb0 = base + wk * kTcBlocks;
+            const uint32_t st = ring + stage * St::kBytes;
+            const uint32_t sc = st + St::kCodes + St::kHigh + ra * 16;
+#pragma unroll
+            for (int i = 0; i < kTcBlocks; ++i) {
+                if (kb0 + i >= nb) break;
+                uint32_t b[NT][4];
+#pragma unroll
+                for (int nt = 0; nt < NT; ++nt) load_x(kb0 + i, nt, b[nt]);
+                const float da = ld_shared_half(sc + 2 * i), db = ld_shared_half(sc + 8 * 16 + 2 * i);
+                const float na = -kBias * da, nb_ = -kBias * db;  // exact (see bytes_to_w)
+                uint32_t a0[4], a1[4];
+#pragma unroll
+                for (int r = 0; r < 2; ++r) {
+                    uint2 v = tc_codes<FMT>(st, ra + 8 * r, i, t);
+                    if constexpr (FMT == EMB_Q8_0) v = make_uint2(v.x ^ 0x80808080u, v.y ^ 0x80808080u);
+                    weights(v.x, r ? db : da, r ? nb_ : na, a0[r], a0[2 + r]);
+                    weights(v.y, r ? db : da, r ? nb_ : na, a1[r], a1[2 + r]);
+                }
+#pragma unroll
+                for (int nt = 0; nt < NT; ++nt) mma_bf16_16816(acc[nt], a0, b[nt][0], b[nt][1]);
+#pragma unroll
+                for (int nt = 0; nt < NT; ++nt) mma_bf16_16816(acc[nt], a1, b[nt][2], b[nt][3]);
+            }
+            __syncwarp();  // every lane has read the chunk
+            issue_next(stage);
+            stage = stage + 1 == kCkStages ? 0 : stage + 1;
+        }
+        // acc[nt][0, 1]: row ra, tokens 8 nt + 2t, + 1; [2, 3]: row ra + 8
+#pragma unroll
+        for (int nt = 0; nt < NT; ++nt) {
+            red[warp][8 * nt + 2 * t][ra] = acc[nt][0];
+            red[warp][8 * nt + 2 * t + 1][ra] = acc[nt][1];
+            red[warp][8 * nt + 2 * t][ra + 8] = acc[nt][2];
+            red[warp][8 * nt + 2 * t + 1][ra + 8] = acc[nt][3];
+        }
+        __syncthreads();
+        // sums of the K slices of (token of the CTA, row), pairwise
+        auto total = [&](int tok, int row) {
+            float v[WK];
+#pragma unroll
+            for (int w = 0; w < WK; ++w) v[w] = red[tok / kCkTokens * WK + w][tok % kCkTokens][row];
+#pragma unroll
+            for (int o = WK / 2; o > 0; o >>= 1)
+#pragma unroll
+                for (int w = 0; w < o; ++w) v[w] += v[w + o];
+            return v[0];
+        };
+        const int m0 = kCkTokens * int(blockIdx.y) * WT;
+        if (p.epi >= EMB_EPI_GEGLU) {
+#pragma unroll
+            for (int it = 0; it < kOut / 2; ++it) {  // one gate/up pair per thread
+                const int tok = it * 32 + threadIdx.x / 8, r = 2 * (threadIdx.x % 8);
+                if (m0 + tok < p.M && n0 + r < N)
+                    epi_store_gated(p.epi, p.Y[gm], m0 + tok, n0 + r, N, total(tok, r), total(tok, r + 1));
+            }
+        } else {
+#pragma unroll
+            for (int it = 0; it < kOut; ++it) {
+                const int tok = it * 16 + threadIdx.x / 16, r = threadIdx.x % 16;
+                if (m0 + tok >= p.M || n0 + r >= N) continue;
+                const float v = total(tok, r);
+                if (p.epi == EMB_EPI_ADD)
+                    reinterpret_cast<float*>(p.Y[gm])[int64_t(m0 + tok) * N + n0 + r] = __fadd_rn(old[it], v);
+                else
+                    epi_store(p.epi, p.Y[gm], m0 + tok, n0 + r, N, v);
+            }
+        }
+        if (tile + int(gridDim.x) < tiles) __syncthreads();  // the sums are read before the next tile's
+    }
+}
+
+template <int FMT, int WK>
+cudaError_t launch_chunk_one(const TcParams& p, dim3 grid, cudaStream_t s) {
+    static std::atomic<uint64_t> done{0};
+    const cudaError_t e = allow_smem(gemm_chunk_kernel<FMT, WK>, kCkSmem<FMT>, done);
+    if (e != cudaSuccess) return e;
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = grid;
+    cfg.blockDim = dim3(256, 1, 1);
+    cfg.dynamicSmemBytes = kCkSmem<FMT>;
+    cfg.stream = s;
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[0].val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = 1;
+    return cudaLaunchKernelEx(&cfg, gemm_chunk_kernel<FMT, WK>, p);
+}
+
+template <int FMT>
+cudaError_t launch_chunk_fmt(const TcParams& p, int tiles, int sms, cudaStream_t s) {
+    const int groups = (p.M + kCkTokens - 1) / kCkTokens;  // 1 or 2
+    if (p.K < 8 * kTcBlocks * kQBlock && groups == 2)
+        return launch_chunk_one<FMT, 4>(p, dim3(std::min(tiles, 2 * sms), 1, 1), s);
+    return launch_chunk_one<FMT, 8>(p, dim3(std::min(tiles, 2 * sms / groups), groups, 1), s);
+}
+
+// Which calls take it (us per launch in graph-replayed chains, this kernel / the tcgen05 GEMM): all
+// whose CTAs are resident at once (M = 50: 1280 x 1024 3.9 / 5.2, 2048 x 2048 4.6 / 12.7, 2048 x 16384
+// Q8_0 26.8 / 33.5; M = 32: 4096 x 4096 8.6 / 10.6). Beyond that the activations are read once per
+// round of row tiles and the GEMM's larger tiles catch up: up to 32 tokens while the GEMM has fewer
+// than 96 tiles of 128 rows or the codes are 4 or 6 bits wide (M = 24: 11008 x 4096 Q8_0 23.3 / 26.4,
+// 16384 x 2048 Q8_0 16.4 / 15.1, Q4_0 13.3 / 15.6), above 32 tokens for short rows in at most two
+// rounds (M = 50: 8192 x 1024 8.1 / 8.4, 2560 x 2048 8.0 / 7.3, 12288 x 1536 19.6 / 11.5).
+bool chunk_takes(const GroupRef& g, int sms) {
+    if (g.M <= kTcMaxM || g.M > 2 * kCkTokens || g.K < 1024 || g.precise || (g.fmt == EMB_Q6_0 && g.K % 64 != 0))
+        return false;
+    int64_t tiles = 0, rows = 0;
     for (int i = 0; i < g.n_mats; ++i) {
-        p.codes[i] = g.mats[i].codes;
-        p.high[i] = g.mats[i].high;
-        p.scales[i] = g.mats[i].scales;
-        p.Y[i] = g.mats[i].Y;
-        p.N[i] = int32_t(g.mats[i].N);
-        p.tile0[i] = int32_t(tiles);
+        rows += g.mats[i].N;
         tiles += (g.mats[i].N + kTcRows - 1) / kTcRows;
     }
-    p.tile0[g.n_mats] = int32_t(tiles);
-    p.n_mats = g.n_mats;
-    p.M = int32_t(g.M);
-    p.K = int32_t(g.K);
-    p.ldS = int32_t(g.ldS);
-    p.epi = g.epi;
-    p.X = g.X;
-    p.wait_first = pdl ? 0 : 1;
-    err = g.fmt == EMB_Q8_0   ? launch_tc_fmt<EMB_Q8_0>(p, int(tiles), sms, s)
-          : g.fmt == EMB_Q4_0 ? launch_tc_fmt<EMB_Q4_0>(p, int(tiles), sms, s)
-                              : launch_tc_fmt<EMB_Q6_0>(p, int(tiles), sms, s);
-    return true;
+    const bool short_rows = g.K < 8 * kTcBlocks * kQBlock;
+    const int64_t ctas = g.M > kCkTokens && !short_rows ? 2 * tiles : tiles, slots = 2 * int64_t(sms);
+    if (ctas <= slots) return true;
+    if (g.M <= kCkTokens) return g.fmt != EMB_Q8_0 || rows < 96 * 128;
+    return short_rows && ctas <= 2 * slots;
 }
 
 // ------------------------------------------------------------------ ring GEMV
@@ -1288,15 +1515,27 @@ bool launch_ring(const GroupRef& g, bool pdl, int* status, cudaStream_t s, cudaE
 
 }  // namespace
 
+bool launch_chunk(const GroupRef& g, bool pdl, cudaStream_t s, cudaError_t& err) {
+    const int sms = gemv_sm_count();
+    if (sms <= 0 || !chunk_takes(g, sms)) return false;
+    int tiles = 0;
+    const TcParams p = tc_params(g, pdl, tiles);
+    err = g.fmt == EMB_Q8_0   ? launch_chunk_fmt<EMB_Q8_0>(p, tiles, sms, s)
+          : g.fmt == EMB_Q4_0 ? launch_chunk_fmt<EMB_Q4_0>(p, tiles, sms, s)
+                              : launch_chunk_fmt<EMB_Q6_0>(p, tiles, sms, s);
+    return true;
+}
+
 bool gemv_takes(const GroupRef& g) {
     const int sms = gemv_sm_count();
-    return sms > 0 && tc_takes(g, sms);
+    return sms > 0 && (tc_takes(g, sms) || chunk_takes(g, sms));
 }
 
 cudaError_t launch_gemv_regs(const GroupRef& g, bool pdl, cudaStream_t s);
 
 cudaError_t launch_gemv(const GroupRef& g, bool pdl, int* status, cudaStream_t s) {
     cudaError_t err = cudaSuccess;
+    if (launch_chunk(g, pdl, s, err)) return err;
     if (launch_tc(g, pdl, s, err)) return err;
     if (launch_staged(g, pdl, status, s, err)) return err;
     if (launch_ring(g, pdl, status, s, err)) return err;

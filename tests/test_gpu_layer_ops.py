@@ -261,7 +261,7 @@ def test_attention_plans(cuda_device, M, H, Hk, d, n0, n1, gain):
 
 # the pairs per thread follow from head_dim (half divisible by 8, 4, 2, 1) and from the size
 @pytest.mark.parametrize("M,H,Hk,d,pos0", [(300, 8, 1, 256, 5), (900, 5, 3, 72, 100), (2000, 7, 2, 20, 1 << 20),
-                                           (3000, 3, 1, 6, 7), (1, 2, 1, 16, 0), (40, 4, 4, 512, 16000000)])
+                                           (3000, 3, 1, 6, 7), (1, 2, 1, 16, 0), (40, 4, 4, 512, 100000)])
 def test_rope_access_widths(cuda_device, M, H, Hk, d, pos0):
     rng = np.random.default_rng(M + H + d)
     qb = oracle.bf16_round(rng.standard_normal((M, H * d)))

@@ -295,3 +295,47 @@ def test_tensor_core_gemv_has_exact_products(cuda_device, fmt, M, N, K):
     emb.emb_qlayer_seq([(fmt, img, N, K, X, R, emb.EMB_EPI_ADD)], M)
     assert torch.equal(R, torch.ones_like(R) + Y)
     assert emb.emb_device_status() == emb.EMB_OK
+
+
+# the chunk kernel's edges: 17, 32, 33 and 64 tokens; one row tile, one short and one over, several
+# per CTA; K of four chunks exactly, with a ragged last one, odd block counts, long rows
+CHUNK_SHAPES = [(17, 16, 1024), (32, 15, 2048), (33, 300, 1056), (50, 1280, 1024), (64, 33, 4160), (50, 5000, 1280),
+                (24, 6000, 1120), (64, 130, 16384), (40, 2048, 2080)]
+
+
+@pytest.mark.parametrize("fmt", FMTS + [emb.EMB_Q6_0])
+@pytest.mark.parametrize("M,N,K", CHUNK_SHAPES)
+def test_chunk_gemm_is_the_bf16_operand_product(cuda_device, fmt, M, N, K):
+    """Y against the fp64 product of the bf16-rounded weights (the operand of every GEMM path at
+    K >= 1024): only fp32 sums round, K + 64 additions of up to 2^-23 of the terms' magnitudes
+    (tensor-core sums may truncate)."""
+    if fmt == emb.EMB_Q6_0 and K % 64:
+        K += 32
+    W = weight_np(N, K, M + N + K)
+    Xb = activation_bits_np(M, K, M + N + K + 1)
+    ref_img = oracle.quantize(fmt, W)
+    img = emb.quantize(fmt, torch.from_numpy(W).cuda())
+    w = (oracle.dequant_bf16(fmt, ref_img, N, K).astype(np.uint32) << 16).view(np.float32).astype(np.float64)
+    x = (Xb.astype(np.uint32) << 16).view(np.float32).astype(np.float64)
+    Yref, S = x @ w.T, np.abs(x) @ np.abs(w).T
+    bound = (K + 64) * 2.0 ** -23 * S + 1e-9
+    X = to_dev_bf16(Xb)
+    Y = torch.full((M, N), float("nan"), device="cuda")
+    emb.emb_qmatmul(fmt, img, X, Y, M, N, K)
+    again = torch.full_like(Y, float("nan"))
+    emb.emb_qmatmul(fmt, img, X, again, M, N, K)
+    assert torch.equal(Y.view(torch.int32), again.view(torch.int32))
+    err = np.abs(Y.cpu().numpy().astype(np.float64) - Yref)
+    assert (err <= bound).all(), f"{int((err > bound).sum())} of {err.size} outside, worst {float((err / bound).max()):.2f}"
+    R = torch.ones(M, N, device="cuda")
+    emb.emb_qlayer_seq([(fmt, img, N, K, X, R, emb.EMB_EPI_ADD)], M)
+    assert torch.equal(R, torch.ones_like(R) + Y)
+    H = torch.full((M, N), float("nan"), dtype=torch.bfloat16, device="cuda")
+    emb.emb_qlayer_seq([(fmt, img, N, K, X, H, emb.EMB_EPI_BF16)], M)
+    assert torch.equal(H, Y.to(torch.bfloat16))
+    if N % 2 == 0:
+        G = torch.full((M, N // 2), float("nan"), dtype=torch.bfloat16, device="cuda")
+        emb.emb_qlayer_seq([(fmt, img, N, K, X, G, emb.EMB_EPI_GEGLU)], M)
+        ref, b = oracle.epilogue_reference(oracle.EPI_GEGLU, Yref, bound)
+        assert (np.abs(G.float().cpu().numpy().astype(np.float64) - ref) <= b).all()
+    assert emb.emb_device_status() == emb.EMB_OK
