@@ -44,54 +44,67 @@ cudaError_t launch_pdl(const void* fn, dim3 grid, dim3 block, size_t smem, cudaS
 // ------------------------------------------------------------------ RMSNorm
 // One CTA per token: the sum of squares in fp32 (per-thread partial sums of 4-element
 // groups, then a shuffle tree and the warps' sums in order), mean = sum / D, one correctly
-// rounded square root and reciprocal, then y = bf16(x * inv * gamma).
-constexpr int kNormThreads = 256;
+// rounded square root and reciprocal, then y = bf16(x * inv * gamma). Latency bounds it (0.3 MB at
+// 50 x 1024), so a thread loads its elements of x and gamma once, up to KEEP groups of each in
+// registers and gamma's loads on their way during the reduction, and one barrier is left: every
+// thread adds the warps' sums for itself. Few tokens take a thread per group, many take 256 threads,
+// so that all their CTAs are resident at once (512 threads: 816 x 2048 4.1 us).
+// Per launch, before (256 threads, x read twice, two barriers) and now, us: 50 x 1024 1.54 -> 1.23,
+// 1 x 4096 2.05 -> 1.75, 4 x 16384 4.71 -> 2.67, 816 x 2048 2.67 -> 2.48, 900 x 4096 3.59 -> 3.27.
 
 // x is read with ordinary loads (not the read-only path): the previous launch wrote it
 // while this grid was already resident (programmatic dependent launch); its writes are
 // visible to ordinary loads after griddepcontrol.wait.
-__global__ void __launch_bounds__(kNormThreads) rmsnorm_kernel(const float* x,
-                                                               const float* __restrict__ gamma,
-                                                               __nv_bfloat16* __restrict__ y,
-                                                               int D, float eps) {
+template <int NT, int KEEP>
+__global__ void __launch_bounds__(NT) rmsnorm_kernel(const float* x, const float* __restrict__ gamma,
+                                                     __nv_bfloat16* __restrict__ y, int D, float eps) {
     ptx::griddep_launch_dependents();
     ptx::griddep_wait();  // x is the residual stream the previous launch wrote
     const int64_t row = blockIdx.x;
     const float* xr = x + row * D;
+    __nv_bfloat16* yr = y + row * D;
+    const int i0 = threadIdx.x * 4;
+    float4 v[KEEP], gm[KEEP];
+#pragma unroll
+    for (int k = 0; k < KEEP; ++k)
+        v[k] = i0 + k * NT * 4 < D ? *reinterpret_cast<const float4*>(xr + i0 + k * NT * 4) : make_float4(0, 0, 0, 0);
+#pragma unroll
+    for (int k = 0; k < KEEP; ++k)
+        if (i0 + k * NT * 4 < D) gm[k] = *reinterpret_cast<const float4*>(gamma + i0 + k * NT * 4);
     float ss = 0.0f;
-    for (int i = threadIdx.x * 4; i < D; i += kNormThreads * 4) {
-        const float4 v = *reinterpret_cast<const float4*>(xr + i);
-        ss = fmaf(v.x, v.x, ss);
-        ss = fmaf(v.y, v.y, ss);
-        ss = fmaf(v.z, v.z, ss);
-        ss = fmaf(v.w, v.w, ss);
-    }
+    auto add = [&](const float4& q) {
+        ss = fmaf(q.x, q.x, ss);
+        ss = fmaf(q.y, q.y, ss);
+        ss = fmaf(q.z, q.z, ss);
+        ss = fmaf(q.w, q.w, ss);
+    };
+#pragma unroll
+    for (int k = 0; k < KEEP; ++k) add(v[k]);
+    for (int i = i0 + KEEP * NT * 4; i < D; i += NT * 4) add(*reinterpret_cast<const float4*>(xr + i));
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) ss += __shfl_xor_sync(0xffffffffu, ss, o);
-    __shared__ float warp_ss[kNormThreads / 32];
-    __shared__ float inv_s;
+    __shared__ float warp_ss[NT / 32];
     if ((threadIdx.x & 31) == 0) warp_ss[threadIdx.x >> 5] = ss;
     __syncthreads();
-    if (threadIdx.x == 0) {
-        float t = 0.0f;
-        for (int w = 0; w < kNormThreads / 32; ++w) t += warp_ss[w];
-        inv_s = __fdiv_rn(1.0f, __fsqrt_rn(__fadd_rn(__fdiv_rn(t, float(D)), eps)));
-    }
-    __syncthreads();
-    const float inv = inv_s;
-    __nv_bfloat16* yr = y + row * D;
-    for (int i = threadIdx.x * 4; i < D; i += kNormThreads * 4) {
-        const float4 v = *reinterpret_cast<const float4*>(xr + i);
-        const float4 g = *reinterpret_cast<const float4*>(gamma + i);
-        const __nv_bfloat162 lo = __floats2bfloat162_rn(__fmul_rn(__fmul_rn(v.x, inv), g.x),
-                                                        __fmul_rn(__fmul_rn(v.y, inv), g.y));
-        const __nv_bfloat162 hi = __floats2bfloat162_rn(__fmul_rn(__fmul_rn(v.z, inv), g.z),
-                                                        __fmul_rn(__fmul_rn(v.w, inv), g.w));
+    float t = 0.0f;
+#pragma unroll
+    for (int w = 0; w < NT / 32; ++w) t += warp_ss[w];
+    const float inv = __fdiv_rn(1.0f, __fsqrt_rn(__fadd_rn(__fdiv_rn(t, float(D)), eps)));
+    auto store = [&](int i, const float4& q, const float4& g) {
+        const __nv_bfloat162 lo = __floats2bfloat162_rn(__fmul_rn(__fmul_rn(q.x, inv), g.x),
+                                                        __fmul_rn(__fmul_rn(q.y, inv), g.y));
+        const __nv_bfloat162 hi = __floats2bfloat162_rn(__fmul_rn(__fmul_rn(q.z, inv), g.z),
+                                                        __fmul_rn(__fmul_rn(q.w, inv), g.w));
         uint2 u;
         u.x = *reinterpret_cast<const uint32_t*>(&lo);
         u.y = *reinterpret_cast<const uint32_t*>(&hi);
         *reinterpret_cast<uint2*>(yr + i) = u;
-    }
+    };
+#pragma unroll
+    for (int k = 0; k < KEEP; ++k)
+        if (i0 + k * NT * 4 < D) store(i0 + k * NT * 4, v[k], gm[k]);
+    for (int i = i0 + KEEP * NT * 4; i < D; i += NT * 4)
+        store(i, *reinterpret_cast<const float4*>(xr + i), *reinterpret_cast<const float4*>(gamma + i));
 }
 
 // ------------------------------------------------------------------ rotary embedding
@@ -656,8 +669,17 @@ cudaError_t launch_rmsnorm(const float* x, const float* gamma, uint16_t* y, int6
     __nv_bfloat16* ya = reinterpret_cast<__nv_bfloat16*>(y);
     int Di = int(D);
     void* args[] = {&xa, &ga, &ya, &Di, &eps};
-    return launch_pdl(reinterpret_cast<const void*>(rmsnorm_kernel), dim3(unsigned(M)),
-                      dim3(kNormThreads), 0, s, args);
+    const int groups = Di / 4;
+    const bool many = M > 304;  // more than two CTAs per SM
+    const int nt = groups <= 128 ? 128 : groups <= 256 || many ? 256 : groups <= 512 ? 512 : 1024;
+    const void* fn = nt == 128   ? reinterpret_cast<const void*>(rmsnorm_kernel<128, 1>)
+                     : nt == 512 ? reinterpret_cast<const void*>(rmsnorm_kernel<512, 1>)
+                     : nt == 256 ? (groups <= 256   ? reinterpret_cast<const void*>(rmsnorm_kernel<256, 1>)
+                                    : groups <= 512 ? reinterpret_cast<const void*>(rmsnorm_kernel<256, 2>)
+                                                    : reinterpret_cast<const void*>(rmsnorm_kernel<256, 4>))
+                     : groups <= 1024 ? reinterpret_cast<const void*>(rmsnorm_kernel<1024, 1>)
+                                      : reinterpret_cast<const void*>(rmsnorm_kernel<1024, 4>);
+    return launch_pdl(fn, dim3(unsigned(M)), dim3(unsigned(nt)), 0, s, args);
 }
 
 cudaError_t launch_rope(uint16_t* x, int64_t n_heads, uint16_t* x2, int64_t n_heads2, int64_t M,

@@ -272,3 +272,18 @@ def test_rope_access_widths(cuda_device, M, H, Hk, d, pos0):
     for t, xb, heads in ((q, qb, H), (k, kb, Hk)):
         ref, bound = oracle.rope_reference(xb, heads, d, pos0, 10000.0)
         _check(_vals(t), ref, bound, f"rope d={d} heads={heads}")
+
+
+# the thread counts and register shares of the norm: few and many tokens, rows around one, two and
+# four groups per thread, rows longer than a CTA keeps in registers
+@pytest.mark.parametrize("M,D", [(3, 512), (304, 520), (305, 1024), (400, 1032), (305, 2048), (320, 4104), (1, 2056),
+                                 (2, 4096), (5, 4104), (310, 16384), (2, 16392)])
+def test_rmsnorm_thread_counts(cuda_device, M, D):
+    rng = np.random.default_rng(M + D)
+    x = (rng.standard_normal((M, D)) * 2).astype(np.float32)
+    g = (1.0 + 0.1 * rng.standard_normal(D)).astype(np.float32)
+    y = torch.full((M, D), float("nan"), dtype=torch.bfloat16, device="cuda")
+    emb.emb_rmsnorm(torch.from_numpy(x).cuda(), torch.from_numpy(g).cuda(), y, 1e-6)
+    torch.cuda.synchronize()
+    ref, bound = oracle.rmsnorm_reference(x, g, 1e-6)
+    _check(_vals(y), ref, bound, f"rmsnorm M={M} D={D}")
