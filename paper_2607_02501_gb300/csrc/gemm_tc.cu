@@ -897,10 +897,10 @@ int sm_count() {
 }
 
 // K splits (1, 2, 4 or 8: one cluster of CTAs per output tile, 8 being the portable
-// cluster size): the count minimising a simple time model -- waves of 148 CTAs, each
-// costing a fixed ~3 us plus its share of the tile's MMA work at ~11.6 TFLOP/s per SM --
-// subject to every split owning at least one 256-k raw stage and the partial tile fitting
-// in the CTA's A/X rings. Eight-way splits lift the M = 50 action expert 48 -> 53 TFLOP/s.
+// cluster size) of the two-operand form and of fewer than 65 tokens: the count minimising a simple
+// time model -- waves of 148 CTAs, each costing a fixed ~3 us plus its share of the tile's MMA work
+// at ~11.6 TFLOP/s per SM -- subject to every split owning at least one 256-k raw stage and the
+// partial tile fitting in the CTA's X ring.
 int pick_splits(int64_t tiles, int T, int64_t K, int stages, bool split_operand) {
     const int64_t nr = (K + kKR - 1) / kKR;
     const double work_us = 2.0 * kBN * T * double(K) / 11.6e12 * 1e6 * (split_operand ? 2 : 1);
@@ -947,6 +947,15 @@ size_t sk_ws_bytes(int G, int P, int T) { return kSkFlagBytes + size_t(G) * sk_s
 // than the loads). An item adds its drain, epilogue and restart.
 double step_cycles(int P, int T) { return std::max(620.0, 2.22 * P * T + 150.0); }
 double item_cycles(int P, int T) { return 6300.0 + 22.6 * P * T; }
+// One launch: waves of CTAs that each take an item's share of K. A K split adds its cluster's
+// exchange, ~2000 + 36 per token of the tile (235 launches of 11 layer shapes with the token tile
+// and the splits forced; the three models together reproduce them to ~12 %).
+double plan_cycles(int64_t items, int P, int T, int splits, int64_t K, int sms) {
+    const int64_t nr = (K + kKR - 1) / kKR, nk = (K + kKC - 1) / kKC;
+    const double steps = double(std::min(nk, (nr + splits - 1) / splits * kStepsPerRaw));
+    const double exchange = splits > 1 ? 2000.0 + 36.0 * T : 0.0;
+    return double((items * splits + sms - 1) / sms) * (steps * step_cycles(P, T) + item_cycles(P, T) + exchange);
+}
 
 // The launch shape of one group. With streamk_ok the plan may take the stream-K schedule,
 // which needs plan.ws_bytes of zero-filled workspace.
@@ -961,36 +970,37 @@ GemmPlan plan_gemm(const GroupRef& g, bool streamk_ok) {
     int S = g.fmt == EMB_Q8_0   ? (split ? pick_stages<EMB_Q8_0, true>(T) : pick_stages<EMB_Q8_0, false>(T))
             : g.fmt == EMB_Q4_0 ? (split ? pick_stages<EMB_Q4_0, true>(T) : pick_stages<EMB_Q4_0, false>(T))
                                 : (split ? pick_stages<EMB_Q6_0, true>(T) : pick_stages<EMB_Q6_0, false>(T));
-    int splits = pick_splits(int64_t(t_tiles) * tiles, T, g.K, S, split);
-    // Prefill shapes whose weight tiles x token tiles leave SMs idle (narrow layers: the
-    // vision tower's 1152-wide ones give 9-36 weight tiles) may take more, smaller token
-    // tiles: up to three more when the cycle model says at least 3 % faster. ViT M = 768: fc1
-    // takes four tiles of 192 instead of three of 256 (108 -> 144 CTAs), q/k/v five of 160
-    // (81 -> 135).
-    if (!split && g.M >= 256) {
-        const int sms = sm_count();
-        if (sms > 0) {
-            const double nk = double((g.K + kKC - 1) / kKC);
-            auto cost = [&](int64_t tt, int Tc, int sp) {
-                return double((tt * tiles * sp + sms - 1) / sms) *
-                       (std::ceil(nk / sp) * step_cycles(1, Tc) + item_cycles(1, Tc));
-            };
-            double best = cost(t_tiles, T, splits);
-            const int64_t t0 = t_tiles;
-            for (int64_t tt = t0 + 1; tt <= t0 + 3; ++tt) {
-                const int Tc = int(roundup((g.M + tt - 1) / tt, 16));
-                if (Tc < 64) break;
-                const int Sc = g.fmt == EMB_Q8_0 ? pick_stages<EMB_Q8_0, false>(Tc)
-                               : g.fmt == EMB_Q4_0 ? pick_stages<EMB_Q4_0, false>(Tc)
-                                                   : pick_stages<EMB_Q6_0, false>(Tc);
-                const int spc = pick_splits(tt * tiles, Tc, g.K, Sc, false);
-                const double c = cost(tt, Tc, spc);
-                if (c < 0.97 * best) {
-                    best = c;
+    const int sms = sm_count();
+    int splits = 1;
+    double one_tile = 0.0;  // cycles of the plan with one token tile per CTA
+    if (split || sms <= 0 || g.M <= 64) {
+        splits = pick_splits(t_tiles * tiles, T, g.K, S, split);
+        one_tile = plan_cycles(t_tiles * tiles, 1, T, splits, g.K, std::max(sms, 1));
+    } else {
+        // Token tiles and K splits together: a launch that leaves SMs idle may take smaller token
+        // tiles, or a K split with its exchange, whichever the model says is at least 3 % faster than
+        // what has fewer tiles. Tiles stay at 96 tokens and more: the model has their steps bound by
+        // the dequantisation, equally long, but 64 measured 9 % slower (they read the weights more
+        // often). Against splitting first (us): ViT M = 768 o, eight tiles of 96 for four of 192 in
+        // four splits, 8.3 / 10.8; 8192 x 1024 at M = 128, one tile for two splits, 8.1 / 10.3;
+        // unchanged: fc1 four tiles of 192, q/k/v five of 160, fc2 four of 192 in four splits.
+        const int64_t tt0 = t_tiles, nr = (g.K + kKR - 1) / kKR;
+        one_tile = 1e30;
+        for (int64_t tt = tt0; tt <= tt0 + 12; ++tt) {
+            const int Tc = int(roundup((g.M + tt - 1) / tt, 16));
+            if (tt > tt0 && Tc < 96) break;
+            const int Sc = g.fmt == EMB_Q8_0   ? pick_stages<EMB_Q8_0, false>(Tc)
+                           : g.fmt == EMB_Q4_0 ? pick_stages<EMB_Q4_0, false>(Tc)
+                                               : pick_stages<EMB_Q6_0, false>(Tc);
+            for (int sp = 1; sp <= 8 && sp <= nr; sp *= 2) {
+                if (sp > 1 && Sc < 4) break;  // the 512 T-byte partial tile lies in the X ring
+                const double c = plan_cycles(tt * tiles, 1, Tc, sp, g.K, sms);
+                if (c < 0.97 * one_tile) {
+                    one_tile = c;
                     t_tiles = tt;
                     T = Tc;
                     S = Sc;
-                    splits = spc;
+                    splits = sp;
                 }
             }
         }
@@ -1007,14 +1017,9 @@ GemmPlan plan_gemm(const GroupRef& g, bool streamk_ok) {
         const int S2 = (g.fmt == EMB_Q8_0)   ? pick_stages_pair<EMB_Q8_0>(T2)
                        : (g.fmt == EMB_Q4_0) ? pick_stages_pair<EMB_Q4_0>(T2)
                                              : pick_stages_pair<EMB_Q6_0>(T2);
-        const int sms = sm_count();
         if (S2 >= 2 && T2 <= 224 && sms > 0) {
-            const double nk = double((g.K + kKC - 1) / kKC);
-            auto waves = [&](int64_t ctas) { return double((ctas + sms - 1) / sms); };
-            const double c1 = waves(int64_t(t_tiles) * tiles * splits) *
-                              (std::ceil(nk / splits) * step_cycles(1, T) + item_cycles(1, T));
-            const double c2 = waves(int64_t(t2 / 2) * tiles) * (nk * step_cycles(2, T2) + item_cycles(2, T2));
-            if (c2 < 0.95 * c1) {
+            const double c2 = plan_cycles(t2 / 2 * tiles, 2, T2, 1, g.K, sms);
+            if (c2 < 0.95 * one_tile) {
                 P = 2;
                 T = T2;
                 S = S2;
@@ -1028,7 +1033,6 @@ GemmPlan plan_gemm(const GroupRef& g, bool streamk_ok) {
     // copies' latency paid once per CTA; the next item's copies overlap this one's epilogue).
     int grid_y = tiles, persist = 0;
     {
-        const int sms = sm_count();
         const int64_t items = int64_t(grid_x) * tiles;
         if (splits == 1 && sms > 0 && items > sms && items < (int64_t(1) << 30)) {
             persist = 1;
@@ -1047,7 +1051,7 @@ GemmPlan plan_gemm(const GroupRef& g, bool streamk_ok) {
     pl.persist = persist;
     // Stream-K: when the waves of whole items leave SMs idle (a last wave that is mostly
     // empty), cut the raw stages of all items into one equal range per SM. Both plans are
-    // costed with the cycle model (and ~5000 for a K split's cluster exchange); stream-K adds, per
+    // costed with the cycle model; stream-K adds, per
     // token of the CTA, 59 cycles for writing, publishing, staging and adding a partial tile and
     // 11.5 for every further tail a head adds (per-CTA %globaltimer stamps at 288 tokens: 147 KB
     // written in ~3 us, staged and added in ~1.7 us, a slower store pass after it). It is taken
@@ -1055,16 +1059,9 @@ GemmPlan plan_gemm(const GroupRef& g, bool streamk_ok) {
     // M = 280 49.8 / 63.8; 24000 x 4096 at M = 130 44.2 / 61.0; 5000 x 5056 at M = 300 30.0 / 35.2;
     // not taken: Llama-7B o 22.9 / 20.2, Gemma-2B gate/up at M = 816 (every CTA ends several
     // items) 108 / 104, ViT q/k/v 19.6 / 11.1.
-    const int sms = sm_count();
     if (streamk_ok && !split && g.M >= 128 && sms > 0) {
         const int64_t nr_all = (g.K + kKR - 1) / kKR;
-        const double nk = double((g.K + kKC - 1) / kKC);
-        double cur;
-        if (pl.persist)
-            cur = double((int64_t(pl.n_items) + sms - 1) / sms) * (nk * step_cycles(P, T) + item_cycles(P, T));
-        else
-            cur = double((int64_t(grid_x) * grid_y * splits + sms - 1) / sms) *
-                  (std::ceil(nk / splits) * step_cycles(P, T) + item_cycles(P, T) + (splits > 1 ? 5000.0 : 0.0));
+        const double cur = plan_cycles(pl.persist ? pl.n_items : int64_t(grid_x) * grid_y, P, T, splits, g.K, sms);
         struct Cand { int P, T, S; int64_t n_tt; };
         Cand cands[2];
         int nc = 0;

@@ -339,3 +339,16 @@ def test_chunk_gemm_is_the_bf16_operand_product(cuda_device, fmt, M, N, K):
         ref, b = oracle.epilogue_reference(oracle.EPI_GEGLU, Yref, bound)
         assert (np.abs(G.float().cpu().numpy().astype(np.float64) - ref) <= b).all()
     assert emb.emb_device_status() == emb.EMB_OK
+
+
+# short rows whose launch leaves SMs idle take more token tiles of 96 and more tokens instead of a K
+# split: tiles that end exactly at M and ragged ones (97, 193, 577, 1030, 1537), the last one row short
+# of or one over a tile, a K of 4.1 raw stages; long rows of few tiles keep the split (97 x 300)
+SHORT_ROW_SHAPES = [(768, 1152, 1152), (577, 1000, 1056), (97, 300, 2112), (193, 130, 1056), (1030, 1100, 1088),
+                    (1537, 900, 1312), (128, 8192, 1024), (65, 40, 1024)]
+
+
+@pytest.mark.parametrize("fmt", FMTS + [emb.EMB_Q6_0])
+@pytest.mark.parametrize("M,N,K", SHORT_ROW_SHAPES)
+def test_short_row_gemm_is_the_bf16_operand_product(cuda_device, fmt, M, N, K):
+    test_chunk_gemm_is_the_bf16_operand_product(cuda_device, fmt, M, N, K)
