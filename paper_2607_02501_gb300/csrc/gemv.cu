@@ -794,7 +794,9 @@ constexpr int kTcDepth = FMT == EMB_Q8_0 && NT == 2 && NW == 8 ? 2 : 3;
 template <int FMT, int NT, int NW>
 constexpr int kTcSmem = NW * kTcDepth<FMT, NT, NW> * TcStage<FMT>::kBytes;
 
-template <int FMT, int NT, int NW>
+// COMP: the sums of a chunk are added to a compensated total (TwoSum), so the fp32 error does not grow
+// with the number of chunks that a warp adds up (see launch_tc_fmt).
+template <int FMT, int NT, int NW, bool COMP>
 __global__ void __launch_bounds__(32 * NW, 16 / NW) gemv_tc_kernel(const __grid_constant__ TcParams p) {
     using St = TcStage<FMT>;
     constexpr int kTcStages = kTcDepth<FMT, NT, NW>;
@@ -843,7 +845,19 @@ __global__ void __launch_bounds__(32 * NW, 16 / NW) gemv_tc_kernel(const __grid_
     };
 
     constexpr int kAcc = NT == 1 ? 4 : 2;  // sums that alternate by block
-    float acc[kAcc][NT][4];
+    float acc[kAcc][NT][4] = {};
+    float tot[COMP ? NT : 1][4], rest[COMP ? NT : 1][4];
+    auto acc_sum = [&](int nt, int e) {
+        float v = acc[0][nt][e] + acc[1][nt][e];
+        if constexpr (kAcc == 4) v += acc[2][nt][e] + acc[3][nt][e];
+        return v;
+    };
+    auto acc_clear = [&] {
+#pragma unroll
+        for (int i = 0; i < kAcc; ++i)
+#pragma unroll
+            for (int nt = 0; nt < NT; ++nt) acc[i][nt][0] = acc[i][nt][1] = acc[i][nt][2] = acc[i][nt][3] = 0.0f;
+    };
     const int ra = tc_row<FMT>(g);
     auto compute = [&](int kb0, uint32_t st) {
         const uint32_t sc = st + St::kCodes + St::kHigh + ra * 16;
@@ -881,14 +895,28 @@ __global__ void __launch_bounds__(32 * NW, 16 / NW) gemv_tc_kernel(const __grid_
                 ac[3] = fmaf(db, d0[3] + d1[3], ac[3]);
             }
         }
+        if constexpr (COMP) {
+#pragma unroll
+            for (int nt = 0; nt < NT; ++nt)
+#pragma unroll
+                for (int e = 0; e < 4; ++e) {
+                    const float a = tot[nt][e], c = acc_sum(nt, e), sum = __fadd_rn(a, c), b = __fsub_rn(sum, a);
+                    rest[nt][e] += __fadd_rn(__fsub_rn(a, __fsub_rn(sum, b)), __fsub_rn(c, b));
+                    tot[nt][e] = sum;
+                }
+            acc_clear();
+        }
     };
     __shared__ float red[kBufs][NW][8 * NT][kTcRows];
     int buf = 0, stage = 0;
     for (int tile = blockIdx.x; tile < tiles; tile += gridDim.x, buf = (buf + 1) % kBufs) {
+        acc_clear();
+        if constexpr (COMP) {
 #pragma unroll
-        for (int i = 0; i < kAcc; ++i)
+            for (int nt = 0; nt < NT; ++nt)
 #pragma unroll
-            for (int nt = 0; nt < NT; ++nt) acc[i][nt][0] = acc[i][nt][1] = acc[i][nt][2] = acc[i][nt][3] = 0.0f;
+                for (int e = 0; e < 4; ++e) tot[nt][e] = rest[nt][e] = 0.0f;
+        }
         for (int base = 0; base < nb; base += stride) {
             asm volatile("cp.async.wait_group %0;" ::"n"(kTcStages - 1) : "memory");
             __syncwarp();  // every lane's copies of this chunk have landed
@@ -905,8 +933,11 @@ __global__ void __launch_bounds__(32 * NW, 16 / NW) gemv_tc_kernel(const __grid_
             float v[4];
 #pragma unroll
             for (int e = 0; e < 4; ++e) {
-                v[e] = acc[0][nt][e] + acc[1][nt][e];
-                if constexpr (kAcc == 4) v[e] += acc[2][nt][e] + acc[3][nt][e];
+                if constexpr (COMP)
+                    // an infinite or NaN total stays as it is: its rounding errors are NaN
+                    v[e] = fabsf(tot[nt][e]) <= 3.402823466e+38f ? tot[nt][e] + rest[nt][e] : tot[nt][e];
+                else
+                    v[e] = acc_sum(nt, e);
             }
             red[buf][warp][8 * nt + 2 * t][ra] = v[0];
             red[buf][warp][8 * nt + 2 * t + 1][ra] = v[1];
@@ -942,7 +973,7 @@ __global__ void __launch_bounds__(32 * NW, 16 / NW) gemv_tc_kernel(const __grid_
 
 int gemv_sm_count();
 
-template <int FMT, int NT, int NW>
+template <int FMT, int NT, int NW, bool COMP = false>
 cudaError_t launch_tc_one(const TcParams& p, int grid, cudaStream_t s) {
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3(grid, 1, 1);
@@ -950,14 +981,14 @@ cudaError_t launch_tc_one(const TcParams& p, int grid, cudaStream_t s) {
     cfg.dynamicSmemBytes = kTcSmem<FMT, NT, NW>;
     cfg.stream = s;
     static std::atomic<uint64_t> done{0};
-    const cudaError_t e = allow_smem(gemv_tc_kernel<FMT, NT, NW>, kTcSmem<FMT, NT, NW>, done);
+    const cudaError_t e = allow_smem(gemv_tc_kernel<FMT, NT, NW, COMP>, kTcSmem<FMT, NT, NW>, done);
     if (e != cudaSuccess) return e;
     cudaLaunchAttribute attr[1];
     attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
     attr[0].val.programmaticStreamSerializationAllowed = 1;
     cfg.attrs = attr;
     cfg.numAttrs = 1;
-    return cudaLaunchKernelEx(&cfg, gemv_tc_kernel<FMT, NT, NW>, p);
+    return cudaLaunchKernelEx(&cfg, gemv_tc_kernel<FMT, NT, NW, COMP>, p);
 }
 
 template <int FMT>
@@ -965,6 +996,14 @@ cudaError_t launch_tc_fmt(const TcParams& p, int tiles, int sms, cudaStream_t s)
     // long rows whose tiles leave each SM at most one CTA: sixteen warps
     const bool wide = tiles <= sms && p.K > 8 * kTcBlocks * kQBlock;
     const int grid = std::min(tiles, 2 * sms);
+    // Many chunks per warp and up to four tokens (more had the GEMM's rounded operand, 1.7e-3): compensated
+    // totals. In plain ones a warp's fp32 chain grows with K and its error passes that of the FFMA2 kernels, whose
+    // 32 to 128 threads have shorter chains (relative to the norm of the result, 6 seeds, plain /
+    // compensated / FFMA2, 1e-8): Q4_0 M = 1 4096 x 11008 8.8 / 7.9 / 8.2, M = 4 4096 x 14336 9.3 / 7.9 / 8.3. It
+    // costs 4 % there (4096 x 11008 9.9 -> 10.3 us). Up to three chunks at eight warps and four at
+    // sixteen plain totals are no worse (K = 4096: within 0.3 %; 2048 x 16384: smaller).
+    if (p.M <= 4 && p.K > (wide ? 4 * 16 : 3 * 8) * kTcBlocks * kQBlock)
+        return wide ? launch_tc_one<FMT, 1, 16, true>(p, tiles, s) : launch_tc_one<FMT, 1, 8, true>(p, grid, s);
     if (p.M <= 8) return wide ? launch_tc_one<FMT, 1, 16>(p, tiles, s) : launch_tc_one<FMT, 1, 8>(p, grid, s);
     return wide ? launch_tc_one<FMT, 2, 16>(p, tiles, s) : launch_tc_one<FMT, 2, 8>(p, grid, s);
 }

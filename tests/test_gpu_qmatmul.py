@@ -352,3 +352,38 @@ SHORT_ROW_SHAPES = [(768, 1152, 1152), (577, 1000, 1056), (97, 300, 2112), (193,
 @pytest.mark.parametrize("M,N,K", SHORT_ROW_SHAPES)
 def test_short_row_gemm_is_the_bf16_operand_product(cuda_device, fmt, M, N, K):
     test_chunk_gemm_is_the_bf16_operand_product(cuda_device, fmt, M, N, K)
+
+
+# the tensor-core GEMV's compensated totals: the last K without and the first with them at eight warps
+# (tiles of two CTAs per SM) and sixteen (one tile per SM), ragged last chunks, few rows
+LONG_ROW_SHAPES = [(4900, 6144), (4900, 6208), (4096, 11008), (300, 16384), (300, 16448), (33, 32768), (2600, 14336)]
+
+
+@pytest.mark.parametrize("fmt", FMTS + [emb.EMB_Q6_0])
+@pytest.mark.parametrize("M", [2, 4])
+@pytest.mark.parametrize("N,K", LONG_ROW_SHAPES)
+def test_long_row_gemv_error_does_not_grow_with_k(cuda_device, fmt, M, N, K):
+    """Exact products; the roundings on a term's way are those of its MMA (16 terms, truncated: 17),
+    the two MMAs' sum, up to eight scaled additions, two levels within the chunk, the total and the warps'
+    levels (three with a total, four without): 32 of 2^-23 of the magnitudes, whatever K. An infinite
+    activation gives the product's own infinities and NaNs in its token and none elsewhere."""
+    W = weight_np(N, K, M + N + K)
+    Xb = activation_bits_np(M, K, M + N + K + 1)
+    img_ref = oracle.quantize(fmt, W)
+    w = oracle.dequant_f32(fmt, img_ref, N, K).astype(np.float64)
+    x = (Xb.astype(np.uint32) << 16).view(np.float32).astype(np.float64)
+    img, X = emb.quantize(fmt, torch.from_numpy(W).cuda()), to_dev_bf16(Xb)
+    Y = torch.full((M, N), float("nan"), device="cuda")
+    emb.emb_qmatmul(fmt, img, X, Y, M, N, K)
+    again = torch.full_like(Y, float("nan"))
+    emb.emb_qmatmul(fmt, img, X, again, M, N, K)
+    assert torch.equal(Y.view(torch.int32), again.view(torch.int32))
+    err, bound = np.abs(Y.cpu().numpy() - x @ w.T), 32 * 2.0 ** -23 * (np.abs(x) @ np.abs(w).T) + 1e-12
+    assert (err <= bound).all(), f"worst {float((err / bound).max()):.2f} of the bound"
+    X[M - 1, 7] = float("inf")
+    emb.emb_qmatmul(fmt, img, X, again, M, N, K)
+    assert torch.equal(again[: M - 1].view(torch.int32), Y[: M - 1].view(torch.int32))
+    with np.errstate(invalid="ignore"):
+        want = np.where(w[:, 7] == 0, np.nan, np.sign(w[:, 7]) * np.inf)
+    assert np.array_equal(again[M - 1].cpu().numpy(), want.astype(np.float32), equal_nan=True)
+    assert emb.emb_device_status() == emb.EMB_OK
