@@ -103,7 +103,9 @@ __device__ __forceinline__ float dot_unit(const uint4 c, const uint2 h, const fl
 // before griddepcontrol.wait, so a layer with long rows has all of its weight bytes in
 // flight while the previous launch drains; the products are summed in the same order as
 // with PF = 1 (bitwise the same results).
-template <int FMT, int R, int NT, int MT, int PF>
+// FIRST: nothing is read before griddepcontrol.wait (the previous launch may have written the weights). A
+// parameter tested at run time costs every other launch 1 to 3 % (Q8_0 1536 x 4608 2.73 -> 2.78 us).
+template <int FMT, int R, int NT, int MT, int PF, bool FIRST>
 __global__ void __launch_bounds__(NT) gemv_kernel(const __grid_constant__ GemvParams p) {
     constexpr int UW = (FMT == EMB_Q8_0) ? 16 : 32;  // weights per 16-byte unit
     constexpr int NWARP = NT / 32;
@@ -123,7 +125,7 @@ __global__ void __launch_bounds__(NT) gemv_kernel(const __grid_constant__ GemvPa
     const int U = p.U;
 
     griddep_launch_dependents();
-    if (p.wait_first) griddep_wait();  // (the previous launch may have written the weights)
+    if constexpr (FIRST) griddep_wait();
     // the activation rows towards L2 while the previous launch finishes (measured on GB300:
     // cold, they arrive ~2 us after the dependency wait, behind the weight stream); one CTA
     // per row block asks, since every CTA reads the same rows
@@ -268,7 +270,8 @@ cudaError_t launch_one(const GemvParams& p, int grid_x, int grid_y, cudaStream_t
     attr[0].val.programmaticStreamSerializationAllowed = 1;
     cfg.attrs = attr;
     cfg.numAttrs = 1;
-    return cudaLaunchKernelEx(&cfg, gemv_kernel<FMT, R, NT, MT, PF>, p);
+    return p.wait_first ? cudaLaunchKernelEx(&cfg, gemv_kernel<FMT, R, NT, MT, PF, true>, p)
+                        : cudaLaunchKernelEx(&cfg, gemv_kernel<FMT, R, NT, MT, PF, false>, p);
 }
 
 template <int FMT, int R, int NT>
@@ -282,12 +285,9 @@ cudaError_t dispatch_mt(const GemvParams& p, int grid_x, int M, cudaStream_t s) 
         if (M == 1 && p.U > NT && p.U <= 4 * NT) return launch_one<FMT, R, NT, 1, 4>(p, grid_x, 1, s);
     }
     if (M == 1) return launch_one<FMT, R, NT, 1>(p, grid_x, 1, s);
-    // more tokens (see tc_takes): small Q8_0 layers at M = 2, Q6_0 with K % 64 != 0 at M <= 4
-    if constexpr (FMT != EMB_Q4_0) {
-        if (M == 2) return launch_one<FMT, R, NT, 2>(p, grid_x, 1, s);
-        if constexpr (FMT == EMB_Q6_0) return launch_one<FMT, R, NT, 4>(p, grid_x, (M + 3) / 4, s);
-    }
-    return cudaErrorInvalidValue;
+    // more tokens (see tc_takes): small or few-row layers at M = 2 and 3, Q6_0 with K % 64 != 0 at M <= 4
+    if (M == 2) return launch_one<FMT, R, NT, 2>(p, grid_x, 1, s);
+    return launch_one<FMT, R, NT, 4>(p, grid_x, (M + 3) / 4, s);
 }
 
 template <int FMT, int R>
@@ -349,7 +349,7 @@ struct StagedParams {
 // (MT, the tokens of a CTA, is 1 in every use. The kernel keeps the loop over tokens: with it
 // written out, ptxas sinks the code loads to their uses, 55 registers become 48, and Gemma-2B gate/up
 // takes 14.9 us instead of 14.4.)
-template <int FMT, int RW, int MT>
+template <int FMT, int RW, int MT, bool FIRST>
 __global__ void __launch_bounds__(kStageThreads) gemv_staged_kernel(const __grid_constant__ StagedParams p) {
     constexpr int UW = (FMT == EMB_Q8_0) ? 16 : 32;
     extern __shared__ __align__(128) uint8_t smem[];
@@ -382,7 +382,7 @@ __global__ void __launch_bounds__(kStageThreads) gemv_staged_kernel(const __grid
         ptx::mbar_init(bar_w, 1);
         ptx::mbar_init(bar_x, 1);
         ptx::fence_mbar_init();
-        if (p.wait_first) ptx::griddep_wait();  // (the previous launch may have written the weights)
+        if constexpr (FIRST) ptx::griddep_wait();
         ptx::mbar_arrive_expect_tx(bar_w, codes_bytes + hi_bytes + scales_bytes);
         ptx::bulk_load(codes_s, p.codes[g] + int64_t(row0) * row_bytes, codes_bytes, bar_w);
         if constexpr (FMT == EMB_Q6_0)
@@ -504,7 +504,7 @@ __global__ void __launch_bounds__(kStageThreads) gemv_staged_kernel(const __grid
     }
 }
 
-template <int FMT, int RW>
+template <int FMT, int RW, bool FIRST>
 cudaError_t launch_staged_one(const StagedParams& p, int tiles, size_t smem, cudaStream_t s) {
     static_assert(kStageHeader + kStageXBytes + kStageBytes + kStageBytes / 8 <= 227 * 1024, "smem");
     cudaLaunchConfig_t cfg = {};
@@ -519,18 +519,22 @@ cudaError_t launch_staged_one(const StagedParams& p, int tiles, size_t smem, cud
     cfg.numAttrs = 1;
     if (smem > 48 * 1024) {
         static std::atomic<uint64_t> done{0};
-        const cudaError_t e = allow_smem(gemv_staged_kernel<FMT, RW, 1>,
+        const cudaError_t e = allow_smem(gemv_staged_kernel<FMT, RW, 1, FIRST>,
                                          int(kStageHeader + kStageXBytes + kStageBytes + kStageBytes / 8), done);
         if (e != cudaSuccess) return e;
     }
-    return cudaLaunchKernelEx(&cfg, gemv_staged_kernel<FMT, RW, 1>, p);
+    return cudaLaunchKernelEx(&cfg, gemv_staged_kernel<FMT, RW, 1, FIRST>, p);
 }
 
 template <int FMT>
 cudaError_t launch_staged_rw(const StagedParams& p, int RW, int tiles, size_t smem, cudaStream_t s) {
-    if (RW == 4) return launch_staged_one<FMT, 4>(p, tiles, smem, s);
-    if (RW == 2) return launch_staged_one<FMT, 2>(p, tiles, smem, s);
-    return launch_staged_one<FMT, 1>(p, tiles, smem, s);
+    if (p.wait_first)
+        return RW == 4 ? launch_staged_one<FMT, 4, true>(p, tiles, smem, s)
+             : RW == 2 ? launch_staged_one<FMT, 2, true>(p, tiles, smem, s)
+                       : launch_staged_one<FMT, 1, true>(p, tiles, smem, s);
+    return RW == 4 ? launch_staged_one<FMT, 4, false>(p, tiles, smem, s)
+         : RW == 2 ? launch_staged_one<FMT, 2, false>(p, tiles, smem, s)
+                   : launch_staged_one<FMT, 1, false>(p, tiles, smem, s);
 }
 
 // Tile shape: rows per warp RW and warps along K WK (TR = RW * 4 / WK rows per tile),
@@ -1035,30 +1039,54 @@ TcParams tc_params(const GroupRef& g, bool pdl, int& n_tiles) {
 bool ring_takes(const GroupRef& g);
 
 // Which calls take it (us per launch in graph-replayed chains, this kernel / the one it leaves):
-//  * M = 3, 4 always, M = 2 but for Q8_0 layers below 1 M weights (640 x 320 1.77 / 1.50, kept on
-//    the register kernel): Q6_0 32768 x 2048 at M = 4 15.4 / 32.9, Q4_0 13.4 / 18.0, Q8_0 16.6 /
-//    22.8; 2048 x 16384 at M = 4 Q8_0 10.0 / 22.6, Q6_0 9.7 / 24.9, Q4_0 8.1 / 23.0;
+//  * M = 3, 4 always (Q6_0 32768 x 2048 at M = 4 15.4 / 32.9, Q4_0 13.4 / 18.0, Q8_0 16.6 / 22.8;
+//    2048 x 16384 at M = 4 Q8_0 10.0 / 22.6, Q6_0 9.7 / 24.9, Q4_0 8.1 / 23.0); M = 2 but for what the
+//    register kernel answers in one short wave: Q8_0 below 1 M weights (640 x 320 1.77 / 1.50), the others
+//    up to 4 M with four of its rows per CTA (2048 x 2048 Q4_0 2.30 / 2.19, Q6_0 2.74 / 2.49; 1024 x
+//    1024 Q4_0 1.61 / 2.89), and at M = 2 and 3 Q6_0 below 256 K (640 x 320 1.91 / 1.82, 300 x 512
+//    1.87 / 1.82) and up to 32 tiles of long rows, which leave SMs idle (512 x 16384 Q8_0 7.6 / 6.5);
 //  * M = 6..16 in place of the tcgen05 GEMM (12288 x 4096 at M = 8 Q8_0 14.6 / 26.7, Q4_0 13.5 /
 //    27.9; 1024 x 4096 at M = 16 4.6 / 6.4), but for Q8_0 above 12 tokens and 32 M weights
 //    (32768 x 2048 30.4 / 27.7), and for five tokens, the count at which the GEMM's bf16 operand
 //    is held to its bits (tests/test_gpu_hotpath_dequant.py);
-//  * M = 1 with rows of at least 4096 k, where its codes-to-bf16 step is cheaper than FFMA2 dot
-//    products and no activation row is staged per CTA: Q4_0 (2048 x 16384 7.5 / 9.3, 4096 x 4096
-//    4.1 / 4.7; with K < 8192 and more than five row tiles per SM the staged kernel keeps it,
-//    22016 x 4096 16.9 / 16.4), Q6_0 (12288 x 4096 12.7 / 16.8, 4096 x 11008 11.6 /
-//    14.4, 2048 x 16384 9.4 / 9.3), Q8_0 only with at most two row tiles per SM (1024 x 4096 2.6 / 3.3, 4096 x 11008
-//    12.1 / 13.3; 12288 x 4096 13.2 / 11.9).
+//  * M = 1, Q4_0 and Q6_0, with rows of at least 4096 k, where its codes-to-bf16 step is cheaper than FFMA2
+//    dot products and no activation row is staged per CTA, if its 16-row tiles are many and fill the SMs:
+//    at least 60 (512 x 16384 Q4_0 6.5 / 4.5, Q6_0 8.0 / 5.2), and where they are more than the SMs at
+//    least 80 % of the slots of their rounds of two CTAs per SM (4096 x 11008 Q4_0, 84 %, 10.3 / 11.3;
+//    2560 x 11008, 53 %, 9.4 / 8.1; 6144 x 11008, 63 %, 18.1 / 15.4; 11008 x 11008, 75 %, 25.6 / 24.6).
+//    At K where the staged kernel's lanes are idle part of the time (Q4_0 4608 to 8192, Q6_0 5120 to 6144) any
+//    fill beyond one round will do (Q4_0 11008 x 4608 12.9 / 15.5, 6144 x 5120 8.3 / 10.7; Q6_0 6144 x 5120 10.4 / 11.2).
+//    With K < 5120 not from 1216 to 4095 rows, where the register kernel has one short wave of four rows per
+//    CTA (2048 x 4096 Q4_0 2.8 / 2.4, Q6_0 3.3 / 2.75), nor Q4_0 beyond five tiles per SM (staged kernel: 22016 x
+//    4096 16.9 / 16.4). Q6_0 only where rows fill the other kernels' passes of 256 threads to less than
+//    70 % (4096 x 4096 4.95 / 7.1, 4096 x 11008 13.3 / 14.4; 4096 x 8192 9.6 / 9.2, 8192 x 16384 35.0 / 30.2, 1300 x 12288
+//    6.6 / 6.3). Q8_0 gains at some row counts and loses at others (1024 x 4096 2.6 / 3.2, 1300 x 4096 2.9 / 2.2).
 bool tc_takes(const GroupRef& g, int sms) {
     if (g.M > kTcMaxM || g.M == 5 || (g.fmt == EMB_Q6_0 && g.K % 64 != 0)) return false;
-    int64_t rows = 0;
-    for (int i = 0; i < g.n_mats; ++i) rows += g.mats[i].N;
-    if (g.M == 1) {
-        if (g.K < 4096) return false;
-        if (g.fmt == EMB_Q4_0) return g.K >= 8192 || rows <= int64_t(5 * kTcRows) * sms;
-        return g.fmt == EMB_Q6_0 || (!ring_takes(g) && rows <= int64_t(2 * kTcRows) * sms);
+    int64_t rows = 0, tiles = 0;
+    for (int i = 0; i < g.n_mats; ++i) {
+        rows += g.mats[i].N;
+        tiles += (g.mats[i].N + kTcRows - 1) / kTcRows;
     }
-    if (g.fmt == EMB_Q8_0 && g.M == 2) return rows * g.K >= (int64_t(1) << 20);
-    if (g.fmt == EMB_Q8_0 && g.M > 12) return rows * g.K <= (int64_t(1) << 25);
+    const int64_t weights = rows * g.K;
+    const bool four_rows = rows >= 4 * 2 * 152;  // per CTA of the register kernel (launch_gemv_regs)
+    if (g.M == 1) {
+        if (g.fmt == EMB_Q8_0 || g.K < 4096 || tiles < 60) return false;
+        const int64_t slots = 2 * int64_t(sms);
+        const bool any_fill = tiles > slots && (g.fmt == EMB_Q4_0 ? g.K >= 4608 && g.K <= 8192 : g.K >= 5120 && g.K <= 6144);
+        if (tiles > sms && !any_fill && 5 * tiles < 4 * slots * ((tiles + slots - 1) / slots)) return false;
+        if (g.K < 5120 && four_rows && rows < 4096) return false;
+        if (g.fmt == EMB_Q4_0) return g.K >= 5120 || tiles <= 5 * int64_t(sms);
+        const int64_t U = g.K / 32, passes = (U + 255) / 256;
+        return U < 256 || 10 * U < 7 * 256 * passes;
+    }
+    if (g.M <= 3) {
+        if (tiles <= 32 && g.K >= 4096) return false;
+        if (g.fmt == EMB_Q6_0 && weights < (int64_t(1) << 18)) return false;
+    }
+    if (g.M == 2)
+        return g.fmt == EMB_Q8_0 ? weights >= (int64_t(1) << 20) : !(four_rows && weights <= (int64_t(1) << 22));
+    if (g.fmt == EMB_Q8_0 && g.M > 12) return weights <= (int64_t(1) << 25);
     return true;
 }
 
@@ -1312,6 +1340,7 @@ constexpr int kRingHeader = 144 + kRingFlush * (kRingThreads / 32) * 4;
 
 struct RingParams {
     const uint8_t* codes[kMaxGroup];
+    const uint8_t* high[kMaxGroup];  // Q6_0: 2-bit high plane of each matrix
     const __half* scales[kMaxGroup];
     void* Y[kMaxGroup];
     int32_t N[kMaxGroup];
@@ -1319,7 +1348,7 @@ struct RingParams {
     int32_t n_mats;
     int32_t K, ldS, U;
     int32_t rows_per_cta, rows_total;
-    int32_t stage_bytes;          // one row of codes + its scales, rounded up to 16
+    int32_t stage_bytes;          // one row of codes (+ Q6_0 high bits) + its scales, rounded up to 16
     int32_t stages;               // ring depth (2..kRingMaxStages)
     int32_t epi;
     int32_t wait_first;            // 1: nothing is read before griddepcontrol.wait
@@ -1327,9 +1356,9 @@ struct RingParams {
     int* status;
 };
 
-template <int PF>
+template <int FMT, int PF, bool FIRST>
 __global__ void __launch_bounds__(kRingThreads, 2) gemv_ring_kernel(const __grid_constant__ RingParams p) {
-    constexpr int UW = 16;
+    constexpr int UW = (FMT == EMB_Q8_0) ? 16 : 32;
     constexpr int NT = kRingThreads, NWARP = NT / 32;
     extern __shared__ __align__(128) uint8_t smem[];
     uint64_t* full = reinterpret_cast<uint64_t*>(smem);              // [stages]
@@ -1340,7 +1369,8 @@ __global__ void __launch_bounds__(kRingThreads, 2) gemv_ring_kernel(const __grid
     const int S = p.stages;
     const int t = threadIdx.x, lane = t & 31, warp = t >> 5;
     const int U = p.U;
-    const int64_t row_bytes = p.K;
+    const int64_t row_bytes = (FMT == EMB_Q8_0) ? int64_t(p.K) : int64_t(p.K) / 2;
+    const int64_t high_bytes = (FMT == EMB_Q6_0) ? int64_t(p.K) / 4 : 0;  // a multiple of 16
     const int r_begin = blockIdx.x * p.rows_per_cta;
     const int n_rows = min(p.rows_per_cta, p.rows_total - r_begin);
     // global row -> (matrix, row within it)
@@ -1356,10 +1386,11 @@ __global__ void __launch_bounds__(kRingThreads, 2) gemv_ring_kernel(const __grid
         locate(r_begin + i, g, n);
         uint8_t* st = ring + stage * p.stage_bytes;
         uint64_t* bar = &full[stage];
-        const uint32_t cb = uint32_t(row_bytes), sb = uint32_t(p.ldS) * 2u;
-        ptx::mbar_arrive_expect_tx(bar, cb + sb);
+        const uint32_t cb = uint32_t(row_bytes), hb = uint32_t(high_bytes), sb = uint32_t(p.ldS) * 2u;
+        ptx::mbar_arrive_expect_tx(bar, cb + hb + sb);
         ptx::bulk_load(st, p.codes[g] + int64_t(n) * row_bytes, cb, bar);
-        ptx::bulk_load(st + row_bytes, p.scales[g] + int64_t(n) * p.ldS, sb, bar);
+        if constexpr (FMT == EMB_Q6_0) ptx::bulk_load(st + row_bytes, p.high[g] + int64_t(n) * high_bytes, hb, bar);
+        ptx::bulk_load(st + row_bytes + high_bytes, p.scales[g] + int64_t(n) * p.ldS, sb, bar);
     };
     if (t == 0) {
         *abort_flag = 0;
@@ -1368,7 +1399,7 @@ __global__ void __launch_bounds__(kRingThreads, 2) gemv_ring_kernel(const __grid
             ptx::mbar_init(&empty[i], NWARP);
         }
         ptx::fence_mbar_init();
-        if (p.wait_first) ptx::griddep_wait();  // (the previous launch may have written the weights)
+        if constexpr (FIRST) ptx::griddep_wait();
         for (int i = 0; i < S && i < n_rows; ++i) issue(i, i);
         // the activation row towards L2 while the previous launch finishes (one CTA asks)
         if (blockIdx.x == 0) ptx::prefetch_l2(p.X, uint32_t(p.K) * 2u);
@@ -1436,15 +1467,17 @@ __global__ void __launch_bounds__(kRingThreads, 2) gemv_ring_kernel(const __grid
         ok = __all_sync(0xffffffffu, ok && ptx::mbar_wait(&full[s], ph, abort_flag, p.status, kWaitLimitNs));
         if (ok) {
             const uint8_t* cs = ring + s * p.stage_bytes;
-            const __half* ss = reinterpret_cast<const __half*>(cs + row_bytes);
+            const __half* ss = reinterpret_cast<const __half*>(cs + row_bytes + high_bytes);
             float acc = 0.0f;
 #pragma unroll
             for (int k = 0; k < PF; ++k) {
                 const int uk = t + k * NT;
                 if (uk < U) {
                     const uint4 c = *reinterpret_cast<const uint4*>(cs + int64_t(uk) * 16);
-                    const float d = __half2float(ss[uk >> 1]);
-                    acc = fmaf(d, dot_q8_unit(c, x[k]), acc);
+                    uint2 hq = make_uint2(0, 0);
+                    if constexpr (FMT == EMB_Q6_0) hq = *reinterpret_cast<const uint2*>(cs + row_bytes + int64_t(uk) * 8);
+                    const float d = __half2float(ss[(FMT == EMB_Q8_0) ? (uk >> 1) : uk]);
+                    acc = fmaf(d, dot_unit<FMT>(c, hq, x[k]), acc);
                 }
             }
             __syncwarp();
@@ -1464,7 +1497,7 @@ __global__ void __launch_bounds__(kRingThreads, 2) gemv_ring_kernel(const __grid
     if (flushed < n_rows) flush(n_rows);  // (a CTA whose wait gave up leaves inside it)
 }
 
-template <int PF>
+template <int FMT, int PF, bool FIRST>
 cudaError_t launch_ring_one(const RingParams& p, int ctas, size_t smem, cudaStream_t s) {
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3(ctas, 1, 1);
@@ -1478,9 +1511,20 @@ cudaError_t launch_ring_one(const RingParams& p, int ctas, size_t smem, cudaStre
     cfg.numAttrs = 1;
     // (two stages of the longest row, 16 KB of codes, fit the budget too)
     static std::atomic<uint64_t> done{0};
-    const cudaError_t e = allow_smem(gemv_ring_kernel<PF>, kRingHeader + kRingBudget, done);
+    const cudaError_t e = allow_smem(gemv_ring_kernel<FMT, PF, FIRST>, kRingHeader + kRingBudget, done);
     if (e != cudaSuccess) return e;
-    return cudaLaunchKernelEx(&cfg, gemv_ring_kernel<PF>, p);
+    return cudaLaunchKernelEx(&cfg, gemv_ring_kernel<FMT, PF, FIRST>, p);
+}
+
+template <int FMT>
+cudaError_t launch_ring_fmt(const RingParams& p, int pf, int ctas, size_t smem, cudaStream_t s) {
+    if (p.wait_first)
+        return pf == 2 ? launch_ring_one<FMT, 2, true>(p, ctas, smem, s)
+             : pf == 3 ? launch_ring_one<FMT, 3, true>(p, ctas, smem, s)
+                       : launch_ring_one<FMT, 4, true>(p, ctas, smem, s);
+    return pf == 2 ? launch_ring_one<FMT, 2, false>(p, ctas, smem, s)
+         : pf == 3 ? launch_ring_one<FMT, 3, false>(p, ctas, smem, s)
+                   : launch_ring_one<FMT, 4, false>(p, ctas, smem, s);
 }
 
 int gemv_sm_count() {
@@ -1494,8 +1538,8 @@ int gemv_sm_count() {
     return counts[dev];
 }
 
-// Which layers take the ring path: M = 1, Q8_0 (the other formats are faster on the tensor-core
-// kernel), rows longer than the staged path takes at M = 1 and than one pass
+// Which layers take the ring path: M = 1, Q8_0 or Q6_0 (K % 64 == 0, for its high plane's 16-byte rows;
+// what of it tc_takes leaves), rows longer than the staged path takes at M = 1 and than one pass
 // of 256 threads (2..4 units per thread), matrices of at least kStageMinBytes; two CTAs per
 // SM, rows split evenly (even runs for gated epilogues).
 // Measured on GB300, Gemma-2B decode step (paired runs on one box, 1000 steps): Q8_0 chain
@@ -1503,17 +1547,20 @@ int gemv_sm_count() {
 // registers and two in shared memory; a 72 KB ring instead of 56 KB was slower for Q8_0,
 // a CTA-wide barrier per row cost ~2 %, and stage indices by integer division ~4 %.
 bool ring_takes(const GroupRef& g) {
-    if (g.M != 1 || g.fmt != EMB_Q8_0) return false;
-    const int64_t U = g.K / 16;
-    if (g.K <= kStageMaxRowBytesM1 || U <= kRingThreads || U > 4 * kRingThreads) return false;
+    if (g.M != 1 || g.fmt == EMB_Q4_0 || (g.fmt == EMB_Q6_0 && g.K % 64 != 0)) return false;
+    const int64_t weight_row_bytes = g.fmt == EMB_Q8_0 ? g.K : g.K / 2 + g.K / 4;
+    const int64_t U = g.fmt == EMB_Q8_0 ? g.K / 16 : g.K / 32;
+    if (weight_row_bytes <= kStageMaxRowBytesM1 || U <= kRingThreads || U > 4 * kRingThreads) return false;
     int64_t rows = 0;
     for (int i = 0; i < g.n_mats; ++i) rows += g.mats[i].N;
-    return rows * g.K >= kStageMinBytes;
+    return rows * weight_row_bytes >= kStageMinBytes;
 }
 
 bool launch_ring(const GroupRef& g, bool pdl, int* status, cudaStream_t s, cudaError_t& err) {
     if (!ring_takes(g)) return false;
-    const int64_t row_bytes = g.K, U = g.K / 16;
+    const int64_t row_bytes = (g.fmt == EMB_Q8_0) ? g.K : g.K / 2;
+    const int64_t high_bytes = (g.fmt == EMB_Q6_0) ? g.K / 4 : 0;
+    const int64_t U = (g.fmt == EMB_Q8_0) ? g.K / 16 : g.K / 32;
     int64_t rows = 0;
     for (int i = 0; i < g.n_mats; ++i) rows += g.mats[i].N;
     const int sms = gemv_sm_count();
@@ -1522,6 +1569,7 @@ bool launch_ring(const GroupRef& g, bool pdl, int* status, cudaStream_t s, cudaE
     int64_t r0 = 0;
     for (int i = 0; i < g.n_mats; ++i) {
         p.codes[i] = g.mats[i].codes;
+        p.high[i] = g.mats[i].high;
         p.scales[i] = g.mats[i].scales;
         p.Y[i] = g.mats[i].Y;
         p.N[i] = int32_t(g.mats[i].N);
@@ -1541,14 +1589,13 @@ bool launch_ring(const GroupRef& g, bool pdl, int* status, cudaStream_t s, cudaE
     if (g.epi >= EMB_EPI_GEGLU) rpc = (rpc + 1) & ~int64_t(1);  // gate/up pairs stay in one CTA
     p.rows_per_cta = int32_t(rpc);
     p.rows_total = int32_t(rows);
-    p.stage_bytes = int32_t((row_bytes + g.ldS * 2 + 15) & ~int64_t(15));
+    p.stage_bytes = int32_t((row_bytes + high_bytes + g.ldS * 2 + 15) & ~int64_t(15));
     p.stages = int32_t(std::min<int64_t>(kRingMaxStages, std::max<int64_t>(2, kRingBudget / p.stage_bytes)));
     const int ctas = int((rows + rpc - 1) / rpc);
     const size_t smem = kRingHeader + size_t(p.stages) * p.stage_bytes;
     const int pf = int((U + kRingThreads - 1) / kRingThreads);
-    err = pf == 2 ? launch_ring_one<2>(p, ctas, smem, s)
-        : pf == 3 ? launch_ring_one<3>(p, ctas, smem, s)
-                  : launch_ring_one<4>(p, ctas, smem, s);
+    err = g.fmt == EMB_Q8_0 ? launch_ring_fmt<EMB_Q8_0>(p, pf, ctas, smem, s)
+                            : launch_ring_fmt<EMB_Q6_0>(p, pf, ctas, smem, s);
     return true;
 }
 
