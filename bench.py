@@ -525,8 +525,8 @@ def measure_workload(name, ws, args, dev, dist, steps, warmup, e2e_steps, clocks
                     "peak_source": f"{peaks['source']} HBM copy bandwidth"}
         roof["frac"] = roof["achieved"] / roof["peak"]
         roof["traffic"] = kernel_traffic(name, c["w"])
-        roof["kernel"] = ("GEMV (gemv_staged_kernel + gemv_ring_kernel + gemv_kernel + gemv_q4_mma_kernel)" if c["w"].M <= 4
-                          else "gemm_tc_kernel") + f" <{wl.FMT_NAMES[c['w'].fmt]}>"
+        roof["kernel"] = ("GEMV (gemv_staged_kernel + gemv_ring_kernel + gemv_kernel + gemv_tc_kernel)" if c["w"].M <= 16
+                          else "gemm_chunk_kernel" if c["w"].M <= 64 else "gemm_tc_kernel") + f" <{wl.FMT_NAMES[c['w'].fmt]}>"
         roof["launches_per_step"] = c["launches"] * c["w"].repeats
         roof["per_launch_us"] = per_launch_ms * 1e3
         return roof
@@ -888,7 +888,7 @@ def run_layer_loop(args):
     if lin_ms >= attn_ms:
         per_launch = lin_ms / lin_launches
         achieved = lin_bytes / lin_launches / (per_launch / 1e3) / 1e9
-        kernel = "gemm_tc_kernel <Q8_0> (q/k/v, o, gate/up, down)"
+        kernel = "gemm_chunk_kernel <Q8_0> (q/k/v, o, gate/up, down)"
         nl = lin_launches
     else:
         qd, kd = L.H * L.d, L.Hk * L.d
