@@ -948,13 +948,15 @@ size_t sk_ws_bytes(int G, int P, int T) { return kSkFlagBytes + size_t(G) * sk_s
 double step_cycles(int P, int T) { return std::max(620.0, 2.22 * P * T + 150.0); }
 double item_cycles(int P, int T) { return 6300.0 + 22.6 * P * T; }
 // One launch: waves of CTAs that each take an item's share of K. A K split adds its cluster's
-// exchange, ~2000 + 36 per token of the tile (235 launches of 11 layer shapes with the token tile
-// and the splits forced; the three models together reproduce them to ~12 %).
+// exchange, ~3000 + 13 per token of the tile (four splits against none at 1000 x 1088 and 1152 x 1152, tiles of
+// 96, 128, 160 and 256 tokens). Twelve clusters of eight CTAs run at once, sixteen do not (512 x 16384: M = 600
+// in twelve 23.2 us, M = 512 in eight 22.3, in sixteen 35.4).
 double plan_cycles(int64_t items, int P, int T, int splits, int64_t K, int sms) {
     const int64_t nr = (K + kKR - 1) / kKR, nk = (K + kKC - 1) / kKC;
     const double steps = double(std::min(nk, (nr + splits - 1) / splits * kStepsPerRaw));
-    const double exchange = splits > 1 ? 2000.0 + 36.0 * T : 0.0;
-    return double((items * splits + sms - 1) / sms) * (steps * step_cycles(P, T) + item_cycles(P, T) + exchange);
+    const double exchange = splits > 1 ? 3000.0 + 13.0 * T : 0.0;
+    const int64_t waves = splits == 8 ? (items + 11) / 12 : (items * splits + sms - 1) / sms;
+    return double(waves) * (steps * step_cycles(P, T) + item_cycles(P, T) + exchange);
 }
 
 // The launch shape of one group. With streamk_ok the plan may take the stream-K schedule,
