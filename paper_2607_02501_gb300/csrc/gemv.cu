@@ -1299,9 +1299,12 @@ cudaError_t launch_chunk_fmt(const TcParams& p, int tiles, int sms, cudaStream_t
 // whose CTAs are resident at once (M = 50: 1280 x 1024 3.9 / 5.2, 2048 x 2048 4.6 / 12.7, 2048 x 16384
 // Q8_0 26.8 / 33.5; M = 32: 4096 x 4096 8.6 / 10.6). Beyond that the activations are read once per
 // round of row tiles and the GEMM's larger tiles catch up: up to 32 tokens while the GEMM has fewer
-// than 96 tiles of 128 rows or the codes are 4 or 6 bits wide (M = 24: 11008 x 4096 Q8_0 23.3 / 26.4,
+// than 96 tiles of 128 rows and the rounds are 70 % full (M = 32: 5120 x 5120, 53 %, 22.0 / 21.4) or the codes are 4 or
+// 6 bits wide (M = 24: 11008 x 4096 Q8_0 23.3 / 26.4,
 // 16384 x 2048 Q8_0 16.4 / 15.1, Q4_0 13.3 / 15.6), above 32 tokens for short rows in at most two
-// rounds (M = 50: 8192 x 1024 8.1 / 8.4, 2560 x 2048 8.0 / 7.3, 12288 x 1536 19.6 / 11.5).
+// rounds (M = 50: 8192 x 1024 8.1 / 8.4, 2560 x 2048 8.0 / 7.3, 12288 x 1536 19.6 / 11.5). Up to 1536 long rows
+// are one wave of the GEMM's eight K splits, while a CTA here walks a whole row (M = 50: 512 x 16384 23.9 / 18.2, 1152 x
+// 16384 25.7 / 19.3, M = 33: 512 x 6144 9.8 / 9.1; M = 50: 1024 x 4096 7.0 / 8.8).
 bool chunk_takes(const GroupRef& g, int sms) {
     if (g.M <= kTcMaxM || g.M > 2 * kCkTokens || g.K < 1024 || g.precise || (g.fmt == EMB_Q6_0 && g.K % 64 != 0))
         return false;
@@ -1310,10 +1313,12 @@ bool chunk_takes(const GroupRef& g, int sms) {
         rows += g.mats[i].N;
         tiles += (g.mats[i].N + kTcRows - 1) / kTcRows;
     }
+    if (rows <= 12 * 128 && g.K > 4608) return false;
     const bool short_rows = g.K < 8 * kTcBlocks * kQBlock;
     const int64_t ctas = g.M > kCkTokens && !short_rows ? 2 * tiles : tiles, slots = 2 * int64_t(sms);
     if (ctas <= slots) return true;
-    if (g.M <= kCkTokens) return g.fmt != EMB_Q8_0 || rows < 96 * 128;
+    if (g.M <= kCkTokens)
+        return g.fmt != EMB_Q8_0 || (rows < 96 * 128 && 10 * ctas >= 7 * slots * ((ctas + slots - 1) / slots));
     return short_rows && ctas <= 2 * slots;
 }
 
