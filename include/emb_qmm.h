@@ -221,10 +221,14 @@ EMB_API emb_status emb_qlayer_seq(const emb_qlayer* layers, int n_layers, int64_
  * As emb_qlayer_seq, for a call inside a chain of this library's launches (a layer's
  * linears between its norm, rotary and attention launches): the first launch of the call
  * also overlaps its weight fetch with the end of the launch before it on `stream`, as
- * every later launch of a call does. Precondition: the weights of the call are not
- * written by the launch enqueued on `stream` just before the call (weights produced
- * further back, e.g. by emb_quantize_* followed by any other launch or a synchronisation,
- * are fine). No workspace: results are bitwise those of emb_qlayer_seq with a NULL
+ * every later launch of a call does. Precondition: between whatever writes the weights of
+ * the call and the call itself, `stream` has something that waits for the writer before it
+ * lets the next launch start: a synchronisation, a copy, a kernel launched without
+ * programmatic stream serialisation (emb_quantize_* of other weights, for one), or a call of
+ * emb_qmatmul, emb_qlayer_seq, emb_qlayer_seq_noalloc or emb_chain_launch. The norm, rotary
+ * and attention calls and this one do not count: they let the next launch start while work
+ * ahead of them may still run (waiting first costs a whole 7B layer at M = 1 5 %).
+ * No workspace: results are bitwise those of emb_qlayer_seq with a NULL
  * workspace. Errors as emb_qlayer_seq. */
 EMB_API emb_status emb_qlayer_seq_chained(const emb_qlayer* layers, int n_layers, int64_t M,
                                           emb_stream_t stream);

@@ -220,7 +220,8 @@ def emb_qlayer_seq(layers, M: int, workspace=None, ws_bytes: int = 0, stream=Non
 
 def emb_qlayer_seq_chained(layers, M: int, stream=None) -> None:
     """emb_qlayer_seq whose first launch also overlaps the previous launch on the stream
-    (the call's weights must not be written by that launch)."""
+    (the call's weights must be complete by then: something that waits for their writer, and is
+    not a norm, rotary, attention or chained call, lies between; see the C header)."""
     arr = layers if isinstance(layers, ctypes.Array) else make_layers(layers)
     _check(lib().emb_qlayer_seq_chained(arr, len(arr), M, _stream(stream)), "emb_qlayer_seq_chained")
 

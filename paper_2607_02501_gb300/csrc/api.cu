@@ -312,10 +312,11 @@ static emb_status attach_workspace(std::vector<GroupRef>& refs, int64_t M, void*
 
 static emb_status enqueue_seq(const std::vector<GroupRef>& refs, cudaStream_t s, bool first_pdl) {
     for (size_t i = 0; i < refs.size(); ++i) {
-        // the first launch must not read weights while whatever the caller enqueued before still
-        // runs (it may have produced them) unless the caller says it did not: it is started early
-        // but waits first (launch latency, barriers and TMEM allocation overlap; one 50 x 1024 x
-        // 1024 GEMM after another 10.2 -> 6.6 us a call). Later ones overlap their weight fetch too
+        // no launch of the call may read weights while whatever the caller enqueued before still
+        // runs (it may have produced them) unless the caller says it did not: the first is started
+        // early but waits before it reads and before it lets the second start (launch latency,
+        // barriers and TMEM allocation overlap; one 50 x 1024 x 1024 GEMM after another 10.2 ->
+        // 6.6 us a call). Later ones overlap their weight fetch too
         const cudaError_t e = launch_group(refs[i], i > 0 || first_pdl, s);
         if (e != cudaSuccess) return EMB_ECUDA;
     }

@@ -285,6 +285,7 @@ __global__ void __launch_bounds__(kThreads, 1) gemm_tc_kernel(const __grid_const
     __syncthreads();
     ptx::tc_fence_after();
     const uint32_t tmem = ptx::warp_uniform(*tmem_slot);
+    if (p.wait_first) ptx::griddep_wait();  // every thread before the trigger: see ptx::griddep_launch_dependents
     ptx::griddep_launch_dependents();
     int items_done = 0;  // this CTA's items started by its role (phase of acc_full / acc_empty)
 
@@ -324,7 +325,6 @@ __global__ void __launch_bounds__(kThreads, 1) gemm_tc_kernel(const __grid_const
                 // the first raw stages before griddepcontrol.wait: weights never depend on
                 // the previous launch; X may be written by it, so only its rows' way towards
                 // L2 starts now (a hint: the TMA loads after the wait read the written values)
-                if (p.wait_first) ptx::griddep_wait();  // (the previous launch may have written the weights)
                 for (; raw_issued < nr && raw_issued < kRawStages; ++raw_issued) issue_raw(raw_issued);
                 const int x_rows = min(M - I.m0, P * T);
                 if (lane == 0 && x_rows > 0 && I.n0 == 0 && I.g == 0 && sg.r0 == 0)  // one CTA per token tile

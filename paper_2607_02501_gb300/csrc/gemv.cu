@@ -124,8 +124,8 @@ __global__ void __launch_bounds__(NT) gemv_kernel(const __grid_constant__ GemvPa
     const __half* sbase = p.scales[g] + int64_t(row0) * p.ldS;
     const int U = p.U;
 
+    if constexpr (FIRST) griddep_wait();  // before the trigger: see ptx::griddep_launch_dependents
     griddep_launch_dependents();
-    if constexpr (FIRST) griddep_wait();
     // the activation rows towards L2 while the previous launch finishes (measured on GB300:
     // cold, they arrive ~2 us after the dependency wait, behind the weight stream); one CTA
     // per row block asks, since every CTA reads the same rows
@@ -393,6 +393,7 @@ __global__ void __launch_bounds__(kStageThreads) gemv_staged_kernel(const __grid
         // one CTA per row block asks, since every CTA reads the same rows
         if (blockIdx.x == 0) ptx::prefetch_l2(p.X + int64_t(m0) * p.K, uint32_t(mt) * uint32_t(p.K) * 2u);
     }
+    if constexpr (FIRST) ptx::griddep_wait();  // every thread before the trigger: see ptx::griddep_launch_dependents
     ptx::griddep_launch_dependents();
     // weights do not depend on earlier launches; X and Y may
     ptx::griddep_wait();
@@ -811,6 +812,7 @@ __global__ void __launch_bounds__(32 * NW, 16 / NW) gemv_tc_kernel(const __grid_
     const int nb = p.K / kQBlock;
     const int tiles = p.tile0[p.n_mats];
     const uint32_t ring = ptx::smem_u32(smem) + warp * kTcStages * St::kBytes;
+    if (p.wait_first) griddep_wait();  // before the trigger: see ptx::griddep_launch_dependents
     griddep_launch_dependents();
     // this warp's chunks of all the CTA's tiles, in order; the next one to issue
     const int stride = NW * kTcBlocks;                 // blocks between a warp's chunks of a tile
@@ -826,7 +828,6 @@ __global__ void __launch_bounds__(32 * NW, 16 / NW) gemv_tc_kernel(const __grid_
         }
         asm volatile("cp.async.commit_group;" ::: "memory");
     };
-    if (p.wait_first) griddep_wait();  // (the previous launch may have written the weights)
 #pragma unroll
     for (int i = 0; i < kTcStages; ++i) issue_next(i);
     if (threadIdx.x == 0 && blockIdx.x == 0) ptx::prefetch_l2(p.X, uint32_t(p.M) * uint32_t(p.K) * 2u);
@@ -1139,6 +1140,7 @@ __global__ void __launch_bounds__(256, 2) gemm_chunk_kernel(const __grid_constan
     const uint32_t ring = ptx::smem_u32(smem) + warp * kCkStages * St::kBytes;
     const int m_base = kCkTokens * (int(blockIdx.y) * WT + wt);  // the warp's first token
 
+    if (p.wait_first) griddep_wait();  // before the trigger: see ptx::griddep_launch_dependents
     griddep_launch_dependents();
     const int stride = WK * kTcBlocks;
     int it_tile = blockIdx.x, it_base = 0;
@@ -1153,7 +1155,6 @@ __global__ void __launch_bounds__(256, 2) gemm_chunk_kernel(const __grid_constan
         }
         asm volatile("cp.async.commit_group;" ::: "memory");
     };
-    if (p.wait_first) griddep_wait();  // (the previous launch may have written the weights)
 #pragma unroll
     for (int i = 0; i < kCkStages; ++i) issue_next(i);
     if (threadIdx.x == 0 && blockIdx.x == 0 && blockIdx.y == 0)
@@ -1409,6 +1410,7 @@ __global__ void __launch_bounds__(kRingThreads, 2) gemv_ring_kernel(const __grid
         // the activation row towards L2 while the previous launch finishes (one CTA asks)
         if (blockIdx.x == 0) ptx::prefetch_l2(p.X, uint32_t(p.K) * 2u);
     }
+    if constexpr (FIRST) griddep_wait();  // every thread before the trigger: see ptx::griddep_launch_dependents
     griddep_launch_dependents();
     __syncthreads();  // the barriers' initialisation is visible to every waiting thread
     // weights do not depend on earlier launches; X and Y may

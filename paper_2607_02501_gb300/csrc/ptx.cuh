@@ -21,6 +21,11 @@ __device__ __forceinline__ uint64_t globaltimer() {
 }
 
 __device__ __forceinline__ void griddep_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+// Lets the next launch of the stream start (once every CTA has called it or ended). That launch may
+// read weights before its own wait, so a kernel launched with wait_first (the first of a call, behind
+// work that may have written any weights of the call) triggers only after griddep_wait has returned:
+// the work before the call is then complete and visible to whatever starts. One thread's trigger
+// counts for its CTA, so every thread waits before it.
 __device__ __forceinline__ void griddep_launch_dependents() {
     asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
 }

@@ -148,3 +148,54 @@ def test_recorded_chain_replays(cuda_device, fmt, M):
     assert emb.emb_device_status() == emb.EMB_OK
     rec.close()
     rec.close()   # idempotent
+
+
+def _norm_rows(total):
+    """Rows and width of the RMSNorm whose bf16 output fills an image of `total` bytes."""
+    D = next(d for d in (4096, 2048, 1024, 512, 256, 128, 64, 8) if total // 2 % d == 0)
+    return total // 2 // D, D
+
+
+@pytest.mark.parametrize("fmt", [emb.EMB_Q8_0, emb.EMB_Q6_0, emb.EMB_Q4_0])
+@pytest.mark.parametrize("M", [1, 4, 50, 280])
+@pytest.mark.parametrize("producer", ["norm", "quantize"])
+def test_weights_written_just_before_the_call(cuda_device, fmt, M, producer):
+    """The image of a call's second launch is written by the work right before the call, without a
+    synchronisation: the call gives the bits it gives after one. The norm is a writer that lets its
+    successor start early; its bf16 output bits are the image (finite fp16 scales: every bf16 pattern
+    below 2^121 is a finite fp16). Two contents alternate, so that stale bytes would show."""
+    N, K = 8192, 4096
+    gen = torch.Generator(device="cuda").manual_seed(11 * M + fmt)
+    rand = lambda *s: torch.randn(*s, generator=gen, device="cuda")
+    img = emb.empty_qweight(fmt, N, K)
+    if producer == "norm":
+        rows, D = _norm_rows(img.numel())
+        src = [rand(rows, D), rand(rows, D)]
+        gamma, out = torch.ones(D, device="cuda"), img.view(torch.bfloat16).view(rows, D)
+        write = lambda i: emb.emb_rmsnorm(src[i], gamma, out, 1e-6)
+    else:
+        pack = {emb.EMB_Q8_0: emb.emb_quantize_q8_0, emb.EMB_Q6_0: emb.emb_quantize_q6_0,
+                emb.EMB_Q4_0: emb.emb_quantize_q4_0}[fmt]
+        src = [rand(N, K), rand(N, K)]
+        write = lambda i: pack(src[i], N, K, img)
+    W1 = emb.quantize(fmt, rand(64, 1024))
+    X1, X2 = rand(M, 1024).to(torch.bfloat16), rand(M, K).to(torch.bfloat16)
+    Y1, Y2 = torch.empty(M, 64, device="cuda"), torch.empty(M, N, device="cuda")
+    layers = emb.make_layers([(fmt, W1, 64, 1024, X1, Y1), (fmt, img, N, K, X2, Y2)])
+    want = []
+    for i in (0, 1):
+        write(i)
+        torch.cuda.synchronize()
+        emb.emb_qlayer_seq(layers, M)
+        torch.cuda.synchronize()
+        want.append(Y2.clone())
+    assert torch.isfinite(want[0]).all() and not torch.equal(want[0], want[1])
+    got = []
+    for r in range(16):
+        write(r % 2)
+        emb.emb_qlayer_seq(layers, M)
+        got.append(Y2.clone())
+    torch.cuda.synchronize()
+    for r, y in enumerate(got):
+        assert torch.equal(y.view(torch.int32), want[r % 2].view(torch.int32)), r
+    assert emb.emb_device_status() == emb.EMB_OK
