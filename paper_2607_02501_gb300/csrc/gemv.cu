@@ -21,10 +21,11 @@
 //     shared memory.
 // The last three dequantise in registers with exact integer->float "magic number"
 // conversions followed by packed fp32x2 FMAs (FFMA2). Every reduction runs in a fixed
-// order, so results are deterministic. Weights are fetched before griddepcontrol.wait (they never depend
-// on an earlier launch) with non-coherent streaming loads; X is read with ordinary
-// (coherent, L1-cached) loads and Y written only after it: the previous launch may have
-// just written X, and after griddepcontrol.wait its writes are visible to ordinary loads.
+// order, so results are deterministic. Weights are fetched before griddepcontrol.wait (within a
+// call they never depend on an earlier launch; the register kernel uses non-coherent streaming
+// loads), but by a call's first launch, behind work that may have written them, after it (the register
+// kernel: with ordinary loads). X is read with ordinary (coherent, L1-cached) loads and Y written only
+// after the wait: the previous launch may have just written X, and its writes are then visible to them.
 // Up to kMaxGroup matrices that read the same X (q/k/v or gate/up) share one launch.
 #include <algorithm>
 #include <atomic>
@@ -71,16 +72,28 @@ struct GemvParams {
     const __nv_bfloat16* X;
 };
 
+// Codes, read once. COHERENT: by ordinary loads, since the launch before may have written them while
+// this grid was already resident; non-coherent ones are for data that nobody writes in its lifetime.
+template <bool COHERENT>
 __device__ __forceinline__ uint4 ld_stream_u4(const void* p) {
     uint4 v;
-    asm volatile("ld.global.nc.L1::no_allocate.v4.u32 {%0, %1, %2, %3}, [%4];"
-                 : "=r"(v.x), "=r"(v.y), "=r"(v.z), "=r"(v.w)
-                 : "l"(p));
+    if constexpr (COHERENT)
+        asm volatile("ld.global.L1::no_allocate.v4.u32 {%0, %1, %2, %3}, [%4];"
+                     : "=r"(v.x), "=r"(v.y), "=r"(v.z), "=r"(v.w)
+                     : "l"(p));
+    else
+        asm volatile("ld.global.nc.L1::no_allocate.v4.u32 {%0, %1, %2, %3}, [%4];"
+                     : "=r"(v.x), "=r"(v.y), "=r"(v.z), "=r"(v.w)
+                     : "l"(p));
     return v;
 }
+template <bool COHERENT>
 __device__ __forceinline__ uint2 ld_stream_u2(const void* p) {
     uint2 v;
-    asm volatile("ld.global.nc.L1::no_allocate.v2.u32 {%0, %1}, [%2];" : "=r"(v.x), "=r"(v.y) : "l"(p));
+    if constexpr (COHERENT)
+        asm volatile("ld.global.L1::no_allocate.v2.u32 {%0, %1}, [%2];" : "=r"(v.x), "=r"(v.y) : "l"(p));
+    else
+        asm volatile("ld.global.nc.L1::no_allocate.v2.u32 {%0, %1}, [%2];" : "=r"(v.x), "=r"(v.y) : "l"(p));
     return v;
 }
 
@@ -139,8 +152,8 @@ __global__ void __launch_bounds__(NT) gemv_kernel(const __grid_constant__ GemvPa
 #pragma unroll
         for (int r = 0; r < R; ++r) {
             if (row0 + r < N) {
-                cc[r] = ld_stream_u4(cbase + r * row_bytes + int64_t(u) * 16);
-                if constexpr (FMT == EMB_Q6_0) hh[r] = ld_stream_u2(hbase + int64_t(r) * (p.K / 4) + int64_t(u) * 8);
+                cc[r] = ld_stream_u4<FIRST>(cbase + r * row_bytes + int64_t(u) * 16);
+                if constexpr (FMT == EMB_Q6_0) hh[r] = ld_stream_u2<FIRST>(hbase + int64_t(r) * (p.K / 4) + int64_t(u) * 8);
                 else hh[r] = make_uint2(0, 0);
                 dd[r] = __half2float(sbase[int64_t(r) * p.ldS + ((FMT == EMB_Q8_0) ? (u >> 1) : u)]);
             } else {

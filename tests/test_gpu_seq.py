@@ -199,3 +199,39 @@ def test_weights_written_just_before_the_call(cuda_device, fmt, M, producer):
     for r, y in enumerate(got):
         assert torch.equal(y.view(torch.int32), want[r % 2].view(torch.int32)), r
     assert emb.emb_device_status() == emb.EMB_OK
+
+
+# one shape per kernel that a call's first launch can take: register (one and four rows per CTA, a
+# whole row in registers), staged, ring, tensor-core GEMV, chunk and tcgen05 GEMM
+FIRST_SHAPES = [(1, 640, 1024), (1, 2048, 2048), (1, 512, 16384), (1, 8192, 2048), (1, 2048, 16384), (4, 8192, 2048),
+                (50, 2048, 2048), (280, 2048, 2048)]
+
+
+@pytest.mark.parametrize("fmt", [emb.EMB_Q8_0, emb.EMB_Q6_0, emb.EMB_Q4_0])
+@pytest.mark.parametrize("M,N,K", FIRST_SHAPES)
+def test_weights_of_a_single_call_written_just_before_it(cuda_device, fmt, M, N, K):
+    """As above for the call's first launch, which is resident while the norm writes its weights."""
+    gen = torch.Generator(device="cuda").manual_seed(M + N + K + fmt)
+    rand = lambda *s: torch.randn(*s, generator=gen, device="cuda")
+    img = emb.empty_qweight(fmt, N, K)
+    rows, D = _norm_rows(img.numel())
+    src, gamma = [rand(rows, D), rand(rows, D)], torch.ones(D, device="cuda")
+    out = img.view(torch.bfloat16).view(rows, D)
+    X, Y = rand(M, K).to(torch.bfloat16), torch.empty(M, N, device="cuda")
+    want = []
+    for i in (0, 1):
+        emb.emb_rmsnorm(src[i], gamma, out, 1e-6)
+        torch.cuda.synchronize()
+        emb.emb_qmatmul(fmt, img, X, Y, M, N, K)
+        torch.cuda.synchronize()
+        want.append(Y.clone())
+    assert torch.isfinite(want[0]).all() and not torch.equal(want[0], want[1])
+    got = []
+    for r in range(16):
+        emb.emb_rmsnorm(src[r % 2], gamma, out, 1e-6)
+        emb.emb_qmatmul(fmt, img, X, Y, M, N, K)
+        got.append(Y.clone())
+    torch.cuda.synchronize()
+    for r, y in enumerate(got):
+        assert torch.equal(y.view(torch.int32), want[r % 2].view(torch.int32)), r
+    assert emb.emb_device_status() == emb.EMB_OK
