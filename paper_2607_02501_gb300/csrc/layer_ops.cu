@@ -508,18 +508,19 @@ __global__ void __launch_bounds__(kAttnThreads) attention_kernel(const __grid_co
 #pragma unroll
         for (int q = 0; q < kCount; ++q)
             mx = fmaxf(mx, qm[q]);
+        const float m0 = mx == -INFINITY ? 0.0f : mx;
         L = 0.0f;
         O = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
 #pragma unroll
         for (int q = 0; q < kCount; ++q) {
-            if (qm[q] != -INFINITY) {  // a partial without keys adds nothing
-                const float w = exp2_fast(qm[q] - mx);
-                L = fmaf(ql[q], w, L);
-                O.x = fmaf(qo[q].x, w, O.x);
-                O.y = fmaf(qo[q].y, w, O.y);
-                O.z = fmaf(qo[q].z, w, O.z);
-                O.w = fmaf(qo[q].w, w, O.w);
-            }
+            // a partial without a finite score has weight 0: its sums are 0 without keys (or with
+            // scores of -inf alone), and NaN with a score of NaN, which has to show
+            const float w = exp2_fast(qm[q] - m0);
+            L = fmaf(ql[q], w, L);
+            O.x = fmaf(qo[q].x, w, O.x);
+            O.y = fmaf(qo[q].y, w, O.y);
+            O.z = fmaf(qo[q].z, w, O.z);
+            O.w = fmaf(qo[q].w, w, O.w);
         }
     };
     if constexpr (WK > 1) {

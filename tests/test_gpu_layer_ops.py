@@ -287,3 +287,36 @@ def test_rmsnorm_thread_counts(cuda_device, M, D):
     torch.cuda.synchronize()
     ref, bound = oracle.rmsnorm_reference(x, g, 1e-6)
     _check(_vals(y), ref, bound, f"rmsnorm M={M} D={D}")
+
+
+# (M, H, Hk, d, n, first and end of the keys that are not finite): keys shared out to the warps, one
+# tile (a warp's share of it; one key; all) and eight splits (a whole split); rows shared out, one split
+# (one tile, one key) and two (a whole split); every key
+ATTN_NOT_FINITE = [(1, 1, 1, 64, 64, 48, 64), (1, 1, 1, 128, 33, 32, 33), (16, 2, 2, 128, 64, 0, 16),
+                   (3, 4, 2, 64, 40, 0, 40), (1, 32, 32, 128, 281, 0, 35), (1, 8, 1, 128, 4001, 250, 501),
+                   (300, 8, 8, 64, 300, 64, 128), (300, 8, 8, 64, 300, 299, 300), (816, 8, 1, 128, 700, 0, 350),
+                   (816, 8, 1, 128, 700, 350, 700), (300, 8, 8, 64, 300, 0, 300)]
+
+
+@pytest.mark.parametrize("M,H,Hk,d,n,lo,hi", ATTN_NOT_FINITE)
+def test_attention_keys_that_are_not_finite(cuda_device, M, H, Hk, d, n, lo, hi):
+    """Keys lo .. hi - 1 of the last key/value head are NaN, give scores of +inf, or of -inf: the
+    softmax is NaN, NaN, and the one over the other keys. Other heads keep their bits."""
+    Qb, _, _, Kb, Vb = _attn_inputs(M, H, Hk, d, 0, n, M + H + n + lo)
+    Qb[:, ::d] = np.abs(Qb[:, ::d]) + 0.5  # the sign of the first product of a score is the key's
+    scale = 1.0 / math.sqrt(d)
+    none = np.zeros((0, Hk * d))
+    first = (H - H // Hk) * d  # output columns of the heads that read the last key/value head
+    clean = _run_attention(Qb, none, none, Kb, Vb, H, Hk, d, scale)
+    for bad in (np.nan, np.inf, -np.inf):
+        K = Kb.copy()
+        K[lo:hi, (Hk - 1) * d] = bad
+        O = _run_attention(Qb, none, none, K, Vb, H, Hk, d, scale)
+        assert torch.equal(O[:, :first].view(torch.int16), clean[:, :first].view(torch.int16)), bad
+        got = _vals(O)[:, first:]
+        if bad != -np.inf or hi - lo == n:
+            assert np.isnan(got).all(), f"{bad}: {int((~np.isnan(got)).sum())} of {got.size} not NaN"
+        else:
+            keep = np.r_[0:lo, hi:n]
+            ref, bound = oracle.attention_reference(Qb, none, none, Kb[keep], Vb[keep], H, Hk, d, scale)
+            _check(got, ref[:, first:], bound[:, first:], "keys of score -inf")
