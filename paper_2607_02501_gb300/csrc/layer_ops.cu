@@ -112,9 +112,10 @@ __global__ void __launch_bounds__(NT) rmsnorm_kernel(const float* x, const float
 // of one token, with one load and store of VEC bf16 for either half. The host
 // passes each pair's inverse frequency base^(-2i/d), computed in fp64, as two floats
 // (hi + lo). The angle p * (hi + lo) is formed as an unevaluated sum A + a with one exact
-// FMA residual (p < 2^24 is exact in fp32), its sine and cosine as sincosf(A) corrected to
-// first order in a: error ~1e-7 at the positions of a prefix plus action chunk, against
-// ~|angle| * 2^-24 for a plain fp32 angle. The frequencies go through shared memory (filled before
+// FMA residual (p < 2^24 is exact in fp32), its sine and cosine as sincosf(A) corrected by a: error
+// ~1e-7 at every position, against ~|angle| * 2^-24 for a plain fp32 angle. To first order while the
+// largest angle stays below 4096 (|a| < 2^-12 + 2^-13, so a^2 / 2 < 7e-8); beyond it (LARGE) a grows
+// to a radian and more and takes its own sine and cosine. The frequencies go through shared memory (filled before
 // the dependency wait): read from the parameter bank, where a warp's 32 different entries take 32
 // turns, and with one pair, a 64-bit division and 2-byte accesses per thread, 816 tokens x 9 heads of
 // 256 took 16.8 us; now 4.3 (15 MB moved), 50 tokens x 9 heads of 128 2.4 -> 1.4 us.
@@ -133,7 +134,7 @@ struct alignas(2 * VEC) BfVec {
     __nv_bfloat16 v[VEC];
 };
 
-template <int VEC>
+template <int VEC, bool LARGE>
 __global__ void __launch_bounds__(256) rope_kernel(const __grid_constant__ RopeParams p) {
     __shared__ float inv_hi[kRopeMaxPairs], inv_lo[kRopeMaxPairs];
     const int half = p.head_dim / 2;
@@ -172,7 +173,19 @@ __global__ void __launch_bounds__(256) rope_kernel(const __grid_constant__ RopeP
             const float a = __fadd_rn(fmaf(pos, hi, -A), __fmul_rn(pos, inv_lo[i + e]));
             float sA, cA;
             sincosf(A, &sA, &cA);
-            const float c = fmaf(-a, sA, cA), s = fmaf(a, cA, sA);
+            float c, s;
+            if constexpr (LARGE) {
+                // sine and cosine of a by their series (error below 1e-10 up to 1/16), then the addition formulas
+                const float a2 = __fmul_rn(a, a);
+                float sa = __fmul_rn(a, fmaf(a2, fmaf(a2, 1.0f / 120.0f, -1.0f / 6.0f), 1.0f));
+                float ca = fmaf(a2, fmaf(a2, 1.0f / 24.0f, -0.5f), 1.0f);
+                if (fabsf(a) > 0.0625f) sincosf(a, &sa, &ca);
+                c = fmaf(cA, ca, -__fmul_rn(sA, sa));
+                s = fmaf(sA, ca, __fmul_rn(cA, sa));
+            } else {
+                c = fmaf(-a, sA, cA);
+                s = fmaf(a, cA, sA);
+            }
             const float xa = __bfloat162float(va.v[e]), xb = __bfloat162float(vb.v[e]);
             oa.v[e] = __float2bfloat16_rn(__fsub_rn(__fmul_rn(xa, c), __fmul_rn(xb, s)));
             ob.v[e] = __float2bfloat16_rn(__fadd_rn(__fmul_rn(xb, c), __fmul_rn(xa, s)));
@@ -180,6 +193,14 @@ __global__ void __launch_bounds__(256) rope_kernel(const __grid_constant__ RopeP
         *reinterpret_cast<BfVec<VEC>*>(xp) = oa;
         *reinterpret_cast<BfVec<VEC>*>(xp + half) = ob;
     }
+}
+
+template <bool LARGE>
+const void* rope_fn(int vec) {
+    return vec == 8   ? reinterpret_cast<const void*>(rope_kernel<8, LARGE>)
+           : vec == 4 ? reinterpret_cast<const void*>(rope_kernel<4, LARGE>)
+           : vec == 2 ? reinterpret_cast<const void*>(rope_kernel<2, LARGE>)
+                      : reinterpret_cast<const void*>(rope_kernel<1, LARGE>);
 }
 
 // ------------------------------------------------------------------ attention
@@ -710,12 +731,10 @@ cudaError_t launch_rope(uint16_t* x, int64_t n_heads, uint16_t* x2, int64_t n_he
     while (vec > 1 && pairs / vec < int64_t(152) * 256) vec /= 2;
     p.units = pairs / vec;
     const int64_t blocks = std::min<int64_t>((p.units + 255) / 256, 152 * 8);
+    // (the frequencies rise or fall with i, as the base is below or above one)
+    const bool large = double(pos0 + M) * std::max(p.inv_hi[0], p.inv_hi[half_d - 1]) >= 4096.0;
     void* args[] = {&p};
-    const void* fn = vec == 8   ? reinterpret_cast<const void*>(rope_kernel<8>)
-                     : vec == 4 ? reinterpret_cast<const void*>(rope_kernel<4>)
-                     : vec == 2 ? reinterpret_cast<const void*>(rope_kernel<2>)
-                                : reinterpret_cast<const void*>(rope_kernel<1>);
-    return launch_pdl(fn, dim3(unsigned(blocks)), dim3(256), 0, s, args);
+    return launch_pdl(large ? rope_fn<true>(vec) : rope_fn<false>(vec), dim3(unsigned(blocks)), dim3(256), 0, s, args);
 }
 
 cudaError_t launch_attention(const uint16_t* Q, const uint16_t* K0, const uint16_t* V0, int64_t n0,

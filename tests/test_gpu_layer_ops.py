@@ -320,3 +320,19 @@ def test_attention_keys_that_are_not_finite(cuda_device, M, H, Hk, d, n, lo, hi)
             keep = np.r_[0:lo, hi:n]
             ref, bound = oracle.attention_reference(Qb, none, none, Kb[keep], Vb[keep], H, Hk, d, scale)
             _check(got, ref[:, first:], bound[:, first:], "keys of score -inf")
+
+
+# the last position of first-order correction and the first beyond it; then ever larger angles
+@pytest.mark.parametrize("M,H,d,pos0,base", [(95, 3, 64, 4000, 1e4), (97, 3, 64, 4000, 1e4), (9, 3, 64, 100000, 1e4),
+                                             (700, 4, 256, 1 << 20, 1e4), (5, 2, 128, 16000000, 1e4),
+                                             (9, 3, 72, (1 << 24) - 9, 5e5), (4, 2, 6, (1 << 24) - 4, 0.5)])
+def test_rope_large_positions(cuda_device, M, H, d, pos0, base):
+    """The angle's residual beyond its fp32 value reaches a radian at the largest: cosine and
+    sine stay within the oracle's 2^-21, which shows where a rotated element is near zero."""
+    rng = np.random.default_rng(pos0 + d)
+    xb = oracle.bf16_round(rng.standard_normal((M, H * d)))
+    x = _bf16_dev(xb)
+    emb.emb_rope(x, H, d, pos0, base)
+    torch.cuda.synchronize()
+    ref, bound = oracle.rope_reference(xb, H, d, pos0, base)
+    _check(_vals(x), ref, bound, f"rope M={M} H={H} d={d} pos0={pos0} base={base}")
