@@ -1,5 +1,8 @@
 """Helpers shared by the GPU parity tests: feed one seeded input to both the CUDA
-path (through the C ABI) and the CPU oracle, and compare."""
+path (through the C ABI) and the CPU oracle, and compare; and read which kernels a call launches."""
+import ctypes
+import re
+
 import numpy as np
 import torch
 
@@ -51,6 +54,58 @@ def run_case(fmt: int, M: int, N: int, K: int, seed: int):
     ref_img = oracle.quantize(fmt, W)
     Yref, B = oracle.qmatmul(fmt, ref_img, Xb, N, K)
     return Y.cpu().numpy(), Yref, B, img, ref_img
+
+
+class _KernelNode(ctypes.Structure):
+    """CUDA_KERNEL_NODE_PARAMS (second version) of the driver API."""
+    _fields_ = [("func", ctypes.c_void_p), ("grid", ctypes.c_uint * 3), ("block", ctypes.c_uint * 3),
+                ("smem", ctypes.c_uint), ("params", ctypes.c_void_p), ("extra", ctypes.c_void_p),
+                ("kern", ctypes.c_void_p), ("ctx", ctypes.c_void_p)]
+
+
+def launches(call):
+    """(kernel, template arguments, grid) of every kernel that `call()` enqueues on the current
+    stream, in order of capture: the call is captured into a graph that never runs."""
+    cu = ctypes.CDLL("libcuda.so.1")
+
+    def ok(status):
+        assert status == 0, f"driver call failed: {status}"
+
+    stream, graph, count = torch.cuda.Stream(), ctypes.c_void_p(), ctypes.c_size_t(0)
+    with torch.cuda.stream(stream):
+        handle = ctypes.c_void_p(stream.cuda_stream)
+        ok(cu.cuStreamBeginCapture_v2(handle, 1))  # thread-local mode
+        try:
+            call()
+        finally:
+            ok(cu.cuStreamEndCapture(handle, ctypes.byref(graph)))
+    out = []
+    try:
+        ok(cu.cuGraphGetNodes(graph, None, ctypes.byref(count)))
+        nodes = (ctypes.c_void_p * count.value)()
+        ok(cu.cuGraphGetNodes(graph, nodes, ctypes.byref(count)))
+        for node in nodes:
+            p, name = _KernelNode(), ctypes.c_char_p()
+            ok(cu.cuGraphKernelNodeGetParams_v2(ctypes.c_void_p(node), ctypes.byref(p)))
+            if p.func:
+                ok(cu.cuFuncGetName(ctypes.byref(name), ctypes.c_void_p(p.func)))
+            else:
+                ok(cu.cuKernelGetName(ctypes.byref(name), ctypes.c_void_p(p.kern)))
+            m = re.search(r"\d([a-z_]+_kernel)(?:I((?:L[a-z]\d+E)+)E)?", name.value.decode())
+            args = re.findall(r"L[a-z](\d+)E", m.group(2) or "")
+            out.append((m.group(1), tuple(int(a) for a in args), tuple(p.grid)))
+    finally:
+        ok(cu.cuGraphDestroy(graph))
+    return out
+
+
+def route(fmt: int, M: int, N: int, K: int, epilogue: int = 0):
+    """The one launch of a layer of this size: (kernel, template arguments, grid)."""
+    img, X = emb.empty_qweight(fmt, N, K), torch.empty(M, K, dtype=torch.bfloat16, device="cuda")
+    Y = torch.empty(M, N, device="cuda")
+    got = launches(lambda: emb.emb_qlayer_seq([(fmt, img, N, K, X, Y, epilogue)], M))
+    assert len(got) == 1
+    return got[0]
 
 
 def layout_rows(fmt: int, img: torch.Tensor, N: int, K: int, rows) -> np.ndarray:

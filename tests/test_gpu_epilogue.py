@@ -1,6 +1,6 @@
 """Fused epilogues of layer chains against the oracle: bf16 output, in-place residual add,
-GeGLU / SwiGLU of interleaved gate/up rows, on every kernel path (register and staged
-GEMV, Q4_0 tensor-core GEMV, tcgen05 GEMM with one or two token tiles per CTA, split K
+GeGLU / SwiGLU of interleaved gate/up rows, on every kernel path (register, staged, ring and
+tensor-core GEMV, chunk GEMM, tcgen05 GEMM with one or two token tiles per CTA, split K
 and the split operand), and a chain whose layers feed each other (gated bf16 output into
 the down projection, residual add)."""
 import numpy as np
@@ -51,13 +51,13 @@ def run_epilogue(fmt, kind, M, N, K, seed):
     return Y
 
 
-# (fmt, M, N, K): register GEMV, staged GEMV (>= 12 MB), register GEMV at M = 4, Q4_0
-# tensor-core GEMV (M = 2..8, >= 12 MB), GEMM split operand (K < 1024), GEMM split K,
-# GEMM one token tile per CTA, GEMM two token tiles per CTA, Q6_0 GEMV and GEMM, Q8_0
+# (fmt, M, N, K): register GEMV, staged GEMV (>= 12 MB), tensor-core GEMV at M = 4 (small and
+# large), GEMM split operand (K < 1024), chunk GEMM, GEMM split K,
+# GEMM two token tiles per CTA, Q6_0 register GEMV and chunk GEMM, Q8_0
 # register GEMV loading whole row shares before the wait (long rows, two rows per CTA), Q4_0
-# staged GEMV at M = 1 with a ragged last tile, GEMM with persistent CTAs (320 tiles), the
-# ring GEMV (long rows, >= 12 MB, M = 1; the second and third with a ragged last CTA, the
-# third with the Q6_0 high plane)
+# staged GEMV at M = 1 with a ragged last tile, GEMM with persistent CTAs (320 tiles), long rows
+# at M = 1: the ring GEMV, the tensor-core GEMV with a ragged last tile, the ring GEMV with a ragged
+# last CTA and the Q6_0 high plane
 PATHS = [(Q8, 1, 256, 1024), (Q8, 1, 24576, 2048), (Q4, 4, 600, 2080), (Q4, 4, 32768, 1024),
          (Q8, 64, 384, 320), (Q8, 50, 1000, 1024), (Q4, 136, 640, 2048), (Q8, 280, 11008, 1024),
          (Q6, 1, 4096, 2048), (Q6, 50, 512, 2048), (Q8, 1, 1300, 7168), (Q4, 1, 16392, 2048),
@@ -67,14 +67,12 @@ PATHS = [(Q8, 1, 256, 1024), (Q8, 1, 24576, 2048), (Q4, 4, 600, 2080), (Q4, 4, 3
 @pytest.mark.parametrize("kind", KINDS)
 @pytest.mark.parametrize("fmt,M,N,K", PATHS)
 def test_epilogue_parity(cuda_device, fmt, M, N, K, kind):
-    if kind >= emb.EMB_EPI_GEGLU and fmt == Q4 and M == 4 and N == 32768:
-        pytest.skip("gated layers do not take the Q4_0 tensor-core GEMV (pairs rows elsewhere)")
     run_epilogue(fmt, kind, M, N, K, seed=M * 3 + N + K + 17 * kind)
 
 
 @pytest.mark.parametrize("kind", [emb.EMB_EPI_GEGLU, emb.EMB_EPI_SWIGLU])
 def test_gated_q4_tensor_core_shape_still_correct(cuda_device, kind):
-    """A gated Q4_0 layer at the tensor-core GEMV's shape runs on the FFMA2 kernels."""
+    """A gated layer on the tensor-core GEMV: gate and up rows meet in its shared-memory sums."""
     run_epilogue(Q4, kind, 4, 32768, 1024, seed=5 + kind)
 
 

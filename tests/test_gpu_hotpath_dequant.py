@@ -2,16 +2,16 @@
 oracle value by value.
 
 emb_dequantize_f32/bf16 run a separate export kernel; the GEMV and GEMM kernels each
-dequantise in their own way (byte-permute magic numbers and FFMA2 in the GEMV, LOP3 nibble
-to bf16 conversion in the Q4_0 mma.sync GEMV, an FFMA2 on a byte-permuted 2^15 + code and
-a bf16 pack in the tcgen05 GEMM). Here they are observed directly through emb_qmatmul: an
+dequantise in their own way (byte-permute magic numbers and FFMA2 in the one-token GEMVs, exact
+bf16 codes in the tensor-core GEMV, an FFMA2 on a byte-permuted 2^15 + code and
+a bf16 pack in the chunk and tcgen05 GEMMs). Here they are observed directly through emb_qmatmul: an
 activation row that is the unit vector e_k turns output m into column k of the dequantised
 matrix, because every product but one is zero and the one left is w' * 1.
 
   * GEMV (M <= 4): the products are exact in fp32 and every sum adds zeros to one term,
     so Y[m][n] must equal the oracle's w'[n][k_m] (Table 3's 8-, 6- and 4-bit weights as
     dequantised by the oracle: w' = d*q, d*(q-32), d*(q-8), exact in fp32).
-  * tcgen05 GEMM at K >= 1024: the MMA operand is bf16(w'), one round-to-nearest-even of
+  * chunk GEMM, and tcgen05 GEMM at K >= 1024: the MMA operand is bf16(w'), one round-to-nearest-even of
     the exact w', so Y[m][n] must equal the oracle's bf16 dequantisation widened to fp32.
   * tcgen05 GEMM at K < 1024: the kernel adds a second operand lo = bf16(w' - bf16(w'))
     (see the kernel's precision note), so Y must equal hi + lo, which is exact in fp32
@@ -32,6 +32,7 @@ import torch
 
 import oracle
 import paper_2607_02501_gb300 as emb
+from tests.gpu_util import route
 
 ONE_BF16 = 0x3F80
 
@@ -160,46 +161,53 @@ def _spread_k(K: int, count: int, seed: int):
 
 
 # ---------------------------------------------------------------- GEMV (M <= 4)
-# (fmt, N, K, M, which kernel the shape routes to, k positions)
+# (fmt, N, K, M, which kernel the shape routes to, k positions); the label's first word is checked
+GEMV_KERNELS = {"register": "gemv_kernel", "staged": "gemv_staged_kernel", "ring": "gemv_ring_kernel",
+                "tensor-core": "gemv_tc_kernel"}
 GEMV_CASES = [
-    # register kernel, one row per CTA (small layer), every k; M = 1, 2 (two tokens per
-    # CTA), 3 and 4 (four-token tiles)
+    # register kernel, one row per CTA (small layer), every k; M = 1 and 2 (two tokens per CTA);
+    # more tokens take the tensor-core kernel
     (emb.EMB_Q8_0, 256, 2048, 1, "register R=1", "all"),
     (emb.EMB_Q8_0, 256, 2048, 2, "register R=1 MT=2", "all"),
-    (emb.EMB_Q8_0, 256, 2048, 3, "register R=1 MT=4", "all"),
+    (emb.EMB_Q8_0, 256, 2048, 3, "tensor-core, few row tiles", "all"),
     (emb.EMB_Q4_0, 256, 2048, 1, "register R=1", "all"),
-    (emb.EMB_Q4_0, 256, 2048, 4, "register R=1 MT=4", "all"),
+    (emb.EMB_Q4_0, 256, 2048, 4, "tensor-core, few row tiles", "all"),
     (emb.EMB_Q6_0, 256, 2048, 1, "register R=1", "all"),
-    (emb.EMB_Q6_0, 256, 2048, 4, "register R=1 MT=4", "all"),
-    # Q6_0 with K % 64 != 0 (no staged or tensor-map path)
+    (emb.EMB_Q6_0, 256, 2048, 4, "tensor-core, few row tiles", "all"),
+    # Q6_0 with K % 64 != 0 (the register kernel at every M <= 4)
     (emb.EMB_Q6_0, 256, 1056, 2, "register R=1", "all"),
     # four rows per CTA (2048 rows, 16-byte units per row < 320)
     (emb.EMB_Q4_0, 2048, 2048, 1, "register R=4", "all"),
-    (emb.EMB_Q8_0, 2048, 2048, 2, "register R=4 MT=2", "all"),
+    (emb.EMB_Q8_0, 2048, 2048, 2, "tensor-core", "all"),
     # long Q8_0 rows below 12 MB: a thread's whole row share loaded before the wait (PF = 4)
     (emb.EMB_Q8_0, 256, 16384, 1, "register PF=4 R=1", "spread"),
     (emb.EMB_Q6_0, 1024, 8192, 1, "register R=2 long rows (< 12 MB)", "spread"),
     (emb.EMB_Q6_0, 2048, 16384, 1, "ring, Q6_0 high plane in the stage", "spread"),
-    # ring kernel (rows > 6 KB, >= 12 MB, M = 1: X in registers, rows through a shared-memory
-    # ring): the Gemma-2B down projection shape, 2..4 units per thread, ragged last CTAs
+    # ring kernel (Q8_0 and Q6_0 rows > 6 KB, >= 12 MB, M = 1: X in registers, rows through a shared-memory
+    # ring): the Gemma-2B down projection shape, 2..4 units per thread, ragged last CTA
     (emb.EMB_Q8_0, 2048, 16384, 1, "ring PF=4", "spread"),
     (emb.EMB_Q8_0, 2048, 8192, 1, "ring PF=2", "spread"),
     (emb.EMB_Q8_0, 1027, 12288, 1, "ring PF=3, ragged last CTA", "spread"),
-    (emb.EMB_Q4_0, 2048, 16384, 1, "ring PF=2", "spread"),
-    (emb.EMB_Q4_0, 1024, 24576, 1, "ring PF=3", "spread"),
-    (emb.EMB_Q4_0, 1538, 16384, 1, "ring, ragged last CTA", "spread"),
-    (emb.EMB_Q4_0, 1539, 16384, 1, "ring, ragged last CTA", "spread"),
-    # staged kernel: >= 12 MB of codes with rows <= 6 KB at M = 1; any rows at M = 2..4
+    # tensor-core kernel at M = 1: long Q4_0 and Q6_0 rows (sixteen warps, ragged last row tiles; eight
+    # warps; both with compensated totals where a warp adds up more chunks)
+    (emb.EMB_Q4_0, 2048, 16384, 1, "tensor-core, long rows", "spread"),
+    (emb.EMB_Q4_0, 1024, 24576, 1, "tensor-core, long rows", "spread"),
+    (emb.EMB_Q4_0, 1538, 16384, 1, "tensor-core, ragged last tile", "spread"),
+    (emb.EMB_Q4_0, 1539, 16384, 1, "tensor-core, ragged last tile", "spread"),
+    (emb.EMB_Q4_0, 4096, 12288, 1, "tensor-core, eight warps", "spread"),
+    (emb.EMB_Q6_0, 4100, 4096, 1, "tensor-core, ragged last tile", "spread"),
+    (emb.EMB_Q6_0, 4096, 11008, 1, "tensor-core, eight warps", "spread"),
+    # staged kernel: >= 12 MB of codes with rows <= 6 KB at M = 1
     (emb.EMB_Q8_0, 6144, 2048, 1, "staged", "all"),
-    (emb.EMB_Q8_0, 6144, 2048, 4, "staged MT=4", "all"),
+    (emb.EMB_Q8_0, 6144, 2048, 4, "tensor-core", "all"),
     (emb.EMB_Q4_0, 12288, 2048, 1, "staged", "all"),
-    (emb.EMB_Q4_0, 4096, 12288, 1, "staged, 6 KB rows", "spread"),
+    (emb.EMB_Q4_0, 2560, 12288, 1, "staged, 6 KB rows", "spread"),
     (emb.EMB_Q6_0, 8192, 2048, 1, "staged", "all"),
-    (emb.EMB_Q6_0, 8192, 2048, 2, "staged MT=2", "all"),
-    # Q4_0 mma.sync kernel: >= 12 MB, rows <= 2 KB, M = 2..4
-    (emb.EMB_Q4_0, 12288, 2048, 2, "q4 mma.sync", "all"),
-    (emb.EMB_Q4_0, 12288, 2048, 3, "q4 mma.sync", "all"),
-    (emb.EMB_Q4_0, 12288, 4096, 4, "q4 mma.sync", "spread"),
+    (emb.EMB_Q6_0, 8192, 2048, 2, "tensor-core", "all"),
+    # large layers at M = 2..4
+    (emb.EMB_Q4_0, 12288, 2048, 2, "tensor-core", "all"),
+    (emb.EMB_Q4_0, 12288, 2048, 3, "tensor-core", "all"),
+    (emb.EMB_Q4_0, 12288, 4096, 4, "tensor-core", "spread"),
 ]
 
 
@@ -208,6 +216,7 @@ GEMV_CASES = [
                          ids=[f"{emb_fmt}-{N}x{K}-M{M}-{path.replace(' ', '_')}"
                               for emb_fmt, N, K, M, path, _ in GEMV_CASES])
 def test_gemv_dequant_exact(cuda_device, fmt, N, K, M, path, which):
+    assert route(fmt, M, N, K)[0] == GEMV_KERNELS[path.replace(",", "").split()[0]]
     img = crafted_image(fmt, N, K, seed=N + K + fmt)
     ks = _all_k(K) if which == "all" else _spread_k(K, 256, seed=K + M)
     Y = run_onehot(fmt, torch.from_numpy(img).cuda(), N, K, M, ks)
@@ -216,7 +225,7 @@ def test_gemv_dequant_exact(cuda_device, fmt, N, K, M, path, which):
 
 
 # ---------------------------------------------------------------- GEMM (M > 4)
-# (fmt, N, K, M, which kernel variant the shape takes, k positions)
+# (fmt, N, K, M, which kernel variant the shape takes, k positions); the variant is checked
 GEMM_CASES = [
     # X = the identity (M = K): Y is the whole dequantised matrix, transposed
     (emb.EMB_Q8_0, 384, 1024, 1024, "identity, bf16 operand", "identity"),
@@ -225,15 +234,19 @@ GEMM_CASES = [
     (emb.EMB_Q8_0, 256, 512, 512, "identity, hi + lo operand", "identity"),
     (emb.EMB_Q4_0, 256, 512, 512, "identity, hi + lo operand", "identity"),
     (emb.EMB_Q6_0, 256, 512, 512, "identity, hi + lo operand", "identity"),
-    # the action chunk (50 tokens): one tile per CTA, K split over a cluster
-    (emb.EMB_Q8_0, 1024, 4096, 50, "M=50 split-K cluster", "spread"),
-    (emb.EMB_Q6_0, 1024, 4096, 50, "M=50 split-K cluster", "spread"),
+    # the action chunk (50 tokens): the mma.sync chunk kernel (its last call, of five tokens, the GEMM)
+    (emb.EMB_Q8_0, 1024, 4096, 50, "M=50 chunk kernel", "spread"),
+    (emb.EMB_Q6_0, 1024, 4096, 50, "M=50 chunk kernel", "spread"),
+    # few tiles of long rows: K split over a cluster of eight
+    (emb.EMB_Q8_0, 256, 4096, 128, "M=128 split-K cluster", "spread"),
+    (emb.EMB_Q4_0, 1000, 4096, 128, "M=128 split-K cluster", "spread"),
+    (emb.EMB_Q6_0, 384, 8192, 110, "M=110 split-K cluster", "spread"),
     (emb.EMB_Q4_0, 256, 640, 50, "M=50 hi + lo operand", "spread"),
     # prefill: two token tiles per CTA sharing each A tile (Llama-style q/k/v at M = 280)
     (emb.EMB_Q4_0, 12288, 4096, 280, "M=280 two token tiles per CTA", "spread"),
-    # prefill: one 208-token tile per CTA (M = 816)
-    (emb.EMB_Q8_0, 2048, 2048, 816, "M=816 one tile per CTA", "spread"),
-    (emb.EMB_Q6_0, 2048, 2048, 816, "M=816 one tile per CTA", "spread"),
+    # prefill: 208-token tiles (M = 816), K split over two CTAs
+    (emb.EMB_Q8_0, 2048, 2048, 816, "M=816 split-K cluster", "spread"),
+    (emb.EMB_Q6_0, 2048, 2048, 816, "M=816 split-K cluster", "spread"),
     # prefill with more tiles than SMs: persistent CTAs looping over (weight, token) tiles
     (emb.EMB_Q8_0, 10240, 1024, 816, "M=816 persistent CTAs", "spread"),
     (emb.EMB_Q4_0, 10240, 1024, 816, "M=816 persistent CTAs", "spread"),
@@ -244,6 +257,13 @@ GEMM_CASES = [
 @pytest.mark.parametrize("fmt,N,K,M,path,which", GEMM_CASES,
                          ids=[f"{emb_fmt}-{N}x{K}-M{M}" for emb_fmt, N, K, M, _, _ in GEMM_CASES])
 def test_gemm_dequant_exact(cuda_device, fmt, N, K, M, path, which):
+    kernel, args, grid = route(fmt, M, N, K)
+    assert kernel == ("gemm_chunk_kernel" if "chunk" in path else "gemm_tc_kernel")
+    if kernel == "gemm_tc_kernel":  # template arguments: format, two-operand form, token tiles, stream-K
+        assert args == (fmt, int("hi + lo" in path), 2 if "two token tiles" in path else args[2], 0)
+        assert (grid[2] > 1) == ("split-K" in path) or "operand" in path
+        sms = torch.cuda.get_device_properties(0).multi_processor_count
+        assert (grid == (sms, 1, 1)) == ("persistent" in path)
     img = crafted_image(fmt, N, K, seed=3 * N + K + fmt)
     ks = _all_k(K) if which == "identity" else _spread_k(K, 2 * M, seed=K + M)
     Y = run_onehot(fmt, torch.from_numpy(img).cuda(), N, K, M, ks)

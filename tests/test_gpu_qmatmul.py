@@ -1,12 +1,12 @@
-"""emb_qmatmul against the oracle: GEMV (M <= 4) and tcgen05 GEMM (M > 4) paths on
-shapes spanning several tiles with ragged tails in every dimension."""
+"""emb_qmatmul against the oracle: GEMV (M <= 4 and most layers up to 16), chunk (M = 17..64)
+and tcgen05 GEMM paths on shapes spanning several tiles with ragged tails in every dimension."""
 import numpy as np
 import pytest
 import torch
 
 import oracle
 import paper_2607_02501_gb300 as emb
-from tests.gpu_util import check_close, run_case, to_dev_bf16
+from tests.gpu_util import check_close, route, run_case, to_dev_bf16
 from workloads import activation_bits_np, weight_np
 
 pytestmark = pytest.mark.gpu
@@ -100,9 +100,9 @@ def test_y_fully_overwritten(cuda_device):
             assert torch.equal(Y0, Y1)
 
 
-# Layers of at least 12 MB of packed weights take the staged (bulk-copy ring) GEMV: ragged
-# row counts (partial last tile and partial last run of tiles per CTA), K not a multiple of
-# the warps' K slices, M = 1..4 and the largest staged activation row (K = 16384 at M = 1).
+# Layers of at least 12 MB of packed weights take the staged GEMV at M = 1 (long rows the ring or
+# tensor-core kernel, more tokens the tensor-core kernel): ragged row counts (partial last tile), K
+# not a multiple of the warps' K slices.
 STAGED_SHAPES = [(1, 24593, 1056), (2, 6151, 4128), (3, 6151, 4096), (4, 12301, 2048),
                  (1, 1543, 16384), (1, 12289, 2048), (2, 12289, 2048), (1, 6151, 4096)]
 
@@ -256,8 +256,8 @@ def test_precise_operand_flag_few_dominant_terms(cuda_device):
 
 # the tensor-core GEMV's edges: a single row, row tiles one short and one over, a 32-weight row, an
 # odd block count, a ragged last 256-k chunk, one and several chunks per warp, sixteen warps per CTA
-# (long rows, few tiles), several row tiles per CTA; one token (long rows only), eight, and both
-# ends of the sixteen-token variant
+# (long rows, few tiles), several row tiles per CTA; eight tokens, and both ends of the
+# sixteen-token variant (the one-token shapes take the other kernels: below are those that do not)
 TC_SHAPES = [(3, 1, 64), (3, 15, 32), (4, 17, 96), (6, 33, 352), (8, 300, 2048), (9, 16, 2080), (16, 31, 256),
              (13, 257, 4160), (1, 100, 4096), (1, 5000, 4128), (8, 70, 16384), (16, 2433, 5056), (7, 9000, 1088)]
 
@@ -297,10 +297,45 @@ def test_tensor_core_gemv_has_exact_products(cuda_device, fmt, M, N, K):
     assert emb.emb_device_status() == emb.EMB_OK
 
 
+# the tensor-core GEMV at one token (long rows of Q4_0 and Q6_0): sixteen warps and few rows, eight
+# warps in one round with ragged last tiles, several rounds; with compensated totals from K = 6208
+# (eight warps) and 16448 (sixteen) on
+TC_ONE_TOKEN = [(emb.EMB_Q4_0, 1000, 4128), (emb.EMB_Q6_0, 1000, 4160), (emb.EMB_Q4_0, 4096, 4096),
+                (emb.EMB_Q6_0, 4100, 4096), (emb.EMB_Q4_0, 4090, 11008), (emb.EMB_Q6_0, 4096, 11008),
+                (emb.EMB_Q4_0, 6144, 5120), (emb.EMB_Q6_0, 6144, 5120), (emb.EMB_Q4_0, 1100, 16448)]
+
+
+@pytest.mark.parametrize("fmt,N,K", TC_ONE_TOKEN)
+def test_tensor_core_gemv_at_one_token(cuda_device, fmt, N, K):
+    assert route(fmt, 1, N, K)[0] == "gemv_tc_kernel"
+    test_tensor_core_gemv_has_exact_products(cuda_device, fmt, 1, N, K)
+
+
+@pytest.mark.parametrize("fmt", FMTS + [emb.EMB_Q6_0])
+def test_shapes_take_the_kernels_they_are_named_for(cuda_device, fmt):
+    k64 = lambda K: K + 32 if fmt == emb.EMB_Q6_0 and K % 64 else K
+    for M, N, K in TC_SHAPES:
+        if M > 3:
+            assert route(fmt, M, N, k64(K))[0] == "gemv_tc_kernel", (M, N, K)
+    for M, N, K in CHUNK_SHAPES:
+        # not: few long rows (the GEMM's K splits), Q8_0 in rounds that are less than 70 % full
+        if (M, N, K) != (64, 130, 16384) and (fmt, M, N) != (emb.EMB_Q8_0, 24, 6000):
+            assert route(fmt, M, N, k64(K))[0] == "gemm_chunk_kernel", (M, N, K)
+    for M, N, K in SHORT_ROW_SHAPES:
+        assert route(fmt, M, N, k64(K))[0] == "gemm_tc_kernel", (M, N, K)
+    for N, K in LONG_ROW_SHAPES:
+        for M in (2, 4):
+            if M == 4 or N > 512:  # two tokens of up to 32 row tiles: the register kernel
+                assert route(fmt, M, N, K)[0] == "gemv_tc_kernel", (M, N, K)
+
+
 # the chunk kernel's edges: 17, 32, 33 and 64 tokens; one row tile, one short and one over, several
-# per CTA; K of four chunks exactly, with a ragged last one, odd block counts, long rows
+# per CTA; K of four chunks exactly, with a ragged last one, odd block counts
 CHUNK_SHAPES = [(17, 16, 1024), (32, 15, 2048), (33, 300, 1056), (50, 1280, 1024), (64, 33, 4160), (50, 5000, 1280),
                 (24, 6000, 1120), (64, 130, 16384), (40, 2048, 2080)]
+# long rows: the longest of a layer of the workloads, a ragged last tile and chunk, one token group; and
+# rounds that are full enough for Q8_0 too
+CHUNK_MORE_SHAPES = [(50, 2048, 16384), (33, 1540, 8256), (20, 4000, 11008), (24, 7000, 1120)]
 
 
 @pytest.mark.parametrize("fmt", FMTS + [emb.EMB_Q6_0])
@@ -339,6 +374,15 @@ def test_chunk_gemm_is_the_bf16_operand_product(cuda_device, fmt, M, N, K):
         ref, b = oracle.epilogue_reference(oracle.EPI_GEGLU, Yref, bound)
         assert (np.abs(G.float().cpu().numpy().astype(np.float64) - ref) <= b).all()
     assert emb.emb_device_status() == emb.EMB_OK
+
+
+@pytest.mark.parametrize("fmt", FMTS + [emb.EMB_Q6_0])
+@pytest.mark.parametrize("M,N,K", CHUNK_MORE_SHAPES)
+def test_chunk_gemm_long_rows_and_rounds(cuda_device, fmt, M, N, K):
+    if fmt == emb.EMB_Q6_0 and K % 64:
+        K += 32
+    assert route(fmt, M, N, K)[0] == "gemm_chunk_kernel"
+    test_chunk_gemm_is_the_bf16_operand_product(cuda_device, fmt, M, N, K)
 
 
 # short rows whose launch leaves SMs idle take more token tiles of 96 and more tokens instead of a K
@@ -387,3 +431,11 @@ def test_long_row_gemv_error_does_not_grow_with_k(cuda_device, fmt, M, N, K):
         want = np.where(w[:, 7] == 0, np.nan, np.sign(w[:, 7]) * np.inf)
     assert np.array_equal(again[M - 1].cpu().numpy(), want.astype(np.float32), equal_nan=True)
     assert emb.emb_device_status() == emb.EMB_OK
+
+
+@pytest.mark.parametrize("fmt,N,K", [(emb.EMB_Q4_0, 4090, 11008), (emb.EMB_Q6_0, 4096, 11008), (emb.EMB_Q4_0, 4864, 14336),
+                                     (emb.EMB_Q4_0, 1100, 16448)])
+def test_long_row_gemv_error_at_one_token(cuda_device, fmt, N, K):
+    kernel, args, _ = route(fmt, 1, N, K)
+    assert kernel == "gemv_tc_kernel" and args[3] == 1  # compensated totals
+    test_long_row_gemv_error_does_not_grow_with_k(cuda_device, fmt, 1, N, K)

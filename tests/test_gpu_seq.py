@@ -54,9 +54,9 @@ def test_seq_equals_single_calls_and_oracle(cuda_device, fmt, M):
 
 @pytest.mark.parametrize("fmt", [emb.EMB_Q8_0, emb.EMB_Q4_0])
 def test_long_rows_group_across_matrices(cuda_device, fmt):
-    """Two long-row matrices sharing X at M = 1 form one launch of the ring kernel, whose
-    CTAs own runs of rows that cross from the first matrix into the second: bitwise the
-    separate calls, within the oracle's bound."""
+    """Two long-row matrices sharing X at M = 1 form one launch of the ring kernel (Q8_0), whose
+    CTAs own runs of rows that cross from the first matrix into the second, or of the tensor-core
+    kernel (Q4_0): bitwise the separate calls, within the oracle's bound."""
     K, Ns, M = 16384, (1000, 1030), 1
     Xb = activation_bits_np(M, K, 77)
     X = to_dev_bf16(Xb)
