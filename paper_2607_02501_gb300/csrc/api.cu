@@ -143,6 +143,17 @@ __global__ void selftest_wait_kernel(uint64_t timeout_ns, int* status) {
 
 }  // namespace
 
+int device_sm_count() {
+    static std::mutex mu;
+    static int counts[64] = {};
+    int dev = 0;
+    if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64) return 0;
+    std::lock_guard<std::mutex> lock(mu);
+    if (!counts[dev] && cudaDeviceGetAttribute(&counts[dev], cudaDevAttrMultiProcessorCount, dev) != cudaSuccess)
+        counts[dev] = 0;
+    return counts[dev];
+}
+
 cudaError_t launch_selftest_wait(uint64_t timeout_ns, int* status, cudaStream_t s) {
     selftest_wait_kernel<<<1, 32, 0, s>>>(timeout_ns, status);
     return cudaGetLastError();

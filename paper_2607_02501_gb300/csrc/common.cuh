@@ -133,6 +133,9 @@ struct GroupRef {
     size_t ws_bytes;
 };
 
+// SMs of the current device (asked once per device); 0 if it cannot be told.
+int device_sm_count();
+
 // Weight-streaming GEMV for small M (register dequant, shuffle reductions).
 // pdl: the kernel reads weights before griddepcontrol.wait (X only after it); otherwise it waits
 // before it reads anything. Both are launched with programmatic stream serialisation.

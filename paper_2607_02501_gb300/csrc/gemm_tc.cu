@@ -885,17 +885,6 @@ cudaError_t launch_kernel(const GemmParams& p, int grid_x, int grid_y, cudaStrea
     return cudaLaunchKernelEx(&cfg, gemm_tc_kernel<FMT, SPLIT, P, SK>, p);
 }
 
-int sm_count() {
-    static std::mutex mu;
-    static int counts[64] = {};
-    int dev = 0;
-    if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64) return 0;
-    std::lock_guard<std::mutex> lock(mu);
-    if (!counts[dev] && cudaDeviceGetAttribute(&counts[dev], cudaDevAttrMultiProcessorCount, dev) != cudaSuccess)
-        counts[dev] = 0;
-    return counts[dev];
-}
-
 // K splits (1, 2, 4 or 8: one cluster of CTAs per output tile, 8 being the portable
 // cluster size) of the two-operand form and of fewer than 65 tokens: the count minimising a simple
 // time model -- waves of 148 CTAs, each costing a fixed ~3 us plus its share of the tile's MMA work
@@ -949,13 +938,14 @@ double step_cycles(int P, int T) { return std::max(620.0, 2.22 * P * T + 150.0);
 double item_cycles(int P, int T) { return 6300.0 + 22.6 * P * T; }
 // One launch: waves of CTAs that each take an item's share of K. A K split adds its cluster's
 // exchange, ~3000 + 13 per token of the tile (four splits against none at 1000 x 1088 and 1152 x 1152, tiles of
-// 96, 128, 160 and 256 tokens). Twelve clusters of eight CTAs run at once, sixteen do not (512 x 16384: M = 600
-// in twelve 23.2 us, M = 512 in eight 22.3, in sixteen 35.4).
+// 96, 128, 160 and 256 tokens). Of clusters of eight CTAs, twelve run at once on 152 SMs, sixteen do not (512 x
+// 16384: M = 600 in twelve 23.2 us, M = 512 in eight 22.3, in sixteen 35.4).
 double plan_cycles(int64_t items, int P, int T, int splits, int64_t K, int sms) {
     const int64_t nr = (K + kKR - 1) / kKR, nk = (K + kKC - 1) / kKC;
     const double steps = double(std::min(nk, (nr + splits - 1) / splits * kStepsPerRaw));
     const double exchange = splits > 1 ? 3000.0 + 13.0 * T : 0.0;
-    const int64_t waves = splits == 8 ? (items + 11) / 12 : (items * splits + sms - 1) / sms;
+    const int64_t eights = std::max(1, sms * 12 / 152);
+    const int64_t waves = splits == 8 ? (items + eights - 1) / eights : (items * splits + sms - 1) / sms;
     return double(waves) * (steps * step_cycles(P, T) + item_cycles(P, T) + exchange);
 }
 
@@ -972,7 +962,7 @@ GemmPlan plan_gemm(const GroupRef& g, bool streamk_ok) {
     int S = g.fmt == EMB_Q8_0   ? (split ? pick_stages<EMB_Q8_0, true>(T) : pick_stages<EMB_Q8_0, false>(T))
             : g.fmt == EMB_Q4_0 ? (split ? pick_stages<EMB_Q4_0, true>(T) : pick_stages<EMB_Q4_0, false>(T))
                                 : (split ? pick_stages<EMB_Q6_0, true>(T) : pick_stages<EMB_Q6_0, false>(T));
-    const int sms = sm_count();
+    const int sms = device_sm_count();
     int splits = 1;
     double one_tile = 0.0;  // cycles of the plan with one token tile per CTA
     if (split || sms <= 0 || g.M <= 64) {

@@ -29,7 +29,6 @@
 // Up to kMaxGroup matrices that read the same X (q/k/v or gate/up) share one launch.
 #include <algorithm>
 #include <atomic>
-#include <mutex>
 
 #include "dequant_dot.cuh"
 #include "ptx.cuh"
@@ -37,7 +36,6 @@
 namespace emb {
 namespace {
 
-using dq::and_or;
 using dq::dot_q4_unit;
 using dq::dot_q6_unit;
 using dq::dot_q8_unit;
@@ -989,8 +987,6 @@ __global__ void __launch_bounds__(32 * NW, 16 / NW) gemv_tc_kernel(const __grid_
     }
 }
 
-int gemv_sm_count();
-
 template <int FMT, int NT, int NW, bool COMP = false>
 cudaError_t launch_tc_one(const TcParams& p, int grid, cudaStream_t s) {
     cudaLaunchConfig_t cfg = {};
@@ -1050,8 +1046,6 @@ TcParams tc_params(const GroupRef& g, bool pdl, int& n_tiles) {
     return p;
 }
 
-bool ring_takes(const GroupRef& g);
-
 // Which calls take it (us per launch in graph-replayed chains, this kernel / the one it leaves):
 //  * M = 3, 4 always (Q6_0 32768 x 2048 at M = 4 15.4 / 32.9, Q4_0 13.4 / 18.0, Q8_0 16.6 / 22.8;
 //    2048 x 16384 at M = 4 Q8_0 10.0 / 22.6, Q6_0 9.7 / 24.9, Q4_0 8.1 / 23.0); M = 2 but for what the
@@ -1105,7 +1099,7 @@ bool tc_takes(const GroupRef& g, int sms) {
 }
 
 bool launch_tc(const GroupRef& g, bool pdl, cudaStream_t s, cudaError_t& err) {
-    const int sms = gemv_sm_count();
+    const int sms = device_sm_count();
     if (sms <= 0 || !tc_takes(g, sms)) return false;
     int tiles = 0;
     const TcParams p = tc_params(g, pdl, tiles);
@@ -1547,17 +1541,6 @@ cudaError_t launch_ring_fmt(const RingParams& p, int pf, int ctas, size_t smem, 
                    : launch_ring_one<FMT, 4, false>(p, ctas, smem, s);
 }
 
-int gemv_sm_count() {
-    static std::mutex mu;
-    static int counts[64] = {};
-    int dev = 0;
-    if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64) return 0;
-    std::lock_guard<std::mutex> lock(mu);
-    if (!counts[dev] && cudaDeviceGetAttribute(&counts[dev], cudaDevAttrMultiProcessorCount, dev) != cudaSuccess)
-        counts[dev] = 0;
-    return counts[dev];
-}
-
 // Which layers take the ring path: M = 1, Q8_0 or Q6_0 (K % 64 == 0, for its high plane's 16-byte rows;
 // what of it tc_takes leaves), rows longer than the staged path takes at M = 1 and than one pass
 // of 256 threads (2..4 units per thread), matrices of at least kStageMinBytes; two CTAs per
@@ -1583,7 +1566,7 @@ bool launch_ring(const GroupRef& g, bool pdl, int* status, cudaStream_t s, cudaE
     const int64_t U = (g.fmt == EMB_Q8_0) ? g.K / 16 : g.K / 32;
     int64_t rows = 0;
     for (int i = 0; i < g.n_mats; ++i) rows += g.mats[i].N;
-    const int sms = gemv_sm_count();
+    const int sms = device_sm_count();
     if (sms <= 0) return false;
     RingParams p = {};
     int64_t r0 = 0;
@@ -1622,7 +1605,7 @@ bool launch_ring(const GroupRef& g, bool pdl, int* status, cudaStream_t s, cudaE
 }  // namespace
 
 bool launch_chunk(const GroupRef& g, bool pdl, cudaStream_t s, cudaError_t& err) {
-    const int sms = gemv_sm_count();
+    const int sms = device_sm_count();
     if (sms <= 0 || !chunk_takes(g, sms)) return false;
     int tiles = 0;
     const TcParams p = tc_params(g, pdl, tiles);
@@ -1633,7 +1616,7 @@ bool launch_chunk(const GroupRef& g, bool pdl, cudaStream_t s, cudaError_t& err)
 }
 
 bool gemv_takes(const GroupRef& g) {
-    const int sms = gemv_sm_count();
+    const int sms = device_sm_count();
     return sms > 0 && (tc_takes(g, sms) || chunk_takes(g, sms));
 }
 

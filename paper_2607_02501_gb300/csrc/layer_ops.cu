@@ -630,7 +630,8 @@ struct AttnPlan {
     int splits;
 };
 AttnPlan plan_attention(int64_t rows, int64_t Hk, int64_t n, int64_t D) {
-    const double sms = 152.0;
+    const int count = device_sm_count();
+    const double sms = count > 0 ? count : 152.0;
     const double per_sm = D == 64 ? 3.0 : 2.0;
     AttnPlan best{false, 1};
     double best_t = 1e30;
