@@ -885,6 +885,43 @@ cudaError_t launch_kernel(const GemmParams& p, int grid_x, int grid_y, cudaStrea
     return cudaLaunchKernelEx(&cfg, gemm_tc_kernel<FMT, SPLIT, P, SK>, p);
 }
 
+// Clusters of 2^i GEMM CTAs (one CTA per SM) that run at once, n[0] = SMs: fewer than SMs / 2^i, since
+// a cluster stays within a part of the chip (GB300, 152 SMs: 76, 36 and 15 of two, four and eight; a
+// 37th cluster of four doubles a launch, 19.4 -> 35.1 us, a 16th of eight too, 13.3 -> 23.5).
+struct Resident {
+    int n[4];
+};
+Resident resident_clusters() {
+    static std::mutex mu;
+    static Resident known[64] = {};
+    int dev = 0;
+    const int sms = device_sm_count();
+    Resident r = {{sms, sms / 2, sms / 4, sms / 8}};
+    if (sms <= 0 || cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64) return r;
+    std::lock_guard<std::mutex> lock(mu);
+    if (known[dev].n[0]) return known[dev];
+    auto* kernel = gemm_tc_kernel<EMB_Q8_0, false, 1, false>;
+    if (cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemLimit) != cudaSuccess) return r;
+    for (int i = 1; i < 4; ++i) {
+        cudaLaunchConfig_t cfg = {};
+        cfg.gridDim = dim3(1, 1, 1u << i);
+        cfg.blockDim = dim3(kThreads, 1, 1);
+        cfg.dynamicSmemBytes = kSmemLimit;
+        cudaLaunchAttribute attr;
+        attr.id = cudaLaunchAttributeClusterDimension;
+        attr.val.clusterDim.x = 1;
+        attr.val.clusterDim.y = 1;
+        attr.val.clusterDim.z = 1u << i;
+        cfg.attrs = &attr;
+        cfg.numAttrs = 1;
+        int n = 0;
+        if (cudaOccupancyMaxActiveClusters(&n, kernel, &cfg) != cudaSuccess || n < 1) return r;
+        r.n[i] = n;
+    }
+    known[dev] = r;
+    return r;
+}
+
 // K splits (1, 2, 4 or 8: one cluster of CTAs per output tile, 8 being the portable
 // cluster size) of the two-operand form and of fewer than 65 tokens: the count minimising a simple
 // time model -- waves of 148 CTAs, each costing a fixed ~3 us plus its share of the tile's MMA work
@@ -938,14 +975,13 @@ double step_cycles(int P, int T) { return std::max(620.0, 2.22 * P * T + 150.0);
 double item_cycles(int P, int T) { return 6300.0 + 22.6 * P * T; }
 // One launch: waves of CTAs that each take an item's share of K. A K split adds its cluster's
 // exchange, ~3000 + 13 per token of the tile (four splits against none at 1000 x 1088 and 1152 x 1152, tiles of
-// 96, 128, 160 and 256 tokens). Of clusters of eight CTAs, twelve run at once on 152 SMs, sixteen do not (512 x
-// 16384: M = 600 in twelve 23.2 us, M = 512 in eight 22.3, in sixteen 35.4).
-double plan_cycles(int64_t items, int P, int T, int splits, int64_t K, int sms) {
+// 96, 128, 160 and 256 tokens).
+double plan_cycles(int64_t items, int P, int T, int splits, int64_t K, const Resident& at_once) {
     const int64_t nr = (K + kKR - 1) / kKR, nk = (K + kKC - 1) / kKC;
     const double steps = double(std::min(nk, (nr + splits - 1) / splits * kStepsPerRaw));
     const double exchange = splits > 1 ? 3000.0 + 13.0 * T : 0.0;
-    const int64_t eights = std::max(1, sms * 12 / 152);
-    const int64_t waves = splits == 8 ? (items + eights - 1) / eights : (items * splits + sms - 1) / sms;
+    const int64_t clusters = std::max(1, at_once.n[splits == 8 ? 3 : splits / 2]);
+    const int64_t waves = (items + clusters - 1) / clusters;
     return double(waves) * (steps * step_cycles(P, T) + item_cycles(P, T) + exchange);
 }
 
@@ -962,12 +998,13 @@ GemmPlan plan_gemm(const GroupRef& g, bool streamk_ok) {
     int S = g.fmt == EMB_Q8_0   ? (split ? pick_stages<EMB_Q8_0, true>(T) : pick_stages<EMB_Q8_0, false>(T))
             : g.fmt == EMB_Q4_0 ? (split ? pick_stages<EMB_Q4_0, true>(T) : pick_stages<EMB_Q4_0, false>(T))
                                 : (split ? pick_stages<EMB_Q6_0, true>(T) : pick_stages<EMB_Q6_0, false>(T));
-    const int sms = device_sm_count();
+    const Resident at_once = resident_clusters();
+    const int sms = at_once.n[0];
     int splits = 1;
     double one_tile = 0.0;  // cycles of the plan with one token tile per CTA
     if (split || sms <= 0 || g.M <= 64) {
         splits = pick_splits(t_tiles * tiles, T, g.K, S, split);
-        one_tile = plan_cycles(t_tiles * tiles, 1, T, splits, g.K, std::max(sms, 1));
+        one_tile = plan_cycles(t_tiles * tiles, 1, T, splits, g.K, at_once);
     } else {
         // Token tiles and K splits together: a launch that leaves SMs idle may take smaller token
         // tiles, or a K split with its exchange, whichever the model says is at least 3 % faster than
@@ -986,7 +1023,7 @@ GemmPlan plan_gemm(const GroupRef& g, bool streamk_ok) {
                                                : pick_stages<EMB_Q6_0, false>(Tc);
             for (int sp = 1; sp <= 8 && sp <= nr; sp *= 2) {
                 if (sp > 1 && Sc < 4) break;  // the 512 T-byte partial tile lies in the X ring
-                const double c = plan_cycles(tt * tiles, 1, Tc, sp, g.K, sms);
+                const double c = plan_cycles(tt * tiles, 1, Tc, sp, g.K, at_once);
                 if (c < 0.97 * one_tile) {
                     one_tile = c;
                     t_tiles = tt;
@@ -1010,7 +1047,7 @@ GemmPlan plan_gemm(const GroupRef& g, bool streamk_ok) {
                        : (g.fmt == EMB_Q4_0) ? pick_stages_pair<EMB_Q4_0>(T2)
                                              : pick_stages_pair<EMB_Q6_0>(T2);
         if (S2 >= 2 && T2 <= 224 && sms > 0) {
-            const double c2 = plan_cycles(t2 / 2 * tiles, 2, T2, 1, g.K, sms);
+            const double c2 = plan_cycles(t2 / 2 * tiles, 2, T2, 1, g.K, at_once);
             if (c2 < 0.95 * one_tile) {
                 P = 2;
                 T = T2;
@@ -1053,7 +1090,7 @@ GemmPlan plan_gemm(const GroupRef& g, bool streamk_ok) {
     // items) 108 / 104, ViT q/k/v 19.6 / 11.1.
     if (streamk_ok && !split && g.M >= 128 && sms > 0) {
         const int64_t nr_all = (g.K + kKR - 1) / kKR;
-        const double cur = plan_cycles(pl.persist ? pl.n_items : int64_t(grid_x) * grid_y, P, T, splits, g.K, sms);
+        const double cur = plan_cycles(pl.persist ? pl.n_items : int64_t(grid_x) * grid_y, P, T, splits, g.K, at_once);
         struct Cand { int P, T, S; int64_t n_tt; };
         Cand cands[2];
         int nc = 0;

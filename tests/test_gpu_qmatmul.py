@@ -439,3 +439,17 @@ def test_long_row_gemv_error_at_one_token(cuda_device, fmt, N, K):
     kernel, args, _ = route(fmt, 1, N, K)
     assert kernel == "gemv_tc_kernel" and args[3] == 1  # compensated totals
     test_long_row_gemv_error_does_not_grow_with_k(cuda_device, fmt, 1, N, K)
+
+
+@pytest.mark.parametrize("fmt,M,N,K,splits", [(emb.EMB_Q4_0, 193, 2432, 8448, 4), (emb.EMB_Q4_0, 481, 2373, 6592, 4),
+                                              (emb.EMB_Q6_0, 151, 4864, 8960, 4), (emb.EMB_Q8_0, 287, 893, 12256, 8)])
+def test_k_splits_are_clusters_that_run_at_once(cuda_device, fmt, M, N, K, splits):
+    """A cluster stays within a part of the chip, so fewer than SMs / splits run at once: 36 of four
+    and 15 of eight on 152 SMs. Nineteen row tiles and two token tiles, or twice the row tiles, are no
+    wave of four splits; seven row tiles and two token tiles are one of eight."""
+    kernel, _, grid = route(fmt, M, N, K)
+    assert kernel == "gemm_tc_kernel"
+    if torch.cuda.get_device_properties(0).multi_processor_count == 152:
+        assert (grid[2] == 8) == (splits == 8) and grid[0] * grid[1] <= {8: 15, 4: 36, 2: 76, 1: 152}[grid[2]]
+    Y, Yref, B, _, _ = run_case(fmt, M, N, K, seed=M + N + K)
+    check_close(Y, Yref, B, f"fmt={fmt} M={M} N={N} K={K}")
