@@ -727,15 +727,16 @@ __global__ void __launch_bounds__(kThreads, 1) gemm_tc_kernel(const __grid_const
         // [s*128/splits, (s+1)*128/splits) over the cluster in a fixed order through
         // distributed shared memory and stores them (deterministic, no global scratch)
         ptx::cluster_sync();
-        if (warp >= 2 && !*abort_flag) {
-            // one thread = 4 consecutive rows of one token: 16-byte remote loads and
+        if (!*abort_flag) {
+            ptx::griddep_wait();  // (the MMA warp has not waited yet)
+            // one thread of any warp = 4 consecutive rows of one token: 16-byte remote loads and
             // 16-byte coalesced stores to Y[m][n..n+3]
             const int rows = kBN / splits, r0 = split * rows, q4 = rows / 4;
             const uint32_t pbase = ptx::smem_u32(part);
             void* Y = p.Y[g];
             const int epi = p.epi;
             const bool vec = (N % 4) == 0;
-            for (int w = threadIdx.x - 64; w < q4 * T; w += kThreads - 64) {
+            for (int w = threadIdx.x; w < q4 * T; w += kThreads) {
                 const int c = w / q4, row = r0 + 4 * (w - c * q4);
                 const int m = m0 + c, n = n0 + row;
                 const uint32_t off = pbase + uint32_t(c * kBN + row) * 4u;
