@@ -647,8 +647,8 @@ bool launch_staged(const GroupRef& g, bool pdl, int* status, cudaStream_t s, cud
 // all in a fixed order: results are deterministic.
 //
 // A row tile is 16 rows of one matrix; a CTA walks row tiles blockIdx.x, + gridDim.x, ... Each of
-// its eight (or, for long rows that give an SM one tile, sixteen) warps takes every eighth
-// 256-k chunk of the tile's rows and streams its chunks through a ring of its own in shared memory
+// its eight warps (sixteen for long rows that give an SM one tile, two for many tiles of short rows)
+// takes every eighth 256-k chunk of the tile's rows and streams its chunks through a ring of its own in shared memory
 // with cp.async (whole 128-byte lines per row, XOR-swizzled 16-byte granules so that fragment loads
 // are conflict-free): no barrier between warps until a tile's sums are added. The first ring's
 // worth is issued before griddepcontrol.wait; the activations come by ordinary cached loads after.
@@ -816,7 +816,7 @@ template <int FMT, int NT, int NW, bool COMP>
 __global__ void __launch_bounds__(32 * NW, 16 / NW) gemv_tc_kernel(const __grid_constant__ TcParams p) {
     using St = TcStage<FMT>;
     constexpr int kTcStages = kTcDepth<FMT, NT, NW>;
-    constexpr int kBufs = NW == 8 ? 2 : 1;  // (sixteen warps: one tile per CTA)
+    constexpr int kBufs = NW < 16 ? 2 : 1;  // (sixteen warps: one tile per CTA)
     extern __shared__ __align__(128) uint8_t smem[];
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int g = lane >> 2, t = lane & 3;
@@ -961,7 +961,7 @@ __global__ void __launch_bounds__(32 * NW, 16 / NW) gemv_tc_kernel(const __grid_
             red[buf][warp][8 * nt + 2 * t + 1][ra + 8] = v[3];
         }
         __syncthreads();
-        const int m = threadIdx.x / kTcRows, r = threadIdx.x % kTcRows;
+        const int m = threadIdx.x / kTcRows, r = threadIdx.x % kTcRows;  // (two warps: up to four tokens)
         if (m < p.M && m < 8 * NT) {
             const int gm = tc_mat_of(p, tile), N = p.N[gm];
             const int n = (tile - p.tile0[gm]) * kTcRows + r;
@@ -1010,6 +1010,14 @@ cudaError_t launch_tc_fmt(const TcParams& p, int tiles, int sms, cudaStream_t s)
     // long rows whose tiles leave each SM at most one CTA: sixteen warps
     const bool wide = tiles <= sms && p.K > 8 * kTcBlocks * kQBlock;
     const int grid = std::min(tiles, 2 * sms);
+    // short rows have fewer chunks than eight warps, and the others idle: pairs of warps on four times as
+    // many CTAs once the tiles fill them (us, eight warps / two / the FFMA2 and mma.sync kernels that were here
+    // before: 32768 x 512 Q8_0 at M = 2 10.3 / 5.7 / 8.9, 32768 x 768 Q4_0 at M = 4 8.9 / 7.2 / 7.9, 16384 x
+    // 1536 Q4_0 at M = 4 7.2 / 5.5 / 6.5; from seven chunks on, or with fewer tiles, eight are faster: 16384 x 1792
+    // Q8_0 at M = 3 by 4 %, 8192 x 768 by 27 %)
+    const int chunks = (p.K + kTcBlocks * kQBlock - 1) / (kTcBlocks * kQBlock);
+    if (p.M <= 4 && tiles > (chunks <= 2 ? 2 : 6) * sms && chunks <= 6)
+        return launch_tc_one<FMT, 1, 2>(p, std::min(tiles, 8 * sms), s);
     // Many chunks per warp and up to four tokens (more had the GEMM's rounded operand, 1.7e-3): compensated
     // totals. In plain ones a warp's fp32 chain grows with K and its error passes that of the FFMA2 kernels, whose
     // 32 to 128 threads have shorter chains (relative to the norm of the result, 6 seeds, plain /

@@ -311,6 +311,22 @@ def test_tensor_core_gemv_at_one_token(cuda_device, fmt, N, K):
     test_tensor_core_gemv_has_exact_products(cuda_device, fmt, 1, N, K)
 
 
+# its two-warp instance: many tiles of short rows, one to six chunks (ragged, fewer than the two warps'),
+# a ragged last tile, just past the least number of tiles, several tiles per CTA
+TC_TWO_WARPS = [(2, 4881, 96), (4, 5003, 512), (3, 14610, 544), (4, 14600, 1536), (2, 32768, 1280)]
+
+
+@pytest.mark.parametrize("fmt", FMTS + [emb.EMB_Q6_0])
+@pytest.mark.parametrize("M,N,K", TC_TWO_WARPS)
+def test_tensor_core_gemv_two_warps(cuda_device, fmt, M, N, K):
+    if fmt == emb.EMB_Q6_0 and K % 64:
+        K += 32
+    kernel, args, _ = route(fmt, M, N, K)
+    if M > 2:  # (two tokens of short rows mostly take the register kernel)
+        assert kernel == "gemv_tc_kernel" and args[2] == 2
+    test_tensor_core_gemv_has_exact_products(cuda_device, fmt, M, N, K)
+
+
 @pytest.mark.parametrize("fmt", FMTS + [emb.EMB_Q6_0])
 def test_shapes_take_the_kernels_they_are_named_for(cuda_device, fmt):
     k64 = lambda K: K + 32 if fmt == emb.EMB_Q6_0 and K % 64 else K
