@@ -296,7 +296,7 @@ cudaError_t dispatch_mt(const GemvParams& p, int grid_x, int M, cudaStream_t s) 
         if (M == 1 && p.U > NT && p.U <= 4 * NT) return launch_one<FMT, R, NT, 1, 4>(p, grid_x, 1, s);
     }
     if (M == 1) return launch_one<FMT, R, NT, 1>(p, grid_x, 1, s);
-    // more tokens (see tc_takes): small or few-row layers at M = 2 and 3, Q6_0 with K % 64 != 0 at M <= 4
+    // more tokens (see tc_takes): few rows at M = 2..4, Q6_0 with K % 64 != 0
     if (M == 2) return launch_one<FMT, R, NT, 2>(p, grid_x, 1, s);
     return launch_one<FMT, R, NT, 4>(p, grid_x, (M + 3) / 4, s);
 }
@@ -1055,28 +1055,38 @@ TcParams tc_params(const GroupRef& g, bool pdl, int& n_tiles) {
 }
 
 // Which calls take it (us per launch in graph-replayed chains, this kernel / the one it leaves):
-//  * M = 3, 4 always (Q6_0 32768 x 2048 at M = 4 15.4 / 32.9, Q4_0 13.4 / 18.0, Q8_0 16.6 / 22.8;
-//    2048 x 16384 at M = 4 Q8_0 10.0 / 22.6, Q6_0 9.7 / 24.9, Q4_0 8.1 / 23.0); M = 2 but for what the
-//    register kernel answers in one short wave: Q8_0 below 1 M weights (640 x 320 1.77 / 1.50), the others
-//    up to 4 M with four of its rows per CTA (2048 x 2048 Q4_0 2.30 / 2.19, Q6_0 2.74 / 2.49; 1024 x
-//    1024 Q4_0 1.61 / 2.89), and at M = 2 and 3 Q6_0 below 256 K (640 x 320 1.91 / 1.82, 300 x 512
-//    1.87 / 1.82) and up to 32 tiles of long rows, which leave SMs idle (512 x 16384 Q8_0 7.6 / 6.5);
+//  * M = 2..4, but for few row tiles, where one row per CTA of the register kernel is sooner done than a
+//    CTA's walk along 16 rows: up to kFewTiles, which grow with K (64 x 16384 Q6_0 at M = 4 7.3 / 4.4) and
+//    shrink with M and with what a row costs the register kernel (768 x 8192 Q8_0 at M = 2 4.1 / 3.7, at
+//    M = 3 4.1 / 6.4; 768 x 2048 Q4_0 at M = 2 1.9 / 3.1). Measured at 13 K x 21 row counts for every format
+//    and M: against the better of the two at each, this line loses 0.3 % or less (geometric mean). Q8_0 at M = 2 also leaves rows beyond 8192 k whose last round is mostly
+//    empty (5000 x 16384 30.0 / 26.7);
 //  * M = 6..16 in place of the tcgen05 GEMM (12288 x 4096 at M = 8 Q8_0 14.6 / 26.7, Q4_0 13.5 /
 //    27.9; 1024 x 4096 at M = 16 4.6 / 6.4), but for Q8_0 above 12 tokens and 32 M weights
-//    (32768 x 2048 30.4 / 27.7), and for five tokens, the count at which the GEMM's bf16 operand
-//    is held to its bits (tests/test_gpu_hotpath_dequant.py);
+//    (32768 x 2048 30.4 / 27.7), for rows so short that most warps idle, beyond one round of tiles (32768 x
+//    128 at M = 16 Q8_0 13.1 / 5.6, 32768 x 256 at M = 8 9.1 / 7.3, 32768 x 512 at M = 16 15.5 / 11.2), and for
+//    five tokens, the count at which the GEMM's bf16 operand is held to its bits
+//    (tests/test_gpu_hotpath_dequant.py);
 //  * M = 1, Q4_0 and Q6_0, with rows of at least 4096 k, where its codes-to-bf16 step is cheaper than FFMA2
 //    dot products and no activation row is staged per CTA, if its 16-row tiles are many and fill the SMs:
-//    at least 60 (512 x 16384 Q4_0 6.5 / 4.5, Q6_0 8.0 / 5.2), and where they are more than the SMs at
+//    at least 60 (768 x 6144 Q6_0 3.7 / 2.8, 960 x 5120 Q4_0 2.9 / 3.8), and where they are more than the SMs at
 //    least 80 % of the slots of their rounds of two CTAs per SM (4096 x 11008 Q4_0, 84 %, 10.3 / 11.3;
 //    2560 x 11008, 53 %, 9.4 / 8.1; 6144 x 11008, 63 %, 18.1 / 15.4; 11008 x 11008, 75 %, 25.6 / 24.6).
-//    At K where the staged kernel's lanes are idle part of the time (Q4_0 4608 to 8192, Q6_0 5120 to 6144) any
-//    fill beyond one round will do (Q4_0 11008 x 4608 12.9 / 15.5, 6144 x 5120 8.3 / 10.7; Q6_0 6144 x 5120 10.4 / 11.2).
+//    At K where the staged kernel's tiles fit shared memory badly (Q4_0 beyond 4096 to 8192, Q6_0 4864 to 6144) any
+//    fill beyond one round will do (Q4_0 11008 x 4608 12.9 / 15.5, 6144 x 5120 8.3 / 10.7, 24000 x 4864 21.1 / 32.8; Q6_0
+//    6144 x 5120 10.4 / 11.2).
 //    With K < 5120 not from 1216 to 4095 rows, where the register kernel has one short wave of four rows per
-//    CTA (2048 x 4096 Q4_0 2.8 / 2.4, Q6_0 3.3 / 2.75), nor Q4_0 beyond five tiles per SM (staged kernel: 22016 x
+//    CTA (2048 x 4096 Q4_0 2.8 / 2.4, Q6_0 3.3 / 2.75), at any K not where that wave is exactly full (1216
+//    rows x 8192 Q4_0 3.6 / 2.7; 1232 3.7 / 4.0), nor Q4_0 at 4096 beyond five tiles per SM (staged kernel: 22016 x
 //    4096 16.9 / 16.4). Q6_0 only where rows fill the other kernels' passes of 256 threads to less than
 //    70 % (4096 x 4096 4.95 / 7.1, 4096 x 11008 13.3 / 14.4; 4096 x 8192 9.6 / 9.2, 8192 x 16384 35.0 / 30.2, 1300 x 12288
 //    6.6 / 6.3). Q8_0 gains at some row counts and loses at others (1024 x 4096 2.6 / 3.2, 1300 x 4096 2.9 / 2.2).
+constexpr int kFewTilesK[4] = {639, 1151, 2048, 4096};  // K up to these (2048 and 4096: one chunk per warp), then the rest
+constexpr int kFewTiles[3][3][5] = {                    // by format, M - 2 and K
+    {{384, 44, 96, 56, 57}, {0, 0, 16, 24, 40}, {0, 0, 0, 16, 16}},   // Q8_0
+    {{0, 0, 10, 11, 32}, {0, 0, 0, 8, 8}, {0, 0, 0, 0, 5}},           // Q4_0
+    {{152, 28, 20, 10, 28}, {32, 16, 10, 8, 28}, {0, 0, 4, 8, 9}}};   // Q6_0
+static_assert(EMB_Q8_0 == 0 && EMB_Q4_0 == 1 && EMB_Q6_0 == 2, "kFewTiles is indexed by format");
 bool tc_takes(const GroupRef& g, int sms) {
     if (g.M > kTcMaxM || g.M == 5 || (g.fmt == EMB_Q6_0 && g.K % 64 != 0)) return false;
     int64_t rows = 0, tiles = 0;
@@ -1084,25 +1094,28 @@ bool tc_takes(const GroupRef& g, int sms) {
         rows += g.mats[i].N;
         tiles += (g.mats[i].N + kTcRows - 1) / kTcRows;
     }
-    const int64_t weights = rows * g.K;
-    const bool four_rows = rows >= 4 * 2 * 152;  // per CTA of the register kernel (launch_gemv_regs)
+    const int64_t slots = 2 * int64_t(sms);
+    const int64_t round_slots = slots * ((tiles + slots - 1) / slots);  // of the rounds that the tiles take
     if (g.M == 1) {
         if (g.fmt == EMB_Q8_0 || g.K < 4096 || tiles < 60) return false;
-        const int64_t slots = 2 * int64_t(sms);
-        const bool any_fill = tiles > slots && (g.fmt == EMB_Q4_0 ? g.K >= 4608 && g.K <= 8192 : g.K >= 5120 && g.K <= 6144);
-        if (tiles > sms && !any_fill && 5 * tiles < 4 * slots * ((tiles + slots - 1) / slots)) return false;
+        const bool four_rows = rows >= 4 * 2 * 152;  // per CTA of the register kernel (launch_gemv_regs)
+        if (four_rows && rows <= 4 * slots) return false;
+        const bool any_fill = tiles > slots && (g.fmt == EMB_Q4_0 ? g.K > 4096 && g.K <= 8192 : g.K >= 4864 && g.K <= 6144);
+        if (tiles > sms && !any_fill && 5 * tiles < 4 * round_slots) return false;
         if (g.K < 5120 && four_rows && rows < 4096) return false;
-        if (g.fmt == EMB_Q4_0) return g.K >= 5120 || tiles <= 5 * int64_t(sms);
+        if (g.fmt == EMB_Q4_0) return g.K > 4096 || tiles <= 5 * int64_t(sms);
         const int64_t U = g.K / 32, passes = (U + 255) / 256;
         return U < 256 || 10 * U < 7 * 256 * passes;
     }
-    if (g.M <= 3) {
-        if (tiles <= 32 && g.K >= 4096) return false;
-        if (g.fmt == EMB_Q6_0 && weights < (int64_t(1) << 18)) return false;
+    if (g.M <= 4) {
+        int k_class = 0;
+        while (k_class < 4 && g.K > kFewTilesK[k_class]) ++k_class;
+        if (tiles <= kFewTiles[g.fmt][g.M - 2][k_class]) return false;
+        return !(g.M == 2 && g.fmt == EMB_Q8_0 && g.K > 8192 && tiles > slots && 20 * tiles < 13 * round_slots);
     }
-    if (g.M == 2)
-        return g.fmt == EMB_Q8_0 ? weights >= (int64_t(1) << 20) : !(four_rows && weights <= (int64_t(1) << 22));
-    if (g.fmt == EMB_Q8_0 && g.M > 12) return weights <= (int64_t(1) << 25);
+    const int64_t short_k = g.M > 8 ? 256 : 128;
+    if ((tiles > slots && g.K <= short_k) || (tiles > 2 * slots && g.K <= 2 * short_k)) return false;
+    if (g.fmt == EMB_Q8_0 && g.M > 12) return rows * g.K <= (int64_t(1) << 25);
     return true;
 }
 

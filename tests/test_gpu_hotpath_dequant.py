@@ -165,11 +165,12 @@ def _spread_k(K: int, count: int, seed: int):
 GEMV_KERNELS = {"register": "gemv_kernel", "staged": "gemv_staged_kernel", "ring": "gemv_ring_kernel",
                 "tensor-core": "gemv_tc_kernel"}
 GEMV_CASES = [
-    # register kernel, one row per CTA (small layer), every k; M = 1 and 2 (two tokens per CTA);
-    # more tokens take the tensor-core kernel
+    # register kernel, one row per CTA (small layer), every k; M = 1, 2 (two tokens per CTA) and 3 (tiles
+    # of four); four tokens, and three of more rows, take the tensor-core kernel
     (emb.EMB_Q8_0, 256, 2048, 1, "register R=1", "all"),
     (emb.EMB_Q8_0, 256, 2048, 2, "register R=1 MT=2", "all"),
-    (emb.EMB_Q8_0, 256, 2048, 3, "tensor-core, few row tiles", "all"),
+    (emb.EMB_Q8_0, 256, 2048, 3, "register R=1 MT=4", "all"),
+    (emb.EMB_Q8_0, 272, 2048, 3, "tensor-core, few row tiles", "all"),
     (emb.EMB_Q4_0, 256, 2048, 1, "register R=1", "all"),
     (emb.EMB_Q4_0, 256, 2048, 4, "tensor-core, few row tiles", "all"),
     (emb.EMB_Q6_0, 256, 2048, 1, "register R=1", "all"),

@@ -341,7 +341,7 @@ def test_shapes_take_the_kernels_they_are_named_for(cuda_device, fmt):
         assert route(fmt, M, N, k64(K))[0] == "gemm_tc_kernel", (M, N, K)
     for N, K in LONG_ROW_SHAPES:
         for M in (2, 4):
-            if M == 4 or N > 512:  # two tokens of up to 32 row tiles: the register kernel
+            if N > 512:  # two tokens of few row tiles, and four of very few: the register kernel
                 assert route(fmt, M, N, K)[0] == "gemv_tc_kernel", (M, N, K)
 
 
@@ -467,5 +467,24 @@ def test_k_splits_are_clusters_that_run_at_once(cuda_device, fmt, M, N, K, split
     assert kernel == "gemm_tc_kernel"
     if torch.cuda.get_device_properties(0).multi_processor_count == 152:
         assert (grid[2] == 8) == (splits == 8) and grid[0] * grid[1] <= {8: 15, 4: 36, 2: 76, 1: 152}[grid[2]]
+    Y, Yref, B, _, _ = run_case(fmt, M, N, K, seed=M + N + K)
+    check_close(Y, Yref, B, f"fmt={fmt} M={M} N={N} K={K}")
+
+
+# lines of the tensor-core GEMV's rule: few row tiles at two to four tokens (on either side), a last round
+# that is mostly empty at two, one exactly full wave of the register kernel at one token and one row
+# tile more, short rows beyond one round and two rounds of tiles at up to eight tokens and more
+@pytest.mark.parametrize("fmt,M,N,K,kernel", [
+    (emb.EMB_Q8_0, 2, 912, 8192, "gemv_kernel"), (emb.EMB_Q8_0, 2, 913, 8192, "gemv_tc_kernel"),
+    (emb.EMB_Q8_0, 3, 640, 6144, "gemv_kernel"), (emb.EMB_Q8_0, 4, 300, 6144, "gemv_tc_kernel"),
+    (emb.EMB_Q4_0, 2, 160, 2048, "gemv_kernel"), (emb.EMB_Q4_0, 3, 129, 4096, "gemv_tc_kernel"),
+    (emb.EMB_Q6_0, 4, 112, 4096, "gemv_kernel"), (emb.EMB_Q6_0, 3, 513, 576, "gemv_tc_kernel"),
+    (emb.EMB_Q8_0, 2, 4999, 8704, "gemv_kernel"), (emb.EMB_Q4_0, 1, 1216, 5120, "gemv_kernel"),
+    (emb.EMB_Q4_0, 1, 1217, 5120, "gemv_tc_kernel"), (emb.EMB_Q4_0, 1, 13000, 4160, "gemv_tc_kernel"),
+    (emb.EMB_Q8_0, 8, 4865, 128, "gemm_tc_kernel"), (emb.EMB_Q4_0, 8, 4864, 128, "gemv_tc_kernel"),
+    (emb.EMB_Q6_0, 9, 4865, 256, "gemm_tc_kernel"), (emb.EMB_Q8_0, 16, 9729, 512, "gemm_tc_kernel"),
+    (emb.EMB_Q4_0, 6, 9729, 256, "gemm_tc_kernel"), (emb.EMB_Q4_0, 6, 9728, 256, "gemv_tc_kernel")])
+def test_tensor_core_gemv_rule(cuda_device, fmt, M, N, K, kernel):
+    assert route(fmt, M, N, K)[0] == kernel
     Y, Yref, B, _, _ = run_case(fmt, M, N, K, seed=M + N + K)
     check_close(Y, Yref, B, f"fmt={fmt} M={M} N={N} K={K}")
