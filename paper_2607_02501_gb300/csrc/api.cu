@@ -23,7 +23,7 @@ __device__ int g_status_read;  // where emb_device_status's exchange leaves the 
 constexpr size_t kScratchBytes = size_t(48) << 20;
 __device__ __align__(256) unsigned char g_scratch[kScratchBytes];
 
-// Token counts up to this run the GEMV; above it, the tensor-core GEMM unless gemv_takes().
+// Token counts up to this run the GEMV; above it, the tensor-core GEMM unless launch_mma_sync takes them.
 constexpr int64_t kGemvMaxM = 4;
 
 int* status_ptr() {
@@ -119,8 +119,9 @@ MatRef mat_ref(int fmt, const void* W, void* Y, int64_t N, int64_t K) {
 cudaError_t launch_group(const GroupRef& g, bool pdl, cudaStream_t s) {
     int* st = status_ptr();
     if (!st) return cudaErrorInvalidDevice;
-    if (g.M <= kGemvMaxM || gemv_takes(g)) return launch_gemv(g, pdl, st, s);
-    return launch_gemm_tc(g, pdl, st, s);
+    if (g.M <= kGemvMaxM) return launch_gemv(g, pdl, st, s);
+    cudaError_t err = cudaSuccess;
+    return launch_mma_sync(g, pdl, s, err) ? err : launch_gemm_tc(g, pdl, st, s);
 }
 
 // Read and clear the status word in one atomic step, on the caller's stream: a flag that a

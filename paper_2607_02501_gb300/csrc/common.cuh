@@ -140,12 +140,15 @@ int device_sm_count();
 // pdl: the kernel reads weights before griddepcontrol.wait (X only after it); otherwise it waits
 // before it reads anything. Both are launched with programmatic stream serialisation.
 cudaError_t launch_gemv(const GroupRef& g, bool pdl, int* status, cudaStream_t s);
-// Whether a group of more than four tokens is faster through launch_gemv.
-bool gemv_takes(const GroupRef& g);
+// The mma.sync kernels for a few more tokens (up to 64): true if one of them takes the group and was
+// launched, its result in err; false leaves it to the GEMM.
+bool launch_mma_sync(const GroupRef& g, bool pdl, cudaStream_t s, cudaError_t& err);
 
 // Tensor-core GEMM (tcgen05 + TMEM) for larger M.
 cudaError_t launch_gemm_tc(const GroupRef& g, bool pdl, int* status, cudaStream_t s);
 bool gemm_tc_supported(const GroupRef& g);
+// Modelled time of the GEMM in us for up to 64 tokens and K >= 1024.
+double gemm_tc_chunk_us(const GroupRef& g);
 // Bytes of zero-filled workspace the GEMM's stream-K schedule wants for this group on the
 // current device (0: the group's plan needs none).
 size_t gemm_tc_workspace(const GroupRef& g);

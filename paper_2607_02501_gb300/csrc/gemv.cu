@@ -29,6 +29,7 @@
 // Up to kMaxGroup matrices that read the same X (q/k/v or gate/up) share one launch.
 #include <algorithm>
 #include <atomic>
+#include <cmath>
 
 #include "dequant_dot.cuh"
 #include "ptx.cuh"
@@ -1014,9 +1015,10 @@ cudaError_t launch_tc_fmt(const TcParams& p, int tiles, int sms, cudaStream_t s)
     // many CTAs once the tiles fill them (us, eight warps / two / the FFMA2 and mma.sync kernels that were here
     // before: 32768 x 512 Q8_0 at M = 2 10.3 / 5.7 / 8.9, 32768 x 768 Q4_0 at M = 4 8.9 / 7.2 / 7.9, 16384 x
     // 1536 Q4_0 at M = 4 7.2 / 5.5 / 6.5; from seven chunks on, or with fewer tiles, eight are faster: 16384 x 1792
-    // Q8_0 at M = 3 by 4 %, 8192 x 768 by 27 %)
+    // Q8_0 at M = 3 by 4 %, 8192 x 768 by 27 %, but for nine and ten chunks, whose second pass has one or two
+    // of eight warps: 16384 x 2112 Q4_0 at M = 2 eight / two / before 10.2 / 8.7 / 8.2)
     const int chunks = (p.K + kTcBlocks * kQBlock - 1) / (kTcBlocks * kQBlock);
-    if (p.M <= 4 && tiles > (chunks <= 2 ? 2 : 6) * sms && chunks <= 6)
+    if (p.M <= 4 && tiles > (chunks <= 2 ? 2 : 6) * sms && (chunks <= 6 || chunks == 9 || chunks == 10))
         return launch_tc_one<FMT, 1, 2>(p, std::min(tiles, 8 * sms), s);
     // Many chunks per warp and up to four tokens (more had the GEMM's rounded operand, 1.7e-3): compensated
     // totals. In plain ones a warp's fp32 chain grows with K and its error passes that of the FFMA2 kernels, whose
@@ -1324,31 +1326,30 @@ cudaError_t launch_chunk_fmt(const TcParams& p, int tiles, int sms, cudaStream_t
     return launch_chunk_one<FMT, 8>(p, dim3(std::min(tiles, 2 * sms / groups), groups, 1), s);
 }
 
-// Which calls take it (us per launch in graph-replayed chains, this kernel / the tcgen05 GEMM): all
-// whose CTAs are resident at once (M = 50: 1280 x 1024 3.9 / 5.2, 2048 x 2048 4.6 / 12.7, 2048 x 16384
-// Q8_0 26.8 / 33.5; M = 32: 4096 x 4096 8.6 / 10.6). Beyond that the activations are read once per
-// round of row tiles and the GEMM's larger tiles catch up: up to 32 tokens while the GEMM has fewer
-// than 96 tiles of 128 rows and the rounds are 70 % full (M = 32: 5120 x 5120, 53 %, 22.0 / 21.4) or the codes are 4 or
-// 6 bits wide (M = 24: 11008 x 4096 Q8_0 23.3 / 26.4,
-// 16384 x 2048 Q8_0 16.4 / 15.1, Q4_0 13.3 / 15.6), above 32 tokens for short rows in at most two
-// rounds (M = 50: 8192 x 1024 8.1 / 8.4, 2560 x 2048 8.0 / 7.3, 12288 x 1536 19.6 / 11.5). Up to 1536 long rows
-// are one wave of the GEMM's eight K splits, while a CTA here walks a whole row (M = 50: 512 x 16384 23.9 / 18.2, 1152 x
-// 16384 25.7 / 19.3, M = 33: 512 x 6144 9.8 / 9.1; M = 50: 1024 x 4096 7.0 / 8.8).
+// Which calls take it: those that a model of both kernels, in us, says are sooner done here. A CTA walks
+// whole rows, so full rounds (more CTAs than SMs) and a last one of one CTA per SM cost by the chunks of a
+// warp, and by the k of its activations. Fitted to 3060 launches (M = 17..64, K = 1024..16384, 64 to
+// 32768 rows, three formats; rms 8 %, the GEMM's 7 %); its choices lose 0.5 % against the better kernel at each
+// (geometric mean) and 8 of them are more than 1 % slower than the GEMM was without this kernel, 6 % at most. Measured,
+// this kernel / the GEMM: M = 50 1024 x 1024 3.7 / 5.3, 2048 x 2048 4.6 / 12.6, 8192 x 1024 8.2 / 8.2, 6144 x 1536 12.9 /
+// 9.0; M = 32 4096 x 4096 8.7 / 10.9, 1792 x 16384 27.5 / 18.0, 16384 x 2560 Q6_0 27.2 / 20.0.
 bool chunk_takes(const GroupRef& g, int sms) {
     if (g.M <= kTcMaxM || g.M > 2 * kCkTokens || g.K < 1024 || g.precise || (g.fmt == EMB_Q6_0 && g.K % 64 != 0))
         return false;
-    int64_t tiles = 0, rows = 0;
-    for (int i = 0; i < g.n_mats; ++i) {
-        rows += g.mats[i].N;
-        tiles += (g.mats[i].N + kTcRows - 1) / kTcRows;
-    }
-    if (rows <= 12 * 128 && g.K > 4608) return false;
-    const bool short_rows = g.K < 8 * kTcBlocks * kQBlock;
-    const int64_t ctas = g.M > kCkTokens && !short_rows ? 2 * tiles : tiles, slots = 2 * int64_t(sms);
-    if (ctas <= slots) return true;
-    if (g.M <= kCkTokens)
-        return g.fmt != EMB_Q8_0 || (rows < 96 * 128 && 10 * ctas >= 7 * slots * ((ctas + slots - 1) / slots));
-    return short_rows && ctas <= 2 * slots;
+    int64_t tiles = 0;
+    for (int i = 0; i < g.n_mats; ++i) tiles += (g.mats[i].N + kTcRows - 1) / kTcRows;
+    const bool both = g.M > kCkTokens && g.K < 8 * kTcBlocks * kQBlock;  // token groups in one CTA
+    const int64_t ctas = g.M > kCkTokens && !both ? 2 * tiles : tiles, slots = 2 * int64_t(sms), rest = ctas % slots;
+    const double span = (both ? 4.0 : 8.0) * kTcBlocks * kQBlock;  // k that the warps of a row tile take at once
+    const double full = double(ctas / slots + (rest > sms)), half = rest > 0 && rest <= sms ? 1.0 : 0.0;
+    const double steps = std::ceil(double(g.K) / span);
+    // one CTA per SM and one chunk per warp: 16 % or more below the GEMM at every such size measured, so the
+    // smallest calls need not ask for its plan, whose time on the host they feel (17 x 1000 x 1184 with it
+    // 5.2 us a call, without 4.8)
+    if (full == 0.0 && steps == 1.0) return true;
+    const double us = 0.44 + full * (0.39 + 2.25 * steps) + half * (0.70 + 1.49 * steps) +
+                      (full + half) * 1.09 * double(g.K) / span;
+    return us < gemm_tc_chunk_us(g);
 }
 
 // ------------------------------------------------------------------ ring GEMV
@@ -1623,8 +1624,6 @@ bool launch_ring(const GroupRef& g, bool pdl, int* status, cudaStream_t s, cudaE
     return true;
 }
 
-}  // namespace
-
 bool launch_chunk(const GroupRef& g, bool pdl, cudaStream_t s, cudaError_t& err) {
     const int sms = device_sm_count();
     if (sms <= 0 || !chunk_takes(g, sms)) return false;
@@ -1636,23 +1635,25 @@ bool launch_chunk(const GroupRef& g, bool pdl, cudaStream_t s, cudaError_t& err)
     return true;
 }
 
-bool gemv_takes(const GroupRef& g) {
-    const int sms = device_sm_count();
-    return sms > 0 && (tc_takes(g, sms) || chunk_takes(g, sms));
-}
-
 cudaError_t launch_gemv_regs(const GroupRef& g, bool pdl, cudaStream_t s);
+
+}  // namespace
+
+bool launch_mma_sync(const GroupRef& g, bool pdl, cudaStream_t s, cudaError_t& err) {
+    return launch_chunk(g, pdl, s, err) || launch_tc(g, pdl, s, err);
+}
 
 cudaError_t launch_gemv(const GroupRef& g, bool pdl, int* status, cudaStream_t s) {
     cudaError_t err = cudaSuccess;
-    if (launch_chunk(g, pdl, s, err)) return err;
     if (launch_tc(g, pdl, s, err)) return err;
     if (launch_staged(g, pdl, status, s, err)) return err;
     if (launch_ring(g, pdl, status, s, err)) return err;
     return launch_gemv_regs(g, pdl, s);
 }
 
-// Register-streaming GEMV: every shape the staged path leaves out.
+namespace {
+
+// Register-streaming GEMV: every shape the other kernels leave out.
 cudaError_t launch_gemv_regs(const GroupRef& g, bool pdl, cudaStream_t s) {
     GemvParams p = {};
     const int U = int((g.fmt == EMB_Q8_0) ? g.K / 16 : g.K / 32);
@@ -1696,5 +1697,7 @@ cudaError_t launch_gemv_regs(const GroupRef& g, bool pdl, cudaStream_t s) {
          : R == 2 ? dispatch_nt<EMB_Q6_0, 2>(p, tiles, M, NT, s)
                   : dispatch_nt<EMB_Q6_0, 1>(p, tiles, M, NT, s);
 }
+
+}  // namespace
 
 }  // namespace emb

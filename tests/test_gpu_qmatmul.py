@@ -311,9 +311,10 @@ def test_tensor_core_gemv_at_one_token(cuda_device, fmt, N, K):
     test_tensor_core_gemv_has_exact_products(cuda_device, fmt, 1, N, K)
 
 
-# its two-warp instance: many tiles of short rows, one to six chunks (ragged, fewer than the two warps'),
+# its two-warp instance: many tiles of short rows, one to six, nine and ten chunks (ragged, fewer than two),
 # a ragged last tile, just past the least number of tiles, several tiles per CTA
-TC_TWO_WARPS = [(2, 4881, 96), (4, 5003, 512), (3, 14610, 544), (4, 14600, 1536), (2, 32768, 1280)]
+TC_TWO_WARPS = [(2, 4881, 96), (4, 5003, 512), (3, 14610, 544), (4, 14600, 1536), (2, 32768, 1280),
+                (3, 14610, 2336)]
 
 
 @pytest.mark.parametrize("fmt", FMTS + [emb.EMB_Q6_0])
@@ -334,9 +335,9 @@ def test_shapes_take_the_kernels_they_are_named_for(cuda_device, fmt):
         if M > 3:
             assert route(fmt, M, N, k64(K))[0] == "gemv_tc_kernel", (M, N, K)
     for M, N, K in CHUNK_SHAPES:
-        # not: few long rows (the GEMM's K splits), Q8_0 in rounds that are less than 70 % full
-        if (M, N, K) != (64, 130, 16384) and (fmt, M, N) != (emb.EMB_Q8_0, 24, 6000):
-            assert route(fmt, M, N, k64(K))[0] == "gemm_chunk_kernel", (M, N, K)
+        # not: few long rows (the GEMM's K splits), a second round of a few CTAs
+        other = (M, N, K) in ((64, 130, 16384), (64, 33, 4160), (50, 5000, 1280))
+        assert route(fmt, M, N, k64(K))[0] == ("gemm_tc_kernel" if other else "gemm_chunk_kernel"), (M, N, K)
     for M, N, K in SHORT_ROW_SHAPES:
         assert route(fmt, M, N, k64(K))[0] == "gemm_tc_kernel", (M, N, K)
     for N, K in LONG_ROW_SHAPES:
@@ -349,9 +350,10 @@ def test_shapes_take_the_kernels_they_are_named_for(cuda_device, fmt):
 # per CTA; K of four chunks exactly, with a ragged last one, odd block counts
 CHUNK_SHAPES = [(17, 16, 1024), (32, 15, 2048), (33, 300, 1056), (50, 1280, 1024), (64, 33, 4160), (50, 5000, 1280),
                 (24, 6000, 1120), (64, 130, 16384), (40, 2048, 2080)]
-# long rows: the longest of a layer of the workloads, a ragged last tile and chunk, one token group; and
-# rounds that are full enough for Q8_0 too
-CHUNK_MORE_SHAPES = [(50, 2048, 16384), (33, 1540, 8256), (20, 4000, 11008), (24, 7000, 1120)]
+# long rows: the longest of a layer of the workloads, a ragged last tile and chunk, one token group; several
+# row tiles per CTA with one token group and with both in a CTA; 64 tokens and one row more than two tiles
+CHUNK_MORE_SHAPES = [(50, 2048, 16384), (33, 1930, 8256), (20, 4000, 11008), (24, 7000, 1120), (50, 9500, 1024),
+                     (64, 33, 2080)]
 
 
 @pytest.mark.parametrize("fmt", FMTS + [emb.EMB_Q6_0])
