@@ -1061,7 +1061,8 @@ TcParams tc_params(const GroupRef& g, bool pdl, int& n_tiles) {
 //    CTA's walk along 16 rows: up to kFewTiles, which grow with K (64 x 16384 Q6_0 at M = 4 7.3 / 4.4) and
 //    shrink with M and with what a row costs the register kernel (768 x 8192 Q8_0 at M = 2 4.1 / 3.7, at
 //    M = 3 4.1 / 6.4; 768 x 2048 Q4_0 at M = 2 1.9 / 3.1). Measured at 13 K x 21 row counts for every format
-//    and M: against the better of the two at each, this line loses 0.3 % or less (geometric mean). Q8_0 at M = 2 also leaves rows beyond 8192 k whose last round is mostly
+//    and M: against the better of the two at each, this line loses 0.3 % or less (geometric mean). For gated
+//    layers, whose register kernel has two rows per CTA, at 11 K x 14 row counts (512 x 8192 Q6_0 at M = 2 4.4 / 2.7). Q8_0 at M = 2 also leaves rows beyond 8192 k whose last round is mostly
 //    empty (5000 x 16384 30.0 / 26.7);
 //  * M = 6..16 in place of the tcgen05 GEMM (12288 x 4096 at M = 8 Q8_0 14.6 / 26.7, Q4_0 13.5 /
 //    27.9; 1024 x 4096 at M = 16 4.6 / 6.4), but for Q8_0 above 12 tokens and 32 M weights
@@ -1084,10 +1085,13 @@ TcParams tc_params(const GroupRef& g, bool pdl, int& n_tiles) {
 //    70 % (4096 x 4096 4.95 / 7.1, 4096 x 11008 13.3 / 14.4; 4096 x 8192 9.6 / 9.2, 8192 x 16384 35.0 / 30.2, 1300 x 12288
 //    6.6 / 6.3). Q8_0 gains at some row counts and loses at others (1024 x 4096 2.6 / 3.2, 1300 x 4096 2.9 / 2.2).
 constexpr int kFewTilesK[4] = {639, 1151, 2048, 4096};  // K up to these (2048 and 4096: one chunk per warp), then the rest
-constexpr int kFewTiles[3][3][5] = {                    // by format, M - 2 and K
-    {{384, 44, 96, 56, 57}, {0, 0, 16, 24, 40}, {0, 0, 0, 16, 16}},   // Q8_0
-    {{0, 0, 10, 11, 32}, {0, 0, 0, 8, 8}, {0, 0, 0, 0, 5}},           // Q4_0
-    {{152, 28, 20, 10, 28}, {32, 16, 10, 8, 28}, {0, 0, 4, 8, 9}}};   // Q6_0
+constexpr int kFewTiles[2][3][3][5] = {                 // by gated or not, format, M - 2 and K
+    {{{384, 44, 96, 56, 57}, {0, 0, 16, 24, 40}, {0, 0, 0, 16, 16}},   // Q8_0
+     {{0, 0, 10, 11, 32}, {0, 0, 0, 8, 8}, {0, 0, 0, 0, 5}},           // Q4_0
+     {{152, 28, 20, 10, 28}, {32, 16, 10, 8, 28}, {0, 0, 4, 8, 9}}},   // Q6_0
+    {{{152, 48, 64, 57, 57}, {0, 8, 28, 32, 32}, {0, 0, 0, 32, 28}},
+     {{0, 0, 16, 20, 32}, {0, 0, 0, 10, 32}, {0, 0, 0, 4, 16}},
+     {{152, 60, 64, 48, 32}, {40, 20, 16, 16, 32}, {0, 0, 0, 8, 32}}}};
 static_assert(EMB_Q8_0 == 0 && EMB_Q4_0 == 1 && EMB_Q6_0 == 2, "kFewTiles is indexed by format");
 bool tc_takes(const GroupRef& g, int sms) {
     if (g.M > kTcMaxM || g.M == 5 || (g.fmt == EMB_Q6_0 && g.K % 64 != 0)) return false;
@@ -1112,7 +1116,7 @@ bool tc_takes(const GroupRef& g, int sms) {
     if (g.M <= 4) {
         int k_class = 0;
         while (k_class < 4 && g.K > kFewTilesK[k_class]) ++k_class;
-        if (tiles <= kFewTiles[g.fmt][g.M - 2][k_class]) return false;
+        if (tiles <= kFewTiles[g.epi >= EMB_EPI_GEGLU][g.fmt][g.M - 2][k_class]) return false;
         return !(g.M == 2 && g.fmt == EMB_Q8_0 && g.K > 8192 && tiles > slots && 20 * tiles < 13 * round_slots);
     }
     const int64_t short_k = g.M > 8 ? 256 : 128;

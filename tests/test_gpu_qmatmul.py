@@ -490,3 +490,17 @@ def test_tensor_core_gemv_rule(cuda_device, fmt, M, N, K, kernel):
     assert route(fmt, M, N, K)[0] == kernel
     Y, Yref, B, _, _ = run_case(fmt, M, N, K, seed=M + N + K)
     check_close(Y, Yref, B, f"fmt={fmt} M={M} N={N} K={K}")
+
+
+# gated layers, two rows per CTA of the register kernel, have lines of their own
+@pytest.mark.parametrize("fmt,M,N,K,kernel", [
+    (emb.EMB_Q6_0, 2, 512, 8192, "gemv_kernel"), (emb.EMB_Q6_0, 2, 514, 8192, "gemv_tc_kernel"),
+    (emb.EMB_Q8_0, 4, 512, 4096, "gemv_kernel"), (emb.EMB_Q8_0, 3, 130, 1024, "gemv_tc_kernel"),
+    (emb.EMB_Q4_0, 3, 160, 2080, "gemv_kernel"), (emb.EMB_Q4_0, 3, 162, 2080, "gemv_tc_kernel")])
+def test_tensor_core_gemv_rule_gated(cuda_device, fmt, M, N, K, kernel):
+    assert route(fmt, M, N, K, emb.EMB_EPI_SWIGLU)[0] == kernel
+    W, Xb = weight_np(N, K, M + N + K), activation_bits_np(M, K, M + N + K + 1)
+    img, Y = emb.quantize(fmt, torch.from_numpy(W).cuda()), torch.empty(M, N // 2, dtype=torch.bfloat16, device="cuda")
+    emb.emb_qlayer_seq([(fmt, img, N, K, to_dev_bf16(Xb), Y, emb.EMB_EPI_SWIGLU)], M)
+    ref, bound = oracle.epilogue_reference(oracle.EPI_SWIGLU, *oracle.qmatmul(fmt, oracle.quantize(fmt, W), Xb, N, K))
+    assert (np.abs(Y.float().cpu().numpy().astype(np.float64) - ref) <= bound).all()
