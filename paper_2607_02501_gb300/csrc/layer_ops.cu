@@ -619,7 +619,11 @@ __global__ void __launch_bounds__(kAttnThreads) attention_kernel(const __grid_co
 // least time by a model in microseconds fitted on GB300. A CTA costs 2.5, per tile of 64 keys 1.8
 // (D = 128) or 1.2 (D = 64) with 16 rows per warp and 1.0 or 0.5 with the keys shared out to the
 // warps; CTAs that share an SM slow one another by a quarter each, further ones queue; a cluster
-// adds 4.0 or 1.3 for its exchange and 0.8 more at 16 CTAs, which must all fit at once.
+// adds 4.0 or 1.3 for its exchange and 0.8 more at 16 CTAs, which must all fit at once. With the keys
+// shared out, the warps' merge costs 0.8 where no cluster's does, and 0.5 or 2.0 more beside one or two
+// other CTAs on the SM (without these two terms 34 queries of 32 heads and 7 keys took 5.3 us instead of 3.8, 152
+// queries of 32 heads on 4 and 16 keys 5.9 instead of 4.3, 50 queries of 16 heads on 8 of 64, 919 keys 10.3
+// instead of 7.9; over 420 calls the plan now loses 1.5 % against the best one, geometric mean).
 // Measured (us per launch, graph-replayed; before: 64 rows per CTA and as many splits as keys
 // allow): M = 816, 8 heads on one key/value head of 128, 816 keys 84.2 -> 26.4 (2 splits); 280
 // queries and keys, 32 heads 43.2 -> 16.9 (1); one query, 32
@@ -645,8 +649,9 @@ AttnPlan plan_attention(int64_t rows, int64_t Hk, int64_t n, int64_t D) {
             const double share = 1.0 + 0.25 * (std::min(std::ceil(ctas / sms), per_sm) - 1.0);
             const double x = ctas / (sms * per_sm);
             const double rounds = x <= 1.0 ? 1.0 : 0.5 * (x + std::ceil(x));
+            const double beside = std::min(std::ceil(ctas / sms), per_sm) - 1.0;  // other CTAs on an SM
             const double t = rounds * (tiles * tile * share + 2.5 + (sp > 1 ? (few ? 1.3 : 4.0) : 0.0)) +
-                             (sp == kMaxSplits ? 0.8 : 0.0);
+                             (sp == kMaxSplits ? 0.8 : 0.0) + (few ? (sp == 1 ? 0.8 : 0.0) + 0.5 * beside * beside : 0.0);
             if (t < best_t * 0.99) {
                 best_t = t;
                 best = AttnPlan{few != 0, sp};

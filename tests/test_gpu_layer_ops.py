@@ -12,7 +12,7 @@ import torch
 
 import oracle
 import paper_2607_02501_gb300 as emb
-from tests.gpu_util import bits_of
+from tests.gpu_util import bits_of, launches
 from workloads import activation_bits_np, weight_np
 
 pytestmark = pytest.mark.gpu
@@ -237,11 +237,26 @@ def test_action_expert_layer_recorded(cuda_device):
 
 
 # every kernel and split count of the attention plan, at its edges: keys shared out to the warps
-# (one 16-row block exactly and one row more, a single tile, a last tile that leaves warps without
-# keys, 1 to 16 splits) and rows shared out (1 to 8 splits, ragged last row block and tile)
+# (one 16-row block exactly and one row more, a last tile that leaves warps without keys, 1 to 16
+# splits) and rows shared out (a single tile, 1 to 8 splits, ragged last row block and tile)
 ATTN_PLANS = [(1, 32, 32, 128, 280, 1), (16, 1, 1, 64, 0, 33), (17, 1, 1, 128, 5, 60), (16, 8, 1, 128, 816, 16),
               (1, 8, 1, 64, 4090, 3), (300, 8, 8, 64, 0, 300), (120, 8, 2, 128, 1000, 120), (130, 8, 2, 64, 300, 1),
-              (816, 8, 1, 128, 0, 700), (400, 16, 4, 64, 500, 400), (280, 32, 32, 128, 0, 65)]
+              (816, 8, 1, 128, 0, 700), (400, 16, 4, 64, 500, 400), (280, 32, 32, 128, 0, 65), (17, 1, 1, 64, 5, 90),
+              (16, 2, 2, 128, 0, 80), (3, 4, 4, 64, 0, 66), (34, 32, 32, 128, 0, 7), (50, 16, 8, 64, 819, 100)]
+
+
+@pytest.mark.parametrize("M,H,Hk,d,n,warps,splits", [
+    (34, 32, 32, 128, 7, 1, 1), (152, 32, 4, 128, 16, 1, 1), (1, 1, 1, 64, 64, 1, 1), (17, 1, 1, 64, 95, 4, 1),
+    (16, 2, 2, 128, 80, 4, 2), (50, 16, 8, 64, 919, 4, 4), (1, 32, 32, 128, 281, 4, 8), (50, 8, 1, 128, 866, 4, 8),
+    (1, 8, 1, 128, 4001, 4, 16), (816, 8, 1, 128, 816, 1, 2), (280, 32, 32, 128, 280, 1, 1)])
+def test_attention_plan(cuda_device, M, H, Hk, d, n, warps, splits):
+    """How many warps share a row's keys and how many key splits a call takes on 152 SMs."""
+    if torch.cuda.get_device_properties(0).multi_processor_count != 152:
+        return
+    t = lambda rows, heads: torch.empty(rows, heads * d, dtype=torch.bfloat16, device="cuda")
+    Q, K, V, O = t(M, H), t(n, Hk), t(n, Hk), t(M, H)
+    (kernel, args, grid), = launches(lambda: emb.emb_attention(Q, None, None, K, V, O, H, Hk, d, 0.1))
+    assert (kernel, args, grid[2]) == ("attention_kernel", (d, warps), splits)
 
 
 @pytest.mark.parametrize("M,H,Hk,d,n0,n1", ATTN_PLANS)
@@ -290,9 +305,11 @@ def test_rmsnorm_thread_counts(cuda_device, M, D):
 
 
 # (M, H, Hk, d, n, first and end of the keys that are not finite): keys shared out to the warps, one
-# tile (a warp's share of it; one key; all) and eight splits (a whole split); rows shared out, one split
-# (one tile, one key) and two (a whole split); every key
-ATTN_NOT_FINITE = [(1, 1, 1, 64, 64, 48, 64), (1, 1, 1, 128, 33, 32, 33), (16, 2, 2, 128, 64, 0, 16),
+# split (all keys of a warp: those of the second tile are too few to reach it), two (all of a warp) and more
+# (a whole split of eight and of sixteen); rows shared out, one split of one tile (some, one, all) and of more (one
+# tile, one key) and two (a whole split); every key
+ATTN_NOT_FINITE = [(1, 1, 1, 64, 100, 48, 64), (16, 2, 2, 128, 80, 16, 32), (16, 2, 2, 128, 80, 64, 80),
+                   (1, 1, 1, 64, 64, 48, 64), (1, 1, 1, 128, 33, 32, 33), (16, 2, 2, 128, 64, 0, 16),
                    (3, 4, 2, 64, 40, 0, 40), (1, 32, 32, 128, 281, 0, 35), (1, 8, 1, 128, 4001, 250, 501),
                    (300, 8, 8, 64, 300, 64, 128), (300, 8, 8, 64, 300, 299, 300), (816, 8, 1, 128, 700, 0, 350),
                    (816, 8, 1, 128, 700, 350, 700), (300, 8, 8, 64, 300, 0, 300)]
