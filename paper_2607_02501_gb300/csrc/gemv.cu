@@ -1116,7 +1116,7 @@ bool tc_takes(const GroupRef& g, int sms) {
     if (g.M <= 4) {
         int k_class = 0;
         while (k_class < 4 && g.K > kFewTilesK[k_class]) ++k_class;
-        if (tiles <= kFewTiles[g.epi >= EMB_EPI_GEGLU][g.fmt][g.M - 2][k_class]) return false;
+        if (rows <= kTcRows * kFewTiles[g.epi >= EMB_EPI_GEGLU][g.fmt][g.M - 2][k_class]) return false;
         return !(g.M == 2 && g.fmt == EMB_Q8_0 && g.K > 8192 && tiles > slots && 20 * tiles < 13 * round_slots);
     }
     const int64_t short_k = g.M > 8 ? 256 : 128;

@@ -47,10 +47,12 @@ cudaError_t launch_pdl(const void* fn, dim3 grid, dim3 block, size_t smem, cudaS
 // rounded square root and reciprocal, then y = bf16(x * inv * gamma). Latency bounds it (0.3 MB at
 // 50 x 1024), so a thread loads its elements of x and gamma once, up to KEEP groups of each in
 // registers and gamma's loads on their way during the reduction, and one barrier is left: every
-// thread adds the warps' sums for itself. Few tokens take a thread per group, many take 256 threads,
-// so that all their CTAs are resident at once (512 threads: 816 x 2048 4.1 us).
-// Per launch, before (256 threads, x read twice, two barriers) and now, us: 50 x 1024 1.54 -> 1.23,
-// 1 x 4096 2.05 -> 1.75, 4 x 16384 4.71 -> 2.67, 816 x 2048 2.67 -> 2.48, 900 x 4096 3.59 -> 3.27.
+// thread adds the warps' sums for itself. A thread takes up to four groups before a CTA takes more
+// threads than 256 (a thread per group, us: 50 x 4096 2.44 instead of 1.41, 150 x 4096 2.85 instead of
+// 1.93), and many tokens take 256 throughout (512: 816 x 2048 4.1).
+// Per launch, before (256 threads, x read twice, two barriers) and now, us: 50 x 1024 1.49 -> 1.13,
+// 1 x 4096 2.00 -> 1.28, 50 x 4096 2.12 -> 1.41, 300 x 8192 4.64 -> 2.51, 816 x 2048 2.62 -> 2.46,
+// 816 x 8192 5.59 -> 5.82, 1200 x 8192 9.48 -> 6.75.
 
 // x is read with ordinary loads (not the read-only path): the previous launch wrote it
 // while this grid was already resident (programmatic dependent launch); its writes are
@@ -698,15 +700,21 @@ cudaError_t launch_rmsnorm(const float* x, const float* gamma, uint16_t* y, int6
     int Di = int(D);
     void* args[] = {&xa, &ga, &ya, &Di, &eps};
     const int groups = Di / 4;
-    const bool many = M > 304;  // more than two CTAs per SM
-    const int nt = groups <= 128 ? 128 : groups <= 256 || many ? 256 : groups <= 512 ? 512 : 1024;
-    const void* fn = nt == 128   ? reinterpret_cast<const void*>(rmsnorm_kernel<128, 1>)
-                     : nt == 512 ? reinterpret_cast<const void*>(rmsnorm_kernel<512, 1>)
-                     : nt == 256 ? (groups <= 256   ? reinterpret_cast<const void*>(rmsnorm_kernel<256, 1>)
-                                    : groups <= 512 ? reinterpret_cast<const void*>(rmsnorm_kernel<256, 2>)
-                                                    : reinterpret_cast<const void*>(rmsnorm_kernel<256, 4>))
-                     : groups <= 1024 ? reinterpret_cast<const void*>(rmsnorm_kernel<1024, 1>)
-                                      : reinterpret_cast<const void*>(rmsnorm_kernel<1024, 4>);
+    const int count = device_sm_count();
+    const int64_t sms = count > 0 ? count : 152;
+    const bool many = M > 2 * sms;
+    // longer rows than four groups per thread hold: 512 threads for few tokens, 1024 for up to one CTA per
+    // SM of the longest; for many, 256 that keep one group where those that keep four, five CTAs per SM at
+    // once, would leave their last wave more than a third empty (816 x 10240 8.0 instead of 6.7)
+    const int64_t at_once = 5 * sms, waves = (M + at_once - 1) / at_once;
+    const bool last_empty = waves > 1 && 3 * M < 2 * at_once * waves;
+    const int nt = groups <= 128 ? 128 : groups <= 1024 || many ? 256 : groups > 2048 && M <= sms ? 1024 : 512;
+    const void* fn = nt == 128    ? reinterpret_cast<const void*>(rmsnorm_kernel<128, 1>)
+                     : nt == 512  ? reinterpret_cast<const void*>(rmsnorm_kernel<512, 4>)
+                     : nt == 1024 ? reinterpret_cast<const void*>(rmsnorm_kernel<1024, 4>)
+                     : groups <= 256 || (groups > 1024 && last_empty) ? reinterpret_cast<const void*>(rmsnorm_kernel<256, 1>)
+                     : groups <= 512                                  ? reinterpret_cast<const void*>(rmsnorm_kernel<256, 2>)
+                                                                      : reinterpret_cast<const void*>(rmsnorm_kernel<256, 4>);
     return launch_pdl(fn, dim3(unsigned(M)), dim3(unsigned(nt)), 0, s, args);
 }
 

@@ -290,8 +290,9 @@ def test_rope_access_widths(cuda_device, M, H, Hk, d, pos0):
 
 
 # the thread counts and register shares of the norm: few and many tokens, rows around one, two and
-# four groups per thread, rows longer than a CTA keeps in registers
-@pytest.mark.parametrize("M,D", [(3, 512), (304, 520), (305, 1024), (400, 1032), (305, 2048), (320, 4104), (1, 2056),
+# four groups per thread, rows longer than a CTA keeps in registers, a mostly empty last wave
+@pytest.mark.parametrize("M,D", [(152, 8200), (153, 8200), (304, 16392), (760, 4104), (761, 4104), (761, 10248), (1100, 4104),
+                                 (3, 512), (304, 520), (305, 1024), (400, 1032), (305, 2048), (320, 4104), (1, 2056),
                                  (2, 4096), (5, 4104), (310, 16384), (2, 16392)])
 def test_rmsnorm_thread_counts(cuda_device, M, D):
     rng = np.random.default_rng(M + D)
