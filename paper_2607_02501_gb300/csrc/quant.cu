@@ -17,7 +17,7 @@ constexpr unsigned kFull = 0xffffffffu;
 
 // The packing kernels read 4 bytes per weight and write 0.56 to 1.06, so HBM bounds them as
 // long as enough loads are in flight and the arithmetic stays near a dozen instructions per
-// weight. A warp owns kPackBlocks = 32 consecutive blocks (4 KB of W, contiguous because rows
+// weight. A warp owns 8 * LOADS = 32 consecutive blocks (4 KB of W, contiguous because rows
 // are whole blocks): eight 16-byte loads per lane, all issued before the first use. Four lanes
 // share a block, lane s of them holding weights 4s .. 4s+3 and 16+4s .. 16+4s+3: the block's
 // extreme takes two shuffles, the per-block divisions are spread over eight weights a lane, and
@@ -26,7 +26,8 @@ constexpr unsigned kFull = 0xffffffffu;
 // Measured (GB300, 0.84 of the copy bandwidth): Q4_0 22016 x 4096 72.0 us (5.7 TB/s) against
 // 362.8 for one weight per lane behind a memset of the whole image; Q8_0 8000 x 4096 28.7 (was
 // 122), Q6_0 8000 x 4128 32.8 (was 165). Eight lanes per block instead of four: 95.8.
-constexpr int kPackBlocks = 32;
+// Matrices of up to 38912 blocks, which would leave SMs without a CTA, go 8 blocks to a warp (LOADS = 1):
+// Q4_0 508 x 32 3.9 -> 2.2 (2.7 with the memset), 1216 x 1024 3.3 -> 2.7.
 constexpr int kPackThreads = 256;
 
 // roundf(w / d) clamped to [lo, hi] for the four weights of v, plus `bias`, one per byte.
@@ -71,7 +72,7 @@ __device__ __forceinline__ float first_of(const float4 v, uint32_t top) {
                                                 : v.w;
 }
 
-template <int FMT>
+template <int FMT, int LOADS>
 __global__ void __launch_bounds__(kPackThreads) pack_kernel(const float* __restrict__ W, int64_t N, int64_t K,
                                                             uint8_t* __restrict__ codes,
                                                             uint8_t* __restrict__ high,
@@ -80,11 +81,11 @@ __global__ void __launch_bounds__(kPackThreads) pack_kernel(const float* __restr
     constexpr float kHi = FMT == EMB_Q8_0 ? 127.0f : FMT == EMB_Q4_0 ? 7.0f : 31.0f;
     constexpr float kDiv = FMT == EMB_Q8_0 ? 127.0f : kLo;
     constexpr uint32_t kBias = FMT == EMB_Q8_0 ? 0u : FMT == EMB_Q4_0 ? 0x08080808u : 0x20202020u;
-    constexpr int kLoads = kPackBlocks / 8;  // pairs of loads per lane
+    constexpr int kBlocks = 8 * LOADS;  // per warp, LOADS pairs of loads per lane
     const int lane = threadIdx.x & 31, sub = lane & 3;
     const int64_t nb = K / kQBlock, total = N * nb;
     const int64_t thread = int64_t(blockIdx.x) * kPackThreads + threadIdx.x;
-    const int64_t b0 = (thread >> 5) * kPackBlocks;  // first block of this warp
+    const int64_t b0 = (thread >> 5) * kBlocks;  // first block of this warp
     // padding bytes of the image (part of the format): between the planes, after each scale row
     if (blockIdx.x == 0) {
         const int64_t gap0 = L.codes_bytes, gap0_end = FMT == EMB_Q6_0 ? L.high_off : L.scales_off;
@@ -98,9 +99,9 @@ __global__ void __launch_bounds__(kPackThreads) pack_kernel(const float* __restr
             scales[(i / pad) * L.ldS + nb + i % pad] = __ushort_as_half(0);
     if (b0 >= total) return;
 
-    float4 v[kLoads][2];
+    float4 v[LOADS][2];
 #pragma unroll
-    for (int i = 0; i < kLoads; ++i) {
+    for (int i = 0; i < LOADS; ++i) {
         const int64_t b = b0 + 8 * i + (lane >> 2);
         const float4* src = reinterpret_cast<const float4*>(W + b * kQBlock) + sub;
         v[i][0] = b < total ? __ldcs(src) : make_float4(0, 0, 0, 0);
@@ -108,7 +109,7 @@ __global__ void __launch_bounds__(kPackThreads) pack_kernel(const float* __restr
     }
     __half mine = __ushort_as_half(0);  // the scale of block b0 + lane
 #pragma unroll
-    for (int i = 0; i < kLoads; ++i) {
+    for (int i = 0; i < LOADS; ++i) {
         const float4 lo = v[i][0], hi = v[i][1];
         const uint32_t top_lo = abs_max(lo), top_hi = abs_max(hi);
         uint32_t top = max(top_lo, top_hi);
@@ -157,7 +158,7 @@ __global__ void __launch_bounds__(kPackThreads) pack_kernel(const float* __restr
         }
     }
     const int64_t b = b0 + lane;
-    if (b < total) {
+    if (lane < kBlocks && b < total) {
         const int64_t n = pad ? b / nb : 0;
         scales[pad ? n * L.ldS + (b - n * nb) : b] = mine;
     }
@@ -210,24 +211,31 @@ int grid_for(int64_t items, int per_block) {
     return int(g < 1 ? 1 : g);
 }
 
+template <int LOADS>
+cudaError_t launch_pack(int fmt, const float* W, int64_t N, int64_t K, uint8_t* base, const Layout& L, cudaStream_t s) {
+    __half* scales = reinterpret_cast<__half*>(base + L.scales_off);
+    const int64_t per_cta = int64_t(8 * LOADS) * (kPackThreads / 32);
+    const int64_t ctas = (N * (K / kQBlock) + per_cta - 1) / per_cta;
+    if (ctas > int64_t(0x7fffffff)) return cudaErrorInvalidConfiguration;
+    const unsigned grid = unsigned(ctas);
+    if (fmt == EMB_Q8_0)
+        pack_kernel<EMB_Q8_0, LOADS><<<grid, kPackThreads, 0, s>>>(W, N, K, base, nullptr, scales, L);
+    else if (fmt == EMB_Q4_0)
+        pack_kernel<EMB_Q4_0, LOADS><<<grid, kPackThreads, 0, s>>>(W, N, K, base, nullptr, scales, L);
+    else
+        pack_kernel<EMB_Q6_0, LOADS><<<grid, kPackThreads, 0, s>>>(W, N, K, base, base + L.high_off, scales, L);
+    return cudaGetLastError();
+}
+
 }  // namespace
 
 cudaError_t launch_quantize(int fmt, const float* W, int64_t N, int64_t K, void* img,
                             cudaStream_t s) {
     const Layout L = layout_of(fmt, N, K);
     uint8_t* base = static_cast<uint8_t*>(img);
-    __half* scales = reinterpret_cast<__half*>(base + L.scales_off);
-    const int64_t per_cta = int64_t(kPackBlocks) * (kPackThreads / 32);
-    const int64_t ctas = (N * (K / kQBlock) + per_cta - 1) / per_cta;
-    const dim3 grid(unsigned(std::min<int64_t>(ctas, int64_t(0x7fffffff))));
-    if (ctas > int64_t(0x7fffffff)) return cudaErrorInvalidConfiguration;
-    if (fmt == EMB_Q8_0)
-        pack_kernel<EMB_Q8_0><<<grid, kPackThreads, 0, s>>>(W, N, K, base, nullptr, scales, L);
-    else if (fmt == EMB_Q4_0)
-        pack_kernel<EMB_Q4_0><<<grid, kPackThreads, 0, s>>>(W, N, K, base, nullptr, scales, L);
-    else
-        pack_kernel<EMB_Q6_0><<<grid, kPackThreads, 0, s>>>(W, N, K, base, base + L.high_off, scales, L);
-    return cudaGetLastError();
+    // fewer blocks per warp while those of 32 would leave SMs without a CTA (see the kernel)
+    return N * (K / kQBlock) <= int64_t(256) * 152 ? launch_pack<1>(fmt, W, N, K, base, L, s)
+                                                   : launch_pack<4>(fmt, W, N, K, base, L, s);
 }
 
 cudaError_t launch_dequant_f32(int fmt, const void* img, int64_t N, int64_t K, float* out,

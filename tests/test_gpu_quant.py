@@ -118,3 +118,11 @@ def test_pack_near_ties_and_padding(cuda_device, fmt, N, K):
     pack(torch.from_numpy(W).cuda(), N, K, out)
     diff = np.nonzero(out.cpu().numpy() != oracle.quantize(fmt, W))[0]
     assert diff.size == 0, f"{diff.size} bytes differ, first at {diff[:8]}"
+
+
+# the warps of 32 blocks that matrices above 38912 blocks take (those above: 8 blocks per warp): the first
+# size over the line, odd block counts, padded scale rows
+@pytest.mark.parametrize("fmt", [emb.EMB_Q8_0, emb.EMB_Q4_0, emb.EMB_Q6_0])
+@pytest.mark.parametrize("N,K", [(38913, 32), (1301, 1056), (304, 4096), (305, 4096)])
+def test_pack_near_ties_and_padding_many_blocks(cuda_device, fmt, N, K):
+    test_pack_near_ties_and_padding(cuda_device, fmt, N, K)
