@@ -525,8 +525,11 @@ def measure_workload(name, ws, args, dev, dist, steps, warmup, e2e_steps, clocks
                     "peak_source": f"{peaks['source']} HBM copy bandwidth"}
         roof["frac"] = roof["achieved"] / roof["peak"]
         roof["traffic"] = kernel_traffic(name, c["w"])
-        roof["kernel"] = ("GEMV (gemv_staged_kernel + gemv_ring_kernel + gemv_kernel + gemv_tc_kernel)" if c["w"].M <= 16
-                          else "gemm_chunk_kernel" if c["w"].M <= 64 else "gemm_tc_kernel") + f" <{wl.FMT_NAMES[c['w'].fmt]}>"
+        # the kernels that the library picks from at this token count
+        roof["kernel"] = ("GEMV (gemv_staged_kernel + gemv_ring_kernel + gemv_kernel + gemv_tc_kernel)" if c["w"].M <= 4
+                          else "gemv_tc_kernel / gemm_tc_kernel" if c["w"].M <= 16
+                          else "gemm_chunk_kernel / gemm_tc_kernel" if c["w"].M <= 64
+                          else "gemm_tc_kernel") + f" <{wl.FMT_NAMES[c['w'].fmt]}>"
         roof["launches_per_step"] = c["launches"] * c["w"].repeats
         roof["per_launch_us"] = per_launch_ms * 1e3
         return roof

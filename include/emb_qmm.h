@@ -126,9 +126,11 @@ EMB_API emb_status emb_quantize_q6_0(const float* W, int64_t N, int64_t K, void*
  * Y [M][N] fp32 = X [M][K] bf16  x  w'^T, w' the dequantised weights of W_blocks.
  * X, Y: device, 16-byte aligned; W_blocks as produced by emb_quantize_*.
  * Small M (M <= 4, action-token decode, and most layers up to M = 16, with the accuracy of
- * M <= 4) runs a weight-streaming GEMV that dequantises
- * in registers; larger M (action-chunk denoising, prefix prefill) runs a tcgen05
- * tensor-core GEMM that dequantises shared-memory tiles to bf16.
+ * M <= 4) runs a weight-streaming GEMV whose products are exact; larger M (action-chunk
+ * denoising, prefix prefill) runs a GEMM on weights rounded to bf16: a tcgen05 one that
+ * dequantises into tensor memory, or for M = 17..64 and K >= 1024, where it is sooner done, one
+ * on mma.sync that streams 16-row tiles. Which of the two never shows beyond the order
+ * of the fp32 sums.
  * Accuracy, per element, with Y_exact from the same dequantised weights w' and the
  * same bf16 X, and S = sum_k |w'[n][k] x[m][k]|:
  *   - M <= 4, or K < 1024:  |Y - Y_exact| <= 1e-3 * S + 1e-6 for every input (the GEMV's
@@ -334,7 +336,11 @@ EMB_API emb_status emb_rope_qk(uint16_t* q, int64_t n_q_heads, uint16_t* k, int6
  * the prefix cache (K0, V0: [n0][n_kv_heads][head_dim]) followed by the chunk's own keys
  * (K1, V1: [n1][n_kv_heads][head_dim]), all visible to every query (no mask). Query head h
  * (Q: [M][n_heads][head_dim]) reads key/value head h / (n_heads / n_kv_heads);
- * O[m][h] = sum_j softmax_j(scale * q.k_j) v_j, in fp32, one bf16 rounding.
+ * O[m][h] = sum_j softmax_j(scale * q.k_j) v_j, in fp32, one bf16 rounding. The scores are
+ * held in base 2 (scale * log2(e) rounded to fp32 once, at most 2^-23 of a score), the weights are
+ * powers of two by the hardware's approximation (relative error about 2^-22; below 2^-126 of
+ * the largest they are zero) and enter the value product as bf16 hi + lo (2^-16). A key whose score
+ * is NaN or +infinity makes its queries' outputs NaN; one of -infinity has weight zero.
  * All bf16, device, 16-byte aligned; K0/V0 may be NULL when n0 == 0, K1/V1 when n1 == 0.
  * n_heads % n_kv_heads == 0; head_dim 64 or 128 (else EMB_EUNSUPPORTED); n0 + n1 >= 1.
  * O may not overlap any input. Errors: EMB_EINVAL, EMB_EALIGN, EMB_EUNSUPPORTED, EMB_ECUDA. */

@@ -561,6 +561,7 @@ const char* emb_status_string(emb_status status) {
 
 const char* emb_build_info(void) {
     return "libembqmm: sm_103a; Q8_0/Q6_0/Q4_0; GEMV (M=1: staged/ring/register FFMA2, long rows and M<=16: mma.sync) + "
+           "chunk GEMM (M=17..64: mma.sync on 16-row tiles) + "
            "tcgen05 GEMM (larger M: TMA, dequant to bf16 A tiles in TMEM, TMEM accumulators; one tile, persistent, "
            "cluster split-K or stream-K schedules); "
            "recorded chains (CUDA graphs); RMSNorm, rotary embedding, grouped-head attention";

@@ -11,7 +11,7 @@
 //     tile of rows plus its activations into shared memory with cp.async.bulk, so many
 //     bytes are in flight per SM and the next layer's tiles load during this layer's
 //     tail (programmatic dependent launch);
-//   * the ring kernel (large Q8_0 layers with long rows at M = 1): activations in
+//   * the ring kernel (large Q8_0 and Q6_0 layers with long rows at M = 1): activations in
 //     registers, rows through a ring of bulk copies;
 //   * the register kernel (what is left: small layers, rows that the others do not take): one CTA
 //     owns R consecutive weight rows; its NT threads split K in 16-byte units (a Q8_0 unit is
@@ -644,7 +644,7 @@ bool launch_staged(const GroupRef& g, bool pdl, int* status, cudaStream_t s, cud
 // M > 8), so up to eight tokens cost what one does and the CUDA cores only turn codes into bf16:
 // codes are small integers, exact in bf16, and every product is exact in fp32. A 32-weight block
 // is two MMAs into one fragment, which is then scaled by the block's fp32 scale as in the plain
-// definition; two such sums alternate by block and are added at the end, the warps' sums pairwise,
+// definition; four such sums (two for M > 8) alternate by block and are added at the end, the warps' sums pairwise,
 // all in a fixed order: results are deterministic.
 //
 // A row tile is 16 rows of one matrix; a CTA walks row tiles blockIdx.x, + gridDim.x, ... Each of
