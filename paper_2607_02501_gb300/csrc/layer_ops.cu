@@ -54,11 +54,11 @@ cudaError_t launch_pdl(const void* fn, dim3 grid, dim3 block, size_t smem, cudaS
 // 1 x 4096 2.00 -> 1.28, 50 x 4096 2.12 -> 1.41, 300 x 8192 4.64 -> 2.51, 816 x 2048 2.62 -> 2.46,
 // 816 x 8192 5.59 -> 5.82, 1200 x 8192 9.48 -> 6.75.
 
-// x is read with ordinary loads (not the read-only path): the previous launch wrote it
-// while this grid was already resident (programmatic dependent launch); its writes are
+// x and gamma are read with ordinary loads (not the read-only path): the previous launch may have
+// written them while this grid was already resident (programmatic dependent launch); its writes are
 // visible to ordinary loads after griddepcontrol.wait.
 template <int NT, int KEEP>
-__global__ void __launch_bounds__(NT) rmsnorm_kernel(const float* x, const float* __restrict__ gamma,
+__global__ void __launch_bounds__(NT) rmsnorm_kernel(const float* x, const float* gamma,
                                                      __nv_bfloat16* __restrict__ y, int D, float eps) {
     ptx::griddep_launch_dependents();
     ptx::griddep_wait();  // x is the residual stream the previous launch wrote
