@@ -1333,15 +1333,18 @@ cudaError_t launch_chunk_fmt(const TcParams& p, int tiles, int sms, cudaStream_t
 // Which calls take it: those that a model of both kernels, in us, says are sooner done here. A CTA walks
 // whole rows, so full rounds (more CTAs than SMs) and a last one of one CTA per SM cost by the chunks of a
 // warp, and by the k of its activations. Fitted to 3060 launches (M = 17..64, K = 1024..16384, 64 to
-// 32768 rows, three formats; rms 8 %, the GEMM's 7 %); its choices lose 0.5 % against the better kernel at each
-// (geometric mean) and 8 of them are more than 1 % slower than the GEMM was without this kernel, 6 % at most. Measured,
+// 32768 rows, three formats; rms 8 %, the GEMM's 7 %); its choices lose 0.4 % against the better kernel at each
+// (geometric mean) and one of them is more than 1 % slower than the GEMM was without this kernel. Measured,
 // this kernel / the GEMM: M = 50 1024 x 1024 3.7 / 5.3, 2048 x 2048 4.6 / 12.6, 8192 x 1024 8.2 / 8.2, 6144 x 1536 12.9 /
 // 9.0; M = 32 4096 x 4096 8.7 / 10.9, 1792 x 16384 27.5 / 18.0, 16384 x 2560 Q6_0 27.2 / 20.0.
 bool chunk_takes(const GroupRef& g, int sms) {
     if (g.M <= kTcMaxM || g.M > 2 * kCkTokens || g.K < 1024 || g.precise || (g.fmt == EMB_Q6_0 && g.K % 64 != 0))
         return false;
-    int64_t tiles = 0;
-    for (int i = 0; i < g.n_mats; ++i) tiles += (g.mats[i].N + kTcRows - 1) / kTcRows;
+    int64_t tiles = 0, rows = 0;
+    for (int i = 0; i < g.n_mats; ++i) {
+        rows += g.mats[i].N;
+        tiles += (g.mats[i].N + kTcRows - 1) / kTcRows;
+    }
     const bool both = g.M > kCkTokens && g.K < 8 * kTcBlocks * kQBlock;  // token groups in one CTA
     const int64_t ctas = g.M > kCkTokens && !both ? 2 * tiles : tiles, slots = 2 * int64_t(sms), rest = ctas % slots;
     const double span = (both ? 4.0 : 8.0) * kTcBlocks * kQBlock;  // k that the warps of a row tile take at once
@@ -1351,8 +1354,10 @@ bool chunk_takes(const GroupRef& g, int sms) {
     // smallest calls need not ask for its plan, whose time on the host they feel (17 x 1000 x 1184 with it
     // 5.2 us a call, without 4.8)
     if (full == 0.0 && steps == 1.0) return true;
+    // (the products of up to 32 tokens do not hide the wider codes' way in)
+    const double codes = g.M > kCkTokens || g.fmt == EMB_Q4_0 ? 0.0 : g.fmt == EMB_Q8_0 ? 0.8e-7 : 0.4e-7;
     const double us = 0.44 + full * (0.39 + 2.25 * steps) + half * (0.70 + 1.49 * steps) +
-                      (full + half) * 1.09 * double(g.K) / span;
+                      (full + half) * 1.09 * double(g.K) / span + codes * double(rows) * double(g.K);
     return us < gemm_tc_chunk_us(g);
 }
 
