@@ -620,8 +620,8 @@ __global__ void __launch_bounds__(kAttnThreads) attention_kernel(const __grid_co
 // Which kernel (WK) and how many key splits (one cluster, a power of two) a call takes: the
 // least time by a model in microseconds fitted on GB300. A CTA costs 2.5, per tile of 64 keys 1.8
 // (D = 128) or 1.2 (D = 64) with 16 rows per warp and 1.0 or 0.5 with the keys shared out to the
-// warps; CTAs that share an SM slow one another by a quarter each, further ones queue; a cluster
-// adds 4.0 or 1.3 for its exchange and 0.8 more at 16 CTAs, which must all fit at once. With the keys
+// warps; CTAs that share an SM slow one another by a quarter each, clusters beyond those that run at
+// once queue; a cluster adds 4.0 or 1.3 for its exchange and 0.8 more at 16 CTAs. With the keys
 // shared out, the warps' merge costs 0.8 where no cluster's does, and 0.5 or 2.0 more beside one or two
 // other CTAs on the SM (without these two terms 34 queries of 32 heads and 7 keys took 5.3 us instead of 3.8, 152
 // queries of 32 heads on 4 and 16 keys 5.9 instead of 4.3, 50 queries of 16 heads on 8 of 64, 919 keys 10.3
@@ -635,21 +635,70 @@ struct AttnPlan {
     bool shared_keys;  // WK = 4
     int splits;
 };
-AttnPlan plan_attention(int64_t rows, int64_t Hk, int64_t n, int64_t D) {
+
+// The opt-in shared-memory size and cluster size are per-device function attributes. Clusters of 2^i CTAs
+// of the kernel that run at once are asked once per device: fewer than the CTAs that do, since a cluster
+// stays within a part of the chip (76 clusters of four in two rounds: 38 queries of 32 heads on 4, 3282 keys
+// 41.7 us, in 20 of eight 25.8).
+constexpr int kSplitKinds = 5;  // 1, 2, 4, 8, 16
+struct AttnResident {
+    int n[kSplitKinds];
+};
+template <int D, int WK>
+cudaError_t prepare_attention(AttnResident& at_once) {
+    static std::mutex mu;
+    static AttnResident known[64] = {};
+    int dev = 0;
+    cudaError_t e = cudaGetDevice(&dev);
+    if (e != cudaSuccess) return e;
+    std::lock_guard<std::mutex> lock(mu);
+    if (dev >= 0 && dev < 64 && known[dev].n[0]) {
+        at_once = known[dev];
+        return cudaSuccess;
+    }
+    auto* kernel = attention_kernel<D, WK>;
+    const int smem = int(sizeof(AttnSmem<D>));
+    e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+    if (e == cudaSuccess) e = cudaFuncSetAttribute(kernel, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
+    for (int i = 0; i < kSplitKinds && e == cudaSuccess; ++i) {
+        cudaLaunchConfig_t cfg = {};
+        cfg.gridDim = dim3(1, 1, 1u << i);
+        cfg.blockDim = dim3(kAttnThreads);
+        cfg.dynamicSmemBytes = size_t(smem);
+        cudaLaunchAttribute attr;
+        attr.id = cudaLaunchAttributeClusterDimension;
+        attr.val.clusterDim.x = 1;
+        attr.val.clusterDim.y = 1;
+        attr.val.clusterDim.z = 1u << i;
+        cfg.attrs = &attr;
+        cfg.numAttrs = 1;
+        e = cudaOccupancyMaxActiveClusters(&at_once.n[i], kernel, &cfg);
+        at_once.n[i] = std::max(1, at_once.n[i]);
+    }
+    if (e == cudaSuccess && dev >= 0 && dev < 64) known[dev] = at_once;
+    return e;
+}
+
+template <int D>
+cudaError_t plan_attention(int64_t rows, int64_t Hk, int64_t n, AttnPlan& best) {
     const int count = device_sm_count();
     const double sms = count > 0 ? count : 152.0;
     const double per_sm = D == 64 ? 3.0 : 2.0;
-    AttnPlan best{false, 1};
+    best = AttnPlan{false, 1};
     double best_t = 1e30;
     for (int few = 0; few < 2; ++few) {
+        AttnResident at_once;
+        const cudaError_t e = few ? prepare_attention<D, 4>(at_once) : prepare_attention<D, 1>(at_once);
+        if (e != cudaSuccess) return e;
         const double blocks = double((rows + (few ? 15 : 63)) / (few ? 16 : 64)) * double(Hk);
         const double tile = few ? (D == 64 ? 0.5 : 1.0) : (D == 64 ? 1.2 : 1.8);
-        for (int sp = 1; sp <= kMaxSplits && (sp == 1 || n >= sp * int64_t(kMinSplitKeys)); sp *= 2) {
+        for (int i = 0; i < kSplitKinds; ++i) {
+            const int sp = 1 << i;
+            if (sp > 1 && n < sp * int64_t(kMinSplitKeys)) break;
             const double ctas = blocks * sp;
-            if (sp == kMaxSplits && ctas > sms) break;
             const double tiles = double((((n + sp - 1) / sp) + kKeyTile - 1) / kKeyTile);
             const double share = 1.0 + 0.25 * (std::min(std::ceil(ctas / sms), per_sm) - 1.0);
-            const double x = ctas / (sms * per_sm);
+            const double x = blocks / double(at_once.n[i]);
             const double rounds = x <= 1.0 ? 1.0 : 0.5 * (x + std::ceil(x));
             const double beside = std::min(std::ceil(ctas / sms), per_sm) - 1.0;  // other CTAs on an SM
             const double t = rounds * (tiles * tile * share + 2.5 + (sp > 1 ? (few ? 1.3 : 4.0) : 0.0)) +
@@ -660,34 +709,25 @@ AttnPlan plan_attention(int64_t rows, int64_t Hk, int64_t n, int64_t D) {
             }
         }
     }
-    return best;
+    return cudaSuccess;
 }
 
 template <int D, int WK>
-cudaError_t launch_attention_d(const AttnParams& p, int splits, cudaStream_t s) {
-    const size_t smem = sizeof(AttnSmem<D>);
-    // the opt-in shared-memory size and cluster size are per-device function attributes
-    static std::mutex mu;
-    static bool attr_done[64] = {};
-    int dev = 0;
-    cudaError_t e = cudaGetDevice(&dev);
-    if (e != cudaSuccess) return e;
-    std::lock_guard<std::mutex> lock(mu);
-    if (dev < 0 || dev >= 64 || !attr_done[dev]) {
-        e = cudaFuncSetAttribute(attention_kernel<D, WK>, cudaFuncAttributeMaxDynamicSharedMemorySize, int(smem));
-        if (e != cudaSuccess) return e;
-        if (kMaxSplits > 8) {
-            e = cudaFuncSetAttribute(attention_kernel<D, WK>, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
-            if (e != cudaSuccess) return e;
-        }
-        if (dev >= 0 && dev < 64) attr_done[dev] = true;
-    }
+cudaError_t launch_attention_wk(const AttnParams& p, int splits, cudaStream_t s) {
     AttnParams pc = p;
     void* args[] = {&pc};
     const int64_t row_blocks = (int64_t(p.M) * (p.H / p.Hk) + kAttnRows<WK> - 1) / kAttnRows<WK>;
     return launch_pdl(reinterpret_cast<const void*>(attention_kernel<D, WK>),
                       dim3(unsigned(row_blocks), unsigned(p.Hk), unsigned(splits)), dim3(kAttnThreads),
-                      smem, s, args, unsigned(splits));
+                      sizeof(AttnSmem<D>), s, args, unsigned(splits));
+}
+
+template <int D>
+cudaError_t launch_attention_d(const AttnParams& p, cudaStream_t s) {
+    AttnPlan pl;
+    const cudaError_t e = plan_attention<D>(int64_t(p.M) * (p.H / p.Hk), p.Hk, p.n0 + p.n1, pl);
+    if (e != cudaSuccess) return e;
+    return pl.shared_keys ? launch_attention_wk<D, 4>(p, pl.splits, s) : launch_attention_wk<D, 1>(p, pl.splits, s);
 }
 
 }  // namespace
@@ -767,10 +807,7 @@ cudaError_t launch_attention(const uint16_t* Q, const uint16_t* K0, const uint16
     p.H = int(H);
     p.Hk = int(Hk);
     p.scale_log2 = float(double(scale) * 1.4426950408889634);
-    const AttnPlan pl = plan_attention(M * (H / Hk), Hk, n0 + n1, D);
-    if (pl.shared_keys)
-        return D == 64 ? launch_attention_d<64, 4>(p, pl.splits, s) : launch_attention_d<128, 4>(p, pl.splits, s);
-    return D == 64 ? launch_attention_d<64, 1>(p, pl.splits, s) : launch_attention_d<128, 1>(p, pl.splits, s);
+    return D == 64 ? launch_attention_d<64>(p, s) : launch_attention_d<128>(p, s);
 }
 
 }  // namespace emb

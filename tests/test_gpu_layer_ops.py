@@ -248,7 +248,7 @@ ATTN_PLANS = [(1, 32, 32, 128, 280, 1), (16, 1, 1, 64, 0, 33), (17, 1, 1, 128, 5
 @pytest.mark.parametrize("M,H,Hk,d,n,warps,splits", [
     (34, 32, 32, 128, 7, 1, 1), (152, 32, 4, 128, 16, 1, 1), (1, 1, 1, 64, 64, 1, 1), (17, 1, 1, 64, 95, 4, 1),
     (16, 2, 2, 128, 80, 4, 2), (50, 16, 8, 64, 919, 4, 4), (1, 32, 32, 128, 281, 4, 8), (50, 8, 1, 128, 866, 4, 8),
-    (1, 8, 1, 128, 4001, 4, 16), (816, 8, 1, 128, 816, 1, 2), (280, 32, 32, 128, 280, 1, 1)])
+    (1, 8, 1, 128, 4001, 4, 16), (38, 32, 4, 128, 3282, 1, 8), (24, 32, 4, 128, 4000, 1, 16), (816, 8, 1, 128, 816, 1, 2), (280, 32, 32, 128, 280, 1, 1)])
 def test_attention_plan(cuda_device, M, H, Hk, d, n, warps, splits):
     """How many warps share a row's keys and how many key splits a call takes on 152 SMs."""
     if torch.cuda.get_device_properties(0).multi_processor_count != 152:
