@@ -235,3 +235,38 @@ def test_weights_of_a_single_call_written_just_before_it(cuda_device, fmt, M, N,
     for r, y in enumerate(got):
         assert torch.equal(y.view(torch.int32), want[r % 2].view(torch.int32)), r
     assert emb.emb_device_status() == emb.EMB_OK
+
+
+@pytest.mark.parametrize("fmt,M", [(emb.EMB_Q8_0, 1), (emb.EMB_Q4_0, 4), (emb.EMB_Q6_0, 50), (emb.EMB_Q8_0, 280)])
+def test_weights_written_just_before_a_replay(cuda_device, fmt, M):
+    """As above for a recorded chain: a replay starts when the norm that writes both images has ended."""
+    N, K = 4096, 2048
+    gen = torch.Generator(device="cuda").manual_seed(3 * M + fmt)
+    rand = lambda *s: torch.randn(*s, generator=gen, device="cuda")
+    bytes_ = emb.empty_qweight(fmt, N, K).numel()
+    both = torch.zeros(2 * bytes_, dtype=torch.uint8, device="cuda")
+    imgs = [both[:bytes_], both[bytes_:]]
+    rows, D = _norm_rows(both.numel())
+    src, gamma = [rand(rows, D), rand(rows, D)], torch.ones(D, device="cuda")
+    out = both.view(torch.bfloat16).view(rows, D)
+    Xs, Ys = [rand(M, K).to(torch.bfloat16) for _ in imgs], [torch.empty(M, N, device="cuda") for _ in imgs]
+    chain = emb.RecordedChain([(fmt, img, N, K, X, Y) for img, X, Y in zip(imgs, Xs, Ys)], M)
+    want = []
+    for i in (0, 1):
+        emb.emb_rmsnorm(src[i], gamma, out, 1e-6)
+        torch.cuda.synchronize()
+        chain.launch()
+        torch.cuda.synchronize()
+        want.append([Y.clone() for Y in Ys])
+    assert not torch.equal(want[0][0], want[1][0]) and not torch.equal(want[0][1], want[1][1])
+    got = []
+    for r in range(16):
+        emb.emb_rmsnorm(src[r % 2], gamma, out, 1e-6)
+        chain.launch()
+        got.append([Y.clone() for Y in Ys])
+    torch.cuda.synchronize()
+    for r, ys in enumerate(got):
+        for y, w in zip(ys, want[r % 2]):
+            assert torch.equal(y.view(torch.int32), w.view(torch.int32)), r
+    chain.close()
+    assert emb.emb_device_status() == emb.EMB_OK
